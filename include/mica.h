@@ -185,7 +185,8 @@ typedef struct {
     uint64_t rev_occ_bytes;  /* their size (0 without them) */
     uint64_t rev_table_bytes; /* the reversed genome's q-mer table (bidirectional search; 0 without it) */
     uint32_t full_sa;        /* 1 if the whole suffix array, its inverse and the 2-bit text are resident */
-    uint64_t full_sa_bytes;  /* their size (0 without them) */
+    uint64_t full_sa_bytes;  /* their size (0 without them); beside each suffix array entry the index
+                                also keeps 4 bytes of the text before it, not counted here */
     uint32_t long_q;         /* q of the longer seed tables of G$ and G~$ the bidirectional search
                                 seeds from (built from the text with full_sa when log4 N + 1 exceeds
                                 kmer_q; at most 15); 0 without them */

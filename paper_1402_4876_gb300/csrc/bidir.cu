@@ -49,22 +49,20 @@
 #include <algorithm>
 #include <mutex>
 
-#include "search_common.cuh"
+#include "bidir_common.cuh"
 
 namespace mica {
 namespace {
 
 constexpr unsigned BFULL = 0xffffffffu;
 constexpr uint32_t BD_DEEP_MIN = 8192;      // entries of each per-warp overflow stack, at least
-constexpr uint32_t SCHEME_FREE = 7;         // the single scheme of reads shorter than k + 1
-constexpr uint32_t BD_BUDGET = 1u << 12;    // node expansions a task may take before it exports its nodes
-constexpr uint32_t BD_VERIFY_MIN = 12;      // matched bases of a one-row node before it is checked against the text
-constexpr uint32_t BD_VERIFY_LEFT = 8;      // ... when at least this many bases are left to match
-constexpr int VCAP = 128;                   // rows waiting for that check (the round choice and the room
-                                            // checks below keep it from overflowing)
-constexpr uint32_t BD_SPLIT_MAX = 8;        // an interval of at most this many rows is checked row by row
+constexpr uint32_t BD_BUDGET = 1u << 10;    // node expansions a task may take before it exports its nodes
+constexpr int VCAP = 64;                    // intervals waiting for that check ...
+constexpr int TCAP = 64;                    // ... and windows of their rows that pass the first look
+constexpr uint32_t BD_SPLIT_LEFT = 32;      // an interval of at most this many rows is checked row by row: while
+constexpr uint32_t BD_SPLIT_RIGHT = 8;      // bases are left to match on the left (the index keeps each row's), after
+constexpr uint32_t BD_RUN = 32;              // steps of a run (nodes whose rows all continue alike) in a round
 constexpr uint32_t BD_CHAIN = 16;           // extension steps a lane may take on one multi-row node in a round
-constexpr uint32_t NSLOT_MAX = 64;          // task slots per warp: 32 (one per lane) or 64 (two)
 constexpr uint32_t BD_ADMIT_LOW = 96;       // admit new tasks while fewer items are pending ...
 constexpr uint32_t BD_ADMIT_FREE = 16;      // ... and at least this many slots are free (or nothing is pending)
 
@@ -82,26 +80,6 @@ __device__ __forceinline__ uint32_t bm_d(uint32_t x) { return (x >> 24) & 3u; }
 __device__ __forceinline__ uint32_t bm_d0(uint32_t x) { return (x >> 26) & 3u; }
 __device__ __forceinline__ uint32_t bm_j(uint32_t x) { return (x >> 28) & 7u; }
 
-// piece boundaries of a pattern of m bases in p pieces
-__device__ __forceinline__ uint32_t bnd(uint32_t i, uint32_t m, uint32_t p) { return i * m / p; }
-
-// The boundaries bnd(0) .. bnd(4) of a task's pieces as 9-bit fields (fields
-// past p hold 511), computed once per task so that a node's scheme check
-// needs no division.
-__device__ __forceinline__ unsigned long long pack_bounds(uint32_t m, uint32_t p)
-{
-    unsigned long long v = 0;
-#pragma unroll
-    for (uint32_t i = 0; i <= 4; i++) v |= (unsigned long long)(i <= p ? bnd(i, m, p) : 511u) << (9 * i);
-    return v;
-}
-__device__ __forceinline__ uint32_t bound_at(unsigned long long v, uint32_t i) { return (uint32_t)(v >> (9 * i)) & 511u; }
-// the piece holding position pos: the boundaries 1..3 at or below it
-__device__ __forceinline__ uint32_t piece_at(unsigned long long v, uint32_t pos)
-{
-    return (pos >= bound_at(v, 1)) + (pos >= bound_at(v, 2)) + (pos >= bound_at(v, 3));
-}
-
 struct BidirArgs {
     IndexView ix;
     OccSide fwd, rev;
@@ -118,6 +96,7 @@ struct BidirArgs {
     // frontier rounds: mode 0 takes (read, strand) tasks, mode 1 the nodes
     // exported by the previous round (task t = 2 read + strand, l, lr, sz; meta)
     uint32_t mode;
+    const uint2 *list;   // mode 0: the tasks and schemes the sweep left; null: every task, every scheme
     const uint4 *fr_in;
     const uint32_t *fr_in_meta;
     uint4 *fr_out;
@@ -132,11 +111,12 @@ template <int SCAP, int NS>
 struct BdSmem {
     uint32_t ml[SCAP], mlr[SCAP], msz[SCAP], mm[SCAP];   // multi-row nodes
     uint32_t sl[SCAP], slr[SCAP], sm[SCAP];              // single-row nodes
-    uint32_t vl[VCAP], vm[VCAP];                         // rows to check against the text (row, meta)
+    uint32_t vl[VCAP], vz[VCAP], vm[VCAP];               // intervals to check row by row (row, rows, meta)
+    uint32_t tp[TCAP], tm[TCAP];                         // windows to check against the text (position, meta)
     uint32_t pat[NS][MAX_WORDS + 1];                  // pattern of each task slot
-    // task slot s: read id, info = m | k << 9 | minus << 11 | p << 12 | end of
-    // its scheme range << 15, next scheme to seed
-    uint32_t sread[NS], sinfo[NS], snext[NS];
+    // task slot s: read id, info = m | k << 9 | minus << 11 | p << 12, and the
+    // schemes still to seed as bits
+    uint32_t sread[NS], sinfo[NS], sleft[NS];
     int live[NS];                                     // nodes of each slot on the stacks
     uint32_t work[NS];                                // node expansions of each slot's task
     unsigned long long bounds[NS];                    // piece boundaries of each slot's pattern
@@ -251,24 +231,19 @@ __device__ __forceinline__ bool bd_allowed(uint32_t j, uint32_t a, uint32_t pos,
 
 // The text check of a one-row node: its pattern `pat` (m bases in p pieces
 // with boundaries `bnds`, scheme j, budget k) has P[A, B) matched at text
-// position t = SA[l].  Below a one-row node the tree is a single path, the
-// text around that occurrence (each row has one preceding and, in the
-// reversed genome's index, one following symbol), so the node has a leaf iff
-// the window G[t - A, t - A + m) lies inside G and meets the scheme: at most
+// position SA[l].  Below a one-row node the tree is a single path, the text
+// around that occurrence (each row has one preceding and, in the reversed
+// genome's index, one following symbol), so the node has a leaf iff the window
+// G[s0, s0 + m), s0 = SA[l] - A, lies inside G and meets the scheme: at most
 // k mismatches in all, none in piece j, at least one in each piece left of j
 // (the free scheme of short reads: the budget alone).  The window's mismatch
 // count goes to d, the text words read to words and the 32-byte sectors
 // they span to sectors.
-__device__ __forceinline__ bool bd_check_window(const uint32_t *__restrict__ text, uint64_t n, const uint32_t *pat,
-                                                uint32_t m, unsigned long long bnds, uint32_t j, uint32_t k,
-                                                uint32_t t, uint32_t A, uint32_t &d, uint32_t &words,
-                                                uint32_t &sectors)
+__device__ __forceinline__ bool bd_check_window(const uint32_t *__restrict__ text, const uint32_t *pat, uint32_t m,
+                                                unsigned long long bnds, uint32_t j, uint32_t k, uint32_t s0,
+                                                uint32_t &d, uint32_t &words, uint32_t &sectors)
 {
-    words = 0;
-    sectors = 0;
-    d = 0;
-    if (t < A || (uint64_t)(t - A) + m > n) return false;
-    const uint32_t s0 = t - A, w0 = s0 >> 4, sh = 2u * (s0 & 15u);
+    const uint32_t w0 = s0 >> 4, sh = 2u * (s0 & 15u);
     const uint32_t Wn = (m + 15) >> 4;
     const int b1 = (int)bound_at(bnds, 1), b2 = (int)bound_at(bnds, 2), b3 = (int)bound_at(bnds, 3);
     uint32_t tot = 0, c1 = 0, c2 = 0, c3 = 0;   // mismatches in all and before boundaries 1, 2, 3
@@ -489,12 +464,13 @@ __device__ __forceinline__ void bd_emit(const BidirArgs &a, uint32_t nleaf, cons
     }
 }
 
-// Rows for the text-check stack: each lane asks for `want` rows (0: none).
-// Lanes are taken in lane order while their rows fit in the stack's room (the
-// taken lanes form a prefix, so their rows lie contiguously from vtop); a
-// lane gets its first position in pos.  vtop grows by the rows taken.
-__device__ __forceinline__ bool bd_take_rows(uint32_t want, uint32_t &vtop, uint32_t &pos, int lane)
+// Entries for the row-check stack: each lane asks for `want` (0: none).
+// Lanes are taken in lane order while theirs fit in the stack's room (the
+// taken lanes form a prefix, so their entries lie contiguously from vtop); a
+// lane gets its first position in pos.  vtop grows by the entries taken.
+__device__ __forceinline__ bool bd_take_entries(uint32_t want, uint32_t &vtop, uint32_t &pos, int lane)
 {
+    if (!__any_sync(BFULL, want)) return false;
     uint32_t end = want;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -506,6 +482,19 @@ __device__ __forceinline__ bool bd_take_rows(uint32_t want, uint32_t &vtop, uint
     vtop += __reduce_max_sync(BFULL, ok ? end : 0u);
     return ok;
 }
+
+// The pattern's 16 bases before position A, as the index keeps a row's.
+__device__ __forceinline__ uint32_t pat_context(const uint32_t *pat, uint32_t A)
+{
+    if (A >= 16u) {
+        const uint32_t p = A - 16u;
+        return __funnelshift_r(pat[p >> 4], pat[(p >> 4) + 1], 2u * (p & 15u));
+    }
+    return A ? pat[0] << (2u * (16u - A)) : 0u;
+}
+
+// Rows an interval with P[a, b) matched may hold to be checked one by one.
+__device__ __forceinline__ uint32_t bd_split(uint32_t a) { return a ? BD_SPLIT_LEFT : BD_SPLIT_RIGHT; }
 
 template <int SCAP, int WARPS, int MINB, int NS>
 __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
@@ -534,13 +523,19 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         W.work[sl] = 0;
         W.sread[sl] = 0;
         W.sinfo[sl] = 0;
-        W.snext[sl] = 0;
+        W.sleft[sl] = 0;
     }
     unsigned used_lo = 0, used_hi = 0;   // slots holding a task (warp-uniform)
     uint32_t mbot = 0, mtop = 0, sbot = 0, stop = 0, dmt = 0, dst = 0;
-    uint32_t vtop = 0;   // nodes waiting for the text check: W.v*[0, vtop)
+    uint32_t vtop = 0, vrows = 0;   // intervals waiting to be checked row by row, W.v*[0, vtop), and their rows
+    uint32_t ttop = 0;              // windows waiting for the text check, W.t*[0, ttop)
     bool tasks_left = true;
-    // once the launch's task counter is spent, a task keeps an eighth of its
+    // tasks a warp takes at a time: no more than its part of the launch's.  What reaches
+    // this kernel after the sweep is a few thousand heavy trees, each a long chain of
+    // dependent steps: spread thinly over every warp the search kernels take 6.4 ms for a
+    // million reads of a 512 Mbp human-like genome, at eight times as many to a warp 8.7 ms
+    const uint32_t share = (uint32_t)max(1ull, min((unsigned long long)NS, ntasks / ((unsigned long long)gridDim.x * WARPS)));
+    // once the launch's task counter is spent, a task keeps a 32nd of its
     // budget: a warp left holding heavy trees hands them to the next round,
     // where every warp takes part, instead of working through them alone
     uint32_t budget = a.budget;
@@ -552,10 +547,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         // a slot frees once its nodes are gone and its schemes are seeded
         const uint32_t lane2 = TWO ? (uint32_t)lane + 32 : (uint32_t)lane;   // the lane's second slot
         bool u0 = (used_lo >> lane) & 1u, u1 = TWO && ((used_hi >> lane) & 1u);
-        const uint32_t i0 = W.sinfo[lane], i1 = W.sinfo[lane2];
-        const uint32_t n0 = W.snext[lane], n1 = W.snext[lane2];
-        if (u0 && W.live[lane] == 0 && n0 >= ((i0 >> 15) & 7u)) u0 = false;
-        if (u1 && W.live[lane2] == 0 && n1 >= ((i1 >> 15) & 7u)) u1 = false;
+        const uint32_t n0 = W.sleft[lane], n1 = W.sleft[lane2];
+        if (u0 && W.live[lane] == 0 && n0 == 0) u0 = false;
+        if (u1 && W.live[lane2] == 0 && n1 == 0) u1 = false;
         used_lo = __ballot_sync(BFULL, u0);
         used_hi = __ballot_sync(BFULL, u1);
         uint32_t mc = mtop - mbot, sc = stop - sbot;
@@ -572,17 +566,17 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         if ((iter & 63) == 63 && budget == a.budget) {
             int spent = 0;
             if (lane == 0) spent = *(volatile unsigned long long *)&ctl->task_head >= ntasks;
-            if (__shfl_sync(BFULL, spent, 0)) budget = max(a.budget >> 3, min(a.budget, 32u));
+            if (__shfl_sync(BFULL, spent, 0)) budget = max(a.budget >> 5, min(a.budget, 32u));
         }
         // ---- slots over their node budget hand their nodes to the next
         // round (one pass over both stacks), and their schemes not yet seeded
         // as seed items (size 0, the scheme in the meta word)
-        const bool over0 = u0 && W.work[lane] >= budget && (W.live[lane] > 0 || n0 < ((i0 >> 15) & 7u));
-        const bool over1 = u1 && W.work[lane2] >= budget && (W.live[lane2] > 0 || n1 < ((i1 >> 15) & 7u));
+        const bool over0 = u0 && W.work[lane] >= budget && (W.live[lane] > 0 || n0);
+        const bool over1 = u1 && W.work[lane2] >= budget && (W.live[lane2] > 0 || n1);
         const unsigned ex_lo = __ballot_sync(BFULL, over0), ex_hi = __ballot_sync(BFULL, over1);
         if (ex_lo | ex_hi) {
             const unsigned long long expm = (unsigned long long)ex_lo | ((unsigned long long)ex_hi << 32);
-            const uint32_t ns0 = over0 ? ((i0 >> 15) & 7u) - n0 : 0u, ns1 = over1 ? ((i1 >> 15) & 7u) - n1 : 0u;
+            const uint32_t ns0 = over0 ? __popc(n0) : 0u, ns1 = over1 ? __popc(n1) : 0u;
             uint32_t pre = ns0 + ns1;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -595,14 +589,15 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                 uint32_t base = 0;
                 if (lane == 0) base = atomicAdd(&ctl->fr_count, tot);
                 base = __shfl_sync(BFULL, base, 0);
-                for (uint32_t i = 0; i < ns0; i++)
-                    bd_export_one(a, base + pre + i, slot_task(W, lane), 0, 0, 0, bd_meta(0, 0, 0, 0, 0, n0 + i));
-                for (uint32_t i = 0; i < ns1; i++)
+                for (uint32_t i = 0, b = n0; i < ns0; i++, b &= b - 1)
+                    bd_export_one(a, base + pre + i, slot_task(W, lane), 0, 0, 0,
+                                  bd_meta(0, 0, 0, 0, 0, (uint32_t)__ffs(b) - 1));
+                for (uint32_t i = 0, b = n1; i < ns1; i++, b &= b - 1)
                     bd_export_one(a, base + pre + ns0 + i, slot_task(W, lane2), 0, 0, 0,
-                                  bd_meta(0, 0, 0, 0, 0, n1 + i));
+                                  bd_meta(0, 0, 0, 0, 0, (uint32_t)__ffs(b) - 1));
             }
-            if (over0) W.snext[lane] = (i0 >> 15) & 7u;
-            if (over1) W.snext[lane2] = (i1 >> 15) & 7u;
+            if (over0) W.sleft[lane] = 0;
+            if (over1) W.sleft[lane2] = 0;
             mtop = mbot + bd_export_stack<SCAP, NS, false, false>(W, a, nullptr, mbot, mtop, expm, lane);
             stop = sbot + bd_export_stack<SCAP, NS, true, false>(W, a, nullptr, sbot, stop, expm, lane);
             if (dmt) dmt = bd_export_stack<SCAP, NS, false, true>(W, a, deep_m, 0, dmt, expm, lane);
@@ -610,10 +605,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             if (over0) W.live[lane] = 0;   // their nodes are gone: the slots free above ...
             if (over1) W.live[lane2] = 0;
             __syncwarp();
-            // ... once the rows they have waiting for the text check are done: those stay here (a row
-            // split from an interval has no row of the reversed genome to travel with)
+            // ... once the rows and windows they have waiting are checked: those stay here (a row split
+            // from an interval has no row of the reversed genome to travel with)
             for (uint32_t e = (uint32_t)lane; e < vtop; e += 32) {
                 const uint32_t sl = bm_slot(W.vm[e]);
+                if ((expm >> sl) & 1ull) atomicAdd(&W.live[sl], 1);
+            }
+            for (uint32_t e = (uint32_t)lane; e < ttop; e += 32) {
+                const uint32_t sl = bm_slot(W.tm[e]);
                 if ((expm >> sl) & 1ull) atomicAdd(&W.live[sl], 1);
             }
             if (over0) W.work[lane] = 0;   // (so that this pass does not repeat while they wait)
@@ -621,10 +620,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             __syncwarp();
             continue;
         }
-        const bool av0 = u0 && n0 < ((i0 >> 15) & 7u), av1 = u1 && n1 < ((i1 >> 15) & 7u);
+        const bool av0 = u0 && n0, av1 = u1 && n1;
         const unsigned avail_lo = __ballot_sync(BFULL, av0), avail_hi = __ballot_sync(BFULL, av1);
         const uint32_t seeds_total = __popc(avail_lo) + __popc(avail_hi);
-        const uint32_t cnt = mc + sc + vtop;
+        const uint32_t cnt = mc + sc + vtop + ttop;
 
         // ---- admission of fresh tasks (or of the last round's exported nodes) into free slots
         const unsigned free_lo = ~used_lo, free_hi = TWO ? ~used_hi : 0u;
@@ -633,7 +632,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         const uint32_t room = a.mode == 1 ? (uint32_t)SCAP - max(mc, sc) : nfree;
         if (tasks_left && nfree != 0 && dmt + dst == 0 && cnt + seeds_total < BD_ADMIT_LOW &&
             (cnt + seeds_total == 0 || nfree >= BD_ADMIT_FREE) && room > 0) {
-            uint32_t want = min(nfree, room), got = 0;
+            uint32_t want = min(min(nfree, room), share), got = 0;
             unsigned long long t0 = 0;
             if (lane == 0) {
                 if (*(volatile unsigned long long *)&ctl->task_head < ntasks) {
@@ -659,6 +658,12 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                     if (!fr || jr >= got) continue;
                     unsigned long long t = t0 + jr;
                     uint32_t seed_j = 8;                   // 8: not a seed item
+                    uint32_t some = 0xfu;                  // the task's schemes to seed
+                    if (a.list) {                          // a task the sweep left, and its schemes
+                        const uint2 x = a.list[t];
+                        t = x.x;
+                        some = x.y;
+                    }
                     if (a.mode == 1) {                     // a node (or a scheme to seed) exported by the last round
                         it[h] = a.fr_in[t];
                         imeta[h] = a.fr_in_meta[t];
@@ -668,13 +673,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                     const uint32_t rid = (uint32_t)(t >> 1), minus = (uint32_t)(t & 1);
                     const uint32_t m = a.rd.len[rid], k = a.rd.k[rid];
                     const uint32_t p = m >= k + 1 ? k + 1 : 1u;
-                    const uint32_t nsch = m >= k + 1 ? p : 1u;
                     const bool given_up = a.mode == 1 && ((a.redo[rid >> 5] >> (rid & 31)) & 1u);
-                    // a seed item seeds its one scheme: the slot's scheme range is [j, j + 1)
-                    const uint32_t send = seed_j < 8 ? seed_j + 1 : nsch;
                     W.sread[sl] = rid;
-                    W.sinfo[sl] = m | (k << 9) | (minus << 11) | (p << 12) | (send << 15);
-                    W.snext[sl] = a.mode == 0 ? 0 : (seed_j < 8 && !given_up ? seed_j : send);
+                    W.sinfo[sl] = m | (k << 9) | (minus << 11) | (p << 12);
+                    // a seed item seeds its one scheme
+                    W.sleft[sl] = a.mode == 0 ? some & ((1u << p) - 1u) : (seed_j < 8 && !given_up ? 1u << seed_j : 0u);
                     // the node of a read already given up is not continued
                     push[h] = a.mode == 1 && seed_j == 8 && !given_up;
                     W.live[sl] = push[h] ? 1 : 0;
@@ -731,18 +734,20 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         }
         c_rounds++;
 
-        // (rounds other than the text check's run only while fewer than 32
-        // rows wait for it; they add rows only while those fit)
+        // (a look at waiting rows adds at most 32 windows: it runs only while fewer than 32 wait)
         int kind;
         const bool seed_room = mc + 32 <= (uint32_t)SCAP && sc + 32 <= (uint32_t)SCAP;
-        if (vtop >= 32) kind = 3;
+        if (ttop >= 32) kind = 3;
+        else if (vrows >= 32) kind = 4;
         else if (mc >= 32) kind = 0;
         else if (sc >= 32) kind = 1;
-        else if (seeds_total > 0 && seed_room && (seeds_total >= 32 || seeds_total >= max(max(mc, sc), vtop)))
+        else if (seeds_total > 0 && seed_room &&
+                 (seeds_total >= 32 || mc + sc < 32u))
             kind = 2;
-        else if (mc && mc >= sc && mc >= vtop) kind = 0;
-        else if (sc && sc >= vtop) kind = 1;
-        else if (vtop) kind = 3;
+        else if (mc) kind = 0;    // (a tree's steps follow one another: they do not wait for part-filled checks)
+        else if (sc) kind = 1;
+        else if (vtop) kind = 4;
+        else if (ttop) kind = 3;
         else kind = 2;
 
         if (kind == 2) {
@@ -759,10 +764,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             uint32_t l = 0, lr = 0, sz = 0, meta = 0;
             if (avail) {
                 const uint32_t m = info & 511u, k = (info >> 9) & 3u, p = (info >> 12) & 7u;
-                const uint32_t nsch = (info >> 15) & 7u;
-                const uint32_t j = W.snext[slot]++;
+                const uint32_t todo = W.sleft[slot], j = (uint32_t)__ffs(todo) - 1;
+                W.sleft[slot] = todo & (todo - 1);
                 const uint32_t *pat = W.pat[slot];
-                if (nsch == 1 && p == 1 && k > 0) {
+                if (p == 1 && k > 0) {
                     // a read shorter than k + 1 bases: the whole tree from the full interval
                     l = 0; lr = 0; sz = ix.rows;
                     meta = bd_meta(slot, m, m, 0, 0, SCHEME_FREE);
@@ -815,14 +820,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             uint32_t cl[4] = {l, 0, 0, 0}, cs[4] = {sz, 0, 0, 0}, cd[4] = {0, 0, 0, 0};
             bd_emit(a, leaf ? 1u : 0u, cl, cs, cd, leaf ? 1u : 0u, W.sread[slot], minus, lane);
             const bool single = sz == 1;
-            // a seed of a few rows, far enough in, goes straight to the text check row by row
+            // a seed of a few rows, far enough in, goes straight to the check row by row
             const uint32_t matched = bm_b(meta) - bm_a(meta);
-            const bool checkable = push && a.verify_min && sz <= BD_SPLIT_MAX && matched >= a.verify_min &&
+            const bool checkable = push && a.verify_min && sz <= bd_split(bm_a(meta)) && matched >= a.verify_min &&
                                    (info & 511u) - matched >= BD_VERIFY_LEFT;
             uint32_t vpos = 0;
-            const bool to_v = bd_take_rows(checkable ? sz : 0u, vtop, vpos, lane);
-            if (to_v)
-                for (uint32_t i = 0; i < sz; i++) { W.vl[vpos + i] = l + i; W.vm[vpos + i] = meta; }
+            const bool to_v = bd_take_entries(checkable ? 1u : 0u, vtop, vpos, lane);
+            if (to_v) { W.vl[vpos] = l; W.vz[vpos] = sz; W.vm[vpos] = meta; }
+            vrows += __reduce_add_sync(BFULL, to_v ? sz : 0u);
             const unsigned bm = __ballot_sync(BFULL, push && !single && !to_v),
                            bs = __ballot_sync(BFULL, push && single && !to_v);
             if (push && !single && !to_v) {
@@ -835,7 +840,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             }
             mtop += __popc(bm);
             stop += __popc(bs);
-            if (push) atomicAdd(&W.live[slot], to_v ? (int)sz : 1);
+            if (push) atomicAdd(&W.live[slot], 1);
         } else if (kind == 1) {
             // ---- single-row nodes: the one possible child is the row's symbol
             const uint32_t npop = min(sc, 32u);
@@ -857,8 +862,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             const bool checkable = has && a.verify_min && matched >= a.verify_min &&
                                    (info & 511u) - matched >= BD_VERIFY_LEFT;
             uint32_t vpos = 0;
-            const bool to_v = bd_take_rows(checkable ? 1u : 0u, vtop, vpos, lane);
-            if (to_v) { W.vl[vpos] = l; W.vm[vpos] = meta; }
+            const bool to_v = bd_take_entries(checkable ? 1u : 0u, vtop, vpos, lane);
+            if (to_v) { W.vl[vpos] = l; W.vz[vpos] = 1; W.vm[vpos] = meta; }
+            vrows += __popc(__ballot_sync(BFULL, to_v));
             const bool live_node = has && !to_v;
             if (live_node) atomicAdd(&W.work[slot], 1u);
             if (live_node) {
@@ -898,37 +904,83 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
             stop += __popc(bsm);
             if (live_node && !child) atomicAdd(&W.live[slot], -1);
         } else if (kind == 3) {
-            // ---- one-row nodes checked against the text: SA gives where the
-            // matched part lies, the text window decides the leaf, ISA its row
-            const uint32_t npop = min(vtop, 32u);
+            // ---- windows checked against the text; a leaf is the position itself (its row is
+            // looked up only where a cap's order needs it)
+            const uint32_t npop = min(ttop, 32u);
             const bool has = (uint32_t)lane < npop;
-            uint32_t l = 0, meta = 0;
+            uint32_t pos = 0, meta = 0;
             if (has) {
-                const uint32_t q = vtop - 1 - lane;
-                l = W.vl[q]; meta = W.vm[q];
+                const uint32_t q = ttop - 1 - lane;
+                pos = W.tp[q]; meta = W.tm[q];
             }
-            vtop -= npop;
+            ttop -= npop;
             __syncwarp();
             const uint32_t slot = bm_slot(meta);
             const uint32_t info = W.sinfo[slot];
             const uint32_t rid = W.sread[slot];
             bool leaf = false;
-            uint32_t row = 0, dn = 0;
+            uint32_t dn = 0;
             if (has) {
                 atomicAdd(&W.work[slot], 1u);
                 const uint32_t m = info & 511u, k = (info >> 9) & 3u;
-                const uint32_t t = __ldg(ix.sa_full + l);
                 uint32_t words = 0, sectors = 0;
-                leaf = bd_check_window(ix.text, ix.n, W.pat[slot], m, W.bounds[slot], bm_j(meta), k, t, bm_a(meta),
-                                       dn, words, sectors);
-                if (leaf) row = __ldg(ix.isa + (t - bm_a(meta)));
+                leaf = bd_check_window(ix.text, W.pat[slot], m, W.bounds[slot], bm_j(meta), k, pos, dn, words, sectors);
                 c_verify++;
-                c_vbytes += 4u + 4u * words + (leaf ? 4u : 0u);
-                c_vsect += 1u + sectors + (leaf ? 1u : 0u);
+                c_vbytes += 4u * words;
+                c_vsect += sectors;
             }
-            uint32_t cl[4] = {row, 0, 0, 0}, cs[4] = {1, 0, 0, 0}, cd[4] = {dn, 0, 0, 0};
+            uint32_t cl[4] = {pos, 0, 0, 0}, cs[4] = {1, 0, 0, 0}, cd[4] = {dn | IV_POS, 0, 0, 0};
             bd_emit(a, leaf ? 1u : 0u, cl, cs, cd, leaf ? 1u : 0u, rid, (info >> 11) & 1u, lane);
             if (has) atomicAdd(&W.live[slot], -1);
+        } else if (kind == 4) {
+            // ---- rows of the newest waiting intervals, 32 at a time: SA gives where the matched
+            // part lies, and a row whose left context already breaks the scheme (a difference in
+            // the exact piece, or more than the budget left) goes no further
+            const uint32_t ne = min(vtop, 32u), e = vtop - 1u - (uint32_t)lane;
+            uint32_t el = 0, sz = 0, em = 0;
+            if ((uint32_t)lane < ne) { el = W.vl[e]; sz = W.vz[e]; em = W.vm[e]; }
+            uint32_t incl = sz;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(BFULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t excl = incl - sz;
+            // row `lane` of the batch belongs to the last entry whose first row is not past it
+            const unsigned heads = __reduce_or_sync(BFULL, (sz && excl < 32u) ? 1u << excl : 0u);
+            const int src = __popc(heads & (0xffffffffu >> (31 - lane))) - 1;
+            const uint32_t take = min(vrows, 32u);
+            const uint32_t row = __shfl_sync(BFULL, el, src) + ((uint32_t)lane - __shfl_sync(BFULL, excl, src));
+            const uint32_t meta = __shfl_sync(BFULL, em, src);
+            const bool gone = sz && incl <= 32u;
+            if (gone) atomicAdd(&W.live[bm_slot(em)], -1);
+            if (sz && excl < 32u && incl > 32u) { W.vl[e] = el + (32u - excl); W.vz[e] = sz - (32u - excl); }
+            vtop -= __popc(__ballot_sync(BFULL, gone));
+            vrows -= take;
+            const uint32_t slot = bm_slot(meta);
+            bool stay = false;
+            uint32_t pos = 0;
+            if ((uint32_t)lane < take) {
+                const uint2 x = __ldg(ix.sa_ctx + row);
+                const uint32_t info = W.sinfo[slot], m = info & 511u, k = (info >> 9) & 3u, A = bm_a(meta), j = bm_j(meta);
+                pos = x.x - A;
+                uint32_t df = x.y ^ pat_context(W.pat[slot], A);
+                df = (df | (df >> 1)) & 0x55555555u;
+                if (A < 16u) df &= A ? ~0u << (2u * (16u - A)) : 0u;
+                const uint32_t aj = j == SCHEME_FREE ? 511u : bound_at(W.bounds[slot], j);
+                const uint32_t ex = A > aj ? min(16u, A - aj) : 0u;          // context bases in the exact piece
+                const bool exact = ex == 0 || (df >> (2u * (16u - ex))) == 0;
+                stay = x.x >= A && (uint64_t)pos + m <= ix.n && exact && __popc(df) + bm_d(meta) <= k;
+                c_vbytes += 8u;
+                c_vsect += (row & 3u) == 0 || lane == 0 || ((heads >> lane) & 1u);
+            }
+            const unsigned bal = __ballot_sync(BFULL, stay);
+            if (stay) {
+                const uint32_t q = ttop + __popc(bal & lt);
+                W.tp[q] = pos; W.tm[q] = meta;
+                atomicAdd(&W.live[slot], 1);
+            }
+            ttop += __popc(bal);
         } else {
             // ---- multi-row nodes: counts of all four symbols at both ends
             // A node whose one child left to push has several rows (a chain
@@ -952,23 +1004,76 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                 const uint32_t slot = bm_slot(meta);
                 const uint32_t info = W.sinfo[slot];
                 const uint32_t rid = W.sread[slot];
+                // ---- runs: while every row of a node has the same next symbol, the node has one
+                // child of the same size and the step is a count and a comparison
+                uint32_t ol[4] = {0, 0, 0, 0}, orr[4] = {0, 0, 0, 0};
+                bool run = has, back = false;                   // back: the node returns to the stack
+                const uint32_t others = (mtop - mbot) + (stop - sbot) + vrows + ttop + seeds_total;
+                for (uint32_t rs = 0;; rs++) {
+                    if (run) {
+                        const uint32_t A = bm_a(meta), B = bm_b(meta);
+                        const bool left = A > 0;
+                        const OccSide &sd = left ? a.fwd : a.rev;
+                        const uint32_t pl = left ? l : lr;      // interval on the side being extended
+                        c_blocks += occ_pair(sd, pl, pl + sz, ol, orr);
+                        c_nodes++;
+                        const uint32_t worked = atomicAdd(&W.work[slot], 1u) + 1u;
+                        uint32_t c = 4;
+#pragma unroll
+                        for (int x = 0; x < 4; x++)
+                            if (orr[x] - ol[x] == sz) c = x;
+                        const uint32_t pos = left ? A - 1 : B;
+                        const uint32_t nA = left ? pos : 0, nB = left ? B : pos + 1;
+                        // (an interval small enough for the text check goes there from the step below)
+                        run = c < 4 && !(nA == 0 && nB == (info & 511u)) && (sz > bd_split(A) || !a.verify_min);
+                        if (run) {
+                            const uint32_t cost = c != pat_base(W.pat[slot], pos) ? 1u : 0u;
+                            uint32_t d0n;
+                            if (bd_allowed(bm_j(meta), A, pos, W.bounds[slot], (info >> 9) & 3u, bm_d(meta),
+                                           bm_d0(meta), cost, d0n)) {
+                                const uint32_t start = side_C(sd, c) + (c == 0 ? ol[0] : c == 1 ? ol[1] : c == 2 ? ol[2] : ol[3]);
+                                if (left) l = start; else lr = start;
+                                meta = bd_meta(slot, nA, nB, bm_d(meta) + cost, d0n, bm_j(meta));
+                                back = worked >= budget;        // over its budget: exported from the stack
+                                run = !back;
+                            } else {
+                                run = false;                    // the only child breaks the scheme
+                                has = false;
+                                atomicAdd(&W.live[slot], -1);
+                            }
+                        }
+                    }
+                    const uint32_t nrun = __popc(__ballot_sync(BFULL, run));
+                    if (nrun == 0) break;
+                    // lanes that are done wait for the others only while that costs little
+                    if (rs + 1 >= BD_RUN || (nrun * 2 < __popc(__ballot_sync(BFULL, has)) && others >= 32u)) {
+                        back = back || run;
+                        break;
+                    }
+                }
+                const unsigned backs = __ballot_sync(BFULL, back);
+                if (backs) {
+                    // (they came from the stack: there is room)
+                    if (back) {
+                        const uint32_t q = (mtop + __popc(backs & lt)) & (SCAP - 1);
+                        W.ml[q] = l; W.mlr[q] = lr; W.msz[q] = sz; W.mm[q] = meta;
+                        has = false;
+                    }
+                    mtop += __popc(backs);
+                    __syncwarp();
+                }
                 uint32_t cl[4] = {0, 0, 0, 0}, clr[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0}, cd[4] = {0, 0, 0, 0};
                 uint32_t cmeta[4] = {0, 0, 0, 0};
                 uint32_t leafmask = 0, nodemask = 0;
                 uint32_t cmatched = 0, cleft = 0;                // the children's matched bases and bases to go
-                const bool live_node = has;
-                if (has) atomicAdd(&W.work[slot], 1u);
-                if (live_node) {
+                if (has) {
                     const uint32_t m = info & 511u, k = (info >> 9) & 3u;
                     const uint32_t A = bm_a(meta), B = bm_b(meta), d = bm_d(meta), d0 = bm_d0(meta), j = bm_j(meta);
                     const bool left = A > 0;
                     cmatched = B - A + 1;
                     cleft = m - cmatched;
                     const OccSide &sd = left ? a.fwd : a.rev;
-                    const uint32_t pl = left ? l : lr;          // interval on the side being extended
-                    uint32_t ol[4], orr[4];
-                    c_blocks += occ_pair(sd, pl, pl + sz, ol, orr);
-                    c_nodes++;
+                    const uint32_t pl = left ? l : lr;
                     const uint32_t pos = left ? A - 1 : B;
                     const uint32_t base = pat_base(W.pat[slot], pos);
                     const uint32_t nA = left ? pos : 0, nB = left ? B : pos + 1;
@@ -992,19 +1097,19 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                     }
                 }
                 bd_emit(a, (uint32_t)__popc(leafmask), cl, cs, cd, leafmask, rid, (info >> 11) & 1u, lane);
-                // children of a few rows, far enough in, go to the text check row by row
-                uint32_t smask = 0, want = 0;
+                // children of a few rows, far enough in, go to the check row by row
+                uint32_t smask = 0, want = 0, srows = 0;
                 if (a.verify_min && cmatched >= a.verify_min && cleft >= BD_VERIFY_LEFT) {
 #pragma unroll
                     for (int c = 0; c < 4; c++)
-                        if ((nodemask >> c & 1u) && cs[c] <= BD_SPLIT_MAX) { smask |= 1u << c; want += cs[c]; }
+                        if ((nodemask >> c & 1u) && cs[c] <= bd_split(bm_a(cmeta[c]))) { smask |= 1u << c; want++; srows += cs[c]; }
                 }
                 uint32_t vpos = 0;
-                if (!bd_take_rows(want, vtop, vpos, lane)) { smask = 0; want = 0; }
+                if (!bd_take_entries(want, vtop, vpos, lane)) { smask = 0; want = 0; srows = 0; }
+                vrows += __reduce_add_sync(BFULL, srows);
 #pragma unroll
                 for (int c = 0; c < 4; c++)
-                    if (smask >> c & 1u)
-                        for (uint32_t i = 0; i < cs[c]; i++) { W.vl[vpos] = cl[c] + i; W.vm[vpos] = cmeta[c]; vpos++; }
+                    if (smask >> c & 1u) { W.vl[vpos] = cl[c]; W.vz[vpos] = cs[c]; W.vm[vpos] = cmeta[c]; vpos++; }
                 nodemask &= ~smask;
                 bool cont = false;
                 uint32_t nl = 0, nlr = 0, nsz = 0, nmeta = 0;
@@ -1220,6 +1325,15 @@ constexpr int BD_GRAPH_ROUNDS = 8;   // frontier rounds a captured batch runs (m
 constexpr int BD_MAX_ROUNDS = 64;
 static uint64_t redo_bytes(uint64_t n) { return redo_bits_bytes(n) + std::max<uint64_t>(n, 1) * 4 + 16; }
 
+// The sweep goes before the kernel when its task list (8 bytes for each of 2n
+// tasks, in the frontier buffer that round 1 writes first) fits and its
+// seeds can be checked.
+static bool use_sweep(const mica_index *idx, uint64_t n)
+{
+    const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
+    return 2 * n <= frontier_cap(n) && vmin < 256 && sweep_available(idx, vmin);
+}
+
 // Reserve the bidirectional search's buffers for n reads; fills the control
 // block template and the grid.
 int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tmpl, int &grid)
@@ -1238,7 +1352,7 @@ int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tm
     // exported nodes: two rounds' buffers of (task, l, lr, sz) and meta
     if ((rc = dev_reserve(w.frontier, 2 * frontier_cap(n) * 20))) return rc;
     tmpl = SearchCtl{};
-    tmpl.ntasks = 2 * n;
+    tmpl.ntasks = use_sweep(idx, n) ? 0 : 2 * n;   // the sweep counts the tasks it leaves
     tmpl.iv_cap = w.iv_cap;
     return 0;
 }
@@ -1268,8 +1382,10 @@ static void bidir_args(const mica_index *idx, Workspace &w, const ReadsView &rd,
     ba.budget = idx->tuning.bidir_budget ? idx->tuning.bidir_budget : BD_BUDGET;
     ba.fr_cap = frontier_cap(rd.n);
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
-    ba.verify_min = (idx->view.sa_full && vmin < 256) ? vmin : 0u;
+    ba.verify_min = (idx->view.sa_ctx && vmin < 256) ? vmin : 0u;
+    ba.list = nullptr;
 }
+
 
 // Frontier buffer b (0 or 1): items, then meta words.
 static uint4 *frontier_items(Workspace &w, uint64_t n, int b)
@@ -1336,6 +1452,11 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         ba.fr_in_meta = nullptr;
         ba.fr_out = frontier_items(w, rd.n, 0);
         ba.fr_out_meta = frontier_meta(w, rd.n, 0);
+        if (use_sweep(idx, rd.n)) {
+            uint2 *list = (uint2 *)frontier_items(w, rd.n, 1);
+            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, list, s, launches)) return rc;
+            ba.list = list;
+        }
         if (int rc = check_vector_alignment(ba)) return rc;
         sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
         launches++;

@@ -721,7 +721,7 @@ void mica_index_free(mica_index *idx)
     dev_release(idx->rocc);
     dev_release(idx->rsuper);
     dev_release(idx->rtable);
-    dev_release(idx->sa_full);
+    dev_release(idx->sa_ctx);
     dev_release(idx->isa);
     dev_release(idx->text);
     dev_release(idx->ltable);

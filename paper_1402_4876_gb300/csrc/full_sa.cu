@@ -1,6 +1,12 @@
 // The whole suffix array, its inverse and the 2-bit text, kept on the device
 // when an index is built with full_sa (GB300's HBM holds them beside the
-// index: 8 (N + 1) + N / 4 bytes, 25 GB for a 3.1 Gbp genome).
+// index: 12 (N + 1) + N / 4 bytes, 38 GB for a 3.1 Gbp genome).
+//
+// Each suffix array entry lies beside the 16 bases before its suffix, so that
+// the rows of an interval, which are contiguous, can be told apart by what
+// precedes the matched bases in one streamed read: of the rows that a repeat
+// family's seed names, nearly all fail there, before their text (a random
+// 64-byte access each) is touched.
 //
 // With them the bidirectional search checks an interval of one row against
 // the text: the row's suffix starts where the matched substring of the
@@ -36,6 +42,28 @@ __global__ void k_isa_scatter(const uint32_t *__restrict__ sa, uint64_t rows, ui
 {
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < rows; j += (uint64_t)gridDim.x * blockDim.x)
         isa[sa[j]] = (uint32_t)j;
+}
+
+__global__ void k_row_contexts(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ text, uint64_t rows,
+                               uint2 *__restrict__ out)
+{
+    for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < rows; j += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t t = sa[j];
+        uint32_t c = 0;
+        if (t >= 16) {
+            const uint32_t p = t - 16, w = p >> 4;
+            c = __funnelshift_r(__ldg(text + w), __ldg(text + w + 1), 2u * (p & 15u));
+        } else if (t) {
+            c = __ldg(text) << (2u * (16u - t));
+        }
+        out[j] = make_uint2(t, c);
+    }
+}
+
+__global__ void k_sa_of(const uint2 *__restrict__ rows, uint64_t n, uint32_t *__restrict__ out)
+{
+    for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x)
+        out[j] = rows[j].x;
 }
 
 __global__ void k_pack_text(const uint8_t *__restrict__ codes, uint64_t n, uint64_t words, uint32_t *__restrict__ text)
@@ -190,22 +218,31 @@ uint64_t full_sa_bytes(uint64_t n) { return 8 * (n + 1) + 4 * full_sa_text_words
 
 void set_full_sa_view(mica_index *idx)
 {
-    idx->view.sa_full = idx->has_full_sa ? (const uint32_t *)idx->sa_full.p : nullptr;
+    idx->view.sa_ctx = idx->has_full_sa ? (const uint2 *)idx->sa_ctx.p : nullptr;
     idx->view.isa = idx->has_full_sa ? (const uint32_t *)idx->isa.p : nullptr;
     idx->view.text = idx->has_full_sa ? (const uint32_t *)idx->text.p : nullptr;
 }
 
-// At build time: takes the suffix array `sa` (rows entries) as the index's
-// own, scatters its inverse and packs the text from the 2-bit codes.
-int build_full_sa(mica_index *idx, DevBuf &sa, const uint8_t *d_codes, uint64_t n, cudaStream_t s)
+// The rows' suffix array entries and left contexts, from both arrays complete.
+static int build_row_contexts(mica_index *idx, const uint32_t *d_sa, uint64_t rows, cudaStream_t s)
+{
+    if (int rc = dev_reserve(idx->sa_ctx, rows * 8)) return rc;
+    k_row_contexts<<<grid_of(rows), 256, 0, s>>>(d_sa, (const uint32_t *)idx->text.p, rows, (uint2 *)idx->sa_ctx.p);
+    MICA_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
+// At build time: from the suffix array `sa` (rows entries) and the 2-bit
+// codes, its inverse, the packed text and the rows' contexts.
+int build_full_sa(mica_index *idx, const DevBuf &sa, const uint8_t *d_codes, uint64_t n, cudaStream_t s)
 {
     const uint64_t rows = n + 1, words = full_sa_text_words(n);
-    std::swap(idx->sa_full, sa);
     int rc;
     if ((rc = dev_reserve(idx->isa, rows * 4)) || (rc = dev_reserve(idx->text, words * 4))) return rc;
-    k_isa_scatter<<<grid_of(rows), 256, 0, s>>>((const uint32_t *)idx->sa_full.p, rows, (uint32_t *)idx->isa.p);
+    k_isa_scatter<<<grid_of(rows), 256, 0, s>>>((const uint32_t *)sa.p, rows, (uint32_t *)idx->isa.p);
     k_pack_text<<<grid_of(words), 256, 0, s>>>(d_codes, n, words, (uint32_t *)idx->text.p);
     MICA_CUDA_TRY(cudaGetLastError());
+    if ((rc = build_row_contexts(idx, (const uint32_t *)sa.p, rows, s))) return rc;
     idx->has_full_sa = true;
     return 0;
 }
@@ -217,29 +254,37 @@ int rebuild_full_sa(mica_index *idx, cudaStream_t s)
 {
     const uint64_t n = idx->n, rows = n + 1, words = full_sa_text_words(n);
     int rc;
-    DevBuf err;
-    if ((rc = dev_reserve(idx->sa_full, rows * 4)) || (rc = dev_reserve(idx->isa, rows * 4)) ||
-        (rc = dev_reserve(idx->text, words * 4)) || (rc = dev_reserve(err, 4)))
+    DevBuf err, sa;
+    if ((rc = dev_reserve(sa, rows * 4)) || (rc = dev_reserve(idx->isa, rows * 4)) ||
+        (rc = dev_reserve(idx->text, words * 4)) || (rc = dev_reserve(err, 4))) {
+        dev_release(sa);
         return rc;
+    }
     unsigned herr = 0;
     cudaError_t e = cudaMemsetAsync(idx->text.p, 0, words * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(err.p, 0, 4, s);
     if (e == cudaSuccess) {
         k_invert_bwt<<<grid_of(idx->n_mark_blocks, 128), 128, 0, s>>>(
-            idx->view, idx->n_mark_blocks, idx->n_samples, (uint32_t *)idx->sa_full.p, (uint32_t *)idx->isa.p,
+            idx->view, idx->n_mark_blocks, idx->n_samples, (uint32_t *)sa.p, (uint32_t *)idx->isa.p,
             (uint32_t *)idx->text.p, (unsigned *)err.p);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err.p, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     dev_release(err);
+    rc = 0;
     if (e != cudaSuccess) {
         set_last_cuda_error(e, "full suffix array rebuild", __FILE__, __LINE__);
-        return MICA_ECUDA;
+        rc = MICA_ECUDA;
+    } else if (herr) {
+        rc = MICA_EIO;
+    } else {
+        rc = build_row_contexts(idx, (const uint32_t *)sa.p, rows, s);
     }
-    if (herr) return MICA_EIO;
-    idx->has_full_sa = true;
-    return 0;
+    if (!rc && cudaStreamSynchronize(s) != cudaSuccess) rc = MICA_ECUDA;
+    dev_release(sa);
+    idx->has_full_sa = rc == 0;
+    return rc;
 }
 
 }  // namespace mica
@@ -290,9 +335,23 @@ extern "C" int mica_debug_full_sa(const mica_index *idx, uint32_t which, uint64_
     const uint64_t len = which == 2 ? full_sa_text_words(idx->n) : idx->n + 1;
     if (first > len || n > len - first) return MICA_EINVAL;
     if (n == 0) return 0;
-    const DevBuf &b = which == 0 ? idx->sa_full : which == 1 ? idx->isa : idx->text;
+    const DevBuf &b = which == 1 ? idx->isa : idx->text;
     DeviceGuard g(idx->device);
     MICA_CUDA_TRY(cudaSetDevice(idx->device));
+    if (which == 0) {   // every other word of the rows, gathered a piece at a time
+        constexpr uint64_t PIECE = 1ull << 24;
+        DevBuf tmp;
+        if (int rc = dev_reserve(tmp, std::min(n, PIECE) * 4)) return rc;
+        cudaError_t e = cudaSuccess;
+        for (uint64_t o = 0; o < n && e == cudaSuccess; o += PIECE) {
+            const uint64_t c = std::min(n - o, PIECE);
+            k_sa_of<<<grid_of(c), 256>>>((const uint2 *)idx->sa_ctx.p + first + o, c, (uint32_t *)tmp.p);
+            e = cudaMemcpy(out + o, tmp.p, c * 4, cudaMemcpyDeviceToHost);
+        }
+        dev_release(tmp);
+        MICA_CUDA_TRY(e);
+        return 0;
+    }
     MICA_CUDA_TRY(cudaMemcpy(out, (const uint32_t *)b.p + first, n * 4, cudaMemcpyDeviceToHost));
     return 0;
 }

@@ -502,7 +502,7 @@ int build_index_from_codes(const uint8_t *d_codes, uint64_t n, const mica_index_
     dev_release(mcnt);
     dev_release(mbase);
 
-    // the whole suffix array (this one), its inverse and the 2-bit text
+    // the whole suffix array with left contexts, its inverse and the 2-bit text
     if (p.full_sa && (rc = build_full_sa(idx, sa, d_codes, n, s))) { cleanup(); return rc; }
 
     // q-mer table
@@ -524,8 +524,7 @@ int build_index_from_codes(const uint8_t *d_codes, uint64_t n, const mica_index_
         DevBuf rcodes;
         if ((rc = dev_reserve(rcodes, std::max<uint64_t>(n, 1)))) { cleanup(); return rc; }
         if (n) k_reverse_codes<<<grid_for(n), 256, 0, s>>>(d_codes, n, (uint8_t *)rcodes.p);
-        rc = dev_reserve(sa, rows * 4);   // (empty when the forward suffix array was kept)
-        if (!rc) rc = build_suffix_array((const uint8_t *)rcodes.p, n, (uint32_t *)sa.p, s);
+        rc = build_suffix_array((const uint8_t *)rcodes.p, n, (uint32_t *)sa.p, s);
         if (!rc) rc = build_occ((const uint8_t *)rcodes.p, n, (const uint32_t *)sa.p, idx->rocc, idx->rsuper,
                                 rdollar, rC, s);
         // and its q-mer table: the seed of a bidirectional search needs the

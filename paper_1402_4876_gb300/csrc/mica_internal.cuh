@@ -89,10 +89,12 @@ struct IndexView {
         uint32_t short_len[MAX_Q];
         unsigned long long short_bloom;
     } rev;
-    // The whole suffix array SA[0, n], its inverse ISA[0, n] and the text G at
-    // 2 bits per base (16 per word, least-significant first, zero words past
-    // the end); all null when the index was built without them.
-    const uint32_t *sa_full;
+    // The whole suffix array SA[0, n] with each row's left context, its inverse
+    // ISA[0, n] and the text G at 2 bits per base (16 per word,
+    // least-significant first, zero words past the end); all null when the
+    // index was built without them.  sa_ctx[j] = (SA[j], the 16 bases before it:
+    // G[SA[j] - 16 + i] at bits 2i, zeros before the text).
+    const uint2 *sa_ctx;
     const uint32_t *isa;
     const uint32_t *text;
     // Seed tables of a longer q (built from the text with full_sa, for the
@@ -112,9 +114,10 @@ struct ReadsView {
 // Leaf interval found by the search.
 struct Interval {
     uint32_t read;
-    uint32_t meta;   // bit 0..1 d, bit 2 strand
+    uint32_t meta;   // bit 0..1 d, bit 2 strand, bit 3 IV_POS
     uint32_t l, r;
 };
+constexpr uint32_t IV_POS = 8u;   // [l, l + 1) is a text position found by the text check, not a row
 
 // Work item in the device queues: a seed range of a (read, strand) task or a
 // continuation node.  meta: bit 30 kind (1 = node), bit 29 strand, bits 0..1
@@ -240,7 +243,7 @@ struct mica_index {
     mica::DevBuf occ, super, marks, samples, table, variants;
     mica::DevBuf rocc, rsuper;   // reversed genome's occurrence blocks (lower bounds, bidirectional search)
     mica::DevBuf rtable;         // reversed genome's q-mer table (bidirectional search)
-    mica::DevBuf sa_full, isa, text;   // whole suffix array, its inverse, 2-bit text (full_sa)
+    mica::DevBuf sa_ctx, isa, text;   // whole suffix array with left contexts, its inverse, 2-bit text (full_sa)
     mica::DevBuf ltable, lrtable;      // longer seed tables of G$ and G~$ (with full_sa)
     bool has_rev = false;
     bool has_full_sa = false;
@@ -296,7 +299,7 @@ int build_suffix_array(const uint8_t *d_codes, uint64_t n, uint32_t *d_sa, cudaS
 uint64_t full_sa_text_words(uint64_t n);   // text words incl. zero padding (a multiple of 4)
 uint64_t full_sa_bytes(uint64_t n);
 void set_full_sa_view(mica_index *idx);
-int build_full_sa(mica_index *idx, DevBuf &sa, const uint8_t *d_codes, uint64_t n, cudaStream_t s);
+int build_full_sa(mica_index *idx, const DevBuf &sa, const uint8_t *d_codes, uint64_t n, cudaStream_t s);
 int rebuild_full_sa(mica_index *idx, cudaStream_t s);
 uint32_t long_seed_q(uint64_t n, uint32_t q);   // q of the longer seed tables (== q: none)
 // the longer seed tables from the genome's codes (or, when d_codes is null,
@@ -356,6 +359,11 @@ int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tm
 int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl *tmpl_src,
                         cudaStream_t s, uint64_t &launches);
 int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s);
+
+// sweep.cu
+bool sweep_available(const mica_index *idx, uint32_t verify_min);
+int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint2 *list,
+                  cudaStream_t s, uint64_t &launches);
 
 // post.cu
 int run_post(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, uint32_t hit_cap,

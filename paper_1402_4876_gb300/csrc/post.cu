@@ -143,6 +143,17 @@ __global__ void k_iv_scatter(const Interval *__restrict__ iv, const unsigned int
     }
 }
 
+// An interval in rows: a text position found by the text check becomes its
+// row (only a capped read's order needs it).
+__device__ __forceinline__ void to_rows(Interval &x, const uint32_t *__restrict__ isa)
+{
+    if (x.meta & IV_POS) {
+        x.l = __ldg(isa + x.l);
+        x.r = x.l + 1u;
+        x.meta &= ~IV_POS;
+    }
+}
+
 __device__ __forceinline__ uint64_t iv_key(const Interval &x)
 {
     return ((uint64_t)(x.meta & 3u) << 33) | ((uint64_t)((x.meta >> 2) & 1u) << 32) | x.l;
@@ -176,7 +187,7 @@ constexpr uint32_t SUMMARY_SMALL = 32;
 __global__ void k_summarize(Interval *__restrict__ ivs, const uint64_t *__restrict__ iv_off, uint64_t n,
                             uint32_t cap, uint64_t *__restrict__ total, uint64_t *__restrict__ keep,
                             uint32_t *__restrict__ many, unsigned int *__restrict__ n_many,
-                            const unsigned int *__restrict__ err)
+                            const uint32_t *__restrict__ isa, const unsigned int *__restrict__ err)
 {
     if (*err) return;
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
@@ -189,8 +200,9 @@ __global__ void k_summarize(Interval *__restrict__ ivs, const uint64_t *__restri
         uint64_t t = 0;
         for (uint64_t i = b; i < e; i++) t += ivs[i].r - ivs[i].l;
         if (cap && t > cap) {
-            for (uint64_t i = b + 1; i < e; i++) {
+            for (uint64_t i = b; i < e; i++) {
                 Interval x = ivs[i];
+                to_rows(x, isa);
                 uint64_t kx = iv_key(x);
                 uint64_t j = i;
                 while (j > b && iv_key(ivs[j - 1]) > kx) { ivs[j] = ivs[j - 1]; j--; }
@@ -231,6 +243,7 @@ __global__ void __launch_bounds__(MANY_THREADS) k_summarize_many(Interval *__res
                                                                  uint64_t *__restrict__ keep,
                                                                  const uint32_t *__restrict__ many,
                                                                  const unsigned int *__restrict__ n_many_p,
+                                                                 const uint32_t *__restrict__ isa,
                                                                  const unsigned int *__restrict__ err)
 {
     if (*err) return;
@@ -248,6 +261,8 @@ __global__ void __launch_bounds__(MANY_THREADS) k_summarize_many(Interval *__res
             keep[r] = (cap && t > cap) ? cap : t;
         }
         if (!(cap && t > cap)) continue;
+        for (uint64_t i = b + threadIdx.x; i < e; i += MANY_THREADS) to_rows(ivs[i], isa);   // (the passes below
+                                                                                            // keep this stride)
         // bitwise search for K over the 35-bit keys
         uint64_t prefix = 0, before = 0;
         for (int bit = 34; bit >= 0; bit--) {
@@ -307,7 +322,7 @@ __global__ void k_expand(const Interval *__restrict__ ivs, const uint64_t *__res
                 h.pos = row;   // resolved to a position by k_locate
                 h.strand = (uint8_t)((x.meta >> 2) & 1u);
                 h.mm = (uint8_t)(x.meta & 3u);
-                h.pad = 0;
+                h.pad = (x.meta & IV_POS) ? 1 : 0;   // a position already
                 hits[q] = h;
             }
         }
@@ -365,7 +380,8 @@ __global__ void k_locate(const IndexView ix, Hit *__restrict__ hits, const uint6
     uint32_t steps = 0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nh;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        hits[i].pos = ix.sa_full ? __ldg(ix.sa_full + hits[i].pos) : locate_row(ix, hits[i].pos, steps);
+        if (hits[i].pad) hits[i].pad = 0;
+        else hits[i].pos = ix.sa_ctx ? __ldg(&ix.sa_ctx[hits[i].pos].x) : locate_row(ix, hits[i].pos, steps);
     }
     unsigned mask = __activemask();
     unsigned s = __reduce_add_sync(mask, steps);
@@ -635,10 +651,11 @@ int enqueue_post_device(const mica_index *idx, Workspace &w, const ReadsView &rd
         L++;
     }
     k_summarize<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, hit_cap, (uint64_t *)w.total.p,
-                                              (uint64_t *)w.keep.p, pl.many, pl.n_many, &ctl->error);
+                                              (uint64_t *)w.keep.p, pl.many, pl.n_many, idx->view.isa,
+                                              &ctl->error);
     k_summarize_many<<<152 * 2, MANY_THREADS, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, hit_cap,
                                                       (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many,
-                                                      pl.n_many, &ctl->error);
+                                                      pl.n_many, idx->view.isa, &ctl->error);
     L += 3;
     if ((rc = exclusive_scan<uint64_t>(w.scan_tmp, (const uint64_t *)w.keep.p, n, hit_off, s, L))) return rc;
     k_expand<<<grid1(n, 128), 128, 0, s>>>((const Interval *)w.iv_sorted.p, iv_off, hit_off, n, (Hit *)w.hits.p,
@@ -710,10 +727,10 @@ int run_post(const mica_index *idx, Workspace &w, mica_stats &stt, const ReadsVi
     if (n) {
         k_summarize<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, hit_cap,
                                                   (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many, pl.n_many,
-                                                  err);
+                                                  idx->view.isa, err);
         k_summarize_many<<<152 * 2, MANY_THREADS, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, hit_cap,
                                                           (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many,
-                                                          pl.n_many, err);
+                                                          pl.n_many, idx->view.isa, err);
         L += 2;
     }
     if ((rc = exclusive_scan<uint64_t>(w.scan_tmp, (const uint64_t *)w.keep.p, n, hit_off, s, L))) return rc;

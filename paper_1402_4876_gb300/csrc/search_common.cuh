@@ -170,26 +170,21 @@ __device__ __forceinline__ void occ_from(const OccSide &ix, uint32_t b, uint32_t
 }
 
 // Occ(c, l) and Occ(c, r) for all c on one side; returns the blocks read.
+// Both blocks and superblock entries are loaded whole and at once even when l
+// and r share a block (one line then): a branch on that had the lanes of a
+// warp wait for one side's loads and then for the other's.
 __device__ __forceinline__ int occ_pair(const OccSide &ix, uint32_t l, uint32_t r, uint32_t (&ol)[4],
                                         uint32_t (&orr)[4])
 {
-    uint32_t bl = l / OCC_ROWS, xl = l - bl * OCC_ROWS;
-    uint32_t br = r / OCC_ROWS, xr = r - br * OCC_ROWS;
-    uint4 sl = ld_nc(ix.super + bl / SB_BLOCKS);
-    OccBlock a;
-    if (bl == br) {
-        load_block(ix, bl, xr, a);
-        occ_from(ix, bl, xl, sl, a, ol);
-        occ_from(ix, br, xr, sl, a, orr);
-        return 1;
-    }
-    uint4 sr = ld_nc(ix.super + br / SB_BLOCKS);
-    OccBlock c;
-    load_block(ix, bl, xl, a);
-    load_block(ix, br, xr, c);
+    const uint32_t bl = l / OCC_ROWS, xl = l - bl * OCC_ROWS;
+    const uint32_t br = r / OCC_ROWS, xr = r - br * OCC_ROWS;
+    const uint4 sl = ld_nc(ix.super + bl / SB_BLOCKS), sr = ld_nc(ix.super + br / SB_BLOCKS);
+    OccBlock a, c;
+    load_block(ix, bl, OCC_ROWS, a);
+    load_block(ix, br, OCC_ROWS, c);
     occ_from(ix, bl, xl, sl, a, ol);
     occ_from(ix, br, xr, sr, c, orr);
-    return 2;
+    return bl == br ? 1 : 2;
 }
 
 // Base t of a packed pattern.
