@@ -148,7 +148,7 @@ void dev_release(DevBuf &b)
 
 void free_workspace(Workspace &w)
 {
-    DevBuf *all[] = {&w.ctl, &w.iv, &w.iv_sorted, &w.iv_cnt, &w.iv_off, &w.total, &w.keep, &w.hit_off,
+    DevBuf *all[] = {&w.ctl, &w.iv, &w.iv_sorted, &w.iv_cnt, &w.iv_off, &w.total, &w.hit_off,
                      &w.hits, &w.spill, &w.big, &w.scan_tmp, &w.reads_words, &w.reads_off, &w.reads_len,
                      &w.reads_k, &w.spill2, &w.lenlist, &w.lb, &w.spill_seq, &w.deep, &w.redo, &w.frontier};
     for (DevBuf *b : all) dev_release(*b);
@@ -268,8 +268,8 @@ static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &s
     launched = false;
     uint64_t n = rd.n;
     if (!w.pin_tmpl) {
-        MICA_CUDA_TRY(cudaMallocHost(&w.pin_tmpl, 256));
-        MICA_CUDA_TRY(cudaMallocHost(&w.pin_status, 256));
+        MICA_CUDA_TRY(cudaMallocHost(&w.pin_tmpl, sizeof(SearchCtl)));
+        MICA_CUDA_TRY(cudaMallocHost(&w.pin_status, sizeof(SearchCtl)));
     }
     if (!w.gstream) MICA_CUDA_TRY(cudaStreamCreateWithFlags(&w.gstream, cudaStreamNonBlocking));
     SearchCtl tmpl;
@@ -293,7 +293,7 @@ static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &s
                                (uint64_t)grid,
                                (uint64_t)w.ctl.p, (uint64_t)w.iv.p, (uint64_t)w.iv_cnt.p, (uint64_t)w.spill.p,
                                (uint64_t)w.lb.p, (uint64_t)w.iv_sorted.p, (uint64_t)w.iv_off.p,
-                               (uint64_t)w.total.p, (uint64_t)w.keep.p, (uint64_t)w.hit_off.p, (uint64_t)w.hits.p,
+                               (uint64_t)w.total.p, (uint64_t)w.hit_off.p, (uint64_t)w.hits.p,
                                (uint64_t)w.big.p, (uint64_t)w.scan_tmp.p, w.hit_capacity, (uint64_t)w.iv_cap,
                                (uint64_t)w.spill_cap, (uint64_t)w.spill_seq.p, (uint64_t)w.deep.p,
                                (uint64_t)p.report | ((uint64_t)idx->tuning.bidir_budget << 32),
@@ -340,12 +340,7 @@ static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd,
     MICA_CUDA_TRY(cudaEventSynchronize(w.ev[2]));
     SearchCtl out;
     memcpy(&out, w.pin_status, sizeof(out));
-    const char *stp = (const char *)w.pin_status + sizeof(SearchCtl);
-    uint64_t nhits, steps;
-    unsigned int cnts[2];
-    memcpy(&nhits, stp, 8);
-    memcpy(&steps, stp + 8, 8);
-    memcpy(cnts, stp + 16, 8);
+    const uint64_t nhits = out.post_hits;
     if (out.error & ERR_TIMEOUT) return MICA_ETIMEOUT;
     if (out.error) {
         // let the regular path grow the buffers and recompute
@@ -359,7 +354,7 @@ static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd,
         return 0;
     }
     if (nhits > w.hit_capacity) { w.hit_capacity = 2 * nhits; return 0; }
-    if (cnts[1]) return 0;   // a read above the shared-memory sort size
+    if (out.n_huge) return 0;   // a read above the shared-memory sort size
     st.tasks = 2 * n;
     st.seeds = out.seeds;
     st.nodes = out.nodes;
@@ -381,7 +376,7 @@ static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd,
     st.verify_sectors = out.verify_sectors;
     st.grid_ctas = (uint64_t)grid;
     st.located = nhits;
-    st.lf_steps = steps;
+    st.lf_steps = out.lf_steps;
     st.launches += w.glaunches;
     st.graph_replays++;
     st.kernel_ms = elapsed_ms(w.kev[0], w.kev[1]);

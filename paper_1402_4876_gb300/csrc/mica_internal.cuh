@@ -162,6 +162,10 @@ struct SearchCtl {
     unsigned long long verified, verify_bytes;        // bidirectional search: one-row intervals checked
                                                       //   against the text, and the bytes that read
     unsigned long long verify_sectors;                // ... and the 32-byte sectors those reads touch
+    // after the search (post.cu)
+    unsigned long long post_hits, lf_steps;           // hits listed; LF steps of locating rows
+    unsigned int n_warp, n_block, n_long, n_huge;     // reads on the finishing kernels' lists
+    unsigned int next_warp, next_block, next_long, pad2_;   // ... and the next one of each to take
 };
 
 constexpr unsigned ERR_IV_OVERFLOW = 1u;
@@ -191,11 +195,11 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-constexpr int GRAPH_KEY = 31;   // words identifying a captured batch shape
+constexpr int GRAPH_KEY = 30;   // words identifying a captured batch shape
 
 // Per-index workspace reused across align calls.
 struct Workspace {
-    DevBuf ctl, iv, iv_sorted, iv_cnt, iv_off, total, keep, hit_off, hits, spill, big, scan_tmp;
+    DevBuf ctl, iv, iv_sorted, iv_cnt, iv_off, total, hit_off, hits, spill, big, scan_tmp;
     DevBuf lb;   // per (read, strand) task: mismatch lower-bound breakpoints (uint64)
     DevBuf spill_seq;   // spill ring: one sequence word per slot
     DevBuf deep;        // per-warp overflow stacks of the persistent kernel

@@ -1,12 +1,25 @@
-// From leaf SA intervals to per-read hit lists:
-//   1. group the intervals by read (prefix sum of per-read counts + scatter);
-//   2. per read: order the intervals by (d, strand, first row), total = sum of
-//      interval sizes (exact), keep = min(total, cap) rows in that order;
-//   3. prefix sum of keep -> CSR offsets; expand the kept rows;
-//   4. resolve each row to a text position by LF walks to the nearest marked
-//      row (SA[j] % s == 0), whose SA value is stored:
-//          SA[j] = SA[LF^t(j)] + t,   LF(j) = C[BWT[j]] + Occ(BWT[j], j);
-//   5. sort each read's hits by (position, strand).
+// From leaf SA intervals to per-read hit lists, in seven kernels (eight for more
+// than 512 reads):
+//   1. k_tile_counts, k_offsets: prefix sum of the per-read interval counts;
+//   2. k_iv_scatter: the intervals grouped by read, and total = the sum of a
+//      read's interval sizes (exact), of which min(total, cap) rows are listed;
+//   3. k_listed: the rows listed per tile of reads;
+//   4. k_finish_small: prefix sum of the listed counts -> CSR offsets, and the
+//      hits of reads with a few; larger reads and reads over their cap go on
+//      lists;
+//   5. k_finish_warp, k_finish_block (two sizes): those reads, a warp or a block each: over
+//      the cap the first cap rows in the order (d, strand, row) are kept, then
+//      rows become text positions, and the hits go out sorted by (position,
+//      strand).
+// A row's position is one read of the suffix array when the index keeps it,
+// else LF walks to the nearest marked row (SA[j] % s == 0), whose SA value is
+// stored: SA[j] = SA[LF^t(j)] + t, LF(j) = C[BWT[j]] + Occ(BWT[j], j).
+//
+// The first form of this had a kernel per step over all hits (fourteen
+// launches, each hit written, located and sorted in global memory); with the
+// hits of a read made, ordered and written in one place each is written once.
+#include <stddef.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -19,12 +32,19 @@ namespace {
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
-constexpr uint32_t SMALL_SORT = 32;
 constexpr unsigned FULL = 0xffffffffu;
-constexpr uint32_t SMEM_SORT = 4096;
-constexpr uint32_t WARP_SORT = 256;            // reads up to this many hits: one warp sorts each ...
-constexpr uint32_t WARP_SORT_WARPS = 8;        // ... 8 warps per block (2 KB of shared memory each);
-constexpr uint32_t BLOCK_SORT_THREADS = 128;   // larger ones (up to SMEM_SORT): a block of 128 threads each
+constexpr uint32_t TILE = 512;                // reads per block of the per-read passes
+constexpr uint32_t TILE_THREADS = 256;
+constexpr uint32_t SMALL_HITS = 8;             // reads up to this many hits: one thread each
+constexpr uint32_t WARP_HITS = 256;            // up to this many hits and intervals: a warp each ...
+constexpr uint32_t WARP_READS = 4;             // ... 4 warps per block;
+constexpr uint32_t WARP_CAP = 65535;           // (and a cap its 32-bit sums hold)
+constexpr uint32_t BLOCK_HITS = 4096;          // up to this many hits: a block each; above: the host's loop
+constexpr uint32_t BLOCK_READ_THREADS = 128;
+constexpr uint32_t LONG_LIST = 1024;           // a read of more intervals than this has a block ...
+constexpr uint32_t LONG_THREADS = 1024;        // ... of this many threads
+constexpr uint32_t WARP_SPAN = 4096;           // hits within this many positions of each other are ordered by counting:
+constexpr uint32_t BLOCK_SPAN = 20480;         // a bit per (position, strand) in shared memory
 
 // ---- exclusive scan (n values -> n + 1 offsets) ----
 
@@ -106,19 +126,77 @@ __global__ void k_scan_add(uint64_t *__restrict__ out, uint64_t n, const uint64_
     if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = tile_sums[ntiles];
 }
 
-template <typename T>
-int exclusive_scan(DevBuf &tmp, const T *in, uint64_t n, uint64_t *out, cudaStream_t s, uint64_t &launches)
+// ---- per-read prefix sums: a block per tile of reads, which adds up the tiles before its own ----
+
+__device__ __forceinline__ uint64_t block_exclusive(uint64_t v, uint64_t *warp_sums, uint64_t &all)
 {
-    uint64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (int rc = dev_reserve(tmp, (ntiles + 1) * 8)) return rc;
-    uint64_t *ts = (uint64_t *)tmp.p;
-    if (ntiles) { k_scan_tiles<T><<<(unsigned)ntiles, SCAN_THREADS, 0, s>>>(in, n, out, ts); launches++; }
-    k_scan_sums<<<1, 1024, 0, s>>>(ts, ntiles);
-    unsigned g = (unsigned)std::min<uint64_t>(std::max<uint64_t>((n + 255) / 256, 1), 152 * 32);
-    k_scan_add<<<g, 256, 0, s>>>(out, n, ts);
-    launches += 2;
-    MICA_CUDA_TRY(cudaGetLastError());
-    return 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __syncthreads();
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    uint64_t before = 0;
+    all = 0;
+    for (uint32_t w = 0; w < TILE_THREADS / 32; w++) {
+        if ((int)w < warp) before += warp_sums[w];
+        all += warp_sums[w];
+    }
+    return before + incl - v;
+}
+
+// Sum of the first `tiles` tile sums.
+__device__ __forceinline__ uint64_t tiles_before(const uint64_t *__restrict__ sums, uint32_t tiles, uint64_t *warp_sums)
+{
+    uint64_t v = 0, all;
+    for (uint32_t i = threadIdx.x; i < tiles; i += TILE_THREADS) v += sums[i];
+    block_exclusive(v, warp_sums, all);
+    return all;
+}
+
+__global__ void __launch_bounds__(TILE_THREADS) k_tile_counts(const uint32_t *__restrict__ cnt, uint64_t n,
+                                                              uint64_t *__restrict__ sums)
+{
+    __shared__ uint64_t ws[TILE_THREADS / 32];
+    uint64_t v = 0, all;
+    for (uint32_t i = threadIdx.x; i < TILE; i += TILE_THREADS) {
+        const uint64_t r = blockIdx.x * (uint64_t)TILE + i;
+        if (r < n) v += cnt[r];
+    }
+    block_exclusive(v, ws, all);
+    if (threadIdx.x == 0) sums[blockIdx.x] = all;
+}
+
+// off[r] = sum of cnt[0, r), r = 0 .. n, and total[r] = 0.  sums: of the tiles
+// before (not read by the first).
+__global__ void __launch_bounds__(TILE_THREADS) k_offsets(const uint32_t *__restrict__ cnt, uint64_t n,
+                                                          const uint64_t *__restrict__ sums, uint64_t *__restrict__ off,
+                                                          uint64_t *__restrict__ total)
+{
+    __shared__ uint64_t ws[TILE_THREADS / 32];
+    uint64_t at = tiles_before(sums, blockIdx.x, ws);
+    constexpr uint32_t PER = TILE / TILE_THREADS;
+    const uint64_t r0 = blockIdx.x * (uint64_t)TILE + threadIdx.x * PER;
+    uint32_t c[PER];
+    uint64_t v = 0, all;
+#pragma unroll
+    for (uint32_t i = 0; i < PER; i++) {
+        c[i] = r0 + i < n ? cnt[r0 + i] : 0u;
+        v += c[i];
+    }
+    at += block_exclusive(v, ws, all);
+#pragma unroll
+    for (uint32_t i = 0; i < PER; i++) {
+        if (r0 + i <= n) off[r0 + i] = at;
+        if (r0 + i < n) total[r0 + i] = 0;
+        at += c[i];
+    }
+    // (the last read's thread writes off[n] above unless n ends a tile)
+    if (r0 + PER == n) off[n] = at;
 }
 
 // ---- intervals grouped by read ----
@@ -131,7 +209,8 @@ int exclusive_scan(DevBuf &tmp, const T *in, uint64_t n, uint64_t *out, cudaStre
 // the buffer's capacity) so the launch needs no host round trip
 __global__ void k_iv_scatter(const Interval *__restrict__ iv, const unsigned int *__restrict__ count_p,
                              uint32_t cap, const uint64_t *__restrict__ iv_off, uint32_t *__restrict__ cursor,
-                             Interval *__restrict__ out, const unsigned int *__restrict__ err)
+                             Interval *__restrict__ out, unsigned long long *__restrict__ total,
+                             const unsigned int *__restrict__ err)
 {
     if (*err) return;
     uint32_t count = min(*count_p, cap);
@@ -140,6 +219,7 @@ __global__ void k_iv_scatter(const Interval *__restrict__ iv, const unsigned int
         if (x.read == IV_PURGED) continue;   // a leaf of a read that was searched again
         uint32_t at = atomicSub(&cursor[x.read], 1u) - 1u;
         out[iv_off[x.read] + at] = x;
+        atomicAdd(&total[x.read], (unsigned long long)(x.r - x.l));
     }
 }
 
@@ -159,174 +239,69 @@ __device__ __forceinline__ uint64_t iv_key(const Interval &x)
     return ((uint64_t)(x.meta & 3u) << 33) | ((uint64_t)((x.meta >> 2) & 1u) << 32) | x.l;
 }
 
+// The tile's listed hits, min(total, cap) per read, to sums.
+__global__ void __launch_bounds__(TILE_THREADS) k_listed(const uint64_t *__restrict__ total, uint64_t n, uint32_t cap,
+                                                         uint64_t *__restrict__ sums)
+{
+    __shared__ uint64_t ws[TILE_THREADS / 32];
+    uint64_t keep = 0, all;
+    for (uint32_t i = threadIdx.x; i < TILE; i += TILE_THREADS) {
+        const uint64_t r = blockIdx.x * (uint64_t)TILE + i;
+        const uint64_t t = r < n ? total[r] : 0;
+        keep += cap && t > cap ? cap : t;
+    }
+    block_exclusive(keep, ws, all);
+    if (threadIdx.x == 0) sums[blockIdx.x] = all;
+}
+
 // Best-stratum reporting: a read keeps only its intervals with the smallest
-// d; the others become empty (r = l) and so count and list nothing.
+// d; the others become empty (r = l) and so count and list nothing.  A read
+// with many intervals is gone through by its warp.
 __global__ void k_stratum(Interval *__restrict__ ivs, const uint64_t *__restrict__ iv_off, uint64_t n,
-                          const unsigned int *__restrict__ err)
+                          uint64_t *__restrict__ total, const unsigned int *__restrict__ err)
 {
     if (*err) return;
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t b = iv_off[r], e = iv_off[r + 1];
-        uint32_t dmin = 3;
-        for (uint64_t i = b; i < e; i++) dmin = min(dmin, ivs[i].meta & 3u);
-        for (uint64_t i = b; i < e; i++)
-            if ((ivs[i].meta & 3u) > dmin) ivs[i].r = ivs[i].l;
-    }
-}
-
-// Per read: total = the sum of its interval sizes (exact) and keep = the
-// rows it lists, min(total, cap).  When total > cap the listed rows are the
-// first cap in the order (d, strand, SA row); k_expand takes rows from the
-// front of the read's interval list until it has `keep`, so that list must
-// start with the kept rows.  A read with at most SUMMARY_SMALL intervals is
-// done here by one thread (insertion sort into key order when over the cap);
-// a longer list goes to `many` for k_summarize_many.
-constexpr uint32_t SUMMARY_SMALL = 32;
-
-__global__ void k_summarize(Interval *__restrict__ ivs, const uint64_t *__restrict__ iv_off, uint64_t n,
-                            uint32_t cap, uint64_t *__restrict__ total, uint64_t *__restrict__ keep,
-                            uint32_t *__restrict__ many, unsigned int *__restrict__ n_many,
-                            const uint32_t *__restrict__ isa, const unsigned int *__restrict__ err)
-{
-    if (*err) return;
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t b = iv_off[r], e = iv_off[r + 1];
-        if (e - b > SUMMARY_SMALL) {
-            many[atomicAdd(n_many, 1u)] = (uint32_t)r;
-            continue;
-        }
-        uint64_t t = 0;
-        for (uint64_t i = b; i < e; i++) t += ivs[i].r - ivs[i].l;
-        if (cap && t > cap) {
-            for (uint64_t i = b; i < e; i++) {
-                Interval x = ivs[i];
-                to_rows(x, isa);
-                uint64_t kx = iv_key(x);
-                uint64_t j = i;
-                while (j > b && iv_key(ivs[j - 1]) > kx) { ivs[j] = ivs[j - 1]; j--; }
-                ivs[j] = x;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint64_t r0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); r0 < n;
+         r0 += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t r = r0 + lane;
+        uint64_t b = 0, e = 0;
+        if (r < n) { b = iv_off[r]; e = iv_off[r + 1]; }
+        const bool many = e - b > 32;
+        if (!many && e - b > 1) {
+            uint32_t dmin = 3;
+            uint64_t gone = 0;
+            for (uint64_t x = b; x < e; x++) dmin = min(dmin, ivs[x].meta & 3u);
+            for (uint64_t x = b; x < e; x++) {
+                const Interval v = ivs[x];
+                if ((v.meta & 3u) > dmin) { ivs[x].r = v.l; gone += v.r - v.l; }
             }
+            if (gone) total[r] -= gone;
         }
-        total[r] = t;
-        keep[r] = (cap && t > cap) ? cap : t;
-    }
-}
-
-// Block-wide sum of one value per thread (blockDim.x = MANY_THREADS).
-constexpr int MANY_THREADS = 256;
-
-__device__ __forceinline__ uint64_t block_sum(uint64_t v, uint64_t *red)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-    __syncthreads();                       // red[] free from the previous use
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    uint64_t s = 0;
-    for (int w = 0; w < MANY_THREADS / 32; w++) s += red[w];
-    return s;
-}
-
-// One block per read with more than SUMMARY_SMALL intervals.  The rows a
-// capped read lists are found without sorting: interval keys (d, strand, l)
-// are distinct, so a bitwise search from the top key bit finds the key K at
-// which the running row count in key order first reaches cap (35 passes,
-// each a block-wide sum of the sizes below the candidate prefix).  Intervals
-// with key < K are kept whole, K's interval keeps its first cap - before
-// rows, and the kept ones are compacted to the front of the read's list in
-// chunks of the block size (each chunk read before any of it is overwritten;
-// writes never pass the chunk being read).
-__global__ void __launch_bounds__(MANY_THREADS) k_summarize_many(Interval *__restrict__ ivs,
-                                                                 const uint64_t *__restrict__ iv_off,
-                                                                 uint32_t cap, uint64_t *__restrict__ total,
-                                                                 uint64_t *__restrict__ keep,
-                                                                 const uint32_t *__restrict__ many,
-                                                                 const unsigned int *__restrict__ n_many_p,
-                                                                 const uint32_t *__restrict__ isa,
-                                                                 const unsigned int *__restrict__ err)
-{
-    if (*err) return;
-    __shared__ uint64_t red[MANY_THREADS / 32];
-    __shared__ uint32_t wsum[MANY_THREADS / 32];
-    const unsigned n_many = *n_many_p;
-    for (unsigned mi = blockIdx.x; mi < n_many; mi += gridDim.x) {
-        const uint32_t r = many[mi];
-        const uint64_t b = iv_off[r], e = iv_off[r + 1];
-        uint64_t part = 0;
-        for (uint64_t i = b + threadIdx.x; i < e; i += MANY_THREADS) part += ivs[i].r - ivs[i].l;
-        const uint64_t t = block_sum(part, red);
-        if (threadIdx.x == 0) {
-            total[r] = t;
-            keep[r] = (cap && t > cap) ? cap : t;
-        }
-        if (!(cap && t > cap)) continue;
-        for (uint64_t i = b + threadIdx.x; i < e; i += MANY_THREADS) to_rows(ivs[i], isa);   // (the passes below
-                                                                                            // keep this stride)
-        // bitwise search for K over the 35-bit keys
-        uint64_t prefix = 0, before = 0;
-        for (int bit = 34; bit >= 0; bit--) {
-            const uint64_t hi = prefix >> (bit + 1);
-            uint64_t z = 0;
-            for (uint64_t i = b + threadIdx.x; i < e; i += MANY_THREADS) {
-                Interval x = ivs[i];
-                uint64_t k = iv_key(x);
-                if ((k >> (bit + 1)) == hi && !((k >> bit) & 1u)) z += x.r - x.l;
+        for (unsigned todo = __ballot_sync(FULL, many); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const uint64_t wb = __shfl_sync(FULL, b, src), we = __shfl_sync(FULL, e, src);
+            uint32_t dmin = 3;
+            for (uint64_t x = wb + lane; x < we; x += 32) dmin = min(dmin, ivs[x].meta & 3u);
+            dmin = __reduce_min_sync(FULL, dmin);
+            uint64_t gone = 0;
+            for (uint64_t x = wb + lane; x < we; x += 32) {
+                const Interval v = ivs[x];
+                if ((v.meta & 3u) > dmin) { ivs[x].r = v.l; gone += v.r - v.l; }
             }
-            z = block_sum(z, red);
-            if (before + z < cap) { before += z; prefix |= 1ull << bit; }
-        }
-        const uint64_t K = prefix;
-        const uint32_t take = (uint32_t)(cap - before);   // rows of K's interval, 1 .. its size
-        // compact the kept intervals to the front
-        uint64_t out = b;
-        for (uint64_t c0 = b; c0 < e; c0 += MANY_THREADS) {
-            uint64_t i = c0 + threadIdx.x;
-            Interval x{};
-            bool kept = false;
-            if (i < e) {
-                x = ivs[i];
-                uint64_t k = iv_key(x);
-                kept = k <= K;
-                if (k == K) x.r = x.l + take;
-            }
-            unsigned bal = __ballot_sync(FULL, kept);
-            __syncthreads();                 // every read of this chunk is done
-            if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = __popc(bal);
-            __syncthreads();
-            uint32_t pre = 0, all = 0;
-            for (int w = 0; w < MANY_THREADS / 32; w++) {
-                if (w < (int)(threadIdx.x >> 5)) pre += wsum[w];
-                all += wsum[w];
-            }
-            pre += __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
-            if (kept) ivs[out + pre] = x;
-            out += all;
-            __syncthreads();                 // writes done before the next chunk is read
+            for (int o = 16; o; o >>= 1) gone += __shfl_xor_sync(FULL, gone, o);
+            if ((int)lane == src) total[r] -= gone;
         }
     }
 }
 
-__global__ void k_expand(const Interval *__restrict__ ivs, const uint64_t *__restrict__ iv_off,
-                         const uint64_t *__restrict__ hit_off, uint64_t n, Hit *__restrict__ hits,
-                         uint64_t capacity, const unsigned int *__restrict__ err)
+// Sum of all tile sums (the hits to be listed), for the host.
+__global__ void __launch_bounds__(TILE_THREADS) k_tiles_total(const uint64_t *__restrict__ sums, uint32_t tiles,
+                                                              uint64_t *__restrict__ out)
 {
-    if (*err) return;
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t q = hit_off[r], qe = min(hit_off[r + 1], capacity);
-        for (uint64_t i = iv_off[r]; i < iv_off[r + 1] && q < qe; i++) {
-            Interval x = ivs[i];
-            for (uint32_t row = x.l; row < x.r && q < qe; row++, q++) {
-                Hit h;
-                h.pos = row;   // resolved to a position by k_locate
-                h.strand = (uint8_t)((x.meta >> 2) & 1u);
-                h.mm = (uint8_t)(x.meta & 3u);
-                h.pad = (x.meta & IV_POS) ? 1 : 0;   // a position already
-                hits[q] = h;
-            }
-        }
-    }
+    __shared__ uint64_t ws[TILE_THREADS / 32];
+    const uint64_t all = tiles_before(sums, tiles, ws);
+    if (threadIdx.x == 0) *out = all;
 }
 
 }  // namespace
@@ -371,52 +346,101 @@ __device__ __forceinline__ uint32_t locate_row(const IndexView &ix, uint32_t j, 
 
 namespace {
 
-__global__ void k_locate(const IndexView ix, Hit *__restrict__ hits, const uint64_t *__restrict__ nh_p,
-                         uint64_t capacity, unsigned long long *__restrict__ steps_out,
-                         const unsigned int *__restrict__ err)
-{
-    if (*err) return;   // hits not expanded: rows would be stale
-    uint64_t nh = min(*nh_p, capacity);
-    uint32_t steps = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nh;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        if (hits[i].pad) hits[i].pad = 0;
-        else hits[i].pos = ix.sa_ctx ? __ldg(&ix.sa_ctx[hits[i].pos].x) : locate_row(ix, hits[i].pos, steps);
-    }
-    unsigned mask = __activemask();
-    unsigned s = __reduce_add_sync(mask, steps);
-    if ((threadIdx.x & 31) == (unsigned)(__ffs(mask) - 1) && s) atomicAdd(steps_out, (unsigned long long)s);
-}
+// What the finishing kernels share.
+struct FinishArgs {
+    IndexView ix;
+    Interval *ivs;
+    const uint64_t *iv_off;
+    const uint64_t *total;
+    uint64_t *hit_off;
+    uint64_t *hits;              // packed: pos | strand << 32 | mm << 40
+    uint64_t n, capacity;
+    uint32_t cap;
+    uint32_t *lists;             // reads for k_finish_warp from the front, for k_finish_block from the back
+    uint32_t *huge;              // reads with more than BLOCK_HITS hits from the front, those of long lists from the back
+    SearchCtl *ctl;
+};
 
 __device__ __forceinline__ uint64_t hit_key(uint64_t raw)
 {
     return ((raw & 0xffffffffull) << 1) | ((raw >> 32) & 1ull);   // (pos, strand)
 }
 
-// per read: sort <= SMALL_SORT hits in place; list larger reads for the
-// block sort (from the front of `lists`) or the global sort (from the back)
-__global__ void k_sort_small(uint64_t *__restrict__ hits, const uint64_t *__restrict__ hit_off, uint64_t n,
-                             uint64_t capacity, uint32_t *__restrict__ lists, unsigned int *__restrict__ counts)
+// The hit of row (or, with IV_POS, position) x of an interval; without the
+// suffix array its position is still the row (locate_hits).
+__device__ __forceinline__ uint64_t hit_of(const IndexView &ix, uint32_t x, uint32_t meta)
 {
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t b = hit_off[r], e = hit_off[r + 1];
-        if (e - b <= 1 || e > capacity) continue;
-        if (e - b > SMEM_SORT) {
-            lists[n - 1 - atomicAdd(&counts[1], 1u)] = (uint32_t)r;
+    const uint32_t pos = (meta & IV_POS) || !ix.sa_ctx ? x : __ldg(&ix.sa_ctx[x].x);
+    return (uint64_t)pos | ((uint64_t)((meta >> 2) & 1u) << 32) | ((uint64_t)(meta & 3u) << 40);
+}
+
+// Without the suffix array: the positions of a read's rows h[0, cnt), every
+// nt-th by this thread (walks of up to s - 1 steps, so that all threads of the
+// warp or block take part whatever the intervals' sizes).
+__device__ __forceinline__ void locate_hits(const IndexView &ix, uint64_t *h, uint64_t cnt, uint32_t tid, uint32_t nt,
+                                            uint32_t &steps)
+{
+    for (uint64_t i = tid; i < cnt; i += nt)
+        h[i] = (h[i] & ~0xffffffffull) | locate_row(ix, (uint32_t)h[i], steps);
+}
+
+__device__ __forceinline__ void count_steps(SearchCtl *ctl, uint32_t steps)
+{
+    const unsigned mask = __activemask();
+    const unsigned s = __reduce_add_sync(mask, steps);
+    if (s && (threadIdx.x & 31) == (unsigned)(__ffs(mask) - 1)) atomicAdd(&ctl->lf_steps, (unsigned long long)s);
+}
+
+// Offsets of the listed hits; reads with at most SMALL_HITS of them, none cut
+// off by the cap, are finished by their thread (an insertion into the hits
+// it has written so far); the others go on a list.
+__global__ void __launch_bounds__(TILE_THREADS) k_finish_small(const FinishArgs a, const uint64_t *__restrict__ sums)
+{
+    __shared__ uint64_t ws[TILE_THREADS / 32];
+    if (*(volatile unsigned *)&a.ctl->error) return;   // (the counts exceed what was stored)
+    uint64_t at = tiles_before(sums, blockIdx.x, ws);
+    uint32_t steps = 0;
+    for (uint32_t i0 = 0; i0 < TILE; i0 += TILE_THREADS) {
+        const uint64_t r = blockIdx.x * (uint64_t)TILE + i0 + threadIdx.x;
+        const uint64_t t = r < a.n ? a.total[r] : 0;
+        const uint64_t keep = a.cap && t > a.cap ? a.cap : t;
+        uint64_t all;
+        const uint64_t q0 = at + block_exclusive(keep, ws, all);
+        at += all;
+        if (r < a.n) a.hit_off[r] = q0;
+        if (r + 1 == a.n || (a.n == 0 && r == 0)) {
+            a.hit_off[a.n] = q0 + keep;
+            a.ctl->post_hits = q0 + keep;
+        }
+        if (keep == 0 || q0 + keep > a.capacity) continue;
+        const uint64_t b = a.iv_off[r], e = a.iv_off[r + 1];
+        // (without the suffix array a hit is a walk: more than one goes to a warp's lanes)
+        if (keep > (a.ix.sa_ctx ? SMALL_HITS : 1u) || t > keep || e - b > 32) {
+            if (keep > BLOCK_HITS) a.huge[atomicAdd(&a.ctl->n_huge, 1u)] = (uint32_t)r;
+            else if (e - b > LONG_LIST) a.huge[a.n - 1 - atomicAdd(&a.ctl->n_long, 1u)] = (uint32_t)r;
+            else if (keep <= WARP_HITS && e - b <= WARP_HITS && (t == keep || a.cap <= WARP_CAP))
+                a.lists[atomicAdd(&a.ctl->n_warp, 1u)] = (uint32_t)r;
+            else a.lists[a.n - 1 - atomicAdd(&a.ctl->n_block, 1u)] = (uint32_t)r;
             continue;
         }
-        if (e - b > SMALL_SORT) {
-            lists[atomicAdd(&counts[0], 1u)] = (uint32_t)r;
-            continue;
-        }
-        for (uint64_t i = b + 1; i < e; i++) {
-            uint64_t x = hits[i], kx = hit_key(x);
-            uint64_t j = i;
-            while (j > b && hit_key(hits[j - 1]) > kx) { hits[j] = hits[j - 1]; j--; }
-            hits[j] = x;
+        uint64_t q = q0;
+        for (uint64_t x = b; x < e; x++) {
+            const Interval v = a.ivs[x];
+            for (uint32_t row = v.l; row < v.r; row++, q++) {
+                uint64_t h = hit_of(a.ix, row, v.meta);
+                if (!a.ix.sa_ctx) locate_hits(a.ix, &h, 1, 0, 1, steps);
+                const uint64_t kh = hit_key(h);
+                uint64_t w = q;
+                for (; w > q0; w--) {
+                    const uint64_t p = a.hits[w - 1];
+                    if (hit_key(p) < kh) break;
+                    a.hits[w] = p;
+                }
+                a.hits[w] = h;
+            }
         }
     }
+    if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
 }
 
 // Bitonic sort of the packed hits sh[0, P) (P a power of two, padding ~0 last)
@@ -453,69 +477,351 @@ __device__ __forceinline__ void bitonic_hits(uint64_t *sh, uint32_t P, uint32_t 
         }
 }
 
-// Reads with SMALL_SORT < hits <= WARP_SORT: one warp each, taken from the
-// listed reads by a counter (reads differ a lot in size: a fixed stride left
-// one warp with the largest); larger listed reads are left to k_sort_block.
-__global__ void __launch_bounds__(WARP_SORT_WARPS * 32) k_sort_warp(uint64_t *__restrict__ hits,
-                                                                    const uint64_t *__restrict__ hit_off,
-                                                                    const uint32_t *__restrict__ big,
-                                                                    const unsigned int *__restrict__ nbig_p,
-                                                                    unsigned int *__restrict__ next)
+// The packed hits sh[0, cnt) of one read to out[0, cnt), sorted by (pos,
+// strand), by the `nt` threads `tid` of a warp or a block.  Hits within `span`
+// positions of each other (those of a tandem array) are ordered by counting:
+// a bit per (position, strand) from the first one (no two hits share one), a
+// prefix sum over the words' bit counts, and each hit goes to the number of
+// bits below its own; else a bitonic sort, for which sh holds a power of two
+// of entries.
+template <bool BLOCK>
+__device__ __forceinline__ void sort_hits(uint64_t *sh, uint32_t cnt, uint32_t *bits, uint32_t *pre, uint32_t span,
+                                          uint64_t *__restrict__ out, uint32_t tid, uint32_t nt)
 {
-    __shared__ uint64_t shw[WARP_SORT_WARPS][WARP_SORT];
-    const unsigned lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    uint64_t *sh = shw[wi];
-    const unsigned nbig = *nbig_p;
-    for (;;) {
-        unsigned bi = 0;
-        if (lane == 0) bi = atomicAdd(next, 1u);
-        bi = __shfl_sync(0xffffffffu, bi, 0);
-        if (bi >= nbig) break;
-        const uint32_t r = big[bi];
-        const uint64_t b = hit_off[r], cnt = hit_off[r + 1] - b;
-        if (cnt > WARP_SORT) continue;
-        uint32_t P = 1;
-        while (P < cnt) P <<= 1;
-        // the packed hits themselves (below 2^48), padded with ~0, ordered by (pos, strand)
-        for (uint32_t i = lane; i < P; i += 32) sh[i] = i < cnt ? hits[b + i] : ~0ull;
-        __syncwarp();
-        bitonic_hits<false>(sh, P, lane, 32);
-        for (uint32_t i = lane; i < cnt; i += 32) hits[b + i] = sh[i];
-        __syncwarp();
+    __shared__ uint32_t red[2][LONG_THREADS / 32];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t lo = 0xffffffffu, hi = 0;
+    for (uint32_t i = tid; i < cnt; i += nt) {
+        const uint32_t p = (uint32_t)sh[i];
+        lo = min(lo, p);
+        hi = max(hi, p);
     }
+    lo = __reduce_min_sync(FULL, lo);
+    hi = __reduce_max_sync(FULL, hi);
+    if (BLOCK) {
+        if (lane == 0) { red[0][warp] = lo; red[1][warp] = hi; }
+        __syncthreads();
+        for (uint32_t w = 0; w < nt / 32; w++) { lo = min(lo, red[0][w]); hi = max(hi, red[1][w]); }
+        __syncthreads();
+    }
+    if (hi - lo < span) {
+        const uint32_t words = (hi - lo) / 16u + 1u, per = (words + nt - 1) / nt;
+        for (uint32_t i = tid; i < words; i += nt) bits[i] = 0;
+        if (BLOCK) __syncthreads(); else __syncwarp();
+        for (uint32_t i = tid; i < cnt; i += nt) {
+            const uint32_t k = 2u * ((uint32_t)sh[i] - lo) + (uint32_t)((sh[i] >> 32) & 1u);
+            atomicOr(&bits[k >> 5], 1u << (k & 31u));
+        }
+        if (BLOCK) __syncthreads(); else __syncwarp();
+        uint32_t sum = 0;
+        for (uint32_t i = tid * per; i < min(words, (tid + 1) * per); i++) sum += __popc(bits[i]);
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, incl, o);
+            if ((int)lane >= o) incl += y;
+        }
+        uint32_t base = incl - sum;
+        if (BLOCK) {
+            if (lane == 31) red[0][warp] = incl;
+            __syncthreads();
+            for (uint32_t w = 0; w < warp; w++) base += red[0][w];
+        }
+        for (uint32_t i = tid * per; i < min(words, (tid + 1) * per); i++) { pre[i] = base; base += __popc(bits[i]); }
+        if (BLOCK) __syncthreads(); else __syncwarp();
+        for (uint32_t i = tid; i < cnt; i += nt) {
+            const uint64_t h = sh[i];
+            const uint32_t k = 2u * ((uint32_t)h - lo) + (uint32_t)((h >> 32) & 1u);
+            out[pre[k >> 5] + __popc(bits[k >> 5] & ((1u << (k & 31u)) - 1u))] = h;
+        }
+        return;
+    }
+    uint32_t P = 1;
+    while (P < cnt) P <<= 1;
+    for (uint32_t i = cnt + tid; i < P; i += nt) sh[i] = ~0ull;
+    if (BLOCK) __syncthreads(); else __syncwarp();
+    bitonic_hits<BLOCK>(sh, P, tid, nt);
+    for (uint32_t i = tid; i < cnt; i += nt) out[i] = sh[i];
 }
 
-// Reads with WARP_SORT < hits <= SMEM_SORT: one block of 128 threads each,
-// taken by a counter.
-__global__ void __launch_bounds__(BLOCK_SORT_THREADS) k_sort_block(uint64_t *__restrict__ hits,
-                                                                   const uint64_t *__restrict__ hit_off,
-                                                                   const uint32_t *__restrict__ big,
-                                                                   const unsigned int *__restrict__ nbig_p,
-                                                                   unsigned int *__restrict__ next)
+// Reads of up to WARP_HITS hits and intervals: one warp each, taken from the
+// list by a counter (reads differ a lot in size: a fixed stride left one warp
+// with the largest).  Each lane holds up to eight intervals in registers.
+__global__ void __launch_bounds__(WARP_READS * 32) k_finish_warp(const FinishArgs a)
 {
-    __shared__ uint64_t sh[SMEM_SORT];
-    __shared__ unsigned bi_s;
-    const unsigned nbig = *nbig_p;
+    __shared__ uint64_t sh_s[WARP_READS][WARP_HITS];
+    __shared__ uint32_t bits_s[WARP_READS][WARP_SPAN / 16], pre_s[WARP_READS][WARP_SPAN / 16];
+    if (*(volatile unsigned *)&a.ctl->error) return;
+    const uint32_t lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    uint64_t *sh = sh_s[wi];
+    const unsigned n_list = a.ctl->n_warp;
+    uint32_t steps = 0;
+    constexpr uint32_t PER = WARP_HITS / 32;
     for (;;) {
-        if (threadIdx.x == 0) bi_s = atomicAdd(next, 1u);
+        unsigned bi = 0;
+        if (lane == 0) bi = atomicAdd(&a.ctl->next_warp, 1u);
+        bi = __shfl_sync(FULL, bi, 0);
+        if (bi >= n_list) break;
+        const uint32_t r = a.lists[bi];
+        const uint64_t b = a.iv_off[r], q0 = a.hit_off[r], t = a.total[r];
+        const uint32_t ni = (uint32_t)(a.iv_off[r + 1] - b), keep = (uint32_t)(a.hit_off[r + 1] - q0);
+        uint32_t l[PER], sz[PER], meta[PER];
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) {
+            const uint32_t x = i * 32 + lane;
+            l[i] = sz[i] = meta[i] = 0;
+            if (x < ni) {
+                const Interval v = a.ivs[b + x];
+                l[i] = v.l; sz[i] = v.r - v.l; meta[i] = v.meta;
+            }
+        }
+        if (t > keep) {
+            // over the cap: the first keep rows in the order (d, strand, row).  Interval keys are
+            // distinct, so a bitwise search from the top key bit finds the key K at which the rows
+            // counted in key order reach keep (sizes cut at 2^16, more than any cap taken here)
+            uint64_t key[PER];
+#pragma unroll
+            for (uint32_t i = 0; i < PER; i++) {
+                Interval v;
+                v.l = l[i]; v.r = l[i] + sz[i]; v.meta = meta[i]; v.read = r;
+                if (sz[i]) to_rows(v, a.ix.isa);
+                l[i] = v.l; meta[i] = v.meta;
+                key[i] = iv_key(v);
+                if (sz[i] == 0) key[i] = ~0ull;
+                sz[i] = min(sz[i], WARP_CAP + 1u);
+            }
+            uint64_t prefix = 0;
+            uint32_t before = 0;
+            for (int bit = 34; bit >= 0; bit--) {
+                const uint64_t hi = prefix >> (bit + 1);
+                uint32_t z = 0;
+#pragma unroll
+                for (uint32_t i = 0; i < PER; i++)
+                    if ((key[i] >> (bit + 1)) == hi && !((key[i] >> bit) & 1u)) z += sz[i];
+                z = __reduce_add_sync(FULL, z);
+                if (before + z < keep) { before += z; prefix |= 1ull << bit; }
+            }
+#pragma unroll
+            for (uint32_t i = 0; i < PER; i++) {
+                if (key[i] == prefix) sz[i] = keep - before;
+                else if (key[i] > prefix) sz[i] = 0;
+            }
+        }
+        // the rows' hits, lane by lane; an interval of several rows by the whole warp
+        uint32_t mine = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) mine += sz[i];
+        uint32_t at = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, at, o);
+            if ((int)lane >= o) at += y;
+        }
+        at -= mine;
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) {
+            if (sz[i] == 1) sh[at] = hit_of(a.ix, l[i], meta[i]);
+            for (unsigned todo = __ballot_sync(FULL, sz[i] > 1); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t wl = __shfl_sync(FULL, l[i], src), wz = __shfl_sync(FULL, sz[i], src);
+                const uint32_t wm = __shfl_sync(FULL, meta[i], src), wa = __shfl_sync(FULL, at, src);
+                for (uint32_t x = lane; x < wz; x += 32) sh[wa + x] = hit_of(a.ix, wl + x, wm);
+            }
+            at += sz[i];
+        }
+        __syncwarp();
+        if (!a.ix.sa_ctx) {
+            locate_hits(a.ix, sh, keep, lane, 32, steps);
+            __syncwarp();
+        }
+        sort_hits<false>(sh, keep, bits_s[wi], pre_s[wi], WARP_SPAN, a.hits + q0, lane, 32);
+        __syncwarp();
+    }
+    if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
+}
+
+// Where a block cuts a read's list of intervals ivs[b, e) with more than cap
+// rows: the first cap rows in the order (d, strand, row) are the intervals of
+// the classes (d, strand) before `cls`, those of cls whose row is below `row`,
+// and the first `take` rows of cls's interval at `row`.
+struct Cut {
+    uint32_t cls, row, take;
+};
+
+__device__ __forceinline__ uint32_t iv_class(const Interval &x) { return ((x.meta & 3u) << 1) | ((x.meta >> 2) & 1u); }
+
+// The rows per class come first (no row is looked up for that); then the class
+// that crosses the cap is searched by its rows, eight bits a pass: a pass sums
+// the rows under each of the 256 next values.
+template <uint32_t NT>
+__device__ __forceinline__ Cut find_cut(Interval *ivs, uint64_t b, uint64_t e, uint32_t cap,
+                                        const uint32_t *__restrict__ isa, unsigned long long *hist, uint32_t *found)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    uint64_t in_class[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (uint64_t i = b + tid; i < e; i += NT) {
+        const Interval x = ivs[i];
+        const uint32_t c = iv_class(x), z = x.r - x.l;
+#pragma unroll
+        for (uint32_t q = 0; q < 8; q++) in_class[q] += c == q ? z : 0u;
+    }
+    if (tid < 8) hist[tid] = 0;
+    __syncthreads();
+#pragma unroll
+    for (uint32_t q = 0; q < 8; q++) {
+        uint64_t v = in_class[q];
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        if (lane == 0 && v) atomicAdd(&hist[q], (unsigned long long)v);
+    }
+    __syncthreads();
+    Cut c{0, 0, 0};
+    uint64_t before = 0;
+    while (before + hist[c.cls] < cap) before += hist[c.cls++];
+    __syncthreads();
+    for (int sh = 24; sh >= 0; sh -= 8) {
+        for (uint32_t i = tid; i < 256; i += NT) hist[i] = 0;
+        __syncthreads();
+        for (uint64_t i = b + tid; i < e; i += NT) {
+            Interval x = ivs[i];
+            if (iv_class(x) != c.cls || x.r <= x.l) continue;
+            if (sh == 24 && (x.meta & IV_POS)) {
+                to_rows(x, isa);
+                ivs[i] = x;   // (the passes keep this stride)
+            }
+            if (((uint64_t)x.l >> (sh + 8)) == ((uint64_t)c.row >> (sh + 8)))
+                atomicAdd(&hist[(x.l >> sh) & 255u], (unsigned long long)(x.r - x.l));
+        }
+        __syncthreads();
+        if (tid < 32) {
+            uint64_t part[8], sum = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++) { part[i] = hist[lane * 8 + i]; sum += part[i]; }
+            uint64_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t y = __shfl_up_sync(FULL, incl, o);
+                if ((int)lane >= o) incl += y;
+            }
+            uint64_t run = before + incl - sum;   // rows before this lane's values
+            // the first value with which the rows counted reach the cap
+            int digit = -1;
+            uint64_t rows = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                if (digit < 0 && run + part[i] >= cap) { digit = (int)lane * 8 + i; rows = run; }
+                run += part[i];
+            }
+            const unsigned has = __ballot_sync(FULL, digit >= 0);
+            if ((int)lane == __ffs(has) - 1) { found[0] = (uint32_t)digit; found[1] = (uint32_t)rows; }
+        }
+        __syncthreads();
+        c.row |= found[0] << sh;
+        before = found[1];   // (less than cap)
+        __syncthreads();
+    }
+    c.take = cap - (uint32_t)before;
+    return c;
+}
+
+// The read's listed rows as hits to out[0, ...), in no order, by a block: all
+// rows of its intervals, or those the cut keeps.  count: in shared memory.
+template <uint32_t NT>
+__device__ __forceinline__ void expand_block(const IndexView &ix, const Interval *ivs, uint64_t b, uint64_t e, bool over,
+                                             const Cut &c, uint64_t *out, unsigned long long *count)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) *count = 0;
+    __syncthreads();
+    for (uint64_t c0 = b + (threadIdx.x & ~31u); c0 < e; c0 += NT) {
+        Interval x{};
+        if (c0 + lane < e) x = ivs[c0 + lane];
+        uint32_t sz = x.r - x.l;
+        if (over && sz) {
+            const uint32_t k = iv_class(x);
+            if (k > c.cls || (k == c.cls && x.l > c.row)) sz = 0;
+            else if (k == c.cls && x.l == c.row) sz = c.take;
+        }
+        uint32_t incl = sz;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, incl, o);
+            if ((int)lane >= o) incl += y;
+        }
+        unsigned long long at = 0;
+        if (lane == 31 && incl) at = atomicAdd(count, (unsigned long long)incl);
+        at = __shfl_sync(FULL, at, 31) + incl - sz;
+        if (sz == 1) out[at] = hit_of(ix, x.l, x.meta);
+        for (unsigned todo = __ballot_sync(FULL, sz > 1); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const uint32_t wl = __shfl_sync(FULL, x.l, src), wz = __shfl_sync(FULL, sz, src);
+            const uint32_t wm = __shfl_sync(FULL, x.meta, src);
+            const unsigned long long wa = __shfl_sync(FULL, at, src);
+            for (uint32_t i = lane; i < wz; i += 32) out[wa + i] = hit_of(ix, wl + i, wm);
+        }
+    }
+    __syncthreads();
+}
+
+// Larger reads (up to BLOCK_HITS hits): one block each, taken by a counter.
+// Those with the longest lists (a read in a diverged tandem array has 10^5
+// intervals of a row each) have blocks of 1,024 threads: 128 took 0.65 ms
+// for the longest of a million reads.
+template <uint32_t NT>
+__global__ void __launch_bounds__(NT) k_finish_block(const FinishArgs a)
+{
+    __shared__ uint64_t sh[BLOCK_HITS];
+    __shared__ uint32_t bits[BLOCK_SPAN / 16], pre[BLOCK_SPAN / 16];
+    __shared__ unsigned long long count;
+    __shared__ uint32_t found[2];
+    __shared__ unsigned bi_s;
+    if (*(volatile unsigned *)&a.ctl->error) return;
+    constexpr bool LONG = NT == LONG_THREADS;
+    const unsigned n_list = LONG ? a.ctl->n_long : a.ctl->n_block;
+    uint32_t steps = 0;
+    for (;;) {
+        if (threadIdx.x == 0) bi_s = atomicAdd(LONG ? &a.ctl->next_long : &a.ctl->next_block, 1u);
         __syncthreads();
         const unsigned bi = bi_s;
         __syncthreads();
-        if (bi >= nbig) break;
-        const uint32_t r = big[bi];
-        const uint64_t b = hit_off[r], cnt = hit_off[r + 1] - b;
-        if (cnt <= WARP_SORT) continue;
-        uint32_t P = 1;
-        while (P < cnt) P <<= 1;
-        for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) sh[i] = i < cnt ? hits[b + i] : ~0ull;
-        __syncthreads();
-        bitonic_hits<true>(sh, P, threadIdx.x, blockDim.x);
-        for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) hits[b + i] = sh[i];
+        if (bi >= n_list) break;
+        const uint32_t r = (LONG ? a.huge : a.lists)[a.n - 1 - bi];
+        const uint64_t b = a.iv_off[r], e = a.iv_off[r + 1], q0 = a.hit_off[r];
+        const uint32_t keep = (uint32_t)(a.hit_off[r + 1] - q0);
+        const bool over = a.total[r] > keep;
+        Cut c{0, 0, 0};
+        if (over) c = find_cut<NT>(a.ivs, b, e, a.cap, a.ix.isa, (unsigned long long *)sh, found);
+        expand_block<NT>(a.ix, a.ivs, b, e, over, c, sh, &count);
+        if (!a.ix.sa_ctx) {
+            locate_hits(a.ix, sh, keep, threadIdx.x, NT, steps);
+            __syncthreads();
+        }
+        sort_hits<true>(sh, keep, bits, pre, BLOCK_SPAN, a.hits + q0, threadIdx.x, NT);
         __syncthreads();
     }
+    if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
 }
 
-// one read with more than SMEM_SORT hits: bitonic network over a global scratch
+// Reads above BLOCK_HITS hits (only without a cap or with a cap above it): a
+// block each writes the hits, not yet in order.
+__global__ void __launch_bounds__(LONG_THREADS) k_finish_huge(const FinishArgs a, uint32_t n_huge)
+{
+    __shared__ unsigned long long hist[256], count;
+    __shared__ uint32_t found[2];
+    uint32_t steps = 0;
+    for (uint32_t i = blockIdx.x; i < n_huge; i += gridDim.x) {
+        const uint32_t r = a.huge[i];
+        const uint64_t b = a.iv_off[r], e = a.iv_off[r + 1], q0 = a.hit_off[r];
+        const bool over = a.total[r] > a.hit_off[r + 1] - q0;
+        Cut c{0, 0, 0};
+        if (over) c = find_cut<LONG_THREADS>(a.ivs, b, e, a.cap, a.ix.isa, hist, found);
+        expand_block<LONG_THREADS>(a.ix, a.ivs, b, e, over, c, a.hits + q0, &count);
+        if (!a.ix.sa_ctx) locate_hits(a.ix, a.hits + q0, count, threadIdx.x, LONG_THREADS, steps);
+        __syncthreads();
+    }
+    if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
+}
+
+// one read with more than BLOCK_HITS hits: bitonic network over a global scratch
 __global__ void __launch_bounds__(1024) k_sort_global(uint64_t *__restrict__ hits, uint64_t cnt,
                                                       uint64_t *__restrict__ scratch, uint64_t P)
 {
@@ -598,81 +904,81 @@ static uint64_t big_list_bytes(uint64_t n)
     return (std::max<uint64_t>(n, 1) * 4 + 15) & ~15ull;
 }
 
-// w.big holds: the sort lists (n u32), 64 bytes of counters (locate steps
-// u64, sort-list counts u32[2], many-interval count u32, the two sort
-// kernels' next-read counters u32[2]), then the list of reads with many
-// intervals (n u32).
-struct PostLists {
-    uint32_t *sort_lists;
-    unsigned long long *steps;
-    unsigned int *nbig;       // [0] reads for the shared-memory sorts, [1] above them
-    unsigned int *n_many;
-    unsigned int *sort_next;  // [0] k_sort_warp's next listed read, [1] k_sort_block's
-    uint32_t *many;
-};
+// w.big holds the list of reads for k_finish_warp and k_finish_block (a read
+// is on one of them: n u32), then the list of larger ones (n u32); w.scan_tmp
+// the tile sums of the interval counts, then of the listed hits.
+static uint64_t post_list_bytes(uint64_t n) { return 2 * big_list_bytes(n); }
+static uint64_t tiles_of(uint64_t n) { return std::max<uint64_t>(1, (n + TILE - 1) / TILE); }
+static uint64_t tile_bytes(uint64_t n) { return (2 * tiles_of(n) + 1) * 8; }
 
-static uint64_t post_list_bytes(uint64_t n) { return 2 * big_list_bytes(n) + 64; }
-
-static PostLists post_lists(Workspace &w, uint64_t n)
+static FinishArgs finish_args(const mica_index *idx, Workspace &w, uint64_t n, uint32_t hit_cap, uint64_t capacity)
 {
-    PostLists p;
-    char *base = (char *)w.big.p;
-    p.sort_lists = (uint32_t *)base;
-    p.steps = (unsigned long long *)(base + big_list_bytes(n));
-    p.nbig = (unsigned int *)(p.steps + 1);
-    p.n_many = p.nbig + 2;
-    p.sort_next = p.nbig + 3;
-    p.many = (uint32_t *)(base + big_list_bytes(n) + 64);
-    return p;
+    FinishArgs a;
+    a.ix = idx->view;
+    a.ivs = (Interval *)w.iv_sorted.p;
+    a.iv_off = (const uint64_t *)w.iv_off.p;
+    a.total = (const uint64_t *)w.total.p;
+    a.hit_off = (uint64_t *)w.hit_off.p;
+    a.hits = (uint64_t *)w.hits.p;
+    a.n = n;
+    a.capacity = capacity;
+    a.cap = hit_cap;
+    a.lists = (uint32_t *)w.big.p;
+    a.huge = (uint32_t *)((char *)w.big.p + big_list_bytes(n));
+    a.ctl = (SearchCtl *)w.ctl.p;
+    return a;
+}
+
+// Steps 1 to 3: intervals grouped by read, totals, tile sums of the listed hits.
+static int enqueue_totals(Workspace &w, uint64_t n, uint32_t hit_cap, uint32_t report, cudaStream_t s, uint64_t &L)
+{
+    uint64_t *iv_off = (uint64_t *)w.iv_off.p, *sums = (uint64_t *)w.scan_tmp.p;
+    SearchCtl *ctl = (SearchCtl *)w.ctl.p;
+    const unsigned tiles = (unsigned)tiles_of(n);
+    if (tiles > 1) {
+        k_tile_counts<<<tiles, TILE_THREADS, 0, s>>>((const uint32_t *)w.iv_cnt.p, n, sums);
+        L++;
+    }
+    unsigned long long *total = (unsigned long long *)w.total.p;
+    k_offsets<<<tiles, TILE_THREADS, 0, s>>>((const uint32_t *)w.iv_cnt.p, n, sums, iv_off, (uint64_t *)total);
+    const unsigned g = (unsigned)std::min<uint64_t>(152 * 16, std::max<uint64_t>(8, n / 64));
+    k_iv_scatter<<<g, 256, 0, s>>>((const Interval *)w.iv.p, &ctl->iv_count, w.iv_cap, iv_off, (uint32_t *)w.iv_cnt.p,
+                                   (Interval *)w.iv_sorted.p, total, &ctl->error);
+    if (report == MICA_REPORT_BEST_STRATUM) {
+        k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, (uint64_t *)total, &ctl->error);
+        L++;
+    }
+    k_listed<<<tiles, TILE_THREADS, 0, s>>>((const uint64_t *)total, n, hit_cap, sums + tiles);
+    L += 3;
+    MICA_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
+// Steps 4 and 5.
+static int enqueue_finish(const FinishArgs &a, Workspace &w, cudaStream_t s, uint64_t &L)
+{
+    const unsigned tiles = (unsigned)tiles_of(a.n);
+    k_finish_small<<<tiles, TILE_THREADS, 0, s>>>(a, (const uint64_t *)w.scan_tmp.p + tiles);
+    const uint64_t n1 = std::max<uint64_t>(a.n, 1);
+    k_finish_block<LONG_THREADS><<<(unsigned)std::min<uint64_t>(152, n1), LONG_THREADS, 0, s>>>(a);
+    k_finish_warp<<<(unsigned)std::min<uint64_t>(152 * 8, n1), WARP_READS * 32, 0, s>>>(a);
+    k_finish_block<BLOCK_READ_THREADS><<<(unsigned)std::min<uint64_t>(152 * 5, n1), BLOCK_READ_THREADS, 0, s>>>(a);
+    L += 4;
+    MICA_CUDA_TRY(cudaGetLastError());
+    return 0;
 }
 
 // The whole post-search pipeline for one batch, enqueued with every count
 // read on the device (fixed grids, capacity-guarded writes) so it can be
 // captured in a CUDA graph.  Buffers must already hold `hit_capacity` hits.
-// Ends with a copy of the status (search control block, hit total, locate
-// steps and sort-list counts) into pinned host memory `status`.
+// Ends with a copy of the control block (the search's counters, the hit
+// total, locate steps and list counts) into pinned host memory `status`.
 int enqueue_post_device(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t hit_cap,
                         uint32_t report, uint64_t hit_capacity, cudaStream_t s, void *status, uint64_t &L)
 {
-    uint64_t n = rd.n;
-    uint64_t *iv_off = (uint64_t *)w.iv_off.p, *hit_off = (uint64_t *)w.hit_off.p;
-    PostLists pl = post_lists(w, n);
-    unsigned long long *steps = pl.steps;
-    unsigned int *nbig = pl.nbig;
-    SearchCtl *ctl = (SearchCtl *)w.ctl.p;
-    const unsigned G = 152 * 16;
-    int rc;
-    MICA_CUDA_TRY(cudaMemsetAsync(steps, 0, 64, s));
-    if ((rc = exclusive_scan<uint32_t>(w.scan_tmp, (const uint32_t *)w.iv_cnt.p, n, iv_off, s, L))) return rc;
-    k_iv_scatter<<<G, 256, 0, s>>>((const Interval *)w.iv.p, &ctl->iv_count, w.iv_cap, iv_off,
-                                   (uint32_t *)w.iv_cnt.p, (Interval *)w.iv_sorted.p, &ctl->error);
-    if (report == MICA_REPORT_BEST_STRATUM) {
-        k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, &ctl->error);
-        L++;
-    }
-    k_summarize<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, hit_cap, (uint64_t *)w.total.p,
-                                              (uint64_t *)w.keep.p, pl.many, pl.n_many, idx->view.isa,
-                                              &ctl->error);
-    k_summarize_many<<<152 * 2, MANY_THREADS, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, hit_cap,
-                                                      (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many,
-                                                      pl.n_many, idx->view.isa, &ctl->error);
-    L += 3;
-    if ((rc = exclusive_scan<uint64_t>(w.scan_tmp, (const uint64_t *)w.keep.p, n, hit_off, s, L))) return rc;
-    k_expand<<<grid1(n, 128), 128, 0, s>>>((const Interval *)w.iv_sorted.p, iv_off, hit_off, n, (Hit *)w.hits.p,
-                                           hit_capacity, &ctl->error);
-    k_locate<<<G, 256, 0, s>>>(idx->view, (Hit *)w.hits.p, hit_off + n, hit_capacity, steps, &ctl->error);
-    k_sort_small<<<grid1(n, 128), 128, 0, s>>>((uint64_t *)w.hits.p, hit_off, n, hit_capacity, (uint32_t *)w.big.p,
-                                               nbig);
-    k_sort_warp<<<152 * 4, WARP_SORT_WARPS * 32, 0, s>>>((uint64_t *)w.hits.p, hit_off, (const uint32_t *)w.big.p,
-                                                        nbig, pl.sort_next);
-    k_sort_block<<<152 * 8, BLOCK_SORT_THREADS, 0, s>>>((uint64_t *)w.hits.p, hit_off, (const uint32_t *)w.big.p,
-                                                        nbig, pl.sort_next + 1);
-    L += 5;
-    char *st = (char *)status;
-    MICA_CUDA_TRY(cudaMemcpyAsync(st, ctl, sizeof(SearchCtl), cudaMemcpyDeviceToHost, s));
-    MICA_CUDA_TRY(cudaMemcpyAsync(st + sizeof(SearchCtl), hit_off + n, 8, cudaMemcpyDeviceToHost, s));
-    MICA_CUDA_TRY(cudaMemcpyAsync(st + sizeof(SearchCtl) + 8, steps, 16, cudaMemcpyDeviceToHost, s));
-    MICA_CUDA_TRY(cudaGetLastError());
+    if (int rc = enqueue_totals(w, rd.n, hit_cap, report, s, L)) return rc;
+    if (int rc = enqueue_finish(finish_args(idx, w, rd.n, hit_cap, hit_capacity), w, s, L)) return rc;
+    MICA_CUDA_TRY(cudaMemcpyAsync(status, w.ctl.p, sizeof(SearchCtl), cudaMemcpyDeviceToHost, s));
     return 0;
 }
 
@@ -680,19 +986,17 @@ int enqueue_post_device(const mica_index *idx, Workspace &w, const ReadsView &rd
 // Device bytes reserve_post takes for n reads (the sizes below).
 uint64_t post_workspace_bytes(uint64_t n, uint64_t iv_cap, uint64_t hit_capacity)
 {
-    uint64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    return std::max<uint64_t>(iv_cap, 1) * sizeof(Interval) + 2 * (n + 1) * 8 + 2 * std::max<uint64_t>(n, 1) * 8 +
-           post_list_bytes(n) + (ntiles + 1) * 8 + std::max<uint64_t>(hit_capacity, 1) * sizeof(Hit) + 64;
+    return std::max<uint64_t>(iv_cap, 1) * sizeof(Interval) + 2 * (n + 1) * 8 + std::max<uint64_t>(n, 1) * 8 +
+           post_list_bytes(n) + tile_bytes(n) + std::max<uint64_t>(hit_capacity, 1) * sizeof(Hit) + 64;
 }
 
 int reserve_post(Workspace &w, uint64_t n, uint32_t iv_cap, uint64_t hit_capacity)
 {
     int rc;
-    uint64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     if ((rc = dev_reserve(w.iv_sorted, std::max<uint64_t>(iv_cap, 1) * sizeof(Interval))) ||
         (rc = dev_reserve(w.iv_off, (n + 1) * 8)) || (rc = dev_reserve(w.total, std::max<uint64_t>(n, 1) * 8)) ||
-        (rc = dev_reserve(w.keep, std::max<uint64_t>(n, 1) * 8)) || (rc = dev_reserve(w.hit_off, (n + 1) * 8)) ||
-        (rc = dev_reserve(w.big, post_list_bytes(n))) || (rc = dev_reserve(w.scan_tmp, (ntiles + 1) * 8)) ||
+        (rc = dev_reserve(w.hit_off, (n + 1) * 8)) || (rc = dev_reserve(w.big, post_list_bytes(n))) ||
+        (rc = dev_reserve(w.scan_tmp, tile_bytes(n))) ||
         (rc = dev_reserve(w.hits, std::max<uint64_t>(hit_capacity, 1) * sizeof(Hit) + 64)))
         return rc;
     return 0;
@@ -701,69 +1005,37 @@ int reserve_post(Workspace &w, uint64_t n, uint32_t iv_cap, uint64_t hit_capacit
 int run_post(const mica_index *idx, Workspace &w, mica_stats &stt, const ReadsView &rd, uint32_t hit_cap,
              uint32_t report, cudaStream_t s, uint64_t *n_hits_out)
 {
-    uint64_t n = rd.n;
-    uint32_t niv = (uint32_t)stt.intervals;
+    const uint64_t n = rd.n;
     int rc;
-    if ((rc = dev_reserve(w.iv_sorted, std::max<uint64_t>(niv, 1) * sizeof(Interval))) ||
-        (rc = dev_reserve(w.iv_off, (n + 1) * 8)) || (rc = dev_reserve(w.total, std::max<uint64_t>(n, 1) * 8)) ||
-        (rc = dev_reserve(w.keep, std::max<uint64_t>(n, 1) * 8)) || (rc = dev_reserve(w.hit_off, (n + 1) * 8)) ||
-        (rc = dev_reserve(w.big, post_list_bytes(n))))
-        return rc;
-    uint64_t *iv_off = (uint64_t *)w.iv_off.p, *hit_off = (uint64_t *)w.hit_off.p;
+    if ((rc = reserve_post(w, n, (uint32_t)stt.intervals, 1))) return rc;
     uint64_t &L = stt.launches;
-    PostLists pl = post_lists(w, n);
-    unsigned long long *steps = pl.steps;
-    unsigned int *nbig = pl.nbig;
-    MICA_CUDA_TRY(cudaMemsetAsync(steps, 0, 64, s));
-    if ((rc = exclusive_scan<uint32_t>(w.scan_tmp, (const uint32_t *)w.iv_cnt.p, n, iv_off, s, L))) return rc;
-    const unsigned int *err = &((SearchCtl *)w.ctl.p)->error;
-    if (niv) { k_iv_scatter<<<grid1(niv), 256, 0, s>>>((const Interval *)w.iv.p, &((SearchCtl *)w.ctl.p)->iv_count,
-                                                       w.iv_cap, iv_off, (uint32_t *)w.iv_cnt.p,
-                                                       (Interval *)w.iv_sorted.p, err); L++; }
-    if (n && report == MICA_REPORT_BEST_STRATUM) {
-        k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, err);
-        L++;
-    }
-    if (n) {
-        k_summarize<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, hit_cap,
-                                                  (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many, pl.n_many,
-                                                  idx->view.isa, err);
-        k_summarize_many<<<152 * 2, MANY_THREADS, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, hit_cap,
-                                                          (uint64_t *)w.total.p, (uint64_t *)w.keep.p, pl.many,
-                                                          pl.n_many, idx->view.isa, err);
-        L += 2;
-    }
-    if ((rc = exclusive_scan<uint64_t>(w.scan_tmp, (const uint64_t *)w.keep.p, n, hit_off, s, L))) return rc;
+    SearchCtl *ctl = (SearchCtl *)w.ctl.p;
+    // the control block's post-search fields (a search may have run in several launches)
+    MICA_CUDA_TRY(cudaMemsetAsync(&ctl->post_hits, 0, sizeof(SearchCtl) - offsetof(SearchCtl, post_hits), s));
+    if ((rc = enqueue_totals(w, n, hit_cap, report, s, L))) return rc;
+    const unsigned tiles = (unsigned)tiles_of(n);
+    uint64_t *sums = (uint64_t *)w.scan_tmp.p;
+    k_tiles_total<<<1, TILE_THREADS, 0, s>>>(sums + tiles, tiles, sums + 2 * tiles);
+    L++;
     uint64_t nh = 0;
-    MICA_CUDA_TRY(cudaMemcpyAsync(&nh, hit_off + n, 8, cudaMemcpyDeviceToHost, s));
+    MICA_CUDA_TRY(cudaMemcpyAsync(&nh, sums + 2 * tiles, 8, cudaMemcpyDeviceToHost, s));
     MICA_CUDA_TRY(cudaStreamSynchronize(s));
     if ((rc = dev_reserve(w.hits, std::max<uint64_t>(nh, 1) * sizeof(Hit) + 64))) return rc;
-    if (n) { k_expand<<<grid1(n, 128), 128, 0, s>>>((const Interval *)w.iv_sorted.p, iv_off, hit_off, n,
-                                                   (Hit *)w.hits.p, nh, err); L++; }
-    if (nh) { k_locate<<<grid1(nh), 256, 0, s>>>(idx->view, (Hit *)w.hits.p, hit_off + n, nh, steps, err); L++; }
-    if (n) { k_sort_small<<<grid1(n, 128), 128, 0, s>>>((uint64_t *)w.hits.p, hit_off, n, nh, (uint32_t *)w.big.p,
-                                                       nbig); L++; }
-    unsigned int hb[2] = {0, 0};
-    unsigned long long st = 0;
-    MICA_CUDA_TRY(cudaMemcpyAsync(&st, steps, 8, cudaMemcpyDeviceToHost, s));
-    MICA_CUDA_TRY(cudaMemcpyAsync(hb, nbig, 8, cudaMemcpyDeviceToHost, s));
+    const FinishArgs a = finish_args(idx, w, n, hit_cap, nh);
+    if ((rc = enqueue_finish(a, w, s, L))) return rc;
+    SearchCtl out;
+    MICA_CUDA_TRY(cudaMemcpyAsync(&out, ctl, sizeof(out), cudaMemcpyDeviceToHost, s));
     MICA_CUDA_TRY(cudaStreamSynchronize(s));
-    if (hb[0]) {
-        k_sort_warp<<<std::min((hb[0] + WARP_SORT_WARPS - 1) / WARP_SORT_WARPS, 152u * 4), WARP_SORT_WARPS * 32, 0,
-                      s>>>((uint64_t *)w.hits.p, hit_off, (const uint32_t *)w.big.p, nbig, pl.sort_next);
-        k_sort_block<<<std::min(hb[0], 152u * 8), BLOCK_SORT_THREADS, 0, s>>>(
-            (uint64_t *)w.hits.p, hit_off, (const uint32_t *)w.big.p, nbig, pl.sort_next + 1);
-        L += 2;
-    }
-    if (hb[1]) {
-        // reads above the shared-memory size (only without a cap or with a cap above it)
-        std::vector<uint32_t> huge(hb[1]);
-        MICA_CUDA_TRY(cudaMemcpyAsync(huge.data(), (const uint32_t *)w.big.p + (n - hb[1]), 4ull * hb[1],
-                                      cudaMemcpyDeviceToHost, s));
+    if (out.n_huge) {
+        k_finish_huge<<<std::min(out.n_huge, 152u), LONG_THREADS, 0, s>>>(a, out.n_huge);
+        L++;
+        std::vector<uint32_t> huge(out.n_huge);
+        MICA_CUDA_TRY(cudaMemcpyAsync(huge.data(), a.huge, 4ull * out.n_huge, cudaMemcpyDeviceToHost, s));
+        MICA_CUDA_TRY(cudaMemcpyAsync(&out, ctl, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
         for (uint32_t r : huge) {
             uint64_t ob[2];
-            MICA_CUDA_TRY(cudaMemcpy(ob, hit_off + r, 16, cudaMemcpyDeviceToHost));
+            MICA_CUDA_TRY(cudaMemcpy(ob, a.hit_off + r, 16, cudaMemcpyDeviceToHost));
             uint64_t cnt = ob[1] - ob[0];
             uint64_t P = 1;
             while (P < cnt) P <<= 1;
@@ -777,7 +1049,7 @@ int run_post(const mica_index *idx, Workspace &w, mica_stats &stt, const ReadsVi
     }
     MICA_CUDA_TRY(cudaGetLastError());
     stt.located = nh;
-    stt.lf_steps = st;
+    stt.lf_steps = out.lf_steps;
     *n_hits_out = nh;
     return 0;
 }
