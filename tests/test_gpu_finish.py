@@ -1,0 +1,98 @@
+"""The kernels that finish reads of different sizes (a thread, a warp, a block,
+a block for long interval lists, the host's loop) and pair mates with few or
+many hits, at the sizes where one hands over to the next."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests import gpu_common as gc
+
+pytestmark = pytest.mark.gpu
+
+
+def _genome_with_copies(copies, unit=60, gap=41, seed=3):
+    """`copies` copies of one random unit, `gap` random bases apart, in a random genome."""
+    rng = np.random.default_rng(seed)
+    u = rng.integers(0, 4, size=unit, dtype=np.uint8)
+    parts = [rng.integers(0, 4, size=500, dtype=np.uint8)]
+    for _ in range(copies):
+        parts += [u, rng.integers(0, 4, size=gap, dtype=np.uint8)]
+    return np.concatenate(parts), u
+
+
+@pytest.mark.parametrize("copies", [1, 2, 8, 9, 31, 33, 255, 256, 257, 4095, 4097])
+@pytest.mark.parametrize("full_sa", [True, False])
+def test_hit_counts_around_the_kernels_limits(copies, full_sa):
+    """A read with exactly `copies` exact placements (spread wider than the
+    counting sort's span from about 40 and 200 copies up), beside an ordinary one, under caps below, at
+    and above that number."""
+    g, u = _genome_with_copies(copies)
+    reads = [u, (3 - u)[::-1].copy(), g[:60].copy()]
+    b = gc.batch_from_reads(reads, [0, 0, 1])
+    fm = oracle.FMIndex(g)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g), kmer_q=10, sa_sample=8, full_sa=full_sa)
+    for cap in sorted({1, max(1, copies - 1), copies, copies + 1, 0}):
+        gc.assert_same(idx.align_batch(b, hit_cap=cap), fm.align(b, cap=cap), f"copies {copies} cap {cap}")
+    idx.free()
+
+
+@pytest.mark.parametrize("cap", [1, 10, 255, 1000, 4096, 5000, 70_000, 0])
+def test_long_interval_lists_under_caps(cap):
+    """Reads inside a diverged array have thousands of one-row intervals in
+    several (d, strand) classes, more than a warp or a small block holds."""
+    rng = np.random.default_rng(11)
+    core = np.resize(np.array([0, 1, 2], np.uint8), 30_000)
+    mut = rng.random(core.size) < 0.03
+    core[mut] = (core[mut] + rng.integers(1, 4, size=int(mut.sum()))) & 3
+    g = np.concatenate([rng.integers(0, 4, 3_000).astype(np.uint8), core])
+    reads = [g[3_000 + 700 * i: 3_000 + 700 * i + 36].copy() for i in range(12)]
+    b = gc.batch_from_reads(reads, [0, 1, 2, 3] * 3)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g), kmer_q=10, sa_sample=8)
+    gc.assert_same(idx.align_batch(b, hit_cap=cap), oracle.FMIndex(g).align(b, cap=cap), f"cap {cap}")
+    idx.free()
+
+
+@pytest.mark.parametrize("n", [1, 511, 512, 513, 1025])
+def test_batch_sizes_around_a_tile(n):
+    """Batches that end before, at and after a tile of the prefix sums."""
+    g = synth.uniform_genome(50_000, 5)
+    rng = np.random.default_rng(n)
+    b = synth.sample_reads(g, rng.integers(20, 90, n), rng.integers(0, 3, n), rng, subs="rate", sub_rate=0.02)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), kmer_q=9, sa_sample=8)
+    gc.assert_same(idx.align_batch(b, hit_cap=3), oracle.FMIndex(g.codes).align(b, cap=3), f"n {n}")
+    idx.free()
+
+
+@pytest.mark.parametrize("sizes", [(4, 4), (4, 5), (1, 40), (33, 64), (300, 500), (0, 9), (1000, 1000)])
+def test_pairs_of_many_hits(sizes):
+    """Mates with few and many hits (some windows hold every hit of the other
+    mate), ties included."""
+    rng = np.random.default_rng(sum(sizes))
+    m = gc.mica()
+    for span, lo, hi in ((400, 0, 5_000), (4_000, 300, 700), (3_000, 450, 450)):
+        lists = []
+        for _ in range(3):
+            for n in sizes:
+                pick = rng.choice(2 * span, size=min(n, 2 * span), replace=False)
+                lists.append(sorted((int(x) // 2, int(x) % 2, int(rng.integers(0, 3))) for x in pick))
+        off = np.concatenate([[0], np.cumsum([len(x) for x in lists])]).astype(np.uint64)
+        hits = np.zeros(int(off[-1]), dtype=m.HIT_DTYPE)
+        for j, h in enumerate(h for x in lists for h in x):
+            hits[j] = (*h, 0)
+
+        class R:
+            offsets = off
+
+            @staticmethod
+            def as_tuples(i):
+                return lists[i]
+
+            @staticmethod
+            def hits_of(i):
+                return lists[i]
+        R.hits = hits
+        lens = np.array([100, 150] * 3, np.uint16)
+        got = [(int(x["n_concordant"]), int(x["n_best"]), int(x["pos_plus"]), int(x["pos_minus"]),
+                int(x["plus_mate"]), int(x["mm"])) for x in m.pair_batch(R, lens, lo, hi)]
+        assert got == oracle.pair(R, lens, lo, hi), (sizes, span)
