@@ -1454,7 +1454,7 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         ba.fr_out_meta = frontier_meta(w, rd.n, 0);
         if (use_sweep(idx, rd.n)) {
             uint2 *list = (uint2 *)frontier_items(w, rd.n, 1);
-            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, list, s, launches)) return rc;
+            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, ba.budget, list, ba.fr_out, ba.fr_cap, s, launches)) return rc;
             ba.list = list;
         }
         if (int rc = check_vector_alignment(ba)) return rc;

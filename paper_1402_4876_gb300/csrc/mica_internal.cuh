@@ -150,7 +150,7 @@ struct SearchCtl {
     unsigned int iv_count;            // intervals written
     unsigned int iv_cap;
     unsigned int error;               // bit 0 interval overflow, bit 1 spill overflow, bit 2 timeout
-    unsigned int pad_;
+    unsigned int row_items;           // seed sweep: items of rows to check
     unsigned long long seeds, nodes, rank_blocks, spills;
     unsigned long long rounds, lane_ops;
     unsigned long long rounds_kind[3];   // multi-row, single-row, seed rounds
@@ -366,8 +366,8 @@ int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const 
 
 // sweep.cu
 bool sweep_available(const mica_index *idx, uint32_t verify_min);
-int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint2 *list,
-                  cudaStream_t s, uint64_t &launches);
+int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint32_t budget, uint2 *list,
+                  uint4 *items, uint32_t item_cap, cudaStream_t s, uint64_t &launches);
 
 // post.cu
 int run_post(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, uint32_t hit_cap,

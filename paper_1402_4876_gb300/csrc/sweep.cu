@@ -31,6 +31,7 @@ namespace {
 constexpr unsigned SFULL = 0xffffffffu;
 constexpr int SWEEP_WARPS = 8;
 constexpr int SWEEP_CTAS = 4;     // per SM
+constexpr uint32_t ROW_ITEM = 128;   // rows of an item (32 .. 256 within 2%)
 constexpr int SWEEP_QUEUE = 64;   // intervals waiting: fewer than 32 left over (each has a row) plus 32 new ones
 
 struct SweepArgs {
@@ -43,7 +44,11 @@ struct SweepArgs {
     Interval *iv;
     uint32_t *iv_cnt;
     uint2 *list;                 // (task, schemes left as bits)
-    uint32_t verify_min, split;
+    // larger intervals, a piece of up to ROW_ITEM rows each: (row l, task, rows | scheme << 9 | context bases in
+    // the exact piece << 11 | budget << 16 | pattern position of the matched bases << 18, the read's context)
+    uint4 *items;
+    uint32_t item_cap;
+    uint32_t verify_min, split, split_max;
 };
 
 // Raw word i of a read, 0 outside it.
@@ -232,6 +237,34 @@ __device__ __forceinline__ void sweep_rows(const SweepArgs &a, SweepQueue &Q, ui
     __syncwarp();
 }
 
+// Put the warp's intervals of many rows (lanes with `want`) on the item list,
+// with one counter update; false for a lane whose items do not fit (what was
+// reserved for them is filled with empty items).
+__device__ __forceinline__ bool sweep_items(const SweepArgs &a, bool want, uint32_t l, uint32_t sz, uint32_t task,
+                                            const uint32_t *w, uint32_t m, uint32_t k, uint32_t j, uint32_t qe,
+                                            int lane)
+{
+    if (!__any_sync(SFULL, want)) return false;
+    const uint32_t n = want ? (sz + ROW_ITEM - 1) / ROW_ITEM : 0u;
+    uint32_t incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(SFULL, incl, o);
+        if (lane >= o) incl += y;
+    }
+    uint32_t q = 0;
+    if (lane == 31) q = atomicAdd(&a.ctl->row_items, incl);
+    q = __shfl_sync(SFULL, q, 31) + incl - n;
+    if (!want || q >= a.item_cap) return false;
+    const bool fits = n <= a.item_cap - q;
+    const uint32_t at = bnd(j + 1, m, k + 1) - qe;
+    const uint32_t meta = (j << 9) | (min(16u, at - bnd(j, m, k + 1)) << 11) | (k << 16) | (at << 18);
+    const uint32_t ctx = read_context(w, task & 1u, m, at);
+    for (uint32_t i = 0; i < n && q + i < a.item_cap; i++)
+        a.items[q + i] = make_uint4(l + i * ROW_ITEM, task, fits ? min(sz - i * ROW_ITEM, ROW_ITEM) | meta : 0u, ctx);
+    return fits;
+}
+
 __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const SweepArgs a)
 {
     __shared__ SweepQueue queues[SWEEP_WARPS];
@@ -287,9 +320,11 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
             const uint32_t qj = j == 0 ? qe[0] : j == 1 ? qe[1] : j == 2 ? qe[2] : qe[3];
             const bool some = qj && lj < rj;
             const uint32_t sz = rj - lj;
-            const bool check = some && sz <= a.split && qj >= a.verify_min && m - qj >= BD_VERIFY_LEFT;
+            const bool rowwise = some && sz <= a.split_max && qj >= a.verify_min && m - qj >= BD_VERIFY_LEFT;
+            const bool check = rowwise && sz <= a.split;
             const bool whole = some && qj == m;            // the seed is the whole read
-            if (some && !check && !whole) left |= 1u << j;
+            const bool larger = sweep_items(a, rowwise && !check, lj, sz, (uint32_t)t, w, m, k, j, qj, lane);
+            if (some && !check && !whole && !larger) left |= 1u << j;
             sweep_emit(a, whole, rid, minus << 2, lj, rj, lane);
             const unsigned bal = __ballot_sync(SFULL, check);
             if (check) {
@@ -331,10 +366,142 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
     }
 }
 
+// One warp's windows of one read (starts st[0, n), n <= 32) against the text:
+// four pattern words at a time, those of the exact piece first (most windows of
+// a repeat family fail there).
+__device__ __forceinline__ void item_windows(const SweepArgs &a, const uint32_t *pat, const uint32_t *st, uint32_t n,
+                                             uint32_t rid, uint32_t minus, uint32_t m, uint32_t k, uint32_t j, int lane,
+                                             uint32_t &c_verify, uint32_t &c_vbytes, uint32_t &c_vsect)
+{
+    const uint32_t p = k + 1;
+    const uint32_t b1 = bnd(1, m, p), b2 = p >= 2 ? bnd(2, m, p) : 511u, b3 = p >= 3 ? bnd(3, m, p) : 511u;
+    const uint32_t wn = (m + 15) >> 4, chunks = (wn + 3) >> 2, first = bnd(j, m, p) >> 6;
+    bool live = (uint32_t)lane < n;
+    const uint32_t s = live ? st[lane] : 0u;
+    const uint32_t *tp = a.text + (s >> 4);
+    const uint32_t sh = 2u * (s & 15u);
+    uint32_t tot = 0, hit = 0;
+    if (live) c_verify++;
+    for (uint32_t i = 0; i < chunks; i++) {
+        const uint32_t q0 = 4u * (first + i < chunks ? first + i : first + i - chunks);
+        if (live) {
+            uint32_t tw[5];
+#pragma unroll
+            for (uint32_t u = 0; u < 5; u++) tw[u] = q0 + u <= wn ? __ldg(tp + q0 + u) : 0u;
+            c_vbytes += 4u * (min(4u, wn - q0) + 1u);
+            c_vsect += ((((s >> 4) + q0) & 7u) * 4u + 4u * min(4u, wn - q0) + 35u) / 32u;
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) {
+                const uint32_t q = q0 + u;
+                uint32_t x = pat[min(q, MAX_WORDS - 1)] ^ __funnelshift_r(tw[u], tw[u + 1], sh);
+                x = (x | (x >> 1)) & 0x55555555u & low_mask(2u * (uint32_t)min(max((int)m - 16 * (int)q, 0), 16));
+                while (x && tot <= k) {
+                    const uint32_t pos = 16u * q + (uint32_t)(__ffs(x) - 1) / 2u;
+                    x &= x - 1;
+                    tot++;
+                    hit |= 1u << ((pos >= b1) + (pos >= b2) + (pos >= b3));
+                }
+            }
+            live = tot <= k && !((hit >> j) & 1u);
+        }
+        if (!__any_sync(SFULL, live)) return;
+    }
+    const bool leaf = live && (hit & ((1u << j) - 1u)) == (1u << j) - 1u;
+    const unsigned bal = __ballot_sync(SFULL, leaf);
+    if (!bal) return;
+    uint32_t at = 0;
+    if (lane == 0) {
+        at = atomicAdd(&a.ctl->iv_count, (unsigned)__popc(bal));
+        atomicAdd(&a.iv_cnt[rid], (unsigned)__popc(bal));
+    }
+    at = __shfl_sync(SFULL, at, 0) + __popc(bal & ((1u << lane) - 1u));
+    if (leaf) {
+        if (at < a.ctl->iv_cap) {
+            Interval x;
+            x.read = rid; x.meta = tot | (minus << 2) | IV_POS; x.l = s; x.r = s + 1u;
+            a.iv[at] = x;
+        } else {
+            atomicOr(&a.ctl->error, ERR_IV_OVERFLOW);
+        }
+    }
+}
+
+// The item list, one item of one read per warp at a time: its rows stream by
+// 32 at a time, those whose left context passes are collected and checked
+// against the text 32 at a time, with the pattern in shared memory.  Intervals
+// of this size come from repeats, a few thousand reads of a batch: here they
+// spread over every warp of the GPU, where the sweep's own warps would each
+// be held by the few they drew.
+__global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const SweepArgs a)
+{
+    __shared__ uint32_t pat_s[SWEEP_WARPS][MAX_WORDS], start_s[SWEEP_WARPS][64];
+    const uint32_t n_items = min(*(volatile unsigned *)&a.ctl->row_items, a.item_cap);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t *pat = pat_s[warp], *st = start_s[warp];
+    uint32_t c_verify = 0, c_vbytes = 0, c_vsect = 0;
+    for (uint32_t it = blockIdx.x * SWEEP_WARPS + warp; it < n_items; it += gridDim.x * SWEEP_WARPS) {
+        const uint4 item = __ldg(a.items + it);
+        const uint32_t cnt = item.z & 511u, j = (item.z >> 9) & 3u, ex = (item.z >> 11) & 31u, k = (item.z >> 16) & 3u;
+        const uint32_t at = item.z >> 18, rid = item.y >> 1, minus = item.y & 1u;
+        if (cnt == 0) continue;
+        const uint32_t m = a.rd.len[rid];
+        const int wn = (int)((m + 15) >> 4);
+        const uint32_t *w = a.rd.words + a.rd.word_off[rid];
+        if (lane < (int)MAX_WORDS)
+            pat[lane] = minus ? rc_word(raw_word(w, wn - 1 - lane, wn), raw_word(w, wn - 2 - lane, wn), m)
+                              : raw_word(w, lane, wn);
+        __syncwarp();
+        uint32_t have = 0;
+        for (uint32_t r0 = 0; r0 < cnt; r0 += 32) {
+            bool stay = false;
+            uint32_t s = 0;
+            if (r0 + (uint32_t)lane < cnt) {
+                const uint2 x = __ldg(a.sa_ctx + item.x + r0 + (uint32_t)lane);
+                s = x.x - at;
+                uint32_t df = x.y ^ item.w;
+                df = (df | (df >> 1)) & 0x55555555u;
+                if (at < 16u) df &= at ? ~0u << (2u * (16u - at)) : 0u;
+                const bool exact = ex == 0 || (df >> (2u * (16u - ex))) == 0;
+                stay = x.x >= at && (uint64_t)s + m <= a.n && exact && __popc(df) <= k;
+                c_vbytes += 8u;
+                c_vsect += (lane & 3) == 0;
+            }
+            const unsigned bal = __ballot_sync(SFULL, stay);
+            if (stay) st[have + __popc(bal & ((1u << lane) - 1u))] = s;
+            have += __popc(bal);
+            __syncwarp();
+            if (have >= 32u) {
+                item_windows(a, pat, st, 32u, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
+                have -= 32u;
+                const uint32_t rest = (uint32_t)lane < have ? st[32 + lane] : 0u;
+                __syncwarp();
+                if ((uint32_t)lane < have) st[lane] = rest;
+                __syncwarp();
+            }
+        }
+        if (have) item_windows(a, pat, st, have, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
+        __syncwarp();
+    }
+    c_verify = __reduce_add_sync(SFULL, c_verify);
+    c_vbytes = __reduce_add_sync(SFULL, c_vbytes);
+    c_vsect = __reduce_add_sync(SFULL, c_vsect);
+    if (lane == 0 && c_vbytes) {
+        atomicAdd(&a.ctl->verified, (unsigned long long)c_verify);
+        atomicAdd(&a.ctl->verify_bytes, (unsigned long long)c_vbytes);
+        atomicAdd(&a.ctl->verify_sectors, (unsigned long long)c_vsect);
+    }
+}
+
 }  // namespace
 
-// Rows of an interval the sweep checks one by one.
+// Rows of an interval the sweep checks itself, and those it puts on the item
+// list.  Up to 32 are a warp's one look.  Past 256 a read's hits outgrow the
+// warp that finishes it: us per pass with 32 (no list) / 128 / 256 / 512 / 1024
+// / 2048, 64 Mbp 1M reads 1378 / 1308 / 1233 / 1225 / 1299 / 1520, uneven 1M 2506
+// / 2428 / 2290 / 2272 / 2404 / 3416, 33k short reads with a cap of 10 313 / 309
+// / 296 / 349 / 334 / 335, a human-like genome within 2%.
 constexpr uint32_t SWEEP_SPLIT = 32;
+constexpr uint32_t SWEEP_SPLIT_MAX = 256;
 
 // May the sweep run for an index and its verify threshold (matched bases)?
 // It needs the suffix array and the text, and seeds long enough to be checked.
@@ -346,8 +513,8 @@ bool sweep_available(const mica_index *idx, uint32_t verify_min)
 
 // Enqueue the sweep of n reads: leaves into iv, the tasks left into list (2 n
 // entries), their number in ctl->ntasks (0 before).
-int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint2 *list,
-                  cudaStream_t s, uint64_t &launches)
+int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint32_t budget, uint2 *list,
+                  uint4 *items, uint32_t item_cap, cudaStream_t s, uint64_t &launches)
 {
     SweepArgs a{};
     const IndexView &v = idx->view;
@@ -373,9 +540,14 @@ int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint
     a.list = list;
     a.verify_min = verify_min;
     a.split = SWEEP_SPLIT;
+    // (a node budget below 64 asks for short turns: then larger intervals stay with the tree, which it governs)
+    a.split_max = budget < 64 ? SWEEP_SPLIT : SWEEP_SPLIT_MAX;
+    a.items = items;
+    a.item_cap = item_cap;
     const uint64_t blocks = (2 * rd.n + SWEEP_WARPS * 32 - 1) / (SWEEP_WARPS * 32);
     k_sweep<<<(unsigned)std::min<uint64_t>(blocks, 152ull * SWEEP_CTAS), SWEEP_WARPS * 32, 0, s>>>(a);
-    launches++;
+    k_rows<<<152 * SWEEP_CTAS, SWEEP_WARPS * 32, 0, s>>>(a);
+    launches += 2;
     MICA_CUDA_TRY(cudaGetLastError());
     return 0;
 }
