@@ -1189,6 +1189,21 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         atomicAdd(&ctl->rounds, (unsigned long long)c_rounds);
         if (c_deep) atomicAdd(&ctl->deep_moves, (unsigned long long)c_deep);
     }
+    // the last CTA to finish turns the nodes this launch exported into the
+    // next round's tasks (a kernel of its own between rounds cost a small batch
+    // as much as its search)
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1) {
+        const uint32_t n = *(volatile unsigned *)&ctl->fr_count;
+        ctl->spills += n;
+        ctl->ntasks = min(n, a.fr_cap);
+        ctl->unfinished = (n ? 1u : 0u) | (*(volatile unsigned *)&ctl->redo_reads ? 2u : 0u);
+        ctl->rounds_run += n != 0;
+        ctl->task_head = 0;
+        ctl->fr_count = 0;
+        ctl->done_ctas = 0;
+    }
 }
 
 // The reads whose bit is set: into list[0, *n_list), with their leaf counts
@@ -1219,22 +1234,23 @@ __global__ void k_iv_purge(Interval *__restrict__ iv, const unsigned int *__rest
     }
 }
 
-// Between frontier rounds: the nodes the last round exported become the
-// next round's tasks.
-__global__ void k_bd_round(SearchCtl *ctl, uint32_t fr_cap)
+// The control block, the per-read interval counts and the give-up bits as a
+// search begins.
+__global__ void k_bd_init(const SearchCtl tmpl, SearchCtl *__restrict__ ctl, uint32_t *__restrict__ iv_cnt, uint64_t n,
+                          uint32_t *__restrict__ redo, uint64_t redo_words)
 {
-    const uint32_t n = min(ctl->fr_count, fr_cap);
-    ctl->spills += ctl->fr_count;
-    ctl->ntasks = n;
-    ctl->task_head = 0;
-    ctl->fr_count = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = tmpl;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        iv_cnt[i] = 0;
+        if (i < redo_words) redo[i] = 0;
+    }
 }
 
 // After the last round: the reads of nodes still in the frontier are given up.
 __global__ void k_bd_give_up_frontier(SearchCtl *ctl, const uint4 *__restrict__ fr, uint32_t fr_cap,
                                       uint32_t *__restrict__ redo)
 {
-    const uint32_t n = min(ctl->fr_count, fr_cap);
+    const uint32_t n = min((uint32_t)ctl->ntasks, fr_cap);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t rid = fr[i].x >> 1, bit = 1u << (rid & 31);
         if (!(atomicOr(&redo[rid >> 5], bit) & bit)) atomicAdd(&ctl->redo_reads, 1u);
@@ -1321,8 +1337,7 @@ static uint32_t frontier_cap(uint64_t n)
 {
     return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(2 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
 }
-constexpr int BD_GRAPH_ROUNDS = 8;   // frontier rounds a captured batch runs (more: the regular path)
-constexpr int BD_MAX_ROUNDS = 64;
+constexpr uint32_t BD_MAX_ROUNDS = 64;
 static uint64_t redo_bytes(uint64_t n) { return redo_bits_bytes(n) + std::max<uint64_t>(n, 1) * 4 + 16; }
 
 // The sweep goes before the kernel when its task list (8 bytes for each of 2n
@@ -1424,25 +1439,30 @@ static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd
     ba.fr_out = frontier_items(w, rd.n, r & 1);
     ba.fr_out_meta = frontier_meta(w, rd.n, r & 1);
     if (int rc = check_vector_alignment(ba)) return rc;
-    k_bd_round<<<1, 1, 0, s>>>(ba.ctl, ba.fr_cap);
     sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
-    launches += 2;
+    launches++;
     MICA_CUDA_TRY(cudaGetLastError());
     return 0;
 }
 
-// Enqueue one bidirectional search (control block from `tmpl_src`, which is
-// pinned host memory when captured; zeroed per-read counters and give-up
-// bits), then `rounds` frontier rounds, between the timing events.  No host
+// Enqueue one bidirectional search from the control block `tmpl`, then `rounds`
+// frontier rounds, between the timing events; with `check` the batch is checked
+// first, and an invalid one leaves everything that follows idle.  No host
 // reads, so it can be captured.
-int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl *tmpl_src,
+int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl &tmpl, bool check,
                   cudaStream_t s, uint64_t &launches, int rounds)
 {
     const BidirShape &sh = g_bd_shapes[bidir_shape_index(idx)];
     SearchCtl *d_ctl = (SearchCtl *)w.ctl.p;
-    MICA_CUDA_TRY(cudaMemcpyAsync(d_ctl, tmpl_src, sizeof(SearchCtl), cudaMemcpyHostToDevice, s));
-    MICA_CUDA_TRY(cudaMemsetAsync(w.iv_cnt.p, 0, std::max<uint64_t>(rd.n, 1) * 4, s));
-    MICA_CUDA_TRY(cudaMemsetAsync(w.redo.p, 0, redo_bits_bytes(rd.n), s));
+    const uint64_t n1 = std::max<uint64_t>(rd.n, 1);   // (at least one give-up word per read: redo_bits_bytes)
+    k_bd_init<<<(unsigned)std::min<uint64_t>((n1 + 255) / 256, 152ull * 8), 256, 0, s>>>(
+        tmpl, d_ctl, (uint32_t *)w.iv_cnt.p, n1, (uint32_t *)w.redo.p, (rd.n + 31) / 32);
+    launches++;
+    MICA_CUDA_TRY(cudaGetLastError());
+    if (check) {
+        if (int rc = enqueue_validate(idx, rd, &d_ctl->error, s)) return rc;
+        launches++;
+    }
     MICA_CUDA_TRY(record_event(w.kev[0], s));
     if (rd.n) {
         BidirArgs ba;
@@ -1468,10 +1488,10 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
     return 0;
 }
 
-int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl *tmpl_src,
-                        cudaStream_t s, uint64_t &launches)
+int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl &tmpl,
+                        bool check, cudaStream_t s, uint64_t &launches)
 {
-    return enqueue_bidir(idx, w, rd, grid, tmpl_src, s, launches, BD_GRAPH_ROUNDS);
+    return enqueue_bidir(idx, w, rd, grid, tmpl, check, s, launches, w.bd_rounds);
 }
 
 // The reads the kernel gave up on: purge their leaves and search them again
@@ -1499,67 +1519,80 @@ int redo_given_up(const mica_index *idx, Workspace &w, mica_stats &st, const Rea
     return run_search_list(idx, w, st, rd, list, nl, out.iv_count, idx->has_rev, s);
 }
 
-// The bidirectional search of a batch, growing the interval buffer when it
-// overflows, then the reads it gave up on.  Returns BIDIR_FALLBACK when the
-// persistent search of those reads overflows a buffer (the caller then runs
-// the persistent search over the whole batch).
-int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s)
+// The rest of a search whose control block after `r - 1` rounds is `out`: the
+// rounds that are left, the reads it gave up on, and the call's counters.
+// Returns BIDIR_FALLBACK when the persistent search of those reads overflows a
+// buffer (the caller then runs the persistent search over the whole batch),
+// BIDIR_GROW when the interval buffer overflowed (it has been given a larger
+// size for the next attempt).
+int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, SearchCtl &out, uint32_t r,
+                 int grid, cudaStream_t s)
 {
     const uint64_t n = rd.n;
+    // four rounds per host read of the control block (a round with nothing
+    // exported to it returns at once)
+    while (r <= BD_MAX_ROUNDS && (out.unfinished & 1u) && !out.error) {
+        for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++)
+            if (int rc = launch_round(idx, w, rd, grid, (int)r, s, st.launches)) return rc;
+        MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
+        MICA_CUDA_TRY(cudaStreamSynchronize(s));
+    }
+    if ((out.unfinished & 1u) && !out.error) {
+        // still exporting after the last round: those reads are given up
+        k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
+                                                  frontier_cap(n), (uint32_t *)w.redo.p);
+        st.launches++;
+        MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
+        MICA_CUDA_TRY(cudaStreamSynchronize(s));
+    }
+    if (out.error & ERR_TIMEOUT) return MICA_ETIMEOUT;
+    if (out.error & ERR_IV_OVERFLOW) {
+        st.retries++;
+        w.iv_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(2ull * out.iv_count, 2ull * w.iv_cap),
+                                                0xfffffff0ull);
+        return BIDIR_GROW;
+    }
+    if (out.error) return BIDIR_FALLBACK;
+    st.tasks = 2 * n;
+    st.seeds = out.seeds;
+    st.nodes = out.nodes;
+    st.rank_blocks = out.rank_blocks;
+    st.intervals = out.iv_count;
+    st.warp_rounds = out.rounds;
+    st.lane_ops = out.lane_ops;
+    st.overflow_moves = out.deep_moves;
+    st.verified = out.verified;
+    st.verify_bytes = out.verify_bytes;
+    st.verify_sectors = out.verify_sectors;
+    st.spills = out.spills;   // nodes exported to later rounds
+    st.grid_ctas = (uint64_t)grid;
+    w.bd_redo_seen = out.redo_reads > 0;
+    // rounds a captured batch of this workspace runs: what its batches needed so far, to a power of two
+    while (w.bd_rounds < out.rounds_run && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
+    if (out.redo_reads) {
+        int rc = redo_given_up(idx, w, st, rd, out, s);
+        if (rc) return rc;
+    }
+    // (what the kernels after the search look at)
+    MICA_CUDA_TRY(cudaMemsetAsync(&((SearchCtl *)w.ctl.p)->unfinished, 0, 4, s));
+    MICA_CUDA_TRY(record_event(w.kev[1], s));   // the kernel time covers the re-search too
+    return 0;
+}
+
+// The bidirectional search of a batch, growing the interval buffer when it
+// overflows, then the reads it gave up on.
+int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s)
+{
     for (int attempt = 0; attempt < 8; attempt++) {
         SearchCtl h{};
         int grid = 0;
-        if (int rc = prepare_bidir(idx, w, n, h, grid)) return rc;
-        if (int rc = enqueue_bidir(idx, w, rd, grid, &h, s, st.launches, 0)) return rc;
+        if (int rc = prepare_bidir(idx, w, rd.n, h, grid)) return rc;
+        if (int rc = enqueue_bidir(idx, w, rd, grid, h, false, s, st.launches, 0)) return rc;
         SearchCtl out;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
-        // frontier rounds while the last one exported nodes (and nothing failed)
-        int r = 1;
-        // four rounds per host read of the control block (a round with
-        // nothing exported to it returns at once)
-        while (r <= BD_MAX_ROUNDS && out.fr_count && !out.error) {
-            for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++)
-                if (int rc = launch_round(idx, w, rd, grid, r, s, st.launches)) return rc;
-            MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
-            MICA_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        if (out.fr_count && !out.error) {
-            // still exporting after the last round: those reads are given up
-            k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
-                                                      frontier_cap(n), (uint32_t *)w.redo.p);
-            st.launches++;
-            MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
-            MICA_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        if (out.error & ERR_TIMEOUT) return MICA_ETIMEOUT;
-        if (out.error & ERR_IV_OVERFLOW) {
-            st.retries++;
-            w.iv_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(2ull * out.iv_count, 2ull * w.iv_cap),
-                                                    0xfffffff0ull);
-            continue;
-        }
-        if (out.error) return BIDIR_FALLBACK;
-        st.tasks = 2 * n;
-        st.seeds = out.seeds;
-        st.nodes = out.nodes;
-        st.rank_blocks = out.rank_blocks;
-        st.intervals = out.iv_count;
-        st.warp_rounds = out.rounds;
-        st.lane_ops = out.lane_ops;
-        st.overflow_moves = out.deep_moves;
-        st.verified = out.verified;
-        st.verify_bytes = out.verify_bytes;
-        st.verify_sectors = out.verify_sectors;
-        st.spills = out.spills + out.fr_count;   // nodes exported to later rounds
-        st.grid_ctas = (uint64_t)grid;
-        w.bd_redo_seen = out.redo_reads > 0 || r > BD_GRAPH_ROUNDS;
-        if (out.redo_reads) {
-            int rc = redo_given_up(idx, w, st, rd, out, s);
-            if (rc) return rc;
-        }
-        MICA_CUDA_TRY(record_event(w.kev[1], s));   // the kernel time covers the re-search too
-        return 0;
+        const int rc = finish_bidir(idx, w, st, rd, out, 1, grid, s);
+        if (rc != BIDIR_GROW) return rc;
     }
     set_last_internal("bidirectional search: interval buffer growth did not converge");
     return MICA_EINTERNAL;

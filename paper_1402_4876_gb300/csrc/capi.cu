@@ -263,7 +263,7 @@ static bool use_prefetch(const mica_index *idx)
 // the batch cannot be captured); align_graph_finish waits for it and reads its
 // status.
 static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
-                              const mica_align_params &p, cudaStream_t s, bool &launched)
+                              const mica_align_params &p, cudaStream_t s, bool check, bool &launched)
 {
     launched = false;
     uint64_t n = rd.n;
@@ -298,12 +298,13 @@ static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &s
                                (uint64_t)w.spill_cap, (uint64_t)w.spill_seq.p, (uint64_t)w.deep.p,
                                (uint64_t)p.report | ((uint64_t)idx->tuning.bidir_budget << 32),
                                ((uint64_t)idx->idle_limit << 32) | idx->spin_limit,
-                               (uint64_t)w.frontier.p, (uint64_t)w.redo.p, (uint64_t)idx->tuning.bidir_verify};
+                               (uint64_t)w.frontier.p, (uint64_t)w.redo.p, (uint64_t)idx->tuning.bidir_verify,
+                               (uint64_t)w.bd_rounds | ((uint64_t)check << 32)};
     if (!w.gexec || memcmp(key, w.gkey, sizeof(key)) != 0) {
         if (w.gexec) { cudaGraphExecDestroy(w.gexec); w.gexec = nullptr; }
         uint64_t L = 0;
         MICA_CUDA_TRY(cudaStreamBeginCapture(w.gstream, cudaStreamCaptureModeThreadLocal));
-        int crc = bidir ? enqueue_bidir_graph(idx, w, rd, grid, (const SearchCtl *)w.pin_tmpl, w.gstream, L)
+        int crc = bidir ? enqueue_bidir_graph(idx, w, rd, grid, tmpl, check, w.gstream, L)
                         : enqueue_persistent(idx, w, rd, shape, grid, (const SearchCtl *)w.pin_tmpl, prune, prefetch,
                                              w.gstream, L);
         if (!crc) crc = enqueue_post_device(idx, w, rd, p.hit_cap, p.report, w.hit_capacity, w.gstream,
@@ -326,12 +327,13 @@ static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &s
     MICA_CUDA_TRY(cudaGraphLaunch(w.gexec, s));
     MICA_CUDA_TRY(cudaEventRecord(w.ev[2], s));
     w.g_grid = grid;
+    w.g_rounds = w.bd_rounds;
     launched = true;
     return 0;
 }
 
-static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd, const mica_align_params &p,
-                              uint64_t *nh, bool &done)
+static int align_graph_finish(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
+                              const mica_align_params &p, cudaStream_t s, uint64_t *nh, bool &done)
 {
     done = false;
     const uint64_t n = rd.n;
@@ -341,16 +343,27 @@ static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd,
     SearchCtl out;
     memcpy(&out, w.pin_status, sizeof(out));
     const uint64_t nhits = out.post_hits;
+    if (out.error & ERR_INVALID) return MICA_EINVAL;
     if (out.error & ERR_TIMEOUT) return MICA_ETIMEOUT;
     if (out.error) {
         // let the regular path grow the buffers and recompute
         return 0;
     }
-    if (bidir && (out.redo_reads || out.fr_count)) {
-        // reads given up, or nodes still exported after the captured rounds:
-        // the regular path runs the rounds to the end and searches the given-up
-        // reads again
-        w.bd_redo_seen = true;
+    if (bidir && out.unfinished) {
+        // nodes left after the captured rounds, or reads given up: the search
+        // goes on from there, then the steps after it, which the replay skipped
+        st.launches += w.glaunches;
+        int rc = finish_bidir(idx, w, st, rd, out, w.g_rounds + 1, grid, s);
+        if (rc == BIDIR_GROW || rc == BIDIR_FALLBACK) return 0;
+        if (rc) return rc;
+        if ((rc = run_post(idx, w, st, rd, p.hit_cap, p.report, s, nh))) return rc;
+        MICA_CUDA_TRY(cudaEventRecord(w.ev[2], s));
+        MICA_CUDA_TRY(cudaEventSynchronize(w.ev[2]));
+        st.graph_replays++;
+        st.kernel_ms = elapsed_ms(w.kev[0], w.kev[1]);
+        st.search_ms = st.kernel_ms;
+        st.total_ms = elapsed_ms(w.ev[0], w.ev[2]);
+        done = true;
         return 0;
     }
     if (nhits > w.hit_capacity) { w.hit_capacity = 2 * nhits; return 0; }
@@ -388,12 +401,11 @@ static int align_graph_finish(Workspace &w, mica_stats &st, const ReadsView &rd,
 }
 
 static int align_graph(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
-                       const mica_align_params &p, cudaStream_t s, uint64_t *nh, bool &done)
+                       const mica_align_params &p, cudaStream_t s, uint64_t *nh, bool check, bool &launched, bool &done)
 {
     done = false;
-    bool launched = false;
-    if (int rc = align_graph_launch(idx, w, st, rd, p, s, launched)) return rc;
-    return launched ? align_graph_finish(w, st, rd, p, nh, done) : 0;
+    if (int rc = align_graph_launch(idx, w, st, rd, p, s, check, launched)) return rc;
+    return launched ? align_graph_finish(idx, w, st, rd, p, s, nh, done) : 0;
 }
 
 // The kernel a call runs: an index without the reversed genome's table runs
@@ -428,18 +440,27 @@ static bool graph_eligible(const Workspace &w, const mica_align_params &p, const
 }
 
 int align_on_device(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
-                    const mica_align_params &p_in, cudaStream_t s, uint64_t *nh, bool allow_graph)
+                    const mica_align_params &p_in, cudaStream_t s, uint64_t *nh, bool allow_graph, bool check)
 {
     const mica_align_params p = effective_params(idx, p_in);
     if (int rc = create_events(w)) return rc;
+    // a bidirectional batch that runs as a captured graph is checked in it: one
+    // wait for the device instead of two
+    const bool graph = allow_graph && graph_eligible(w, p, rd);
+    const bool check_inside = check && graph && p.kernel == MICA_KERNEL_BIDIRECTIONAL;
+    if (check && !check_inside)
+        if (int rc = validate_device_batch(idx, w, st, rd, s)) return rc;
     uint64_t launches = st.launches;   // the batch check already counted
     st = mica_stats{};
     st.launches = launches;
     const bool deepen = p.report == MICA_REPORT_BEST_STRATUM && p.kernel == MICA_KERNEL_PERSISTENT && rd.n > 0;
-    if (allow_graph && graph_eligible(w, p, rd)) {
-        bool done = false;
-        if (int rc = align_graph(idx, w, st, rd, p, s, nh, done)) return rc;
+    if (graph) {
+        bool launched = false, done = false;
+        if (int rc = align_graph(idx, w, st, rd, p, s, nh, check_inside, launched, done)) return rc;
         if (done) return 0;
+        if (check_inside && !launched) {
+            if (int rc = validate_device_batch(idx, w, st, rd, s)) return rc;
+        }
         st.graph_fallbacks++;
     }
     MICA_CUDA_TRY(cudaEventRecord(w.ev[0], s));
@@ -811,11 +832,22 @@ __global__ void k_validate(ReadsView rd, uint64_t genome_len, unsigned int *bad)
         uint64_t off = rd.word_off[i];
         if (m == 0 || m > MICA_MAX_READ_LEN || m > genome_len || rd.k[i] > MICA_MAX_K ||
             off > total_words || total_words - off < (m + 15) / 16)
-            atomicOr(bad, 1u);
+            atomicOr(bad, ERR_INVALID);
     }
 }
 
 }  // namespace
+
+// Queue the batch check: ERR_INVALID in *error when a read is not one the
+// search takes.
+int enqueue_validate(const mica_index *idx, const ReadsView &rd, unsigned int *error, cudaStream_t s)
+{
+    if (rd.n == 0) return 0;
+    const unsigned g = (unsigned)std::min<uint64_t>((rd.n + 255) / 256, 152 * 32);
+    k_validate<<<g, 256, 0, s>>>(rd, idx->n, error);
+    MICA_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
 
 int validate_device_batch(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
                           cudaStream_t s)
@@ -937,9 +969,8 @@ int mica_align_device(mica_index *idx, const uint32_t *d_packed_reads, const uin
     cudaStream_t s = (cudaStream_t)p.cuda_stream;
     ReadsView rd{d_packed_reads, d_word_offsets, d_lengths, d_k, n_reads};
     idx->stats.launches = 0;
-    if (int rc = validate_device_batch(idx, idx->ws, idx->stats, rd, s)) return rc;
     uint64_t nh = 0;
-    if (int rc = align_on_device(idx, idx->ws, idx->stats, rd, p, s, &nh)) return rc;
+    if (int rc = align_on_device(idx, idx->ws, idx->stats, rd, p, s, &nh, true, true)) return rc;
     out->n_reads = n_reads;
     out->n_hits = nh;
     out->total = (const uint64_t *)idx->ws.total.p;
@@ -999,7 +1030,7 @@ int mica_align_submit(mica_index *idx, const uint32_t *packed_reads, const uint6
     slot->st = mica_stats{};
     slot->launched = false;
     if (graph_eligible(w, p, rd)) {
-        if (!(rc = create_events(w))) rc = align_graph_launch(idx, w, slot->st, rd, p, slot->stream, slot->launched);
+        if (!(rc = create_events(w))) rc = align_graph_launch(idx, w, slot->st, rd, p, slot->stream, false, slot->launched);
         if (rc) {
             // no ticket, so the caller may free its buffers on return: let the copies finish first
             cudaStreamSynchronize(slot->stream);
@@ -1031,7 +1062,7 @@ int mica_align_collect(mica_index *idx, uint64_t ticket, mica_result **out)
     uint64_t nh = 0;
     bool done = false;
     int rc = 0;
-    if (slot->launched) rc = align_graph_finish(w, slot->st, rd, slot->p, &nh, done);
+    if (slot->launched) rc = align_graph_finish(idx, w, slot->st, rd, slot->p, slot->stream, &nh, done);
     if (!rc && !done) {
         // not captured, or the replay needs the regular path: run it now
         rc = align_on_device(idx, w, slot->st, rd, slot->p, slot->stream, &nh, false);

@@ -159,6 +159,10 @@ struct SearchCtl {
     unsigned long long deep_moves;                    // nodes moved to per-warp overflow stacks
     unsigned int redo_reads;                          // bidirectional search: reads given up, to be re-searched
     unsigned int fr_count;                            // bidirectional search: nodes exported this round
+    unsigned int unfinished;                          // ... bit 0 nodes wait for a further round, bit 1 reads
+                                                      //   were given up
+    unsigned int rounds_run, done_ctas;               // ... rounds with tasks; CTAs of this launch that are done
+    unsigned int pad3_;
     unsigned long long verified, verify_bytes;        // bidirectional search: one-row intervals checked
                                                       //   against the text, and the bytes that read
     unsigned long long verify_sectors;                // ... and the 32-byte sectors those reads touch
@@ -172,6 +176,7 @@ constexpr unsigned ERR_IV_OVERFLOW = 1u;
 constexpr unsigned ERR_SPILL_OVERFLOW = 2u;
 constexpr unsigned ERR_TIMEOUT = 4u;
 constexpr unsigned ERR_HIT_OVERFLOW = 8u;
+constexpr unsigned ERR_INVALID = 16u;   // the batch check (when it is part of a captured batch)
 constexpr uint32_t IV_PURGED = 0xffffffffu;   // Interval::read of a leaf dropped after the search
 
 // ---------------------------------------------------------------------------
@@ -195,7 +200,7 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-constexpr int GRAPH_KEY = 30;   // words identifying a captured batch shape
+constexpr int GRAPH_KEY = 31;   // words identifying a captured batch shape
 
 // Per-index workspace reused across align calls.
 struct Workspace {
@@ -210,6 +215,7 @@ struct Workspace {
     DevBuf frontier;                                      // bidirectional search: exported nodes, two rounds
     uint32_t iv_cap = 0, spill_cap = 0;
     uint32_t bd_deep_cap = 0;   // bidirectional search: entries of each warp's overflow stacks
+    uint32_t bd_rounds = 2;     // bidirectional search: frontier rounds of a captured batch
     bool bd_redo_seen = false;  // bidirectional search: the last call gave reads up (no graph replay then)
     uint64_t hit_cap_total = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};   // call timing
@@ -221,7 +227,8 @@ struct Workspace {
     uint64_t gkey[GRAPH_KEY] = {};
     uint64_t hit_capacity = 0;
     uint64_t glaunches = 0;   // kernels in the captured graph
-    int g_grid = 0;           // grid of the launched replay's search kernel
+    int g_grid = 0;           // grid of the launched replay's search kernel,
+    uint32_t g_rounds = 0;    //   and its frontier rounds
 };
 
 // One of an index's two slots for pipelined host batches
@@ -360,8 +367,11 @@ bool bidir_available(const mica_index *idx);
 int bidir_shape_index(const mica_index *idx);   // compiled bidirectional shape a call uses
 int bidir_shape_count();
 int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tmpl, int &grid);
-int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl *tmpl_src,
-                        cudaStream_t s, uint64_t &launches);
+constexpr int BIDIR_GROW = 3;       // finish_bidir: the interval buffer overflowed
+int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl &tmpl,
+                        bool check, cudaStream_t s, uint64_t &launches);
+int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, SearchCtl &out, uint32_t r,
+                 int grid, cudaStream_t s);
 int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s);
 
 // sweep.cu
@@ -374,9 +384,11 @@ int run_post(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsVie
              uint32_t report, cudaStream_t s, uint64_t *n_hits_out);
 // capi.cu: the whole path on one workspace (validation of device batches included)
 int align_on_device(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
-                    const mica_align_params &p, cudaStream_t s, uint64_t *nh, bool allow_graph = true);
+                    const mica_align_params &p, cudaStream_t s, uint64_t *nh, bool allow_graph = true,
+                    bool check = false);
 int validate_device_batch(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd,
                           cudaStream_t s);
+int enqueue_validate(const mica_index *idx, const ReadsView &rd, unsigned int *error, cudaStream_t s);
 int validate_host_batch(const mica_index *idx, const uint64_t *off, const uint16_t *len, const uint8_t *k,
                         uint64_t n);
 void free_workspace(Workspace &w);

@@ -201,19 +201,23 @@ __global__ void __launch_bounds__(TILE_THREADS) k_offsets(const uint32_t *__rest
 
 // ---- intervals grouped by read ----
 
-// Every post kernel that indexes by the search's per-read counts first reads
-// the search's error word: after an overflow the counts exceed what was
-// stored, so these kernels do nothing and the caller recomputes the batch.
-//
-// count: the search's interval counter on the device, read here (capped at
-// the buffer's capacity) so the launch needs no host round trip
-__global__ void k_iv_scatter(const Interval *__restrict__ iv, const unsigned int *__restrict__ count_p,
-                             uint32_t cap, const uint64_t *__restrict__ iv_off, uint32_t *__restrict__ cursor,
-                             Interval *__restrict__ out, unsigned long long *__restrict__ total,
-                             const unsigned int *__restrict__ err)
+// Every post kernel that indexes by the search's per-read counts first looks
+// at how the search ended: after an overflow the counts exceed what was
+// stored, and after rounds that left nodes or gave reads up they are not
+// complete.  Then these kernels do nothing, and the caller finishes the
+// search or runs it again before it calls them again.
+__device__ __forceinline__ bool search_open(const SearchCtl *ctl)
 {
-    if (*err) return;
-    uint32_t count = min(*count_p, cap);
+    return (*(const volatile unsigned *)&ctl->error | *(const volatile unsigned *)&ctl->unfinished) != 0;
+}
+
+// The interval count is read on the device (capped at the buffer's capacity) so
+// the launch needs no host round trip.
+__global__ void k_iv_scatter(const Interval *__restrict__ iv, const SearchCtl *__restrict__ ctl, uint32_t cap, const uint64_t *__restrict__ iv_off, uint32_t *__restrict__ cursor,
+                             Interval *__restrict__ out, unsigned long long *__restrict__ total)
+{
+    if (search_open(ctl)) return;
+    const uint32_t count = min(ctl->iv_count, cap);
     for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
         Interval x = iv[e];
         if (x.read == IV_PURGED) continue;   // a leaf of a read that was searched again
@@ -258,9 +262,9 @@ __global__ void __launch_bounds__(TILE_THREADS) k_listed(const uint64_t *__restr
 // d; the others become empty (r = l) and so count and list nothing.  A read
 // with many intervals is gone through by its warp.
 __global__ void k_stratum(Interval *__restrict__ ivs, const uint64_t *__restrict__ iv_off, uint64_t n,
-                          uint64_t *__restrict__ total, const unsigned int *__restrict__ err)
+                          uint64_t *__restrict__ total, const SearchCtl *__restrict__ ctl)
 {
-    if (*err) return;
+    if (search_open(ctl)) return;
     const uint32_t lane = threadIdx.x & 31;
     for (uint64_t r0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); r0 < n;
          r0 += (uint64_t)gridDim.x * blockDim.x) {
@@ -397,7 +401,7 @@ __device__ __forceinline__ void count_steps(SearchCtl *ctl, uint32_t steps)
 __global__ void __launch_bounds__(TILE_THREADS) k_finish_small(const FinishArgs a, const uint64_t *__restrict__ sums)
 {
     __shared__ uint64_t ws[TILE_THREADS / 32];
-    if (*(volatile unsigned *)&a.ctl->error) return;   // (the counts exceed what was stored)
+    if (search_open(a.ctl)) return;
     uint64_t at = tiles_before(sums, blockIdx.x, ws);
     uint32_t steps = 0;
     for (uint32_t i0 = 0; i0 < TILE; i0 += TILE_THREADS) {
@@ -551,7 +555,7 @@ __global__ void __launch_bounds__(WARP_READS * 32) k_finish_warp(const FinishArg
 {
     __shared__ uint64_t sh_s[WARP_READS][WARP_HITS];
     __shared__ uint32_t bits_s[WARP_READS][WARP_SPAN / 16], pre_s[WARP_READS][WARP_SPAN / 16];
-    if (*(volatile unsigned *)&a.ctl->error) return;
+    if (search_open(a.ctl)) return;
     const uint32_t lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     uint64_t *sh = sh_s[wi];
     const unsigned n_list = a.ctl->n_warp;
@@ -774,7 +778,7 @@ __global__ void __launch_bounds__(NT) k_finish_block(const FinishArgs a)
     __shared__ unsigned long long count;
     __shared__ uint32_t found[2];
     __shared__ unsigned bi_s;
-    if (*(volatile unsigned *)&a.ctl->error) return;
+    if (search_open(a.ctl)) return;
     constexpr bool LONG = NT == LONG_THREADS;
     const unsigned n_list = LONG ? a.ctl->n_long : a.ctl->n_block;
     uint32_t steps = 0;
@@ -942,10 +946,10 @@ static int enqueue_totals(Workspace &w, uint64_t n, uint32_t hit_cap, uint32_t r
     unsigned long long *total = (unsigned long long *)w.total.p;
     k_offsets<<<tiles, TILE_THREADS, 0, s>>>((const uint32_t *)w.iv_cnt.p, n, sums, iv_off, (uint64_t *)total);
     const unsigned g = (unsigned)std::min<uint64_t>(152 * 16, std::max<uint64_t>(8, n / 64));
-    k_iv_scatter<<<g, 256, 0, s>>>((const Interval *)w.iv.p, &ctl->iv_count, w.iv_cap, iv_off, (uint32_t *)w.iv_cnt.p,
-                                   (Interval *)w.iv_sorted.p, total, &ctl->error);
+    k_iv_scatter<<<g, 256, 0, s>>>((const Interval *)w.iv.p, ctl, w.iv_cap, iv_off, (uint32_t *)w.iv_cnt.p,
+                                   (Interval *)w.iv_sorted.p, total);
     if (report == MICA_REPORT_BEST_STRATUM) {
-        k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, (uint64_t *)total, &ctl->error);
+        k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, (uint64_t *)total, ctl);
         L++;
     }
     k_listed<<<tiles, TILE_THREADS, 0, s>>>((const uint64_t *)total, n, hit_cap, sums + tiles);

@@ -268,6 +268,7 @@ __device__ __forceinline__ bool sweep_items(const SweepArgs &a, bool want, uint3
 __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const SweepArgs a)
 {
     __shared__ SweepQueue queues[SWEEP_WARPS];
+    if (*(volatile unsigned *)&a.ctl->error) return;   // (the batch check failed)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     SweepQueue &Q = queues[warp];

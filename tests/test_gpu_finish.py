@@ -96,3 +96,31 @@ def test_pairs_of_many_hits(sizes):
         got = [(int(x["n_concordant"]), int(x["n_best"]), int(x["pos_plus"]), int(x["pos_minus"]),
                 int(x["plus_mate"]), int(x["mm"])) for x in m.pair_batch(R, lens, lo, hi)]
         assert got == oracle.pair(R, lens, lo, hi), (sizes, span)
+
+
+def test_invalid_device_batches_are_refused_in_the_captured_batch():
+    """The check of a device batch runs inside the captured batch: a read of no
+    bases, a budget of 4 and an offset past the words are refused every time,
+    and the valid batch in the same buffers is not."""
+    import torch
+    m = gc.mica()
+    g = synth.uniform_genome(20_000, 8)
+    rng = np.random.default_rng(2)
+    b = synth.sample_reads(g, np.full(300, 50), np.full(300, 1), rng, subs="rate", sub_rate=0.01)
+    idx = m.Index.build(synth.to_acgt_bytes(g.codes), kmer_q=8, sa_sample=8)
+    d = [torch.from_numpy(b.words.view(np.int32)).cuda(), torch.from_numpy(b.word_off.view(np.int64)).cuda(),
+         torch.from_numpy(b.lengths.view(np.int16)).cuda(), torch.from_numpy(b.k).cuda()]
+    want = oracle.FMIndex(g.codes).align(b, cap=1000)
+    for which, value in ((2, 0), (3, 4), (1, 1 << 40), (2, 300)):
+        for _ in range(2):
+            keep = d[which][7].clone()
+            d[which][7] = value
+            with pytest.raises(m.MicaError) as e:
+                idx.align_device(*d, b.n)
+            assert e.value.code == m.MICA_EINVAL
+            d[which][7] = keep
+            t, o, h = idx.align_device(*d, b.n).tensors()
+            got = m.Result(t.cpu().numpy().view(np.uint64), o.cpu().numpy().view(np.uint64),
+                           h.cpu().numpy().view(m.HIT_DTYPE))
+            gc.assert_same(got, want, f"{which} {value}")
+    idx.free()
