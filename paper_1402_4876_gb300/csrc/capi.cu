@@ -171,23 +171,48 @@ static int validate_params(const mica_index_params &p)
     return 0;
 }
 
-// ASCII genome -> base codes (host), rejecting anything but A/C/G/T.
-static int encode_genome(const uint8_t *acgt, uint64_t len, std::vector<uint8_t> &codes)
+// ASCII genome -> base codes in place, four bytes a thread; *bad when a byte is
+// none of A/C/G/T in either case.  (A, C, G, T differ in bits 1 and 2: 0, 1, 3,
+// 2.  One host thread took longer over this than the GPU over the suffix sort.)
+__global__ void k_encode(uint32_t *__restrict__ text, uint64_t words, uint64_t len, unsigned *__restrict__ bad)
 {
-    static uint8_t lut[256];
-    static std::once_flag once;
-    std::call_once(once, [] {
-        memset(lut, 0xff, sizeof(lut));
-        lut['A'] = lut['a'] = 0; lut['C'] = lut['c'] = 1;
-        lut['G'] = lut['g'] = 2; lut['T'] = lut['t'] = 3;
-    });
-    codes.resize(len);
-    for (uint64_t i = 0; i < len; i++) {
-        uint8_t c = lut[acgt[i]];
-        if (c > 3) return MICA_EINVAL;
-        codes[i] = c;
+    bool wrong = false;
+    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t v = text[w];
+        uint32_t out = 0;
+#pragma unroll
+        for (uint32_t b = 0; b < 4; b++) {
+            const uint32_t c = (v >> (8 * b)) & 0xdfu;
+            const uint32_t x = (c >> 1) & 3u;
+            out |= (x ^ (x >> 1)) << (8 * b);
+            if (4 * w + b < len) wrong |= c != 'A' && c != 'C' && c != 'G' && c != 'T';
+        }
+        text[w] = out;
     }
-    return 0;
+    if (wrong) atomicOr(bad, 1u);
+}
+
+// The genome's base codes on the device, rejecting anything but A/C/G/T.
+static int encode_genome(const uint8_t *acgt, uint64_t len, DevBuf &codes)
+{
+    const uint64_t words = (len + 3) / 4;
+    DevBuf bad;
+    int rc = dev_reserve(codes, std::max<uint64_t>(words, 1) * 4);
+    if (!rc) rc = dev_reserve(bad, 4);
+    unsigned wrong = 0;
+    if (!rc && len) {
+        cudaError_t e = cudaMemset(bad.p, 0, 4);
+        if (e == cudaSuccess) e = cudaMemcpy(codes.p, acgt, len, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) {
+            k_encode<<<(unsigned)std::min<uint64_t>((words + 255) / 256, 152ull * 16), 256>>>(
+                (uint32_t *)codes.p, words, len, (unsigned *)bad.p);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpy(&wrong, bad.p, 4, cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) { set_last_cuda_error(e, "genome upload", __FILE__, __LINE__); rc = MICA_ECUDA; }
+    }
+    dev_release(bad);
+    return rc ? rc : wrong ? MICA_EINVAL : 0;
 }
 
 
@@ -548,18 +573,12 @@ int mica_index_build_resident(const uint8_t *genome_acgt, uint64_t len, const mi
     if (params) p = *params;
     if (int rc = validate_params(p)) return rc;
     if (len + 1 >= (1ull << 32)) return MICA_EINVAL;
-    std::vector<uint8_t> codes;
-    if (int rc = encode_genome(genome_acgt, len, codes)) return rc;
     DeviceGuard g(device);
     MICA_CUDA_TRY(cudaSetDevice(device));
     mica_index *idx = new mica_index();
     idx->device = device;
     DevBuf dcodes;
-    int rc = dev_reserve(dcodes, std::max<uint64_t>(len, 1));
-    if (!rc && len) {
-        cudaError_t e = cudaMemcpy(dcodes.p, codes.data(), len, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { set_last_cuda_error(e, "cudaMemcpy genome", __FILE__, __LINE__); rc = MICA_ECUDA; }
-    }
+    int rc = encode_genome(genome_acgt, len, dcodes);
     if (!rc) rc = build_index_from_codes((const uint8_t *)dcodes.p, len, p, idx, 0);
     dev_release(dcodes);
     if (rc) { mica_index_free(idx); return rc; }
@@ -1090,14 +1109,11 @@ void mica_result_free(mica_result *res)
 int mica_debug_suffix_array(const uint8_t *genome_acgt, uint64_t len, int device, uint32_t *sa_out)
 {
     if ((!genome_acgt && len) || !sa_out || len + 1 >= (1ull << 32)) return MICA_EINVAL;
-    std::vector<uint8_t> codes;
-    if (int rc = encode_genome(genome_acgt, len, codes)) return rc;
     DeviceGuard g(device);
     MICA_CUDA_TRY(cudaSetDevice(device));
     DevBuf dc, dsa;
-    int rc = dev_reserve(dc, std::max<uint64_t>(len, 1));
+    int rc = encode_genome(genome_acgt, len, dc);
     if (!rc) rc = dev_reserve(dsa, (len + 1) * 4);
-    if (!rc && len && cudaMemcpy(dc.p, codes.data(), len, cudaMemcpyHostToDevice) != cudaSuccess) rc = MICA_ECUDA;
     if (!rc) rc = build_suffix_array((const uint8_t *)dc.p, len, (uint32_t *)dsa.p, 0);
     if (!rc && cudaMemcpy(sa_out, dsa.p, (len + 1) * 4, cudaMemcpyDeviceToHost) != cudaSuccess) rc = MICA_ECUDA;
     dev_release(dc);

@@ -3,8 +3,12 @@
 // memory transactions per query).
 //
 //   1. suffix array of T = G$ by prefix doubling: sort positions by their
-//      first 21 symbols (3 bits each), then repeatedly by (rank[i], rank[i+h])
-//      with h doubling, until all ranks are distinct;
+//      first 16 bases (32-bit keys), then the positions that still share a
+//      rank with others by (rank[i], rank[i+h]) with h doubling, until none
+//      do.  A position alone in its group has its final place and leaves the
+//      sorts: most do at once (of a genome's 16-mers only those of repeats and
+//      a few by chance occur twice), where sorting all of them by 21 symbols and
+//      then by rank pairs round after round moved every key 50 times;
 //   2. BWT[j] = T[SA[j]-1] as two bit planes in 32-byte blocks of 96 rows
 //      that start with Occ(A..T, block start) relative to a superblock of
 //      682 blocks, whose absolute counts sit in a small separate table;
@@ -30,35 +34,42 @@ namespace mica {
 
 namespace {
 
-constexpr int KEY_SYMS = 21;   // symbols in the initial 63-bit key
+constexpr uint32_t KEY_SYMS = 16;   // bases in the initial 32-bit key
 
-__global__ void k_init_keys(const uint8_t *__restrict__ codes, uint64_t n,
-                            uint64_t *__restrict__ keys, uint32_t *__restrict__ vals)
+// The suffixes shorter than KEY_SYMS bases, shortest first, then the others in
+// text order: padded with A, a short suffix sorts before every longer one
+// with its key, which the stable sort keeps from this order.
+__global__ void k_init_keys(const uint8_t *__restrict__ codes, uint64_t n, uint64_t n_short,
+                            uint32_t *__restrict__ keys, uint32_t *__restrict__ vals)
 {
-    uint64_t rows = n + 1;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < rows;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t key = 0;
+    const uint64_t rows = n + 1;
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < rows; t += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t i = t < n_short ? n - t : t - n_short;
+        uint32_t key = 0;
 #pragma unroll
-        for (int j = 0; j < KEY_SYMS; j++) {
-            uint64_t p = i + j;
-            uint64_t s = p < n ? (uint64_t)codes[p] + 1 : 0;   // $ and beyond: 0
-            key = (key << 3) | s;
-        }
-        keys[i] = key;
-        vals[i] = (uint32_t)i;
+        for (uint32_t j = 0; j < KEY_SYMS; j++) key = (key << 2) | (i + j < n ? (uint32_t)codes[i + j] : 0u);
+        keys[t] = key;
+        vals[t] = (uint32_t)i;
     }
 }
 
-// head flag -> group head index (inclusive max-scan input); flags "not done"
-__global__ void k_heads(const uint64_t *__restrict__ keys, uint64_t rows,
-                        uint32_t *__restrict__ hv, int *__restrict__ not_done)
+__device__ __forceinline__ bool first_head(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ sa, uint64_t p,
+                                           uint64_t n)
 {
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < rows;
-         p += (uint64_t)gridDim.x * blockDim.x) {
-        bool head = (p == 0) || keys[p] != keys[p - 1];
+    // (short suffixes, i + KEY_SYMS > n, are alone in their groups)
+    return p == 0 || keys[p] != keys[p - 1] || (uint64_t)sa[p] + KEY_SYMS > n || (uint64_t)sa[p - 1] + KEY_SYMS > n;
+}
+
+// Group heads of the first sort: their index (input of a max-scan), and
+// whether a position shares its group.
+__global__ void k_first_heads(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ sa, uint64_t n,
+                              uint32_t *__restrict__ hv, uint8_t *__restrict__ open)
+{
+    const uint64_t rows = n + 1;
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < rows; p += (uint64_t)gridDim.x * blockDim.x) {
+        const bool head = first_head(keys, sa, p, n);
         hv[p] = head ? (uint32_t)p : 0u;
-        if (!head) *not_done = 1;
+        open[p] = !(head && (p + 1 == rows || first_head(keys, sa, p + 1, n)));
     }
 }
 
@@ -70,21 +81,53 @@ __global__ void k_scatter_rank(const uint32_t *__restrict__ sa, const uint32_t *
         rank[sa[p]] = grp[p];
 }
 
-__global__ void k_pair_keys(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ rank,
+// Keys of the m positions that share a rank: (rank[i], rank[i + h]).
+__global__ void k_pair_keys(const uint32_t *__restrict__ pos, const uint32_t *__restrict__ rank, uint64_t m,
                             uint64_t n, uint64_t h, int bits, uint64_t *__restrict__ keys)
 {
-    uint64_t rows = n + 1;
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < rows;
-         p += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t i = sa[p];
-        uint64_t r1 = rank[i];
-        uint64_t r2 = (i + h <= n) ? (uint64_t)rank[i + h] + 1 : 0;
-        keys[p] = (r1 << bits) | r2;
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t i = pos[p];
+        const uint64_t r2 = (i + h <= n) ? (uint64_t)rank[i + h] + 1 : 0;
+        keys[p] = ((uint64_t)rank[i] << bits) | r2;
+    }
+}
+
+// After their sort: where the old group and the new one of each begin (input
+// of a max-scan of both).
+__global__ void k_pair_heads(const uint64_t *__restrict__ keys, uint64_t m, int bits, uint2 *__restrict__ hv)
+{
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = keys[p], b = p ? keys[p - 1] : 0;
+        hv[p] = make_uint2(p && (k >> bits) == (b >> bits) ? 0u : (uint32_t)p, p && k == b ? 0u : (uint32_t)p);
+    }
+}
+
+// A group's positions fill the rows from its rank on, in the order of the
+// sort: each position's row, its new rank (the row of its new group's head)
+// and whether it still shares it.
+__global__ void k_place(const uint64_t *__restrict__ keys, const uint32_t *__restrict__ pos, const uint2 *__restrict__ hv,
+                        uint64_t m, int bits, uint32_t *__restrict__ sa, uint32_t *__restrict__ rank,
+                        uint8_t *__restrict__ open)
+{
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = keys[p];
+        const uint2 h = hv[p];                        // (old group's first, new group's first)
+        const uint32_t base = (uint32_t)(k >> bits);
+        sa[base + ((uint32_t)p - h.x)] = pos[p];
+        rank[pos[p]] = base + (h.y - h.x);
+        open[p] = !(h.y == (uint32_t)p && (p + 1 == m || keys[p + 1] != k));
     }
 }
 
 struct MaxOp {
     __device__ __forceinline__ uint32_t operator()(uint32_t a, uint32_t b) const { return a > b ? a : b; }
+};
+
+struct MaxOp2 {
+    __device__ __forceinline__ uint2 operator()(const uint2 &a, const uint2 &b) const
+    {
+        return make_uint2(a.x > b.x ? a.x : b.x, a.y > b.y ? a.y : b.y);
+    }
 };
 
 struct Sum4 {
@@ -100,8 +143,8 @@ int grid_for(uint64_t n, int block = 256)
     return (int)std::min<uint64_t>(std::max<uint64_t>(g, 1), 152ull * 64);
 }
 
-template <typename NumT>
-int sort_pairs(DevBuf &tmp, cub::DoubleBuffer<uint64_t> &keys, cub::DoubleBuffer<uint32_t> &vals,
+template <typename KeyT, typename NumT>
+int sort_pairs(DevBuf &tmp, cub::DoubleBuffer<KeyT> &keys, cub::DoubleBuffer<uint32_t> &vals,
                NumT rows, int end_bit, cudaStream_t s)
 {
     size_t need = 0;
@@ -111,57 +154,92 @@ int sort_pairs(DevBuf &tmp, cub::DoubleBuffer<uint64_t> &keys, cub::DoubleBuffer
     return 0;
 }
 
-template <typename NumT>
-int max_scan(DevBuf &tmp, const uint32_t *in, uint32_t *out, NumT rows, cudaStream_t s)
+template <typename T, typename Op, typename NumT>
+int scan_in_place(DevBuf &tmp, T *v, Op op, NumT rows, cudaStream_t s)
 {
     size_t need = 0;
-    MICA_CUDA_TRY(cub::DeviceScan::InclusiveScan(nullptr, need, in, out, MaxOp(), rows, s));
+    MICA_CUDA_TRY(cub::DeviceScan::InclusiveScan(nullptr, need, v, v, op, rows, s));
     if (int rc = dev_reserve(tmp, need)) return rc;
-    MICA_CUDA_TRY(cub::DeviceScan::InclusiveScan(tmp.p, need, in, out, MaxOp(), rows, s));
+    MICA_CUDA_TRY(cub::DeviceScan::InclusiveScan(tmp.p, need, v, v, op, rows, s));
     return 0;
 }
+
+// The entries of in[0, rows) whose flag is set, in their order; their number to the host.
+template <typename NumT>
+int keep_open(DevBuf &tmp, const uint32_t *in, const uint8_t *flags, uint32_t *out, uint64_t *d_count, NumT rows,
+              uint64_t &count, cudaStream_t s)
+{
+    size_t need = 0;
+    MICA_CUDA_TRY(cub::DeviceSelect::Flagged(nullptr, need, in, flags, out, d_count, rows, s));
+    if (int rc = dev_reserve(tmp, need)) return rc;
+    MICA_CUDA_TRY(cub::DeviceSelect::Flagged(tmp.p, need, in, flags, out, d_count, rows, s));
+    MICA_CUDA_TRY(cudaMemcpyAsync(&count, d_count, 8, cudaMemcpyDeviceToHost, s));
+    MICA_CUDA_TRY(cudaStreamSynchronize(s));
+    return 0;
+}
+
+struct DoublingBufs {
+    DevBuf k0, k1, v1, rank, open, count, tmp, key_a, key_b, pos_a, pos_b;
+    ~DoublingBufs()
+    {
+        for (DevBuf *b : {&k0, &k1, &v1, &rank, &open, &count, &tmp, &key_a, &key_b, &pos_a, &pos_b}) dev_release(*b);
+    }
+};
 
 template <typename NumT>
 int doubling(const uint8_t *d_codes, uint64_t n, uint32_t *d_sa, cudaStream_t s)
 {
-    uint64_t rows = n + 1;
-    DevBuf k0, k1, v1, rank, tmp, flag;
+    const uint64_t rows = n + 1;
+    DoublingBufs B;
     int rc = 0;
-    auto cleanup = [&]() { dev_release(k0); dev_release(k1); dev_release(v1); dev_release(rank);
-                           dev_release(tmp); dev_release(flag); };
-    if ((rc = dev_reserve(k0, rows * 8)) || (rc = dev_reserve(k1, rows * 8)) ||
-        (rc = dev_reserve(v1, rows * 4)) || (rc = dev_reserve(rank, rows * 4)) ||
-        (rc = dev_reserve(flag, 16))) { cleanup(); return rc; }
-    cub::DoubleBuffer<uint64_t> keys((uint64_t *)k0.p, (uint64_t *)k1.p);
-    cub::DoubleBuffer<uint32_t> vals(d_sa, (uint32_t *)v1.p);
+    if ((rc = dev_reserve(B.k0, rows * 4)) || (rc = dev_reserve(B.k1, rows * 4)) || (rc = dev_reserve(B.v1, rows * 4)) ||
+        (rc = dev_reserve(B.rank, rows * 4)) || (rc = dev_reserve(B.open, rows)) || (rc = dev_reserve(B.count, 16)))
+        return rc;
+    uint32_t *rank = (uint32_t *)B.rank.p;
+    uint8_t *open = (uint8_t *)B.open.p;
+    uint64_t *d_count = (uint64_t *)B.count.p;
     int bits = 1;
     while ((1ull << bits) < rows + 1) bits++;          // rank + 1 <= rows fits in `bits`
-    int g = grid_for(rows);
-    k_init_keys<<<g, 256, 0, s>>>(d_codes, n, keys.Current(), vals.Current());
-    if ((rc = sort_pairs<NumT>(tmp, keys, vals, (NumT)rows, 3 * KEY_SYMS, s))) { cleanup(); return rc; }
-    uint64_t h = KEY_SYMS;
-    for (int iter = 0; iter < 64; iter++) {
-        uint32_t *hv = (uint32_t *)keys.Alternate();            // free after the sort
-        uint32_t *grp = hv + rows;
-        int *nd = (int *)flag.p;
-        cudaMemsetAsync(nd, 0, sizeof(int), s);
-        k_heads<<<g, 256, 0, s>>>(keys.Current(), rows, hv, nd);
-        int not_done = 0;
-        MICA_CUDA_TRY(cudaMemcpyAsync(&not_done, nd, sizeof(int), cudaMemcpyDeviceToHost, s));
-        MICA_CUDA_TRY(cudaStreamSynchronize(s));
-        if (!not_done) break;
-        if ((rc = max_scan<NumT>(tmp, hv, grp, (NumT)rows, s))) { cleanup(); return rc; }
-        k_scatter_rank<<<g, 256, 0, s>>>(vals.Current(), grp, rows, (uint32_t *)rank.p);
-        k_pair_keys<<<g, 256, 0, s>>>(vals.Current(), (const uint32_t *)rank.p, n, h, bits,
-                                      keys.Current());
-        if ((rc = sort_pairs<NumT>(tmp, keys, vals, (NumT)rows, 2 * bits, s))) { cleanup(); return rc; }
-        h *= 2;
-    }
+    const int g = grid_for(rows);
+
+    // by the first 16 bases
+    cub::DoubleBuffer<uint32_t> keys((uint32_t *)B.k0.p, (uint32_t *)B.k1.p);
+    cub::DoubleBuffer<uint32_t> vals(d_sa, (uint32_t *)B.v1.p);
+    k_init_keys<<<g, 256, 0, s>>>(d_codes, n, std::min<uint64_t>(KEY_SYMS, rows), keys.Current(), vals.Current());
+    if ((rc = sort_pairs<uint32_t, NumT>(B.tmp, keys, vals, (NumT)rows, 32, s))) return rc;
     if (vals.Current() != d_sa)
         MICA_CUDA_TRY(cudaMemcpyAsync(d_sa, vals.Current(), rows * 4, cudaMemcpyDeviceToDevice, s));
+    uint32_t *hv = keys.Alternate();                   // free after the sort
+    k_first_heads<<<g, 256, 0, s>>>(keys.Current(), d_sa, n, hv, open);
+    if ((rc = scan_in_place(B.tmp, hv, MaxOp(), (NumT)rows, s))) return rc;
+    k_scatter_rank<<<g, 256, 0, s>>>(d_sa, hv, rows, rank);
+    uint64_t m = 0;
+    if ((rc = keep_open<NumT>(B.tmp, d_sa, open, (uint32_t *)B.v1.p, d_count, (NumT)rows, m, s))) return rc;
+    if (m) {
+        dev_release(B.k0);
+        dev_release(B.k1);
+        if ((rc = dev_reserve(B.key_a, m * 8)) || (rc = dev_reserve(B.key_b, m * 8)) ||
+            (rc = dev_reserve(B.pos_a, m * 4)) || (rc = dev_reserve(B.pos_b, m * 4)))
+            return rc;
+        MICA_CUDA_TRY(cudaMemcpyAsync(B.pos_a.p, B.v1.p, m * 4, cudaMemcpyDeviceToDevice, s));
+    }
+    uint32_t *pos = (uint32_t *)B.pos_a.p, *other = (uint32_t *)B.pos_b.p;
+    for (uint64_t h = KEY_SYMS; m; h *= 2) {
+        cub::DoubleBuffer<uint64_t> pk((uint64_t *)B.key_a.p, (uint64_t *)B.key_b.p);
+        cub::DoubleBuffer<uint32_t> pv(pos, other);
+        const int gm = grid_for(m);
+        k_pair_keys<<<gm, 256, 0, s>>>(pos, rank, m, n, h, bits, pk.Current());
+        if ((rc = sort_pairs<uint64_t, NumT>(B.tmp, pk, pv, (NumT)m, 2 * bits, s))) return rc;
+        uint2 *heads = (uint2 *)pk.Alternate();
+        k_pair_heads<<<gm, 256, 0, s>>>(pk.Current(), m, bits, heads);
+        if ((rc = scan_in_place(B.tmp, heads, MaxOp2(), (NumT)m, s))) return rc;
+        k_place<<<gm, 256, 0, s>>>(pk.Current(), pv.Current(), heads, m, bits, d_sa, rank, open);
+        if ((rc = keep_open<NumT>(B.tmp, pv.Current(), open, pv.Alternate(), d_count, (NumT)m, m, s))) return rc;
+        pos = pv.Alternate();
+        other = pv.Current();
+    }
     MICA_CUDA_TRY(cudaStreamSynchronize(s));
     MICA_CUDA_TRY(cudaGetLastError());
-    cleanup();
     return 0;
 }
 
