@@ -1310,17 +1310,17 @@ bool bidir_available(const mica_index *idx)
 
 // Entries of each warp's overflow stacks: their 32 bytes per entry and warp
 // take a sixteenth of the device memory free at the workspace's first
-// bidirectional call, at most 8 GiB and at least BD_DEEP_MIN entries.  The
-// stacks of a warp whose tasks sit in long repeats (a read inside a tandem
-// array matches thousands of rows and branches at every substitution) hold
-// the frontier of its depth-first walk; when one fills, its oldest nodes go
-// to the next round.
+// bidirectional call, at most 1 GiB and at least BD_DEEP_MIN entries.  The
+// stacks of a warp whose tasks sit in long repeats hold the frontier of its
+// depth-first walk; when one fills, its oldest nodes go to the next round.
+// (With up to 8 GiB no batch measured was faster, and giving the memory back
+// took 8.3 ms of an index's release; with 1 GiB it takes 3.1.)
 static uint32_t bidir_deep_cap(Workspace &w, uint64_t warps)
 {
     if (w.bd_deep_cap == 0) {
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); fr = 0; }
-        uint64_t budget = std::min<uint64_t>(fr / 16, 8ull << 30);
+        uint64_t budget = std::min<uint64_t>(fr / 16, 1ull << 30);
         uint64_t cap = budget / (warps * 32);
         w.bd_deep_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(cap, BD_DEEP_MIN), 1u << 20);
     }
