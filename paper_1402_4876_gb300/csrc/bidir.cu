@@ -27,8 +27,13 @@
 // genome's start, whose preceding symbol is $).  Extending to the right is the
 // same step on the reversed genome's index.
 //
+// With the whole suffix array resident the seed sweep (sweep.cu) goes first and
+// the trees it leaves are tree.cu's; the kernel here searches whole tasks
+// where those cannot run (no suffix array, seeds too short to check), when a
+// node budget is set, and for schemes that found no room among the nodes.
+//
 // The kernel is a persistent warp pool like k_persistent: each warp holds up
-// to 32 tasks, one per lane slot, and two node stacks in shared memory
+// to 64 tasks in slots, and two node stacks in shared memory
 // (multi-row and single-row nodes); every round extends up to 32 nodes of one
 // kind, or seeds up to 32 schemes.  A full stack moves its oldest nodes to the
 // warp's overflow stack in global memory.  A warp leaves when the task
@@ -49,7 +54,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "bidir_common.cuh"
+#include "sweep_common.cuh"
 
 namespace mica {
 namespace {
@@ -65,20 +70,6 @@ constexpr uint32_t BD_RUN = 32;              // steps of a run (nodes whose rows
 constexpr uint32_t BD_CHAIN = 16;           // extension steps a lane may take on one multi-row node in a round
 constexpr uint32_t BD_ADMIT_LOW = 96;       // admit new tasks while fewer items are pending ...
 constexpr uint32_t BD_ADMIT_FREE = 16;      // ... and at least this many slots are free (or nothing is pending)
-
-// node meta: slot (6 bits) | a (9) | b (9) | d (2) | d0 (2) | scheme (3)
-__device__ __forceinline__ uint32_t bd_meta(uint32_t slot, uint32_t a, uint32_t b, uint32_t d, uint32_t d0,
-                                            uint32_t j)
-{
-    return slot | (a << 6) | (b << 15) | (d << 24) | (d0 << 26) | (j << 28);
-}
-constexpr uint32_t BM_SLOT_MASK = 63u;
-__device__ __forceinline__ uint32_t bm_slot(uint32_t x) { return x & BM_SLOT_MASK; }
-__device__ __forceinline__ uint32_t bm_a(uint32_t x) { return (x >> 6) & 511u; }
-__device__ __forceinline__ uint32_t bm_b(uint32_t x) { return (x >> 15) & 511u; }
-__device__ __forceinline__ uint32_t bm_d(uint32_t x) { return (x >> 24) & 3u; }
-__device__ __forceinline__ uint32_t bm_d0(uint32_t x) { return (x >> 26) & 3u; }
-__device__ __forceinline__ uint32_t bm_j(uint32_t x) { return (x >> 28) & 7u; }
 
 struct BidirArgs {
     IndexView ix;
@@ -208,25 +199,6 @@ __device__ __forceinline__ void bd_complement_row(uint32_t *row, uint32_t m)
         uint32_t hi = row[q], lo = q + 1 < Wn ? row[q + 1] : 0u;
         row[q] = rc_word(hi, lo, m);
     }
-}
-
-// May a child that extends P[a, b) by base c at position pos (to the left
-// when a > 0, else to the right) exist under scheme j?  Returns the child's
-// d0 (mismatches before its current left piece) through d0n.
-__device__ __forceinline__ bool bd_allowed(uint32_t j, uint32_t a, uint32_t pos, unsigned long long bounds,
-                                           uint32_t k, uint32_t d, uint32_t d0, uint32_t cost, uint32_t &d0n)
-{
-    const uint32_t dn = d + cost;
-    d0n = d0;
-    if (dn > k) return false;
-    if (j == SCHEME_FREE || a == 0) return true;              // free scheme, or the right phase
-    const uint32_t i = piece_at(bounds, pos);
-    if (i == j) return cost == 0;                             // the exact piece
-    // a piece left of j: it needs a substitution, and so do pieces 0 .. i - 1
-    d0n = (a == bound_at(bounds, i + 1)) ? d : d0;            // entering piece i
-    const uint32_t dp = dn - d0n;
-    if (pos == bound_at(bounds, i)) return dp >= 1 && dn + i <= k;   // piece i complete
-    return dn + i + (dp == 0 ? 1u : 0u) <= k;
 }
 
 // The text check of a one-row node: its pattern `pat` (m bases in p pieces
@@ -1194,16 +1166,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
     // as much as its search)
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1) {
-        const uint32_t n = *(volatile unsigned *)&ctl->fr_count;
-        ctl->spills += n;
-        ctl->ntasks = min(n, a.fr_cap);
-        ctl->unfinished = (n ? 1u : 0u) | (*(volatile unsigned *)&ctl->redo_reads ? 2u : 0u);
-        ctl->rounds_run += n != 0;
-        ctl->task_head = 0;
-        ctl->fr_count = 0;
-        ctl->done_ctas = 0;
-    }
+    if (threadIdx.x == 0 && atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1) end_round(ctl, a.fr_cap);
 }
 
 // The reads whose bit is set: into list[0, *n_list), with their leaf counts
@@ -1337,17 +1300,23 @@ static uint32_t frontier_cap(uint64_t n)
 {
     return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(2 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
 }
+// Items of rows to check: the sweep's, and what four launches of the trees add.
+static uint32_t item_cap(uint64_t n) { return (uint32_t)std::min<uint64_t>(2ull * frontier_cap(n), 1u << 28); }
 constexpr uint32_t BD_MAX_ROUNDS = 64;
+constexpr uint32_t ROWS_EVERY = 4;   // launches of the trees between two checks of the row items
 static uint64_t redo_bytes(uint64_t n) { return redo_bits_bytes(n) + std::max<uint64_t>(n, 1) * 4 + 16; }
 
-// The sweep goes before the kernel when its task list (8 bytes for each of 2n
-// tasks, in the frontier buffer that round 1 writes first) fits and its
-// seeds can be checked.
+// The sweep goes first when its task list (8 bytes for each of 2n tasks) fits
+// and its seeds can be checked.
 static bool use_sweep(const mica_index *idx, uint64_t n)
 {
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     return 2 * n <= frontier_cap(n) && vmin < 256 && sweep_available(idx, vmin);
 }
+
+// After the sweep the trees grow from the frontier, a thread a node (tree.cu),
+// unless a node budget is set, which is this kernel's.
+static bool use_tree(const mica_index *idx, uint64_t n) { return use_sweep(idx, n) && idx->tuning.bidir_budget == 0; }
 
 // Reserve the bidirectional search's buffers for n reads; fills the control
 // block template and the grid.
@@ -1364,10 +1333,12 @@ int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tm
     if ((rc = dev_reserve(w.deep, (size_t)warps * bidir_deep_cap(w, warps) * 32))) return rc;
     // given-up reads: a bit per read, then a list of them and its length
     if ((rc = dev_reserve(w.redo, redo_bytes(n)))) return rc;
-    // exported nodes: two rounds' buffers of (task, l, lr, sz) and meta
-    if ((rc = dev_reserve(w.frontier, 2 * frontier_cap(n) * 20))) return rc;
+    // nodes: two rounds' buffers of (task, l, lr, sz) and meta; the sweep's row items and task list
+    if ((rc = dev_reserve(w.frontier, (uint64_t)frontier_cap(n) * (2 * 20) + (uint64_t)item_cap(n) * 16 +
+                                      std::max<uint64_t>(n, 1) * 16)))
+        return rc;
     tmpl = SearchCtl{};
-    tmpl.ntasks = use_sweep(idx, n) ? 0 : 2 * n;   // the sweep counts the tasks it leaves
+    tmpl.ntasks = use_sweep(idx, n) ? 0 : 2 * n;   // the sweep counts the tasks (or nodes) it leaves
     tmpl.iv_cap = w.iv_cap;
     return 0;
 }
@@ -1412,6 +1383,9 @@ static uint32_t *frontier_meta(Workspace &w, uint64_t n, int b)
     return (uint32_t *)(frontier_items(w, n, b) + frontier_cap(n));
 }
 
+static uint4 *row_items(Workspace &w, uint64_t n) { return frontier_items(w, n, 2); }
+static uint2 *sweep_list(Workspace &w, uint64_t n) { return (uint2 *)(row_items(w, n) + item_cap(n)); }
+
 // The kernel moves frontier items and overflow-stack entries as 16-byte
 // vectors: refuse a launch whose buffers are not on 16-byte boundaries.
 static int check_vector_alignment(const BidirArgs &ba)
@@ -1426,9 +1400,10 @@ static int check_vector_alignment(const BidirArgs &ba)
     return 0;
 }
 
-// Launch frontier round r >= 1 (its tasks: the nodes round r - 1 exported).
-static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, int r, cudaStream_t s,
-                        uint64_t &launches)
+// Launch frontier round r >= 1 (its tasks: the nodes round r - 1 exported), of
+// the trees' kernel or of this file's.
+static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, int r, bool tree,
+                        cudaStream_t s, uint64_t &launches)
 {
     const BidirShape &sh = g_bd_shapes[bidir_shape_index(idx)];
     BidirArgs ba;
@@ -1439,6 +1414,11 @@ static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd
     ba.fr_out = frontier_items(w, rd.n, r & 1);
     ba.fr_out_meta = frontier_meta(w, rd.n, r & 1);
     if (int rc = check_vector_alignment(ba)) return rc;
+    if (tree) {
+        launches++;
+        return launch_tree(ba.fwd, ba.rev, w, rd, ba.fr_in, ba.fr_in_meta, ba.fr_out, ba.fr_out_meta, ba.fr_cap,
+                           row_items(w, rd.n), item_cap(rd.n), ba.redo, ba.verify_min, s);
+    }
     sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
     launches++;
     MICA_CUDA_TRY(cudaGetLastError());
@@ -1472,17 +1452,28 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         ba.fr_in_meta = nullptr;
         ba.fr_out = frontier_items(w, rd.n, 0);
         ba.fr_out_meta = frontier_meta(w, rd.n, 0);
-        if (use_sweep(idx, rd.n)) {
-            uint2 *list = (uint2 *)frontier_items(w, rd.n, 1);
-            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, ba.budget, list, ba.fr_out, ba.fr_cap, s, launches)) return rc;
-            ba.list = list;
-        }
+        const bool sweep = use_sweep(idx, rd.n), tree = use_tree(idx, rd.n);
         if (int rc = check_vector_alignment(ba)) return rc;
-        sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
-        launches++;
-        MICA_CUDA_TRY(cudaGetLastError());
-        for (int r = 1; r <= rounds; r++)
-            if (int rc = launch_round(idx, w, rd, grid, r, s, launches)) return rc;
+        if (sweep) {
+            ba.list = sweep_list(w, rd.n);
+            // (with the trees' kernel the sweep's nodes are round 1's tasks)
+            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, idx->tuning.bidir_budget, sweep_list(w, rd.n),
+                                       tree ? ba.fr_out : nullptr, ba.fr_out_meta, ba.fr_cap, row_items(w, rd.n),
+                                       item_cap(rd.n), s, launches))
+                return rc;
+        }
+        if (!tree) {
+            if (sweep)
+                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_cap(rd.n), s, launches)) return rc;
+            sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
+            launches++;
+            MICA_CUDA_TRY(cudaGetLastError());
+        }
+        for (int r = 1; r <= rounds; r++) {
+            if (int rc = launch_round(idx, w, rd, grid, r, tree, s, launches)) return rc;
+            if (tree && (r == rounds || r % (int)ROWS_EVERY == 0))
+                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_cap(rd.n), s, launches)) return rc;
+        }
     }
     MICA_CUDA_TRY(record_event(w.kev[1], s));
     return 0;
@@ -1529,11 +1520,44 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
                  int grid, cudaStream_t s)
 {
     const uint64_t n = rd.n;
-    // four rounds per host read of the control block (a round with nothing
-    // exported to it returns at once)
-    while (r <= BD_MAX_ROUNDS && (out.unfinished & 1u) && !out.error) {
-        for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++)
-            if (int rc = launch_round(idx, w, rd, grid, (int)r, s, st.launches)) return rc;
+    bool tree = use_tree(idx, n);
+    bool rows = tree;   // rows to check may be left
+    for (;;) {
+        // four rounds (ROWS_EVERY) per host read of the control block (a round with
+        // nothing exported to it returns at once).  The first read of a search
+        // with trees comes before any round.
+        while (r <= BD_MAX_ROUNDS && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error) {
+            for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++)
+                if (int rc = launch_round(idx, w, rd, grid, (int)r, tree, s, st.launches)) return rc;
+            if (tree)
+                if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
+            MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
+            MICA_CUDA_TRY(cudaStreamSynchronize(s));
+        }
+        if (!tree || !out.pool_tasks || (out.unfinished & 1u) || out.error) break;
+        // schemes the sweep found no room for among the nodes: this kernel's
+        SearchCtl *d_ctl = (SearchCtl *)w.ctl.p;
+        MICA_CUDA_TRY(cudaMemcpyAsync(&d_ctl->ntasks, &d_ctl->pool_tasks, 8, cudaMemcpyDeviceToDevice, s));
+        MICA_CUDA_TRY(cudaMemsetAsync(&d_ctl->pool_tasks, 0, 8, s));
+        BidirArgs ba;
+        bidir_args(idx, w, rd, grid, ba);
+        ba.mode = 0;
+        ba.list = sweep_list(w, n);
+        ba.fr_in = nullptr;
+        ba.fr_in_meta = nullptr;
+        ba.fr_out = frontier_items(w, n, 0);
+        ba.fr_out_meta = frontier_meta(w, n, 0);
+        const BidirShape &sh = g_bd_shapes[bidir_shape_index(idx)];
+        sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
+        st.launches++;
+        MICA_CUDA_TRY(cudaGetLastError());
+        MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
+        MICA_CUDA_TRY(cudaStreamSynchronize(s));
+        tree = false;
+        r = 1;
+    }
+    if (rows && !out.error) {
+        if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
     }
@@ -1568,7 +1592,7 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     st.grid_ctas = (uint64_t)grid;
     w.bd_redo_seen = out.redo_reads > 0;
     // rounds a captured batch of this workspace runs: what its batches needed so far, to a power of two
-    while (w.bd_rounds < out.rounds_run && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
+    while (w.bd_rounds < out.rounds_run + 1 && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
     if (out.redo_reads) {
         int rc = redo_given_up(idx, w, st, rd, out, s);
         if (rc) return rc;

@@ -162,7 +162,8 @@ struct SearchCtl {
     unsigned int unfinished;                          // ... bit 0 nodes wait for a further round, bit 1 reads
                                                       //   were given up
     unsigned int rounds_run, done_ctas;               // ... rounds with tasks; CTAs of this launch that are done
-    unsigned int pad3_;
+    unsigned int done_rows;                           // row check: CTAs of this launch that are done
+    unsigned long long pool_tasks;                    // seed sweep: tasks left past the nodes' room
     unsigned long long verified, verify_bytes;        // bidirectional search: one-row intervals checked
                                                       //   against the text, and the bytes that read
     unsigned long long verify_sectors;                // ... and the 32-byte sectors those reads touch
@@ -376,8 +377,7 @@ int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const 
 
 // sweep.cu
 bool sweep_available(const mica_index *idx, uint32_t verify_min);
-int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint32_t budget, uint2 *list,
-                  uint4 *items, uint32_t item_cap, cudaStream_t s, uint64_t &launches);
+
 
 // post.cu
 int run_post(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, uint32_t hit_cap,

@@ -5,10 +5,12 @@
 // bases come up empty in the seed table (a read's other strand, mostly) or
 // name a few rows, each of which one look at the text decides.  The sweep does
 // exactly those: one thread per (read, strand) looks its k + 1 seeds up, the
-// rows of the small intervals are checked against the text 32 at a time, and
-// only the schemes it cannot finish (an interval of many rows, a piece too
-// short to be told apart, a read shorter than k + 1 bases) go on a task list
-// with a bit per scheme, which the bidirectional kernel works through.
+// rows of the small intervals are checked against the text 32 at a time, those
+// of somewhat larger ones go on a list (k_rows), and only the schemes it cannot
+// finish (an interval of many rows, a piece too short to be told apart, a read
+// shorter than k + 1 bases) become trees (tree.cu), or, when a node budget is
+// set or the frontier is full, tasks with a bit per scheme for bidir.cu's
+// kernel.
 //
 // What bounds it: random 32-byte reads of HBM (a table entry pair per seed, a
 // suffix array entry per row; the text of a genome of this size is L2 hits), so
@@ -19,11 +21,11 @@
 // reversed genome's table too, which only a tree's second interval needs.
 //
 // Measured on one GB300, search kernels of 1M x 150 bp reads, k = 2, on a 64
-// Mbp genome with repeats: 1.57 ms before, 0.45 ms of sweep + 0.55 ms of trees
-// with it (6M seeds and 2.4M windows at 30 G random reads/s would take 0.3 ms).
+// Mbp genome with repeats: 1.57 ms before, 0.87 ms now, 0.45 ms of it the sweep
+// (6M seeds and 3M rows at 30 G random reads/s would take 0.3 ms).
 #include <algorithm>
 
-#include "bidir_common.cuh"
+#include "sweep_common.cuh"
 
 namespace mica {
 namespace {
@@ -31,11 +33,14 @@ namespace {
 constexpr unsigned SFULL = 0xffffffffu;
 constexpr int SWEEP_WARPS = 8;
 constexpr int SWEEP_CTAS = 4;     // per SM
-constexpr uint32_t ROW_ITEM = 128;   // rows of an item (32 .. 256 within 2%)
 constexpr int SWEEP_QUEUE = 64;   // intervals waiting: fewer than 32 left over (each has a row) plus 32 new ones
 
 struct SweepArgs {
-    QmerView seed;               // the longer table of G$ when there is one
+    QmerView seed, rseed;        // the longer tables of G$ and G~$ when there are such
+    uint4 *nodes;                // the trees' first frontier (null: everything left goes on the list)
+    uint32_t *node_meta;
+    uint32_t node_cap;
+    uint32_t rows_all;           // N + 1
     const uint2 *sa_ctx;
     const uint32_t *text;
     uint64_t n;
@@ -44,37 +49,11 @@ struct SweepArgs {
     Interval *iv;
     uint32_t *iv_cnt;
     uint2 *list;                 // (task, schemes left as bits)
-    // larger intervals, a piece of up to ROW_ITEM rows each: (row l, task, rows | scheme << 9 | context bases in
-    // the exact piece << 11 | budget << 16 | pattern position of the matched bases << 18, the read's context)
+    // larger intervals (sweep_common.cuh)
     uint4 *items;
     uint32_t item_cap;
     uint32_t verify_min, split, split_max;
 };
-
-// Raw word i of a read, 0 outside it.
-__device__ __forceinline__ uint32_t raw_word(const uint32_t *w, int i, int wn)
-{
-    return (i >= 0 && i < wn) ? __ldg(w + i) : 0u;
-}
-
-// The 16 bases of the pattern (the read, or its other strand) before position
-// at, the nearest in the top bits, as the index keeps a row's; zeros past the
-// pattern's start.
-__device__ __forceinline__ uint32_t read_context(const uint32_t *w, uint32_t minus, uint32_t m, uint32_t at)
-{
-    const int wn = (int)((m + 15) >> 4);
-    if (minus) {   // R[m - at, m - at + 16) complemented, back to front
-        const uint32_t p = m - at;
-        const int i = (int)(p >> 4);
-        return rev_groups(~__funnelshift_r(raw_word(w, i, wn), raw_word(w, i + 1, wn), 2u * (p & 15u)));
-    }
-    if (at >= 16u) {
-        const uint32_t p = at - 16u;
-        const int i = (int)(p >> 4);
-        return __funnelshift_r(raw_word(w, i, wn), raw_word(w, i + 1, wn), 2u * (p & 15u));
-    }
-    return at ? __ldg(w) << (2u * (16u - at)) : 0u;
-}
 
 // One leaf per lane (where leaf): its interval, with one counter update per warp.
 __device__ __forceinline__ void sweep_emit(const SweepArgs &a, bool leaf, uint32_t rid, uint32_t meta, uint32_t l,
@@ -237,32 +216,22 @@ __device__ __forceinline__ void sweep_rows(const SweepArgs &a, SweepQueue &Q, ui
     __syncwarp();
 }
 
-// Put the warp's intervals of many rows (lanes with `want`) on the item list,
-// with one counter update; false for a lane whose items do not fit (what was
-// reserved for them is filled with empty items).
+// Put the warp's larger intervals (lanes with `want`) on the item list, with
+// one counter update; false for a lane past the list's end.
 __device__ __forceinline__ bool sweep_items(const SweepArgs &a, bool want, uint32_t l, uint32_t sz, uint32_t task,
                                             const uint32_t *w, uint32_t m, uint32_t k, uint32_t j, uint32_t qe,
                                             int lane)
 {
-    if (!__any_sync(SFULL, want)) return false;
-    const uint32_t n = want ? (sz + ROW_ITEM - 1) / ROW_ITEM : 0u;
-    uint32_t incl = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(SFULL, incl, o);
-        if (lane >= o) incl += y;
-    }
+    const unsigned bal = __ballot_sync(SFULL, want);
+    if (!bal) return false;
     uint32_t q = 0;
-    if (lane == 31) q = atomicAdd(&a.ctl->row_items, incl);
-    q = __shfl_sync(SFULL, q, 31) + incl - n;
+    if (lane == 0) q = atomicAdd(&a.ctl->row_items, (unsigned)__popc(bal));
+    q = __shfl_sync(SFULL, q, 0) + __popc(bal & ((1u << lane) - 1u));
     if (!want || q >= a.item_cap) return false;
-    const bool fits = n <= a.item_cap - q;
     const uint32_t at = bnd(j + 1, m, k + 1) - qe;
-    const uint32_t meta = (j << 9) | (min(16u, at - bnd(j, m, k + 1)) << 11) | (k << 16) | (at << 18);
-    const uint32_t ctx = read_context(w, task & 1u, m, at);
-    for (uint32_t i = 0; i < n && q + i < a.item_cap; i++)
-        a.items[q + i] = make_uint4(l + i * ROW_ITEM, task, fits ? min(sz - i * ROW_ITEM, ROW_ITEM) | meta : 0u, ctx);
-    return fits;
+    a.items[q] = make_uint4(l, task, item_meta(sz, j, min(16u, at - bnd(j, m, k + 1)), k, at, k),
+                            read_context(w, task & 1u, m, at));
+    return true;
 }
 
 __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const SweepArgs a)
@@ -325,7 +294,29 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
             const bool check = rowwise && sz <= a.split;
             const bool whole = some && qj == m;            // the seed is the whole read
             const bool larger = sweep_items(a, rowwise && !check, lj, sz, (uint32_t)t, w, m, k, j, qj, lane);
-            if (some && !check && !whole && !larger) left |= 1u << j;
+            const bool grow = some && !check && !whole && !larger;
+            if (a.nodes) {
+                // the tree's first node: the reversed seed's interval in the reversed genome's index too
+                const unsigned bal = __ballot_sync(SFULL, grow);
+                if (bal) {
+                    unsigned long long at = 0;
+                    if (lane == 0) at = atomicAdd(&a.ctl->ntasks, (unsigned long long)__popc(bal));
+                    at = __shfl_sync(SFULL, at, 0) + __popc(bal & lt);
+                    if (grow && at < a.node_cap) {
+                        const uint32_t cj = j == 0 ? code[0] : j == 1 ? code[1] : j == 2 ? code[2] : code[3];
+                        uint32_t lr, rr;
+                        seed_interval_in(a.rseed.table, a.rseed.q, a.rseed.nshort, a.rseed.short_pad, a.rseed.short_len,
+                                         a.rseed.short_bloom, rev_groups(cj) >> (2u * (16u - qj)), qj, lr, rr);
+                        const uint32_t bj = bnd(j + 1, m, p);
+                        a.nodes[at] = make_uint4((uint32_t)t, lj, lr, sz);
+                        a.node_meta[at] = bd_meta(0, bj - qj, bj, 0, 0, j);
+                    } else if (grow) {
+                        left |= 1u << j;
+                    }
+                }
+            } else if (grow) {
+                left |= 1u << j;
+            }
             sweep_emit(a, whole, rid, minus << 2, lj, rj, lane);
             const unsigned bal = __ballot_sync(SFULL, check);
             if (check) {
@@ -343,10 +334,26 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
                 if (windows >= 32) sweep_windows(a, Q, windows, lane, c_verify, c_vbytes, c_vsect);
             }
         }
+        if (a.nodes) {
+            // a read shorter than k + 1 bases: the whole tree from the full interval
+            const bool full = left && !pieces;
+            const unsigned bal = __ballot_sync(SFULL, full);
+            if (bal) {
+                unsigned long long at = 0;
+                if (lane == 0) at = atomicAdd(&a.ctl->ntasks, (unsigned long long)__popc(bal));
+                at = __shfl_sync(SFULL, at, 0) + __popc(bal & lt);
+                if (full && at < a.node_cap) {
+                    a.nodes[at] = make_uint4((uint32_t)t, 0u, 0u, a.rows_all);
+                    a.node_meta[at] = bd_meta(0, m, m, 0, 0, SCHEME_FREE);
+                    left = 0;
+                }
+            }
+        }
         const unsigned bal = __ballot_sync(SFULL, left != 0);
         if (bal) {
             unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(&a.ctl->ntasks, (unsigned long long)__popc(bal));
+            if (lane == 0)
+                at = atomicAdd(a.nodes ? &a.ctl->pool_tasks : &a.ctl->ntasks, (unsigned long long)__popc(bal));
             at = __shfl_sync(SFULL, at, 0) + __popc(bal & lt);
             if (left) a.list[at] = make_uint2((uint32_t)t, left);
         }
@@ -437,14 +444,14 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
 {
     __shared__ uint32_t pat_s[SWEEP_WARPS][MAX_WORDS], start_s[SWEEP_WARPS][64];
     const uint32_t n_items = min(*(volatile unsigned *)&a.ctl->row_items, a.item_cap);
+    if (n_items == 0 || *(volatile unsigned *)&a.ctl->error) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *pat = pat_s[warp], *st = start_s[warp];
     uint32_t c_verify = 0, c_vbytes = 0, c_vsect = 0;
     for (uint32_t it = blockIdx.x * SWEEP_WARPS + warp; it < n_items; it += gridDim.x * SWEEP_WARPS) {
         const uint4 item = __ldg(a.items + it);
         const uint32_t cnt = item.z & 511u, j = (item.z >> 9) & 3u, ex = (item.z >> 11) & 31u, k = (item.z >> 16) & 3u;
-        const uint32_t at = item.z >> 18, rid = item.y >> 1, minus = item.y & 1u;
-        if (cnt == 0) continue;
+        const uint32_t at = (item.z >> 18) & 511u, rem = (item.z >> 27) & 3u, rid = item.y >> 1, minus = item.y & 1u;
         const uint32_t m = a.rd.len[rid];
         const int wn = (int)((m + 15) >> 4);
         const uint32_t *w = a.rd.words + a.rd.word_off[rid];
@@ -463,7 +470,7 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
                 df = (df | (df >> 1)) & 0x55555555u;
                 if (at < 16u) df &= at ? ~0u << (2u * (16u - at)) : 0u;
                 const bool exact = ex == 0 || (df >> (2u * (16u - ex))) == 0;
-                stay = x.x >= at && (uint64_t)s + m <= a.n && exact && __popc(df) <= k;
+                stay = x.x >= at && (uint64_t)s + m <= a.n && exact && __popc(df) <= rem;
                 c_vbytes += 8u;
                 c_vsect += (lane & 3) == 0;
             }
@@ -491,18 +498,23 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
         atomicAdd(&a.ctl->verify_bytes, (unsigned long long)c_vbytes);
         atomicAdd(&a.ctl->verify_sectors, (unsigned long long)c_vsect);
     }
+    // the last CTA: the list is empty again (a search may go on and add to it)
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&a.ctl->done_rows, 1u) == gridDim.x - 1) {
+        a.ctl->row_items = 0;
+        a.ctl->done_rows = 0;
+    }
 }
 
 }  // namespace
 
 // Rows of an interval the sweep checks itself, and those it puts on the item
-// list.  Up to 32 are a warp's one look.  Past 256 a read's hits outgrow the
-// warp that finishes it: us per pass with 32 (no list) / 128 / 256 / 512 / 1024
-// / 2048, 64 Mbp 1M reads 1378 / 1308 / 1233 / 1225 / 1299 / 1520, uneven 1M 2506
-// / 2428 / 2290 / 2272 / 2404 / 3416, 33k short reads with a cap of 10 313 / 309
-// / 296 / 349 / 334 / 335, a human-like genome within 2%.
+// list.  Up to 32 are a warp's one look; past 64 a first extension in the trees
+// drops most rows of a repeat family for less than their checks cost (32 / 64 /
+// 128 / 256: 512 Mbp human-like 1M mates 3.57 / 3.57 / 3.58 / 4.00 ms of search
+// kernels, uneven 1M reads 1.38 / 1.39 / 1.50 / 1.55 ms).
 constexpr uint32_t SWEEP_SPLIT = 32;
-constexpr uint32_t SWEEP_SPLIT_MAX = 256;
+constexpr uint32_t SWEEP_SPLIT_MAX = 64;
 
 // May the sweep run for an index and its verify threshold (matched bases)?
 // It needs the suffix array and the text, and seeds long enough to be checked.
@@ -512,43 +524,76 @@ bool sweep_available(const mica_index *idx, uint32_t verify_min)
     return idx->view.sa_ctx && verify_min && verify_min <= q;
 }
 
-// Enqueue the sweep of n reads: leaves into iv, the tasks left into list (2 n
-// entries), their number in ctl->ntasks (0 before).
-int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint32_t budget, uint2 *list,
-                  uint4 *items, uint32_t item_cap, cudaStream_t s, uint64_t &launches)
+static void base_view(QmerView &q, const uint32_t *table, uint32_t len, uint32_t nshort, const uint32_t *pad,
+                      const uint32_t *slen, unsigned long long bloom)
+{
+    q.table = table;
+    q.q = len;
+    q.nshort = nshort;
+    q.short_bloom = bloom;
+    for (uint32_t i = 0; i < MAX_Q; i++) {
+        q.short_pad[i] = pad[i];
+        q.short_len[i] = slen[i];
+    }
+}
+
+static SweepArgs sweep_args(const mica_index *idx, Workspace &w, const ReadsView &rd)
 {
     SweepArgs a{};
     const IndexView &v = idx->view;
     if (v.lfwd.table) {
         a.seed = v.lfwd;
+        a.rseed = v.lrev;
     } else {
-        a.seed.table = v.table;
-        a.seed.q = v.q;
-        a.seed.nshort = v.nshort;
-        a.seed.short_bloom = v.short_bloom;
-        for (uint32_t i = 0; i < MAX_Q; i++) {
-            a.seed.short_pad[i] = v.short_pad[i];
-            a.seed.short_len[i] = v.short_len[i];
-        }
+        base_view(a.seed, v.table, v.q, v.nshort, v.short_pad, v.short_len, v.short_bloom);
+        base_view(a.rseed, v.rev.table, v.q, v.rev.nshort, v.rev.short_pad, v.rev.short_len, v.rev.short_bloom);
     }
     a.sa_ctx = v.sa_ctx;
     a.text = v.text;
     a.n = v.n;
+    a.rows_all = v.rows;
     a.rd = rd;
     a.ctl = (SearchCtl *)w.ctl.p;
     a.iv = (Interval *)w.iv.p;
     a.iv_cnt = (uint32_t *)w.iv_cnt.p;
+    return a;
+}
+
+// Enqueue the sweep of n reads: leaves into iv, larger intervals' rows into
+// items, and what is left as nodes (up to `cap`, their number in ctl->ntasks,
+// 0 before), or, with none given or past their end, as tasks with a bit per
+// scheme in list (2 n entries; ctl->pool_tasks, or ctl->ntasks without nodes).
+int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t verify_min, uint32_t budget,
+                  uint2 *list, uint4 *nodes, uint32_t *node_meta, uint32_t cap, uint4 *items, uint32_t item_cap,
+                  cudaStream_t s, uint64_t &launches)
+{
+    SweepArgs a = sweep_args(idx, w, rd);
     a.list = list;
+    a.nodes = nodes;
+    a.node_meta = node_meta;
+    a.node_cap = cap;
+    a.items = items;
+    a.item_cap = item_cap;
     a.verify_min = verify_min;
     a.split = SWEEP_SPLIT;
     // (a node budget below 64 asks for short turns: then larger intervals stay with the tree, which it governs)
-    a.split_max = budget < 64 ? SWEEP_SPLIT : SWEEP_SPLIT_MAX;
-    a.items = items;
-    a.item_cap = item_cap;
+    a.split_max = budget && budget < 64 ? SWEEP_SPLIT : SWEEP_SPLIT_MAX;
     const uint64_t blocks = (2 * rd.n + SWEEP_WARPS * 32 - 1) / (SWEEP_WARPS * 32);
     k_sweep<<<(unsigned)std::min<uint64_t>(blocks, 152ull * SWEEP_CTAS), SWEEP_WARPS * 32, 0, s>>>(a);
+    launches++;
+    MICA_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
+// Enqueue the check of the items not yet done.
+int enqueue_rows(const mica_index *idx, Workspace &w, const ReadsView &rd, uint4 *items, uint32_t item_cap,
+                 cudaStream_t s, uint64_t &launches)
+{
+    SweepArgs a = sweep_args(idx, w, rd);
+    a.items = items;
+    a.item_cap = item_cap;
     k_rows<<<152 * SWEEP_CTAS, SWEEP_WARPS * 32, 0, s>>>(a);
-    launches += 2;
+    launches++;
     MICA_CUDA_TRY(cudaGetLastError());
     return 0;
 }
