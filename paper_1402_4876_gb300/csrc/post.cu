@@ -1,4 +1,4 @@
-// From leaf SA intervals to per-read hit lists, in seven kernels (eight for more
+// From leaf SA intervals to per-read hit lists, in five kernels (seven for more
 // than 512 reads):
 //   1. k_tile_counts, k_offsets: prefix sum of the per-read interval counts;
 //   2. k_iv_scatter: the intervals grouped by read, and total = the sum of a
@@ -7,7 +7,7 @@
 //   4. k_finish_small: prefix sum of the listed counts -> CSR offsets, and the
 //      hits of reads with a few; larger reads and reads over their cap go on
 //      lists;
-//   5. k_finish_warp, k_finish_block (two sizes): those reads, a warp or a block each: over
+//   5. k_finish_block (blocks of two sizes): those reads, a warp or a block each: over
 //      the cap the first cap rows in the order (d, strand, row) are kept, then
 //      rows become text positions, and the hits go out sorted by (position,
 //      strand).
@@ -36,8 +36,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t TILE = 512;                // reads per block of the per-read passes
 constexpr uint32_t TILE_THREADS = 256;
 constexpr uint32_t SMALL_HITS = 8;             // reads up to this many hits: one thread each
-constexpr uint32_t WARP_HITS = 256;            // up to this many hits and intervals: a warp each ...
-constexpr uint32_t WARP_READS = 4;             // ... 4 warps per block;
+constexpr uint32_t WARP_HITS = 256;            // up to this many hits and intervals: a warp each
 constexpr uint32_t WARP_CAP = 65535;           // (and a cap its 32-bit sums hold)
 constexpr uint32_t BLOCK_HITS = 4096;          // up to this many hits: a block each; above: the host's loop
 constexpr uint32_t BLOCK_READ_THREADS = 128;
@@ -360,7 +359,7 @@ struct FinishArgs {
     uint64_t *hits;              // packed: pos | strand << 32 | mm << 40
     uint64_t n, capacity;
     uint32_t cap;
-    uint32_t *lists;             // reads for k_finish_warp from the front, for k_finish_block from the back
+    uint32_t *lists;             // reads for a warp each from the front, for a block each from the back
     uint32_t *huge;              // reads with more than BLOCK_HITS hits from the front, those of long lists from the back
     SearchCtl *ctl;
 };
@@ -548,102 +547,6 @@ __device__ __forceinline__ void sort_hits(uint64_t *sh, uint32_t cnt, uint32_t *
     for (uint32_t i = tid; i < cnt; i += nt) out[i] = sh[i];
 }
 
-// Reads of up to WARP_HITS hits and intervals: one warp each, taken from the
-// list by a counter (reads differ a lot in size: a fixed stride left one warp
-// with the largest).  Each lane holds up to eight intervals in registers.
-__global__ void __launch_bounds__(WARP_READS * 32) k_finish_warp(const FinishArgs a)
-{
-    __shared__ uint64_t sh_s[WARP_READS][WARP_HITS];
-    __shared__ uint32_t bits_s[WARP_READS][WARP_SPAN / 16], pre_s[WARP_READS][WARP_SPAN / 16];
-    if (search_open(a.ctl)) return;
-    const uint32_t lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    uint64_t *sh = sh_s[wi];
-    const unsigned n_list = a.ctl->n_warp;
-    uint32_t steps = 0;
-    constexpr uint32_t PER = WARP_HITS / 32;
-    for (;;) {
-        unsigned bi = 0;
-        if (lane == 0) bi = atomicAdd(&a.ctl->next_warp, 1u);
-        bi = __shfl_sync(FULL, bi, 0);
-        if (bi >= n_list) break;
-        const uint32_t r = a.lists[bi];
-        const uint64_t b = a.iv_off[r], q0 = a.hit_off[r], t = a.total[r];
-        const uint32_t ni = (uint32_t)(a.iv_off[r + 1] - b), keep = (uint32_t)(a.hit_off[r + 1] - q0);
-        uint32_t l[PER], sz[PER], meta[PER];
-#pragma unroll
-        for (uint32_t i = 0; i < PER; i++) {
-            const uint32_t x = i * 32 + lane;
-            l[i] = sz[i] = meta[i] = 0;
-            if (x < ni) {
-                const Interval v = a.ivs[b + x];
-                l[i] = v.l; sz[i] = v.r - v.l; meta[i] = v.meta;
-            }
-        }
-        if (t > keep) {
-            // over the cap: the first keep rows in the order (d, strand, row).  Interval keys are
-            // distinct, so a bitwise search from the top key bit finds the key K at which the rows
-            // counted in key order reach keep (sizes cut at 2^16, more than any cap taken here)
-            uint64_t key[PER];
-#pragma unroll
-            for (uint32_t i = 0; i < PER; i++) {
-                Interval v;
-                v.l = l[i]; v.r = l[i] + sz[i]; v.meta = meta[i]; v.read = r;
-                if (sz[i]) to_rows(v, a.ix.isa);
-                l[i] = v.l; meta[i] = v.meta;
-                key[i] = iv_key(v);
-                if (sz[i] == 0) key[i] = ~0ull;
-                sz[i] = min(sz[i], WARP_CAP + 1u);
-            }
-            uint64_t prefix = 0;
-            uint32_t before = 0;
-            for (int bit = 34; bit >= 0; bit--) {
-                const uint64_t hi = prefix >> (bit + 1);
-                uint32_t z = 0;
-#pragma unroll
-                for (uint32_t i = 0; i < PER; i++)
-                    if ((key[i] >> (bit + 1)) == hi && !((key[i] >> bit) & 1u)) z += sz[i];
-                z = __reduce_add_sync(FULL, z);
-                if (before + z < keep) { before += z; prefix |= 1ull << bit; }
-            }
-#pragma unroll
-            for (uint32_t i = 0; i < PER; i++) {
-                if (key[i] == prefix) sz[i] = keep - before;
-                else if (key[i] > prefix) sz[i] = 0;
-            }
-        }
-        // the rows' hits, lane by lane; an interval of several rows by the whole warp
-        uint32_t mine = 0;
-#pragma unroll
-        for (uint32_t i = 0; i < PER; i++) mine += sz[i];
-        uint32_t at = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, at, o);
-            if ((int)lane >= o) at += y;
-        }
-        at -= mine;
-#pragma unroll
-        for (uint32_t i = 0; i < PER; i++) {
-            if (sz[i] == 1) sh[at] = hit_of(a.ix, l[i], meta[i]);
-            for (unsigned todo = __ballot_sync(FULL, sz[i] > 1); todo; todo &= todo - 1) {
-                const int src = __ffs(todo) - 1;
-                const uint32_t wl = __shfl_sync(FULL, l[i], src), wz = __shfl_sync(FULL, sz[i], src);
-                const uint32_t wm = __shfl_sync(FULL, meta[i], src), wa = __shfl_sync(FULL, at, src);
-                for (uint32_t x = lane; x < wz; x += 32) sh[wa + x] = hit_of(a.ix, wl + x, wm);
-            }
-            at += sz[i];
-        }
-        __syncwarp();
-        if (!a.ix.sa_ctx) {
-            locate_hits(a.ix, sh, keep, lane, 32, steps);
-            __syncwarp();
-        }
-        sort_hits<false>(sh, keep, bits_s[wi], pre_s[wi], WARP_SPAN, a.hits + q0, lane, 32);
-        __syncwarp();
-    }
-    if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
-}
-
 // Where a block cuts a read's list of intervals ivs[b, e) with more than cap
 // rows: the first cap rows in the order (d, strand, row) are the intervals of
 // the classes (d, strand) before `cls`, those of cls whose row is below `row`,
@@ -766,7 +669,101 @@ __device__ __forceinline__ void expand_block(const IndexView &ix, const Interval
     __syncthreads();
 }
 
-// Larger reads (up to BLOCK_HITS hits): one block each, taken by a counter.
+// Reads of up to WARP_HITS hits and intervals: one warp each, taken from the
+// list by a counter (reads differ a lot in size: a fixed stride left one warp
+// with the largest).  Each lane holds up to eight intervals in registers.
+// sh, bits, pre: the warp's own shared memory.
+__device__ __forceinline__ void finish_by_warps(const FinishArgs &a, uint64_t *sh, uint32_t *bits, uint32_t *pre,
+                                                uint32_t &steps)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const unsigned n_list = a.ctl->n_warp;
+    constexpr uint32_t PER = WARP_HITS / 32;
+    for (;;) {
+        unsigned bi = 0;
+        if (lane == 0) bi = atomicAdd(&a.ctl->next_warp, 1u);
+        bi = __shfl_sync(FULL, bi, 0);
+        if (bi >= n_list) break;
+        const uint32_t r = a.lists[bi];
+        const uint64_t b = a.iv_off[r], q0 = a.hit_off[r], t = a.total[r];
+        const uint32_t ni = (uint32_t)(a.iv_off[r + 1] - b), keep = (uint32_t)(a.hit_off[r + 1] - q0);
+        uint32_t l[PER], sz[PER], meta[PER];
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) {
+            const uint32_t x = i * 32 + lane;
+            l[i] = sz[i] = meta[i] = 0;
+            if (x < ni) {
+                const Interval v = a.ivs[b + x];
+                l[i] = v.l; sz[i] = v.r - v.l; meta[i] = v.meta;
+            }
+        }
+        if (t > keep) {
+            // over the cap: the first keep rows in the order (d, strand, row).  Interval keys are
+            // distinct, so a bitwise search from the top key bit finds the key K at which the rows
+            // counted in key order reach keep (sizes cut at 2^16, more than any cap taken here)
+            uint64_t key[PER];
+#pragma unroll
+            for (uint32_t i = 0; i < PER; i++) {
+                Interval v;
+                v.l = l[i]; v.r = l[i] + sz[i]; v.meta = meta[i]; v.read = r;
+                if (sz[i]) to_rows(v, a.ix.isa);
+                l[i] = v.l; meta[i] = v.meta;
+                key[i] = iv_key(v);
+                if (sz[i] == 0) key[i] = ~0ull;
+                sz[i] = min(sz[i], WARP_CAP + 1u);
+            }
+            uint64_t prefix = 0;
+            uint32_t before = 0;
+            for (int bit = 34; bit >= 0; bit--) {
+                const uint64_t hi = prefix >> (bit + 1);
+                uint32_t z = 0;
+#pragma unroll
+                for (uint32_t i = 0; i < PER; i++)
+                    if ((key[i] >> (bit + 1)) == hi && !((key[i] >> bit) & 1u)) z += sz[i];
+                z = __reduce_add_sync(FULL, z);
+                if (before + z < keep) { before += z; prefix |= 1ull << bit; }
+            }
+#pragma unroll
+            for (uint32_t i = 0; i < PER; i++) {
+                if (key[i] == prefix) sz[i] = keep - before;
+                else if (key[i] > prefix) sz[i] = 0;
+            }
+        }
+        // the rows' hits, lane by lane; an interval of several rows by the whole warp
+        uint32_t mine = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) mine += sz[i];
+        uint32_t at = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, at, o);
+            if ((int)lane >= o) at += y;
+        }
+        at -= mine;
+#pragma unroll
+        for (uint32_t i = 0; i < PER; i++) {
+            if (sz[i] == 1) sh[at] = hit_of(a.ix, l[i], meta[i]);
+            for (unsigned todo = __ballot_sync(FULL, sz[i] > 1); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t wl = __shfl_sync(FULL, l[i], src), wz = __shfl_sync(FULL, sz[i], src);
+                const uint32_t wm = __shfl_sync(FULL, meta[i], src), wa = __shfl_sync(FULL, at, src);
+                for (uint32_t x = lane; x < wz; x += 32) sh[wa + x] = hit_of(a.ix, wl + x, wm);
+            }
+            at += sz[i];
+        }
+        __syncwarp();
+        if (!a.ix.sa_ctx) {
+            locate_hits(a.ix, sh, keep, lane, 32, steps);
+            __syncwarp();
+        }
+        sort_hits<false>(sh, keep, bits, pre, WARP_SPAN, a.hits + q0, lane, 32);
+        __syncwarp();
+    }
+}
+
+// Larger reads (up to BLOCK_HITS hits): one block each, taken by a counter;
+// then, in the small blocks, a warp each for the others (the largest first: a
+// kernel for each kind had every kind's last reads run alone).
 // Those with the longest lists (a read in a diverged tandem array has 10^5
 // intervals of a row each) have blocks of 1,024 threads: 128 took 0.65 ms
 // for the longest of a million reads.
@@ -801,6 +798,12 @@ __global__ void __launch_bounds__(NT) k_finish_block(const FinishArgs a)
         }
         sort_hits<true>(sh, keep, bits, pre, BLOCK_SPAN, a.hits + q0, threadIdx.x, NT);
         __syncthreads();
+    }
+    if (!LONG) {
+        const uint32_t wi = threadIdx.x >> 5;
+        static_assert(WARP_HITS * (BLOCK_READ_THREADS / 32) <= BLOCK_HITS &&
+                      WARP_SPAN * (BLOCK_READ_THREADS / 32) <= BLOCK_SPAN, "the warps' shares of the block's arrays");
+        finish_by_warps(a, sh + wi * WARP_HITS, bits + wi * (WARP_SPAN / 16), pre + wi * (WARP_SPAN / 16), steps);
     }
     if (!a.ix.sa_ctx) count_steps(a.ctl, steps);
 }
@@ -908,7 +911,7 @@ static uint64_t big_list_bytes(uint64_t n)
     return (std::max<uint64_t>(n, 1) * 4 + 15) & ~15ull;
 }
 
-// w.big holds the list of reads for k_finish_warp and k_finish_block (a read
+// w.big holds the list of reads for warps and blocks of their own (a read
 // is on one of them: n u32), then the list of larger ones (n u32); w.scan_tmp
 // the tile sums of the interval counts, then of the listed hits.
 static uint64_t post_list_bytes(uint64_t n) { return 2 * big_list_bytes(n); }
@@ -934,7 +937,8 @@ static FinishArgs finish_args(const mica_index *idx, Workspace &w, uint64_t n, u
 }
 
 // Steps 1 to 3: intervals grouped by read, totals, tile sums of the listed hits.
-static int enqueue_totals(Workspace &w, uint64_t n, uint32_t hit_cap, uint32_t report, cudaStream_t s, uint64_t &L)
+static int enqueue_totals(Workspace &w, uint64_t n, uint32_t hit_cap, uint32_t report, bool need_total,
+                          cudaStream_t s, uint64_t &L)
 {
     uint64_t *iv_off = (uint64_t *)w.iv_off.p, *sums = (uint64_t *)w.scan_tmp.p;
     SearchCtl *ctl = (SearchCtl *)w.ctl.p;
@@ -952,8 +956,11 @@ static int enqueue_totals(Workspace &w, uint64_t n, uint32_t hit_cap, uint32_t r
         k_stratum<<<grid1(n, 128), 128, 0, s>>>((Interval *)w.iv_sorted.p, iv_off, n, (uint64_t *)total, ctl);
         L++;
     }
-    k_listed<<<tiles, TILE_THREADS, 0, s>>>((const uint64_t *)total, n, hit_cap, sums + tiles);
-    L += 3;
+    if (tiles > 1 || need_total) {   // (a single tile has none before it)
+        k_listed<<<tiles, TILE_THREADS, 0, s>>>((const uint64_t *)total, n, hit_cap, sums + tiles);
+        L++;
+    }
+    L += 2;
     MICA_CUDA_TRY(cudaGetLastError());
     return 0;
 }
@@ -965,9 +972,8 @@ static int enqueue_finish(const FinishArgs &a, Workspace &w, cudaStream_t s, uin
     k_finish_small<<<tiles, TILE_THREADS, 0, s>>>(a, (const uint64_t *)w.scan_tmp.p + tiles);
     const uint64_t n1 = std::max<uint64_t>(a.n, 1);
     k_finish_block<LONG_THREADS><<<(unsigned)std::min<uint64_t>(152, n1), LONG_THREADS, 0, s>>>(a);
-    k_finish_warp<<<(unsigned)std::min<uint64_t>(152 * 8, n1), WARP_READS * 32, 0, s>>>(a);
     k_finish_block<BLOCK_READ_THREADS><<<(unsigned)std::min<uint64_t>(152 * 5, n1), BLOCK_READ_THREADS, 0, s>>>(a);
-    L += 4;
+    L += 3;
     MICA_CUDA_TRY(cudaGetLastError());
     return 0;
 }
@@ -980,7 +986,7 @@ static int enqueue_finish(const FinishArgs &a, Workspace &w, cudaStream_t s, uin
 int enqueue_post_device(const mica_index *idx, Workspace &w, const ReadsView &rd, uint32_t hit_cap,
                         uint32_t report, uint64_t hit_capacity, cudaStream_t s, void *status, uint64_t &L)
 {
-    if (int rc = enqueue_totals(w, rd.n, hit_cap, report, s, L)) return rc;
+    if (int rc = enqueue_totals(w, rd.n, hit_cap, report, false, s, L)) return rc;
     if (int rc = enqueue_finish(finish_args(idx, w, rd.n, hit_cap, hit_capacity), w, s, L)) return rc;
     MICA_CUDA_TRY(cudaMemcpyAsync(status, w.ctl.p, sizeof(SearchCtl), cudaMemcpyDeviceToHost, s));
     return 0;
@@ -1016,7 +1022,7 @@ int run_post(const mica_index *idx, Workspace &w, mica_stats &stt, const ReadsVi
     SearchCtl *ctl = (SearchCtl *)w.ctl.p;
     // the control block's post-search fields (a search may have run in several launches)
     MICA_CUDA_TRY(cudaMemsetAsync(&ctl->post_hits, 0, sizeof(SearchCtl) - offsetof(SearchCtl, post_hits), s));
-    if ((rc = enqueue_totals(w, n, hit_cap, report, s, L))) return rc;
+    if ((rc = enqueue_totals(w, n, hit_cap, report, true, s, L))) return rc;
     const unsigned tiles = (unsigned)tiles_of(n);
     uint64_t *sums = (uint64_t *)w.scan_tmp.p;
     k_tiles_total<<<1, TILE_THREADS, 0, s>>>(sums + tiles, tiles, sums + 2 * tiles);
