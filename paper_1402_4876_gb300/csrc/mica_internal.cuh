@@ -376,7 +376,7 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
 int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s);
 
 // sweep.cu
-bool sweep_available(const mica_index *idx, uint32_t verify_min);
+bool sweep_checks(const mica_index *idx, uint32_t verify_min);
 
 
 // post.cu

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
             const uint32_t qj = j == 0 ? qe[0] : j == 1 ? qe[1] : j == 2 ? qe[2] : qe[3];
             const bool some = qj && lj < rj;
             const uint32_t sz = rj - lj;
-            const bool rowwise = some && sz <= a.split_max && qj >= a.verify_min && m - qj >= BD_VERIFY_LEFT;
+            const bool rowwise = some && a.verify_min && sz <= a.split_max && qj >= a.verify_min && m - qj >= BD_VERIFY_LEFT;
             const bool check = rowwise && sz <= a.split;
             const bool whole = some && qj == m;            // the seed is the whole read
             const bool larger = sweep_items(a, rowwise && !check, lj, sz, (uint32_t)t, w, m, k, j, qj, lane);
@@ -516,9 +516,9 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
 constexpr uint32_t SWEEP_SPLIT = 32;
 constexpr uint32_t SWEEP_SPLIT_MAX = 64;
 
-// May the sweep run for an index and its verify threshold (matched bases)?
-// It needs the suffix array and the text, and seeds long enough to be checked.
-bool sweep_available(const mica_index *idx, uint32_t verify_min)
+// Are a seed's bases enough to check its rows against the text, at this verify
+// threshold (matched bases)?
+bool sweep_checks(const mica_index *idx, uint32_t verify_min)
 {
     const uint32_t q = idx->view.lfwd.table ? idx->view.lfwd.q : idx->view.q;
     return idx->view.sa_ctx && verify_min && verify_min <= q;

@@ -124,3 +124,45 @@ def test_invalid_device_batches_are_refused_in_the_captured_batch():
                            h.cpu().numpy().view(m.HIT_DTYPE))
             gc.assert_same(got, want, f"{which} {value}")
     idx.free()
+
+
+@pytest.mark.parametrize("full_sa", [True, False])
+def test_more_trees_than_the_frontier_holds(full_sa):
+    """300,000 reads whose seeds are too short to be checked (40 bases in four
+    pieces) leave more first nodes than the frontier's 2^20: the rest go to the
+    warp pool as tasks.  Every result equals the persistent kernel's, on repeated
+    calls, and a sample the oracle's."""
+    g = synth.uniform_genome(300_000, 21)
+    rng = np.random.default_rng(4)
+    b = synth.sample_reads(g, np.full(300_000, 40), np.full(300_000, 3), rng, subs="rate", sub_rate=0.02)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), kmer_q=10, sa_sample=8, full_sa=full_sa)
+    want = idx.align_batch(b, hit_cap=10, kernel="persistent")
+    for call in range(2):
+        gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"call {call}")
+    assert idx.stats()["fallback_reads"] == 0
+    some = b.subset(np.arange(0, b.n, 600))
+    gc.assert_same(idx.align_batch(some, hit_cap=10), oracle.FMIndex(g.codes).align(some, cap=10), "sample")
+    idx.free()
+
+
+@pytest.mark.parametrize("m,k", [(1, 0), (2, 3), (3, 3), (4, 3), (11, 0), (12, 0), (20, 1), (32, 1), (33, 1), (48, 3), (256, 3)])
+@pytest.mark.parametrize("full_sa", [True, False])
+def test_tree_shapes(m, k, full_sa):
+    """Reads shorter than k + 1 bases (one tree from the full interval), whole-read
+    seeds, pieces around the verify threshold and the longest reads, inside an
+    exact tandem array, at both ends of the genome and elsewhere."""
+    rng = np.random.default_rng(100 * m + k)
+    g = np.concatenate([rng.integers(0, 4, 3_000).astype(np.uint8), np.resize(rng.integers(0, 4, 7).astype(np.uint8), 4_000),
+                        rng.integers(0, 4, 3_000).astype(np.uint8)])
+    at = [0, g.size - m, 1_500, 3_500, 4_200, 6_990, 8_000]
+    reads = []
+    for i, a in enumerate(at):
+        r = g[a:a + m].copy()
+        if m > 20:
+            synth.substitute(r, rng.choice(m, size=i % (k + 1), replace=False), rng)
+        reads.append(r if i % 2 else (3 - r)[::-1].copy())
+    b = gc.batch_from_reads(reads, [k] * len(reads))
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g), kmer_q=8, sa_sample=8, full_sa=full_sa)
+    for cap in (0, 50):
+        gc.assert_same(idx.align_batch(b, hit_cap=cap), oracle.FMIndex(g).align(b, cap=cap), f"m {m} k {k} cap {cap}")
+    idx.free()
