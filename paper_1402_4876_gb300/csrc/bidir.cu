@@ -29,7 +29,7 @@
 //
 // With the whole suffix array resident the seed sweep (sweep.cu) goes first and
 // the trees it leaves are tree.cu's; the kernel here searches whole tasks
-// where those cannot run (no suffix array, seeds too short to check), when a
+// where those cannot run (the check off or seeds too short for it), when a small
 // node budget is set, and for schemes that found no room among the nodes.
 //
 // The kernel is a persistent warp pool like k_persistent: each warp holds up
@@ -1306,6 +1306,14 @@ constexpr uint32_t BD_MAX_ROUNDS = 64;
 constexpr uint32_t ROWS_EVERY = 4;   // launches of the trees between two checks of the row items
 static uint64_t redo_bytes(uint64_t n) { return redo_bits_bytes(n) + std::max<uint64_t>(n, 1) * 4 + 16; }
 
+// Does the tuning leave the trees to tree.cu?  A node budget of less than 1,024
+// asks for short turns, which this file's kernel takes (the autotuner's budgets
+// are not below it).
+static bool frontier_trees(const mica_index *idx)
+{
+    return idx->tuning.bidir_budget == 0 || idx->tuning.bidir_budget >= 1024;
+}
+
 // The sweep goes first when its task list (8 bytes for each of 2n tasks) fits
 // and its seeds can be checked.  Without the suffix array nothing is checked:
 // it then only turns every seed into a tree's first node (a chain of one row
@@ -1315,13 +1323,12 @@ static bool use_sweep(const mica_index *idx, uint64_t n)
 {
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     if (2 * n > frontier_cap(n)) return false;
-    if (!idx->view.sa_ctx) return idx->tuning.bidir_budget == 0;
+    if (!idx->view.sa_ctx) return frontier_trees(idx);
     return vmin < 256 && sweep_checks(idx, vmin);
 }
 
-// After the sweep the trees grow from the frontier, a thread a node (tree.cu),
-// unless a node budget is set, which is this kernel's.
-static bool use_tree(const mica_index *idx, uint64_t n) { return use_sweep(idx, n) && idx->tuning.bidir_budget == 0; }
+// After the sweep the trees grow from the frontier, a thread a node.
+static bool use_tree(const mica_index *idx, uint64_t n) { return use_sweep(idx, n) && frontier_trees(idx); }
 
 // Reserve the bidirectional search's buffers for n reads; fills the control
 // block template and the grid.

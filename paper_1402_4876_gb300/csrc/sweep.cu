@@ -8,8 +8,8 @@
 // rows of the small intervals are checked against the text 32 at a time, those
 // of somewhat larger ones go on a list (k_rows), and only the schemes it cannot
 // finish (an interval of many rows, a piece too short to be told apart, a read
-// shorter than k + 1 bases) become trees (tree.cu), or, when a node budget is
-// set or the frontier is full, tasks with a bit per scheme for bidir.cu's
+// shorter than k + 1 bases) become trees (tree.cu), or, when a small node budget
+// is set or the frontier is full, tasks with a bit per scheme for bidir.cu's
 // kernel.
 //
 // What bounds it: random 32-byte reads of HBM (a table entry pair per seed, a

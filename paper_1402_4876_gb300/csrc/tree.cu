@@ -1,6 +1,6 @@
 // The search trees the sweep leaves: the nodes of every tree in one frontier
 // in global memory, one thread a node (bidir.cu has the scheme search itself,
-// and the warp pool that works from it when a node budget is set).
+// and the warp pool that works from it when a small node budget is set).
 //
 // A tree comes from a seed in a long repeat: an interval of hundreds to tens of
 // thousands of rows whose extension is a chain of 100-250 dependent steps with

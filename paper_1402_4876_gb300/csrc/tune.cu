@@ -96,7 +96,7 @@ int mica_autotune(mica_index *idx, const uint32_t *packed_reads, const uint64_t 
         float tbest = 1e30f;
         // bidirectional shapes (task slots and warps per CTA) and node budgets
         if (bidir_available(idx)) {
-            const uint32_t budgets[] = {0, 1024, 4096};   // (0: the default, trees from the frontier)
+            const uint32_t budgets[] = {1024, 4096};
             for (int s = 0; s < bidir_shape_count(); s++)
                 for (uint32_t b : budgets) {
                     idx->tuning.bidir_shape = s;
