@@ -1291,19 +1291,23 @@ static uint32_t bidir_deep_cap(Workspace &w, uint64_t warps)
 }
 
 static uint64_t redo_bits_bytes(uint64_t n) { return ((n + 31) / 32 * 4 + 15) & ~15ull; }
-// Items per frontier buffer: 2n, at least 2^20, at most 2^28, and a multiple
+// Nodes per frontier buffer: 4n, at least 2^20, at most 2^28, and a multiple
 // of 4 so that the second buffer and both meta arrays (20 B per item in all)
 // start on a 16-byte boundary, as the kernel's 16-byte item loads and stores
-// require (an odd batch above 2^19 reads would otherwise put the second
+// require (an odd batch above 2^18 reads would otherwise put the second
 // buffer 8 bytes off).
 static uint32_t frontier_cap(uint64_t n)
 {
-    return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(2 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
+    return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(4 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
 }
-// Items of rows to check: the sweep's, and what four launches of the trees add.
-static uint32_t item_cap(uint64_t n) { return (uint32_t)std::min<uint64_t>(2ull * frontier_cap(n), 1u << 28); }
+// Items of rows to check: the sweep's (half of them), and what the trees add
+// between two checks of the list; when it is full small intervals stay nodes.
+// (2M mates on a 3.1 Gbp human-like genome need some 10M in one launch.)
+static uint32_t item_cap(uint64_t n) { return (uint32_t)std::min<uint64_t>(4ull * frontier_cap(n), 1u << 28); }
 constexpr uint32_t BD_MAX_ROUNDS = 64;
-constexpr uint32_t ROWS_EVERY = 4;   // launches of the trees between two checks of the row items
+// The row items are checked after every launch of the trees for a batch of this
+// many reads, else at the end.
+constexpr uint64_t ROWS_EACH = 1u << 16;
 static uint64_t redo_bytes(uint64_t n) { return redo_bits_bytes(n) + std::max<uint64_t>(n, 1) * 4 + 16; }
 
 // Does the tuning leave the trees to tree.cu?  A node budget of less than 1,024
@@ -1471,7 +1475,7 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
             // (with the trees' kernel the sweep's nodes are round 1's tasks)
             if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, idx->tuning.bidir_budget, sweep_list(w, rd.n),
                                        tree ? ba.fr_out : nullptr, ba.fr_out_meta, ba.fr_cap, row_items(w, rd.n),
-                                       item_cap(rd.n), s, launches))
+                                       item_cap(rd.n) / 2, s, launches))
                 return rc;
         }
         if (!tree) {
@@ -1483,7 +1487,7 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         }
         for (int r = 1; r <= rounds; r++) {
             if (int rc = launch_round(idx, w, rd, grid, r, tree, s, launches)) return rc;
-            if (tree && (r == rounds || r % (int)ROWS_EVERY == 0))
+            if (tree && (r == rounds || rd.n >= ROWS_EACH))
                 if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_cap(rd.n), s, launches)) return rc;
         }
     }
@@ -1535,14 +1539,15 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     bool tree = use_tree(idx, n);
     bool rows = tree;   // rows to check may be left
     for (;;) {
-        // four rounds (ROWS_EVERY) per host read of the control block (a round with
+        // four rounds per host read of the control block (a round with
         // nothing exported to it returns at once).  The first read of a search
         // with trees comes before any round.
         while (r <= BD_MAX_ROUNDS && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error) {
-            for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++)
+            for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++) {
                 if (int rc = launch_round(idx, w, rd, grid, (int)r, tree, s, st.launches)) return rc;
-            if (tree)
-                if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
+                if (tree)
+                    if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
+            }
             MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
             MICA_CUDA_TRY(cudaStreamSynchronize(s));
         }

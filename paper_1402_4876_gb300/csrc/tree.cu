@@ -77,20 +77,17 @@ __device__ __forceinline__ void push_node(const TreeArgs &a, uint32_t q, uint32_
     }
 }
 
-// The staged items to their list.  (It holds what a search's rounds add between
-// two checks of it in all but degenerate batches; a read whose rows find it
-// full is given up.)
-__device__ __forceinline__ void flush_items(const TreeArgs &a, const TreeStage &S, uint32_t n, int lane)
+// The staged items to their list; false when it has room for only one more
+// such flush by every warp (TreeArgs::item_cap is less than its size by that):
+// from then on this launch's small intervals stay nodes.
+__device__ __forceinline__ bool flush_items(const TreeArgs &a, const TreeStage &S, uint32_t n, int lane)
 {
     uint32_t at = 0;
     if (lane == 0) at = atomicAdd(&a.ctl->row_items, n);
     at = __shfl_sync(TFULL, at, 0);
-    for (uint32_t i = lane; i < n; i += 32) {
-        const uint4 x = S.item[i];
-        if (at + i < a.item_cap) a.items[at + i] = x;
-        else push_node(a, a.cap, x.y, 0, 0, 0, 0);
-    }
+    for (uint32_t i = lane; i < n; i += 32) a.items[at + i] = S.item[i];
     __syncwarp();
+    return at + n < a.item_cap;
 }
 
 // The staged nodes [from, n) to the frontier.
@@ -118,6 +115,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
     // nodes a warp takes at a time: no more than its part of the launch's
     const uint32_t share = max(1u, min(32u, ntasks / (gridDim.x * (TREE_THREADS / 32))));
     bool active = false, more = true;
+    bool item_room = *(volatile unsigned *)&ctl->row_items < a.item_cap;
     uint32_t task = 0, l = 0, lr = 0, sz = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
     unsigned long long bounds = 0;
     const uint32_t *w = nullptr;
@@ -200,7 +198,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             // the other side's interval start: rows of lower symbols (and a $) come first
             uint32_t acc = (left ? lr : l) + ((sd.dollar_row >= pl && sd.dollar_row < pl + sz) ? 1u : 0u);
             const bool whole = nA == 0 && nB == m;
-            const bool checkable = a.verify_min && nB - nA >= a.verify_min && m - (nB - nA) >= BD_VERIFY_LEFT;
+            const bool checkable = item_room && a.verify_min && nB - nA >= a.verify_min && m - (nB - nA) >= BD_VERIFY_LEFT;
             const uint32_t split = nA ? TREE_SPLIT_LEFT : TREE_SPLIT_RIGHT;
             uint32_t most = 0;
 #pragma unroll
@@ -283,7 +281,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
                 nn = STAGE_LOW;
             }
             if (ni > STAGE_LOW) {
-                flush_items(a, S, ni, lane);
+                item_room = flush_items(a, S, ni, lane);
                 ni = 0;
             }
         }
@@ -327,7 +325,7 @@ int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const Read
     a.out_meta = out_meta;
     a.cap = cap;
     a.items = items;
-    a.item_cap = item_cap;
+    a.item_cap = item_cap - 152u * TREE_CTAS * (TREE_THREADS / 32) * STAGE_ITEMS;
     a.redo = redo;
     a.verify_min = verify_min;
     constexpr size_t smem = sizeof(TreeStage) * (TREE_THREADS / 32);
