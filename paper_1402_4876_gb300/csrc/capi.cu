@@ -171,48 +171,53 @@ static int validate_params(const mica_index_params &p)
     return 0;
 }
 
-// ASCII genome -> base codes in place, four bytes a thread; *bad when a byte is
-// none of A/C/G/T in either case.  (A, C, G, T differ in bits 1 and 2: 0, 1, 3,
-// 2.  One host thread took longer over this than the GPU over the suffix sort.)
-__global__ void k_encode(uint32_t *__restrict__ text, uint64_t words, uint64_t len, unsigned *__restrict__ bad)
+// Is every byte one of A/C/G/T in either case?  On the host threads, before any
+// device call; every byte's condition is evaluated, so that the loop vectorises.
+static bool genome_is_acgt(const uint8_t *acgt, uint64_t len)
 {
-    bool wrong = false;
-    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t v = text[w];
-        uint32_t out = 0;
-#pragma unroll
-        for (uint32_t b = 0; b < 4; b++) {
-            const uint32_t c = (v >> (8 * b)) & 0xdfu;
-            const uint32_t x = (c >> 1) & 3u;
-            out |= (x ^ (x >> 1)) << (8 * b);
-            if (4 * w + b < len) wrong |= c != 'A' && c != 'C' && c != 'G' && c != 'T';
+    auto bad_in = [=](uint64_t i0, uint64_t i1) {
+        uint8_t bad = 0;
+        for (uint64_t i = i0; i < i1; i++) {
+            const uint8_t c = acgt[i] & 0xdf;
+            bad |= (uint8_t)((c != 'A') & (c != 'C') & (c != 'G') & (c != 'T'));
         }
-        text[w] = out;
-    }
-    if (wrong) atomicOr(bad, 1u);
+        return bad != 0;
+    };
+    constexpr uint64_t CHUNK = 1u << 21;
+    if (len <= CHUNK) return !bad_in(0, len);
+    std::atomic<bool> bad{false};
+    parallel_chunks((len + CHUNK - 1) / CHUNK, host_threads(), [&](uint64_t c) {
+        if (!bad.load(std::memory_order_relaxed) && bad_in(c * CHUNK, std::min(len, (c + 1) * CHUNK)))
+            bad.store(true, std::memory_order_relaxed);
+    });
+    return !bad.load();
 }
 
-// The genome's base codes on the device, rejecting anything but A/C/G/T.
+// ASCII genome -> base codes in place, four bytes a thread.  (A, C, G, T differ in
+// bits 1 and 2: 0, 1, 3, 2.  One host thread took longer over this than the GPU over
+// the suffix sort.)
+__global__ void k_encode(uint32_t *__restrict__ text, uint64_t words)
+{
+    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t x = (text[w] >> 1) & 0x03030303u;
+        text[w] = x ^ ((x >> 1) & 0x01010101u);
+    }
+}
+
+// A checked genome's base codes on the device.
 static int encode_genome(const uint8_t *acgt, uint64_t len, DevBuf &codes)
 {
     const uint64_t words = (len + 3) / 4;
-    DevBuf bad;
     int rc = dev_reserve(codes, std::max<uint64_t>(words, 1) * 4);
-    if (!rc) rc = dev_reserve(bad, 4);
-    unsigned wrong = 0;
     if (!rc && len) {
-        cudaError_t e = cudaMemset(bad.p, 0, 4);
-        if (e == cudaSuccess) e = cudaMemcpy(codes.p, acgt, len, cudaMemcpyHostToDevice);
+        cudaError_t e = cudaMemcpy(codes.p, acgt, len, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) {
-            k_encode<<<(unsigned)std::min<uint64_t>((words + 255) / 256, 152ull * 16), 256>>>(
-                (uint32_t *)codes.p, words, len, (unsigned *)bad.p);
+            k_encode<<<(unsigned)std::min<uint64_t>((words + 255) / 256, 152ull * 16), 256>>>((uint32_t *)codes.p, words);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = cudaMemcpy(&wrong, bad.p, 4, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) { set_last_cuda_error(e, "genome upload", __FILE__, __LINE__); rc = MICA_ECUDA; }
     }
-    dev_release(bad);
-    return rc ? rc : wrong ? MICA_EINVAL : 0;
+    return rc;
 }
 
 
@@ -573,6 +578,7 @@ int mica_index_build_resident(const uint8_t *genome_acgt, uint64_t len, const mi
     if (params) p = *params;
     if (int rc = validate_params(p)) return rc;
     if (len + 1 >= (1ull << 32)) return MICA_EINVAL;
+    if (!genome_is_acgt(genome_acgt, len)) return MICA_EINVAL;
     DeviceGuard g(device);
     MICA_CUDA_TRY(cudaSetDevice(device));
     mica_index *idx = new mica_index();
@@ -1112,6 +1118,7 @@ void mica_result_free(mica_result *res)
 int mica_debug_suffix_array(const uint8_t *genome_acgt, uint64_t len, int device, uint32_t *sa_out)
 {
     if ((!genome_acgt && len) || !sa_out || len + 1 >= (1ull << 32)) return MICA_EINVAL;
+    if (!genome_is_acgt(genome_acgt, len)) return MICA_EINVAL;
     DeviceGuard g(device);
     MICA_CUDA_TRY(cudaSetDevice(device));
     DevBuf dc, dsa;
