@@ -53,15 +53,15 @@ BIDIR_CU = os.path.join(ROOT, "paper_1402_4876_gb300", "csrc", "bidir.cu")
 PROFILE_BIDIR = os.path.join(ROOT, "profiles", "k_bidir_64m_1m150.txt")
 PROFILE_BIDIR_HUMAN = os.path.join(ROOT, "profiles", "k_bidir_3g_human2m.txt")
 KERNEL_NAMES = {"bidirectional": "k_bidir", "persistent": "k_lower_bounds + k_persistent"}
-KERNEL_LABEL = {"bidirectional": "bidirectional warp-pool (one persistent launch)",
+KERNEL_LABEL = {"bidirectional": "bidirectional (seed sweep, search trees, row checks)",
                 "persistent": "one-directional persistent warp-pool"}
 SEARCH_LABEL = {"bidirectional": "k + 1 pieces, one search per leftmost exact piece over the genome's and the "
                                  "reversed genome's index (same result as exhaustive backtracking)",
                 "persistent": "exhaustive backtracking from the read's end, pruned by mismatch lower bounds "
                               "(same result as unpruned)"}
-ALG_LABEL = {"bidirectional": "32 B x occurrence blocks read + 16 B x seeds (two table entries in each of two "
-                              "tables) + the packed reads once + 16 B x leaf intervals + the bytes of the text "
-                              "checks (4 B of SA and the window's text words per check, 4 B of ISA per leaf)",
+ALG_LABEL = {"bidirectional": "32 B x occurrence blocks read + 8 B x seeds (two entries of one table) + the packed "
+                              "reads once + 16 B x leaf intervals + the bytes of the text checks (8 B of suffix "
+                              "array entry and left context per row, the window's text words per row that passes)",
              "persistent": "32 B x occurrence blocks read (search and lower-bound pass) + 8 B x seeds + the "
                            "packed reads twice + 16 B x leaf intervals"}
 
@@ -69,7 +69,7 @@ ALG_LABEL = {"bidirectional": "32 B x occurrence blocks read + 16 B x seeds (two
 def search_alg_bytes(kernel: str, st: dict, read_bytes: int) -> int:
     """Algorithmic bytes of one search step from the on-device work counters."""
     if kernel == "bidirectional":
-        return (32 * st["rank_blocks"] + 16 * st["seeds"] + read_bytes + 16 * st["intervals"] +
+        return (32 * st["rank_blocks"] + 8 * st["seeds"] + read_bytes + 16 * st["intervals"] +
                 st.get("verify_bytes", 0))
     return 32 * st["rank_blocks"] + 8 * st["seeds"] + 2 * read_bytes + 16 * st["intervals"]
 
@@ -77,13 +77,12 @@ def search_alg_bytes(kernel: str, st: dict, read_bytes: int) -> int:
 def gather_floor(kernel: str, st: dict, read_bytes: int, index_gbs: float, text_gbs: float, copy_gbs: float):
     """The least time a search step's memory accesses can take at the measured
     ceilings: every 32-byte sector it gathers from the index (occurrence
-    blocks, one q-mer table sector per table and seed, leaf writes) at the
+    blocks, one q-mer table sector per seed, leaf writes) at the
     random-gather rate of the level the index lives in (L2 when it fits, else
-    HBM), every sector of the text checks (SA, ISA, text windows: HBM) at the
+    HBM), every sector of the text checks (SA rows, text windows: HBM) at the
     HBM random-gather rate, and the packed reads streamed at copy bandwidth.
     Returns (seconds, parts in ms)."""
-    seed_sectors = (2 if kernel == "bidirectional" else 1) * st["seeds"]
-    index_sectors = st["rank_blocks"] + seed_sectors + (st["intervals"] + 1) // 2
+    index_sectors = st["rank_blocks"] + st["seeds"] + (st["intervals"] + 1) // 2
     t_index = index_sectors * 32 / (index_gbs * 1e9)
     t_text = st.get("verify_sectors", 0) * 32 / (text_gbs * 1e9)
     t_reads = (read_bytes if kernel == "bidirectional" else 2 * read_bytes) / (copy_gbs * 1e9)

@@ -163,10 +163,10 @@ typedef struct {
     uint64_t grid_ctas;      /* persistent kernel: CTAs of the launch (SMs x resident CTAs per SM) */
     uint64_t fallback_reads; /* bidirectional kernel: reads it gave up on (over the node budget, or on a
                                 warp whose overflow stack filled), searched again by the persistent kernel */
-    uint64_t verified;       /* bidirectional kernel: one-row intervals checked against the genome's text */
-    uint64_t verify_bytes;   /* bytes those checks read: suffix array and inverse entries, text words */
-    uint64_t verify_sectors; /* 32-byte sectors those reads touch (one per SA or ISA entry, the text
-                                window's span) */
+    uint64_t verified;       /* bidirectional search: windows checked against the genome's text (rows whose
+                                left context passed) */
+    uint64_t verify_bytes;   /* bytes the row and text checks read: 8 per row looked at, text words */
+    uint64_t verify_sectors; /* 32-byte sectors those reads touch */
     float search_ms;         /* device time of the search phase (kernel + its control copies) */
     float kernel_ms;         /* device time of the search kernel launch(es) alone, with the
                                 lower-bound pass when pruning */
@@ -292,10 +292,11 @@ typedef struct {
                                occurrence blocks of the next round's nodes.  -1 = automatic (on
                                when the occurrence blocks exceed 96 MiB and so do not stay in
                                L2), 0 = off, 1 = on */
-    uint32_t bidir_budget;  /* bidirectional kernel: node expansions a task may take before it hands
+    uint32_t bidir_budget;  /* bidirectional warp pool: node expansions a task may take before it hands
                                its pending nodes to the next launch round, where they are tasks of
                                their own on every warp (bounds each round's tail; no effect on
-                               results); 0 = 4096 */
+                               results); 0 = 1024.  The pool runs instead of the trees' kernel when
+                               this is 1 .. 1023, and where the trees cannot */
     uint32_t bidir_verify;  /* bidirectional kernel with full_sa: an interval of one row whose matched
                                part is at least this many bases (and which has at least 8 bases
                                left to match) is checked against the genome's text in one step
