@@ -52,7 +52,7 @@ SEARCH_CU = os.path.join(ROOT, "paper_1402_4876_gb300", "csrc", "search.cu")
 BIDIR_CU = os.path.join(ROOT, "paper_1402_4876_gb300", "csrc", "bidir.cu")
 PROFILE_BIDIR = os.path.join(ROOT, "profiles", "k_bidir_64m_1m150.txt")
 PROFILE_BIDIR_HUMAN = os.path.join(ROOT, "profiles", "k_bidir_3g_human2m.txt")
-KERNEL_NAMES = {"bidirectional": "k_bidir", "persistent": "k_lower_bounds + k_persistent"}
+KERNEL_NAMES = {"bidirectional": "k_sweep + k_tree + k_rows", "persistent": "k_lower_bounds + k_persistent"}
 KERNEL_LABEL = {"bidirectional": "bidirectional (seed sweep, search trees, row checks)",
                 "persistent": "one-directional persistent warp-pool"}
 SEARCH_LABEL = {"bidirectional": "k + 1 pieces, one search per leftmost exact piece over the genome's and the "

@@ -1322,7 +1322,7 @@ static bool frontier_trees(const mica_index *idx)
 // and its seeds can be checked.  Without the suffix array nothing is checked:
 // it then only turns every seed into a tree's first node (a chain of one row
 // at a time for most, which a lane of tree.cu follows in registers; the warp
-// pool took 0.81 ms for 50k x 100 bp reads on a 16 Mbp genome, this 0.28).
+// pool took 0.81 ms for 50k x 100 bp reads on a 16 Mbp genome, 0.31 here).
 static bool use_sweep(const mica_index *idx, uint64_t n)
 {
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;

@@ -11,9 +11,11 @@
 // TREE_TAIL more steps are done, goes to the frontier of the next launch, which
 // spreads them over all warps again.
 //
-// What bounds it: two random reads of occurrence blocks a step (both loaded
-// whole at once; L2 hits for a genome of up to some 150 Mbp), then the integer
-// work on them.  The warp pool spent 3,000-14,000 cycles a round on its
+// What bounds it: the longest tree of a block.  Of 16.9 cycles between a warp's
+// issues 10.5 are at the barrier before the block's end, 1.4 on global loads (300k x
+// 150 bp reads, 64 Mbp genome with repeats).  A step reads two occurrence blocks
+// (both loaded whole at once; L2 for a genome of up to some 150 Mbp) and does
+// integer work on them.  The warp pool spent 3,000-14,000 cycles a round on its
 // stacks and slots, with 1-5 of 32 lanes at work on these trees.  Measured,
 // search kernels with the pool / with this: 100k reads of 100-250 bp on a 32 Mbp
 // human-like genome 2.36 / 0.39 ms, 1M mates on a 512 Mbp one 5.8 / 3.3 ms, 100k x
