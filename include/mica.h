@@ -764,6 +764,16 @@ int mica_debug_seed_interval(const mica_index *idx, const uint32_t *codes, uint3
 int mica_debug_table_interval(const mica_index *idx, uint32_t which, const uint32_t *codes, uint32_t len,
                               uint64_t n, uint32_t *lr_out);
 
+/* Lower limits of the bidirectional search's device lists and launches (0 =
+   the built-in limit; no effect on results), to make each run out on a small
+   batch: nodes a frontier buffer takes (built in: 4 per read, at least 2^20),
+   items of rows to check (16 per read, at least 2^22, of which the trees leave
+   the last 583,680 for nodes they already staged), steps a warp of the trees'
+   kernel takes once a launch's nodes are all taken (200), and launches of the
+   trees, or rounds of the warp pool, before the reads of the nodes left are
+   given up to the persistent kernel (64).  Not while a call runs on the index. */
+int mica_debug_set_search_limits(mica_index *idx, uint32_t nodes, uint32_t row_items, uint32_t steps, uint32_t rounds);
+
 /* Mismatch lower bounds of every (read, strand) task as the pruned search
    computes them (host in/out; the index must have lower_bounds).  Task
    2i + s is read i on strand s (0 = the read, 1 = its reverse complement):

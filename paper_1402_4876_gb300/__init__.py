@@ -145,6 +145,7 @@ SIGNATURES = {
     "mica_set_tuning": (_i32, [P, P]),
     "mica_get_tuning": (_i32, [P, P]),
     "mica_set_wait_limits": (_i32, [P, _u32, _u32]),
+    "mica_debug_set_search_limits": (_i32, [P, _u32, _u32, _u32, _u32]),
     "mica_autotune": (_i32, [P, P, P, P, P, _u64, _u32, _u32, P]),
     "mica_tuning_cache_store": (_i32, [ctypes.c_char_p, P, _u32, _u32, P]),
     "mica_tuning_cache_lookup": (_i32, [ctypes.c_char_p, P, _u32, _u32, P]),
@@ -392,6 +393,12 @@ class Index:
     def set_wait_limits(self, idle_rounds: int = 0, ring_spins: int = 0):
         """Bounds of the persistent kernel's device waits (0 = defaults); see mica_set_wait_limits."""
         _check(_lib.mica_set_wait_limits(self._h, idle_rounds, ring_spins), "mica_set_wait_limits")
+
+    def debug_search_limits(self, nodes: int = 0, row_items: int = 0, steps: int = 0, rounds: int = 0):
+        """Lower limits of the bidirectional search's lists and launches (0 = built in); see
+        mica_debug_set_search_limits."""
+        _check(_lib.mica_debug_set_search_limits(self._h, nodes, row_items, steps, rounds),
+               "mica_debug_set_search_limits")
 
     def tuning(self) -> dict:
         t = Tuning()

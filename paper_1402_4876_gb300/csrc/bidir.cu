@@ -1300,11 +1300,18 @@ static uint32_t frontier_cap(uint64_t n)
 {
     return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(4 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
 }
-// Items of rows to check: the sweep's (half of them), and what the trees add
-// between two checks of the list; when it is full small intervals stay nodes.
+// Items of rows to check: the sweep's, and what the trees add between two
+// checks of the list; when it is full small intervals stay nodes.  One
+// capacity for all who write or read the list: the counter runs past the end
+// when an item finds no room, and every entry before the end is then written.
 // (2M mates on a 3.1 Gbp human-like genome need some 10M in one launch.)
 static uint32_t item_cap(uint64_t n) { return (uint32_t)std::min<uint64_t>(4ull * frontier_cap(n), 1u << 28); }
+// What of both the kernels use: all, or less under a debug limit (the buffers keep their layout).
+static uint32_t limited(uint32_t cap, uint32_t limit) { return limit ? std::min(cap, limit) : cap; }
+static uint32_t node_room(const mica_index *idx, uint64_t n) { return limited(frontier_cap(n), idx->limits.nodes); }
+static uint32_t item_room(const mica_index *idx, uint64_t n) { return limited(item_cap(n), idx->limits.row_items); }
 constexpr uint32_t BD_MAX_ROUNDS = 64;
+static uint32_t max_rounds(const mica_index *idx) { return limited(BD_MAX_ROUNDS, idx->limits.rounds); }
 // The row items are checked after every launch of the trees for a batch of this
 // many reads, else at the end.
 constexpr uint64_t ROWS_EACH = 1u << 16;
@@ -1382,7 +1389,7 @@ static void bidir_args(const mica_index *idx, Workspace &w, const ReadsView &rd,
     ba.deep_s = (uint4 *)((char *)w.deep.p + (size_t)grid * sh.warps * w.bd_deep_cap * 16);
     ba.redo = (uint32_t *)w.redo.p;
     ba.budget = idx->tuning.bidir_budget ? idx->tuning.bidir_budget : BD_BUDGET;
-    ba.fr_cap = frontier_cap(rd.n);
+    ba.fr_cap = node_room(idx, rd.n);
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     ba.verify_min = (idx->view.sa_ctx && vmin < 256) ? vmin : 0u;
     ba.list = nullptr;
@@ -1433,7 +1440,7 @@ static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd
     if (tree) {
         launches++;
         return launch_tree(ba.fwd, ba.rev, w, rd, ba.fr_in, ba.fr_in_meta, ba.fr_out, ba.fr_out_meta, ba.fr_cap,
-                           row_items(w, rd.n), item_cap(rd.n), ba.redo, ba.verify_min, s);
+                           row_items(w, rd.n), item_room(idx, rd.n), ba.redo, ba.verify_min, idx->limits.steps, s);
     }
     sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
     launches++;
@@ -1475,12 +1482,12 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
             // (with the trees' kernel the sweep's nodes are round 1's tasks)
             if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, idx->tuning.bidir_budget, sweep_list(w, rd.n),
                                        tree ? ba.fr_out : nullptr, ba.fr_out_meta, ba.fr_cap, row_items(w, rd.n),
-                                       item_cap(rd.n) / 2, s, launches))
+                                       item_room(idx, rd.n), s, launches))
                 return rc;
         }
         if (!tree) {
             if (sweep)
-                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_cap(rd.n), s, launches)) return rc;
+                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
             sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
             launches++;
             MICA_CUDA_TRY(cudaGetLastError());
@@ -1488,7 +1495,7 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         for (int r = 1; r <= rounds; r++) {
             if (int rc = launch_round(idx, w, rd, grid, r, tree, s, launches)) return rc;
             if (tree && (r == rounds || rd.n >= ROWS_EACH))
-                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_cap(rd.n), s, launches)) return rc;
+                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
         }
     }
     MICA_CUDA_TRY(record_event(w.kev[1], s));
@@ -1542,11 +1549,11 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
         // four rounds per host read of the control block (a round with
         // nothing exported to it returns at once).  The first read of a search
         // with trees comes before any round.
-        while (r <= BD_MAX_ROUNDS && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error) {
-            for (int q = 0; q < 4 && r <= BD_MAX_ROUNDS; q++, r++) {
+        while (r <= max_rounds(idx) && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error) {
+            for (int q = 0; q < 4 && r <= max_rounds(idx); q++, r++) {
                 if (int rc = launch_round(idx, w, rd, grid, (int)r, tree, s, st.launches)) return rc;
                 if (tree)
-                    if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
+                    if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
             }
             MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
             MICA_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1574,14 +1581,14 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
         r = 1;
     }
     if (rows && !out.error) {
-        if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_cap(n), s, st.launches)) return rc;
+        if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
     }
     if ((out.unfinished & 1u) && !out.error) {
         // still exporting after the last round: those reads are given up
         k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
-                                                  frontier_cap(n), (uint32_t *)w.redo.p);
+                                                  node_room(idx, n), (uint32_t *)w.redo.p);
         st.launches++;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));

@@ -329,7 +329,9 @@ static int align_graph_launch(const mica_index *idx, Workspace &w, mica_stats &s
                                (uint64_t)p.report | ((uint64_t)idx->tuning.bidir_budget << 32),
                                ((uint64_t)idx->idle_limit << 32) | idx->spin_limit,
                                (uint64_t)w.frontier.p, (uint64_t)w.redo.p, (uint64_t)idx->tuning.bidir_verify,
-                               (uint64_t)w.bd_rounds | ((uint64_t)check << 32)};
+                               (uint64_t)w.bd_rounds | ((uint64_t)check << 32),
+                               (uint64_t)idx->limits.nodes | ((uint64_t)idx->limits.row_items << 32),
+                               (uint64_t)idx->limits.steps | ((uint64_t)idx->limits.rounds << 32)};
     if (!w.gexec || memcmp(key, w.gkey, sizeof(key)) != 0) {
         if (w.gexec) { cudaGraphExecDestroy(w.gexec); w.gexec = nullptr; }
         uint64_t L = 0;
@@ -840,6 +842,13 @@ int mica_set_wait_limits(mica_index *idx, uint32_t idle_rounds, uint32_t ring_sp
     if (!idx) return MICA_EINVAL;
     idx->idle_limit = idle_rounds;
     idx->spin_limit = ring_spins;
+    return 0;
+}
+
+int mica_debug_set_search_limits(mica_index *idx, uint32_t nodes, uint32_t row_items, uint32_t steps, uint32_t rounds)
+{
+    if (!idx) return MICA_EINVAL;
+    idx->limits = SearchLimits{nodes, row_items, steps, rounds};
     return 0;
 }
 

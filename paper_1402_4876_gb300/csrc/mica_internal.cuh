@@ -201,7 +201,7 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-constexpr int GRAPH_KEY = 31;   // words identifying a captured batch shape
+constexpr int GRAPH_KEY = 33;   // words identifying a captured batch shape
 
 // Per-index workspace reused across align calls.
 struct Workspace {
@@ -230,6 +230,15 @@ struct Workspace {
     uint64_t glaunches = 0;   // kernels in the captured graph
     int g_grid = 0;           // grid of the launched replay's search kernel,
     uint32_t g_rounds = 0;    //   and its frontier rounds
+};
+
+// Lower limits of the bidirectional search's device lists and launches, for
+// tests that make each run out (0: the built-in one).
+struct SearchLimits {
+    uint32_t nodes = 0;       // nodes per frontier buffer
+    uint32_t row_items = 0;   // items of rows to check
+    uint32_t steps = 0;       // steps of a warp of the trees' kernel once a launch's nodes are all taken
+    uint32_t rounds = 0;      // launches of the trees (rounds of the warp pool) before reads are given up
 };
 
 // One of an index's two slots for pipelined host batches
@@ -263,6 +272,7 @@ struct mica_index {
     mica_stats stats{};
     mica_tuning tuning{-1, 0, 0, {0, 0, 0, 0}, -1, 0, 0, -1};
     uint32_t idle_limit = 0, spin_limit = 0;   // persistent kernel wait bounds; 0 = built-in defaults
+    mica::SearchLimits limits;                 // bidirectional search (mica_debug_set_search_limits)
     mica::PipeSlot pipe[2];                    // pipelined host batches
     uint64_t next_ticket = 0;
 };

@@ -217,7 +217,9 @@ __device__ __forceinline__ void sweep_rows(const SweepArgs &a, SweepQueue &Q, ui
 }
 
 // Put the warp's larger intervals (lanes with `want`) on the item list, with
-// one counter update; false for a lane past the list's end.
+// one counter update; false for a lane past the list's end (the counter then
+// stays above it, and item_cap is what k_rows and the trees go by too, so that
+// no entry that nobody wrote is read).
 __device__ __forceinline__ bool sweep_items(const SweepArgs &a, bool want, uint32_t l, uint32_t sz, uint32_t task,
                                             const uint32_t *w, uint32_t m, uint32_t k, uint32_t j, uint32_t qe,
                                             int lane)

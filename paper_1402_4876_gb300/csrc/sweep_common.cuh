@@ -56,6 +56,6 @@ int enqueue_rows(const mica_index *idx, Workspace &w, const ReadsView &rd, uint4
                  cudaStream_t s, uint64_t &launches);
 int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, const uint4 *in,
                 const uint32_t *in_meta, uint4 *out, uint32_t *out_meta, uint32_t cap, uint4 *items, uint32_t item_cap,
-                uint32_t *redo, uint32_t verify_min, cudaStream_t s);
+                uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s);
 
 }  // namespace mica

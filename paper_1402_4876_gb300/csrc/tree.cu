@@ -58,6 +58,7 @@ struct TreeArgs {
     uint32_t item_cap;
     uint32_t *redo;
     uint32_t verify_min;
+    uint32_t tail;               // TREE_TAIL, or a debug limit
 };
 
 __device__ __forceinline__ uint32_t tree_C(const OccSide &s, uint32_t c)
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             if (!more && nn == 0) break;
             continue;
         }
-        if (!more && ++tail > TREE_TAIL) {
+        if (!more && ++tail > a.tail) {
             // the rest to the next launch
             const unsigned act = __ballot_sync(TFULL, active);
             if (active) {
@@ -310,9 +311,10 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
 }  // namespace
 
 // One launch of the trees: the nodes of `in` (their number in ctl->ntasks), their children to `out`.
+// tail: steps after the launch's nodes are all taken (0: TREE_TAIL).
 int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, const uint4 *in,
                 const uint32_t *in_meta, uint4 *out, uint32_t *out_meta, uint32_t cap, uint4 *items, uint32_t item_cap,
-                uint32_t *redo, uint32_t verify_min, cudaStream_t s)
+                uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s)
 {
     TreeArgs a;
     a.fwd = fwd;
@@ -327,9 +329,11 @@ int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const Read
     a.out_meta = out_meta;
     a.cap = cap;
     a.items = items;
-    a.item_cap = item_cap - 152u * TREE_CTAS * (TREE_THREADS / 32) * STAGE_ITEMS;
+    constexpr uint32_t LAST_FLUSHES = 152u * TREE_CTAS * (TREE_THREADS / 32) * STAGE_ITEMS;
+    a.item_cap = item_cap > LAST_FLUSHES ? item_cap - LAST_FLUSHES : 0u;
     a.redo = redo;
     a.verify_min = verify_min;
+    a.tail = tail ? tail : TREE_TAIL;
     constexpr size_t smem = sizeof(TreeStage) * (TREE_THREADS / 32);
     MICA_CUDA_TRY(cudaFuncSetAttribute(k_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_tree<<<152 * TREE_CTAS, TREE_THREADS, smem, s>>>(a);

@@ -1,0 +1,95 @@
+"""The bidirectional search's default path (seed sweep, trees from a frontier, row
+checks) with each of its lists and launch limits made to run out: results stay
+the oracle's, alone and in combination, on repeated calls."""
+import functools
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests import gpu_common as gc
+
+pytestmark = pytest.mark.gpu
+
+# Of the row items' list the trees leave this many for what they staged before it was full.
+LAST_FLUSHES = 152 * 3 * 8 * 160
+
+
+def _copies(unit, n, div, rng):
+    """n copies of a unit at divergence div, 20-60 random bases apart."""
+    parts = []
+    for _ in range(n):
+        u = unit.copy()
+        hit = rng.random(u.size) < div
+        u[hit] = (u[hit] + rng.integers(1, 4, int(hit.sum()))) & 3
+        parts += [u, rng.integers(0, 4, int(rng.integers(20, 60)))]
+    return np.concatenate(parts)
+
+
+@functools.lru_cache(maxsize=None)
+def _inputs():
+    """A genome of repeats whose seeds name a few dozen rows (row items), hundreds
+    (trees) and thousands (trees of many branches), reads of each and two batches
+    of them in different orders."""
+    rng = np.random.default_rng(31)
+    unit = lambda n: rng.integers(0, 4, n)
+    parts = [unit(30_000), _copies(unit(300), 40, 0.0, rng), _copies(unit(250), 300, 0.03, rng),
+             _copies(np.resize(unit(7), 5_000), 1, 0.03, rng), unit(5_000)]
+    g = np.concatenate(parts).astype(np.uint8)
+    at = np.cumsum([0] + [p.size for p in parts])
+    reads, ks = [], []
+
+    def some(i, count, m, k):
+        for _ in range(count):
+            a = int(rng.integers(at[i], min(at[i + 1], g.size - m)))
+            r = g[a:a + m].copy()
+            hit = rng.random(m) < 0.01
+            r[hit] = (r[hit] + rng.integers(1, 4, int(hit.sum()))) & 3
+            reads.append(r if rng.random() < 0.5 else (3 - r)[::-1].copy())
+            ks.append(k)
+
+    for k in (0, 1, 2, 3):
+        some(0, 20, 100, k)
+        some(1, 120, 101, k)
+        some(2, 100, 150, k)
+        some(3, 12, 60, k)
+    some(2, 60, 33, 3)      # pieces too short for a row check: every seed is a tree
+    some(0, 20, 3, 3)       # no pieces: one tree from the full interval
+    order = rng.permutation(len(reads))
+    a = gc.batch_from_reads([reads[i] for i in order], [ks[i] for i in order])
+    order = order[::-1]
+    b = gc.batch_from_reads([reads[i] for i in order], [ks[i] for i in order])
+    fm = oracle.FMIndex(g)
+    return g, a, b, {cap: fm.align(a, cap=cap) for cap in (0, 20)}
+
+
+def _index(full_sa=True):
+    return gc.mica().Index.build(synth.to_acgt_bytes(_inputs()[0]), kmer_q=12, sa_sample=8, full_sa=full_sa)
+
+
+def _path_is_the_trees(idx):
+    assert idx.stats()["warp_rounds"] == 0, "the warp pool took part"
+
+
+@pytest.mark.parametrize("row_items", [1, 33, 500, LAST_FLUSHES + 1, LAST_FLUSHES + 2_000])
+def test_the_row_item_list_runs_out(row_items):
+    """A list with room for fewer row items than the sweep (up to 500) or the
+    trees want, after a batch of the same reads in another order has filled
+    it: what finds no room stays with the trees, and no entry that another
+    batch left behind is looked at."""
+    g, a, b, want = _inputs()
+    idx = _index()
+    idx.align_batch(b, hit_cap=20)
+    gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], "built-in limits")
+    _path_is_the_trees(idx)
+    free = idx.stats()
+    assert free["verified"] > 0
+    idx.align_batch(b, hit_cap=20)
+    idx.debug_search_limits(row_items=row_items)
+    for call in range(2):
+        for cap in (20, 0):
+            gc.assert_same(idx.align_batch(a, hit_cap=cap), want[cap], f"items {row_items} call {call} cap {cap}")
+    _path_is_the_trees(idx)
+    assert idx.stats()["nodes"] > free["nodes"]       # what found no room was extended instead
+    idx.free()
