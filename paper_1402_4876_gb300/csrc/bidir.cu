@@ -1544,7 +1544,8 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
 {
     const uint64_t n = rd.n;
     bool tree = use_tree(idx, n);
-    bool rows = tree;   // rows to check may be left
+    const bool rows = tree;   // rows to check may be left
+    bool changed = rows;      // the control block is read once more
     for (;;) {
         // four rounds per host read of the control block (a round with
         // nothing exported to it returns at once).  The first read of a search
@@ -1558,8 +1559,18 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
             MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
             MICA_CUDA_TRY(cudaStreamSynchronize(s));
         }
-        if (!tree || !out.pool_tasks || (out.unfinished & 1u) || out.error) break;
-        // schemes the sweep found no room for among the nodes: this kernel's
+        if (out.error) break;
+        if (out.unfinished & 1u) {
+            // still exporting after the last round: those reads are given up
+            k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
+                                                      node_room(idx, n), (uint32_t *)w.redo.p);
+            MICA_CUDA_TRY(cudaGetLastError());
+            st.launches++;
+            changed = true;
+        }
+        if (!tree || !out.pool_tasks) break;
+        // schemes the sweep found no room for among the nodes: this kernel's, whether or not
+        // the trees came to their end
         SearchCtl *d_ctl = (SearchCtl *)w.ctl.p;
         MICA_CUDA_TRY(cudaMemcpyAsync(&d_ctl->ntasks, &d_ctl->pool_tasks, 8, cudaMemcpyDeviceToDevice, s));
         MICA_CUDA_TRY(cudaMemsetAsync(&d_ctl->pool_tasks, 0, 8, s));
@@ -1580,16 +1591,9 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
         tree = false;
         r = 1;
     }
-    if (rows && !out.error) {
-        if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
-        MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
-        MICA_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-    if ((out.unfinished & 1u) && !out.error) {
-        // still exporting after the last round: those reads are given up
-        k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
-                                                  node_room(idx, n), (uint32_t *)w.redo.p);
-        st.launches++;
+    if (changed && !out.error) {
+        if (rows)
+            if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
     }

@@ -93,3 +93,29 @@ def test_the_row_item_list_runs_out(row_items):
     _path_is_the_trees(idx)
     assert idx.stats()["nodes"] > free["nodes"]       # what found no room was extended instead
     idx.free()
+
+
+@pytest.mark.parametrize("full_sa", [True, False])
+@pytest.mark.parametrize("limits", [
+    dict(nodes=64), dict(steps=1), dict(rounds=1, steps=1), dict(rounds=2, steps=2), dict(nodes=4096, steps=3),
+    dict(nodes=400, rounds=1, steps=1),      # tasks left to the warp pool, and trees that outlast their rounds
+    dict(nodes=64, rounds=1, steps=1), dict(nodes=400, rounds=3, steps=2, row_items=40),
+    dict(nodes=4, rounds=64, steps=1, row_items=1)], ids=str)
+def test_limits_of_the_trees(limits, full_sa):
+    """The frontier's nodes (first nodes past its end are the warp pool's tasks,
+    later ones give their reads up), a launch's steps, the launches, and these
+    together: every read's hits are the oracle's, through a call that captures,
+    one that replays, and the pipelined calls."""
+    _, a, b, want = _inputs()
+    idx = _index(full_sa)
+    idx.align_batch(b, hit_cap=20)
+    idx.debug_search_limits(**limits)
+    for cap in (20, 0):
+        for call in range(2):
+            gc.assert_same(idx.align_batch(a, hit_cap=cap), want[cap], f"{limits} cap {cap} call {call}")
+    gc.assert_same(idx.collect(idx.submit_batch(a, hit_cap=20)), want[20], f"{limits} pipelined")
+    if "rounds" in limits and limits["rounds"] < 64:
+        assert idx.stats()["fallback_reads"] > 0
+    idx.debug_search_limits()
+    gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], "built-in limits again")
+    idx.free()
