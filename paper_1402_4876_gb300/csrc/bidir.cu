@@ -1025,7 +1025,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                 }
                 const unsigned backs = __ballot_sync(BFULL, back);
                 if (backs) {
-                    // (they came from the stack: there is room)
+                    // (after a first step the others' children may have filled the stack)
+                    bd_make_room<SCAP, NS, false>(W, a, deep_m, dmt, mbot, mtop, (uint32_t)__popc(backs), lane, c_deep);
                     if (back) {
                         const uint32_t q = (mtop + __popc(backs & lt)) & (SCAP - 1);
                         W.ml[q] = l; W.mlr[q] = lr; W.msz[q] = sz; W.mm[q] = meta;

@@ -119,3 +119,25 @@ def test_limits_of_the_trees(limits, full_sa):
     idx.debug_search_limits()
     gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], "built-in limits again")
     idx.free()
+
+
+@pytest.mark.parametrize("budget", [8, 200, 512, 1023])
+def test_runs_return_to_a_full_stack(budget):
+    """The warp pool: short reads with a large budget fill a warp's stack with
+    children of several rows while other lanes' runs (nodes whose rows all
+    continue alike) end early and go back to it.  Which lanes meet depends on
+    the launch, so two batches are searched 80 times each; the result is the
+    persistent kernel's each time."""
+    g = synth.genome_64m(1 << 24)
+    rng = np.random.default_rng(78)
+    batches = [synth.sample_reads(g, rng.integers(36, 61, 50_000), np.full(50_000, 3), rng, subs="rate", sub_rate=0.01,
+                                  repeat_frac=0.3) for _ in range(2)]
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), kmer_q=12, sa_sample=16)
+    for b in batches:
+        idx.set_tuning()
+        want = idx.align_batch(b, hit_cap=10, kernel="persistent")
+        idx.set_tuning(bidir_budget=budget)
+        for call in range(80):
+            gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"budget {budget} call {call}")
+            assert idx.stats()["warp_rounds"] > 0
+    idx.free()
