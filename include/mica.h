@@ -295,7 +295,7 @@ typedef struct {
     uint32_t bidir_budget;  /* bidirectional warp pool: node expansions a task may take before it hands
                                its pending nodes to the next launch round, where they are tasks of
                                their own on every warp (bounds each round's tail; no effect on
-                               results); 0 = 1024.  The pool runs instead of the trees' kernel when
+                               results); 0 = 4096.  The pool runs instead of the trees' kernel when
                                this is 1 .. 1023, and where the trees cannot */
     uint32_t bidir_verify;  /* bidirectional kernel with full_sa: an interval of one row whose matched
                                part is at least this many bases (and which has at least 8 bases
@@ -766,9 +766,10 @@ int mica_debug_table_interval(const mica_index *idx, uint32_t which, const uint3
 
 /* Lower limits of the bidirectional search's device lists and launches (0 =
    the built-in limit; no effect on results), to make each run out on a small
-   batch: nodes a frontier buffer takes (built in: 4 per read, at least 2^20),
-   items of rows to check (16 per read, at least 2^22, of which the trees leave
-   the last 583,680 for nodes they already staged), steps a warp of the trees'
+   batch: first nodes the sweep makes and nodes a launch of the trees stops at
+   (built in: 4 and 6 per read, at least 2^20 and 1.5 * 2^20; without the suffix
+   array 6 and 8), items of rows to check (16 per read, at least 2^22; a launch
+   of the trees stops at 583,680 fewer), steps a warp of the trees'
    kernel takes once a launch's nodes are all taken (200), and launches of the
    trees, or rounds of the warp pool, before the reads of the nodes left are
    given up to the persistent kernel (64).  Not while a call runs on the index. */

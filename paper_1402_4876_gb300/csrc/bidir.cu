@@ -61,7 +61,7 @@ namespace {
 
 constexpr unsigned BFULL = 0xffffffffu;
 constexpr uint32_t BD_DEEP_MIN = 8192;      // entries of each per-warp overflow stack, at least
-constexpr uint32_t BD_BUDGET = 1u << 10;    // node expansions a task may take before it exports its nodes
+constexpr uint32_t BD_BUDGET = 1u << 12;    // node expansions a task may take before it exports its nodes
 constexpr int VCAP = 64;                    // intervals waiting for that check ...
 constexpr int TCAP = 64;                    // ... and windows of their rows that pass the first look
 constexpr uint32_t BD_SPLIT_LEFT = 32;      // an interval of at most this many rows is checked row by row: while
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
     // dependent steps: spread thinly over every warp the search kernels take 6.4 ms for a
     // million reads of a 512 Mbp human-like genome, at eight times as many to a warp 8.7 ms
     const uint32_t share = (uint32_t)max(1ull, min((unsigned long long)NS, ntasks / ((unsigned long long)gridDim.x * WARPS)));
-    // once the launch's task counter is spent, a task keeps a 32nd of its
+    // once the launch's task counter is spent, a task keeps an eighth of its
     // budget: a warp left holding heavy trees hands them to the next round,
     // where every warp takes part, instead of working through them alone
     uint32_t budget = a.budget;
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
         if ((iter & 63) == 63 && budget == a.budget) {
             int spent = 0;
             if (lane == 0) spent = *(volatile unsigned long long *)&ctl->task_head >= ntasks;
-            if (__shfl_sync(BFULL, spent, 0)) budget = max(a.budget >> 5, min(a.budget, 32u));
+            if (__shfl_sync(BFULL, spent, 0)) budget = max(a.budget >> 3, min(a.budget, 32u));
         }
         // ---- slots over their node budget hand their nodes to the next
         // round (one pass over both stacks), and their schemes not yet seeded
@@ -1210,6 +1210,25 @@ __global__ void k_bd_init(const SearchCtl tmpl, SearchCtl *__restrict__ ctl, uin
     }
 }
 
+// Of a launch of the trees that stopped early, the nodes `in` that no warp took,
+// behind the `base` ones it left: `out` then holds the next round's tasks.
+__global__ void k_bd_carry(SearchCtl *ctl, const uint4 *__restrict__ in, const uint32_t *__restrict__ in_meta, uint32_t n,
+                           uint4 *__restrict__ out, uint32_t *__restrict__ out_meta, uint32_t base, uint32_t cap,
+                           uint32_t *__restrict__ redo)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->ntasks = min((unsigned long long)base + n, (unsigned long long)cap);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t q = base + i;
+        if (q < cap) {
+            out[q] = in[i];
+            out_meta[q] = in_meta[i];
+        } else {   // (a launch that stops in time leaves no more than `out` holds)
+            const uint32_t rid = in[i].x >> 1, bit = 1u << (rid & 31);
+            if (!(atomicOr(&redo[rid >> 5], bit) & bit)) atomicAdd(&ctl->redo_reads, 1u);
+        }
+    }
+}
+
 // After the last round: the reads of nodes still in the frontier are given up.
 __global__ void k_bd_give_up_frontier(SearchCtl *ctl, const uint4 *__restrict__ fr, uint32_t fr_cap,
                                       uint32_t *__restrict__ redo)
@@ -1292,25 +1311,43 @@ static uint32_t bidir_deep_cap(Workspace &w, uint64_t warps)
 }
 
 static uint64_t redo_bits_bytes(uint64_t n) { return ((n + 31) / 32 * 4 + 15) & ~15ull; }
-// Nodes per frontier buffer: 4n, at least 2^20, at most 2^28, and a multiple
-// of 4 so that the second buffer and both meta arrays (20 B per item in all)
-// start on a 16-byte boundary, as the kernel's 16-byte item loads and stores
-// require (an odd batch above 2^18 reads would otherwise put the second
-// buffer 8 bytes off).
-static uint32_t frontier_cap(uint64_t n)
+// First nodes of the trees the sweep may make: 4n, at least 2^20 and at most
+// 2^28; without the suffix array, where every seed is one, 6n.
+static uint64_t first_nodes(const mica_index *idx, uint64_t n)
 {
-    return (uint32_t)((std::min<uint64_t>(std::max<uint64_t>(4 * n, 1u << 20), 1u << 28) + 3) & ~3ull);
+    const uint64_t per = idx->view.sa_ctx ? 4 : 6;
+    return std::min<uint64_t>(std::max<uint64_t>(per * n, per << 18), 1ull << 28);
+}
+// Nodes a launch of the trees stops at (its children and the nodes it has not
+// taken): the first nodes and as many as half (a third) of them more, since a
+// launch's children outnumber the nodes it has finished.
+static uint64_t stop_nodes(const mica_index *idx, uint64_t n)
+{
+    return first_nodes(idx, n) + first_nodes(idx, n) / (idx->view.sa_ctx ? 2 : 3);
+}
+// Nodes per frontier buffer: a multiple of 4 so that the second buffer and
+// both meta arrays (20 B per node in all) start on a 16-byte boundary, as the
+// kernels' 16-byte loads and stores require.
+static uint32_t frontier_cap(const mica_index *idx, uint64_t n)
+{
+    return (uint32_t)((stop_nodes(idx, n) + TREE_LAST + 3) & ~3ull);
 }
 // Items of rows to check: the sweep's, and what the trees add between two
-// checks of the list; when it is full small intervals stay nodes.  One
+// checks of the list; a launch of the trees stops when it is nearly full.  One
 // capacity for all who write or read the list: the counter runs past the end
-// when an item finds no room, and every entry before the end is then written.
-// (2M mates on a 3.1 Gbp human-like genome need some 10M in one launch.)
-static uint32_t item_cap(uint64_t n) { return (uint32_t)std::min<uint64_t>(4ull * frontier_cap(n), 1u << 28); }
-// What of both the kernels use: all, or less under a debug limit (the buffers keep their layout).
-static uint32_t limited(uint32_t cap, uint32_t limit) { return limit ? std::min(cap, limit) : cap; }
-static uint32_t node_room(const mica_index *idx, uint64_t n) { return limited(frontier_cap(n), idx->limits.nodes); }
-static uint32_t item_room(const mica_index *idx, uint64_t n) { return limited(item_cap(n), idx->limits.row_items); }
+// when an item of the sweep finds no room, and every entry before the end is
+// then written.  (2M mates on a 3.1 Gbp human-like genome need some 10M in one
+// launch.)  Without the suffix array there are none.
+static uint32_t item_cap(const mica_index *idx, uint64_t n)
+{
+    return idx->view.sa_ctx ? (uint32_t)std::min<uint64_t>(4 * first_nodes(idx, n), 1ull << 28) : 0u;
+}
+// What of these the kernels use: all, or less under a debug limit (the buffers keep their layout).
+static uint32_t limited(uint64_t cap, uint32_t limit) { return (uint32_t)(limit ? std::min<uint64_t>(cap, limit) : cap); }
+static uint32_t first_room(const mica_index *idx, uint64_t n) { return limited(first_nodes(idx, n), idx->limits.nodes); }
+static uint32_t stop_room(const mica_index *idx, uint64_t n) { return limited(stop_nodes(idx, n), idx->limits.nodes); }
+static uint32_t pool_room(const mica_index *idx, uint64_t n) { return limited(frontier_cap(idx, n), idx->limits.nodes); }
+static uint32_t item_room(const mica_index *idx, uint64_t n) { return limited(item_cap(idx, n), idx->limits.row_items); }
 constexpr uint32_t BD_MAX_ROUNDS = 64;
 static uint32_t max_rounds(const mica_index *idx) { return limited(BD_MAX_ROUNDS, idx->limits.rounds); }
 // The row items are checked after every launch of the trees for a batch of this
@@ -1334,7 +1371,7 @@ static bool frontier_trees(const mica_index *idx)
 static bool use_sweep(const mica_index *idx, uint64_t n)
 {
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
-    if (2 * n > frontier_cap(n)) return false;
+    if (n > 1ull << 27) return false;
     if (!idx->view.sa_ctx) return frontier_trees(idx);
     return vmin < 256 && sweep_checks(idx, vmin);
 }
@@ -1358,7 +1395,7 @@ int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tm
     // given-up reads: a bit per read, then a list of them and its length
     if ((rc = dev_reserve(w.redo, redo_bytes(n)))) return rc;
     // nodes: two rounds' buffers of (task, l, lr, sz) and meta; the sweep's row items and task list
-    if ((rc = dev_reserve(w.frontier, (uint64_t)frontier_cap(n) * (2 * 20) + (uint64_t)item_cap(n) * 16 +
+    if ((rc = dev_reserve(w.frontier, (uint64_t)frontier_cap(idx, n) * (2 * 20) + (uint64_t)item_cap(idx, n) * 16 +
                                       std::max<uint64_t>(n, 1) * 16)))
         return rc;
     tmpl = SearchCtl{};
@@ -1390,7 +1427,7 @@ static void bidir_args(const mica_index *idx, Workspace &w, const ReadsView &rd,
     ba.deep_s = (uint4 *)((char *)w.deep.p + (size_t)grid * sh.warps * w.bd_deep_cap * 16);
     ba.redo = (uint32_t *)w.redo.p;
     ba.budget = idx->tuning.bidir_budget ? idx->tuning.bidir_budget : BD_BUDGET;
-    ba.fr_cap = node_room(idx, rd.n);
+    ba.fr_cap = pool_room(idx, rd.n);
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     ba.verify_min = (idx->view.sa_ctx && vmin < 256) ? vmin : 0u;
     ba.list = nullptr;
@@ -1398,17 +1435,20 @@ static void bidir_args(const mica_index *idx, Workspace &w, const ReadsView &rd,
 
 
 // Frontier buffer b (0 or 1): items, then meta words.
-static uint4 *frontier_items(Workspace &w, uint64_t n, int b)
+static uint4 *frontier_items(const mica_index *idx, Workspace &w, uint64_t n, int b)
 {
-    return (uint4 *)((char *)w.frontier.p + (size_t)b * frontier_cap(n) * 20);
+    return (uint4 *)((char *)w.frontier.p + (size_t)b * frontier_cap(idx, n) * 20);
 }
-static uint32_t *frontier_meta(Workspace &w, uint64_t n, int b)
+static uint32_t *frontier_meta(const mica_index *idx, Workspace &w, uint64_t n, int b)
 {
-    return (uint32_t *)(frontier_items(w, n, b) + frontier_cap(n));
+    return (uint32_t *)(frontier_items(idx, w, n, b) + frontier_cap(idx, n));
 }
 
-static uint4 *row_items(Workspace &w, uint64_t n) { return frontier_items(w, n, 2); }
-static uint2 *sweep_list(Workspace &w, uint64_t n) { return (uint2 *)(row_items(w, n) + item_cap(n)); }
+static uint4 *row_items(const mica_index *idx, Workspace &w, uint64_t n) { return frontier_items(idx, w, n, 2); }
+static uint2 *sweep_list(const mica_index *idx, Workspace &w, uint64_t n)
+{
+    return (uint2 *)(row_items(idx, w, n) + item_cap(idx, n));
+}
 
 // The kernel moves frontier items and overflow-stack entries as 16-byte
 // vectors: refuse a launch whose buffers are not on 16-byte boundaries.
@@ -1433,15 +1473,18 @@ static int launch_round(const mica_index *idx, Workspace &w, const ReadsView &rd
     BidirArgs ba;
     bidir_args(idx, w, rd, grid, ba);
     ba.mode = 1;
-    ba.fr_in = frontier_items(w, rd.n, (r + 1) & 1);
-    ba.fr_in_meta = frontier_meta(w, rd.n, (r + 1) & 1);
-    ba.fr_out = frontier_items(w, rd.n, r & 1);
-    ba.fr_out_meta = frontier_meta(w, rd.n, r & 1);
+    ba.fr_in = frontier_items(idx, w, rd.n, (r + 1) & 1);
+    ba.fr_in_meta = frontier_meta(idx, w, rd.n, (r + 1) & 1);
+    ba.fr_out = frontier_items(idx, w, rd.n, r & 1);
+    ba.fr_out_meta = frontier_meta(idx, w, rd.n, r & 1);
     if (int rc = check_vector_alignment(ba)) return rc;
     if (tree) {
         launches++;
-        return launch_tree(ba.fwd, ba.rev, w, rd, ba.fr_in, ba.fr_in_meta, ba.fr_out, ba.fr_out_meta, ba.fr_cap,
-                           row_items(w, rd.n), item_room(idx, rd.n), ba.redo, ba.verify_min, idx->limits.steps, s);
+        // (round 1's nodes are the sweep's)
+        const uint32_t stop = stop_room(idx, rd.n), in_cap = r == 1 ? first_room(idx, rd.n) : stop + TREE_LAST;
+        return launch_tree(ba.fwd, ba.rev, w, rd, (uint32_t)r, ba.fr_in, ba.fr_in_meta, in_cap, ba.fr_out,
+                           ba.fr_out_meta, stop, row_items(idx, w, rd.n), item_room(idx, rd.n), ba.redo, ba.verify_min,
+                           idx->limits.steps, s);
     }
     sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
     launches++;
@@ -1474,21 +1517,21 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         ba.mode = 0;
         ba.fr_in = nullptr;
         ba.fr_in_meta = nullptr;
-        ba.fr_out = frontier_items(w, rd.n, 0);
-        ba.fr_out_meta = frontier_meta(w, rd.n, 0);
+        ba.fr_out = frontier_items(idx, w, rd.n, 0);
+        ba.fr_out_meta = frontier_meta(idx, w, rd.n, 0);
         const bool sweep = use_sweep(idx, rd.n), tree = use_tree(idx, rd.n);
         if (int rc = check_vector_alignment(ba)) return rc;
         if (sweep) {
-            ba.list = sweep_list(w, rd.n);
+            ba.list = sweep_list(idx, w, rd.n);
             // (with the trees' kernel the sweep's nodes are round 1's tasks)
-            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, idx->tuning.bidir_budget, sweep_list(w, rd.n),
-                                       tree ? ba.fr_out : nullptr, ba.fr_out_meta, ba.fr_cap, row_items(w, rd.n),
+            if (int rc = enqueue_sweep(idx, w, rd, ba.verify_min, idx->tuning.bidir_budget, sweep_list(idx, w, rd.n),
+                                       tree ? ba.fr_out : nullptr, ba.fr_out_meta, first_room(idx, rd.n), row_items(idx, w, rd.n),
                                        item_room(idx, rd.n), s, launches))
                 return rc;
         }
         if (!tree) {
             if (sweep)
-                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
+                if (int rc = enqueue_rows(idx, w, rd, row_items(idx, w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
             sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
             launches++;
             MICA_CUDA_TRY(cudaGetLastError());
@@ -1496,7 +1539,7 @@ int enqueue_bidir(const mica_index *idx, Workspace &w, const ReadsView &rd, int 
         for (int r = 1; r <= rounds; r++) {
             if (int rc = launch_round(idx, w, rd, grid, r, tree, s, launches)) return rc;
             if (tree && (r == rounds || rd.n >= ROWS_EACH))
-                if (int rc = enqueue_rows(idx, w, rd, row_items(w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
+                if (int rc = enqueue_rows(idx, w, rd, row_items(idx, w, rd.n), item_room(idx, rd.n), s, launches)) return rc;
         }
     }
     MICA_CUDA_TRY(record_event(w.kev[1], s));
@@ -1547,29 +1590,50 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     bool tree = use_tree(idx, n);
     const bool rows = tree;   // rows to check may be left
     bool changed = rows;      // the control block is read once more
+    uint32_t rounds_run = 0;  // of the trees
     for (;;) {
         // four rounds per host read of the control block (a round with
         // nothing exported to it returns at once).  The first read of a search
         // with trees comes before any round.
-        while (r <= max_rounds(idx) && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error) {
+        while (r <= max_rounds(idx) && ((out.unfinished & 1u) || (tree && out.ntasks)) && !out.error &&
+               !(tree && out.stop)) {
             for (int q = 0; q < 4 && r <= max_rounds(idx); q++, r++) {
                 if (int rc = launch_round(idx, w, rd, grid, (int)r, tree, s, st.launches)) return rc;
                 if (tree)
-                    if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
+                    if (int rc = enqueue_rows(idx, w, rd, row_items(idx, w, n), item_room(idx, n), s, st.launches)) return rc;
             }
             MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
             MICA_CUDA_TRY(cudaStreamSynchronize(s));
         }
+        if (tree) rounds_run = out.rounds_run;
         if (out.error) break;
+        if (tree && out.stop) {
+            // the trees stopped early: their nodes, and the launch's that no warp took, are this kernel's
+            const int from = (int)((out.stop + 1) & 1u), to = (int)(out.stop & 1u);
+            const uint32_t left = out.left_to - out.left_from, base = (uint32_t)out.ntasks;
+            k_bd_carry<<<(unsigned)std::min<uint64_t>(left / 256 + 1, 152ull * 8), 256, 0, s>>>(
+                (SearchCtl *)w.ctl.p, frontier_items(idx, w, n, from) + out.left_from,
+                frontier_meta(idx, w, n, from) + out.left_from, left, frontier_items(idx, w, n, to),
+                frontier_meta(idx, w, n, to), base, frontier_cap(idx, n), (uint32_t *)w.redo.p);
+            MICA_CUDA_TRY(cudaGetLastError());
+            st.launches++;
+            tree = false;
+            r = 1 + (out.stop & 1u);   // (a round whose input is that buffer)
+            if (base + left) {
+                out.unfinished |= 1u;
+                continue;
+            }
+            out.unfinished &= ~1u;
+        }
         if (out.unfinished & 1u) {
             // still exporting after the last round: those reads are given up
-            k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(w, n, (r - 1) & 1),
-                                                      node_room(idx, n), (uint32_t *)w.redo.p);
+            k_bd_give_up_frontier<<<152, 256, 0, s>>>((SearchCtl *)w.ctl.p, frontier_items(idx, w, n, (r - 1) & 1),
+                                                      frontier_cap(idx, n), (uint32_t *)w.redo.p);
             MICA_CUDA_TRY(cudaGetLastError());
             st.launches++;
             changed = true;
         }
-        if (!tree || !out.pool_tasks) break;
+        if (!out.pool_tasks) break;
         // schemes the sweep found no room for among the nodes: this kernel's, whether or not
         // the trees came to their end
         SearchCtl *d_ctl = (SearchCtl *)w.ctl.p;
@@ -1578,11 +1642,11 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
         BidirArgs ba;
         bidir_args(idx, w, rd, grid, ba);
         ba.mode = 0;
-        ba.list = sweep_list(w, n);
+        ba.list = sweep_list(idx, w, n);
         ba.fr_in = nullptr;
         ba.fr_in_meta = nullptr;
-        ba.fr_out = frontier_items(w, n, 0);
-        ba.fr_out_meta = frontier_meta(w, n, 0);
+        ba.fr_out = frontier_items(idx, w, n, 0);
+        ba.fr_out_meta = frontier_meta(idx, w, n, 0);
         const BidirShape &sh = g_bd_shapes[bidir_shape_index(idx)];
         sh.fn<<<grid, sh.warps * 32, sh.smem, s>>>(ba);
         st.launches++;
@@ -1594,7 +1658,7 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     }
     if (changed && !out.error) {
         if (rows)
-            if (int rc = enqueue_rows(idx, w, rd, row_items(w, n), item_room(idx, n), s, st.launches)) return rc;
+            if (int rc = enqueue_rows(idx, w, rd, row_items(idx, w, n), item_room(idx, n), s, st.launches)) return rc;
         MICA_CUDA_TRY(cudaMemcpyAsync(&out, w.ctl.p, sizeof(out), cudaMemcpyDeviceToHost, s));
         MICA_CUDA_TRY(cudaStreamSynchronize(s));
     }
@@ -1621,7 +1685,7 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     st.grid_ctas = (uint64_t)grid;
     w.bd_redo_seen = out.redo_reads > 0;
     // rounds a captured batch of this workspace runs: what its batches needed so far, to a power of two
-    while (w.bd_rounds < out.rounds_run + 1 && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
+    while (w.bd_rounds < (rows ? rounds_run : out.rounds_run) + 1 && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
     if (out.redo_reads) {
         int rc = redo_given_up(idx, w, st, rd, out, s);
         if (rc) return rc;

@@ -160,10 +160,13 @@ struct SearchCtl {
     unsigned int redo_reads;                          // bidirectional search: reads given up, to be re-searched
     unsigned int fr_count;                            // bidirectional search: nodes exported this round
     unsigned int unfinished;                          // ... bit 0 nodes wait for a further round, bit 1 reads
-                                                      //   were given up
+                                                      //   were given up, bit 2 tasks wait for the warp pool,
+                                                      //   bit 3 the trees stopped early
     unsigned int rounds_run, done_ctas;               // ... rounds with tasks; CTAs of this launch that are done
     unsigned int done_rows;                           // row check: CTAs of this launch that are done
     unsigned long long pool_tasks;                    // seed sweep: tasks left past the nodes' room
+    unsigned int stop;                                // trees: the round that stopped with its lists nearly full ...
+    unsigned int left_from, left_to;                  //   ... and its nodes that no warp took
     unsigned long long verified, verify_bytes;        // bidirectional search: one-row intervals checked
                                                       //   against the text, and the bytes that read
     unsigned long long verify_sectors;                // ... and the 32-byte sectors those reads touch

@@ -54,8 +54,12 @@ int enqueue_sweep(const mica_index *idx, Workspace &w, const ReadsView &rd, uint
                   cudaStream_t s, uint64_t &launches);
 int enqueue_rows(const mica_index *idx, Workspace &w, const ReadsView &rd, uint4 *items, uint32_t item_cap,
                  cudaStream_t s, uint64_t &launches);
-int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, const uint4 *in,
-                const uint32_t *in_meta, uint4 *out, uint32_t *out_meta, uint32_t cap, uint4 *items, uint32_t item_cap,
-                uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s);
+int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, uint32_t round,
+                const uint4 *in, const uint32_t *in_meta, uint32_t in_cap, uint4 *out, uint32_t *out_meta, uint32_t cap,
+                uint4 *items, uint32_t item_cap, uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s);
+// What the trees' warps may still add to a list once it is found full: the
+// nodes (items) each has staged, and those its lanes are at.
+constexpr uint32_t TREE_WARPS = 152u * 3u * 8u;
+constexpr uint32_t TREE_LAST = TREE_WARPS * 160u;
 
 }  // namespace mica

@@ -11,6 +11,17 @@
 // TREE_TAIL more steps are done, goes to the frontier of the next launch, which
 // spreads them over all warps again.
 //
+// A launch stops early when the list of rows to check is nearly full, or the
+// next frontier with the nodes not yet taken: the warp that finds it so says
+// so, every warp puts its nodes in the frontier, and the warp pool, which checks
+// rows itself and has overflow stacks, goes on from all that is left.  Such
+// batches have tens of millions of row items (short reads with a large budget,
+// reads of a family of a thousand copies).  Going on here instead, with small
+// intervals as nodes and the reads of nodes without room given up to the
+// one-directional search, took 25.8 ms for 200k reads of 36-60 bp, k = 3, on a
+// 64 Mbp genome (now 4.8; the pool alone 3.9) and 21.2 ms for 100k reads of 100
+// bp in a family of 1,000 copies at 0.5% (now 9.7).
+//
 // What bounds it: the longest tree of a block.  Of 16.9 cycles between a warp's
 // issues 10.5 are at the barrier before the block's end, 1.4 on global loads (300k x
 // 150 bp reads, 64 Mbp genome with repeats).  A step reads two occurrence blocks
@@ -31,11 +42,14 @@ namespace {
 constexpr unsigned TFULL = 0xffffffffu;
 constexpr int TREE_THREADS = 256;
 constexpr int TREE_CTAS = 3;            // per SM
+static_assert(TREE_WARPS == 152u * TREE_CTAS * (TREE_THREADS / 32), "warps of a launch");
 constexpr uint32_t TREE_TAIL = 200;      // steps of a warp after the launch's nodes are all taken
 constexpr uint32_t TREE_REFILL = 8;     // idle lanes of a warp before it takes new nodes
 constexpr uint32_t STAGE_LOW = 32;      // staged nodes (items) kept; a step adds at most 96 (128)
 constexpr uint32_t STAGE_NODES = 128;
 constexpr uint32_t STAGE_ITEMS = 160;
+
+static_assert(STAGE_ITEMS <= 160 && STAGE_NODES + 32 <= 160, "TREE_LAST");
 
 struct TreeStage {
     uint4 node[STAGE_NODES];
@@ -49,13 +63,15 @@ struct TreeArgs {
     SearchCtl *ctl;
     Interval *iv;
     uint32_t *iv_cnt;
+    uint32_t in_cap;             // nodes `in` may hold (the sweep's counter runs past its own)
     const uint4 *in;             // (task, l, lr, rows)
     const uint32_t *in_meta;
     uint4 *out;
     uint32_t *out_meta;
-    uint32_t cap;
+    uint32_t cap;                // nodes the launch stops at; `out` has room for TREE_LAST more
     uint4 *items;                // rows to check (sweep_common.cuh)
-    uint32_t item_cap;
+    uint32_t item_cap;           // items the launch stops at
+    uint32_t round;
     uint32_t *redo;
     uint32_t verify_min;
     uint32_t tail;               // TREE_TAIL, or a debug limit
@@ -66,12 +82,12 @@ __device__ __forceinline__ uint32_t tree_C(const OccSide &s, uint32_t c)
     return c == 0 ? s.C[0] : c == 1 ? s.C[1] : c == 2 ? s.C[2] : s.C[3];
 }
 
-// A node for the next launch (past the end: its read is given up, to be
-// searched again by the persistent kernel).
+// A node for the next launch.  (One past the end, which a launch that stops in
+// time has none of, gives its read up to the persistent kernel.)
 __device__ __forceinline__ void push_node(const TreeArgs &a, uint32_t q, uint32_t task, uint32_t l, uint32_t lr,
                                           uint32_t sz, uint32_t meta)
 {
-    if (q < a.cap) {
+    if (q < a.cap + TREE_LAST) {
         a.out[q] = make_uint4(task, l, lr, sz);
         a.out_meta[q] = meta;
     } else {
@@ -80,9 +96,7 @@ __device__ __forceinline__ void push_node(const TreeArgs &a, uint32_t q, uint32_
     }
 }
 
-// The staged items to their list; false when it has room for only one more
-// such flush by every warp (TreeArgs::item_cap is less than its size by that):
-// from then on this launch's small intervals stay nodes.
+// The staged items to their list; false when it is nearly full.
 __device__ __forceinline__ bool flush_items(const TreeArgs &a, const TreeStage &S, uint32_t n, int lane)
 {
     uint32_t at = 0;
@@ -93,32 +107,41 @@ __device__ __forceinline__ bool flush_items(const TreeArgs &a, const TreeStage &
     return at + n < a.item_cap;
 }
 
-// The staged nodes [from, n) to the frontier.
-__device__ __forceinline__ void flush_nodes(const TreeArgs &a, const TreeStage &S, uint32_t from, uint32_t n, int lane)
+// The staged nodes [from, n) to the frontier; false when it is nearly full with
+// the launch's nodes that are not yet taken.
+__device__ __forceinline__ bool flush_nodes(const TreeArgs &a, const TreeStage &S, uint32_t from, uint32_t n,
+                                            uint32_t ntasks, int lane)
 {
-    uint32_t at = 0;
-    if (lane == 0) at = atomicAdd(&a.ctl->fr_count, n - from);
+    uint32_t at = 0, left = 0;
+    if (lane == 0) {
+        const unsigned long long head = *(volatile unsigned long long *)&a.ctl->task_head;
+        at = atomicAdd(&a.ctl->fr_count, n - from);
+        left = head < ntasks ? ntasks - (uint32_t)head : 0u;
+    }
     at = __shfl_sync(TFULL, at, 0);
+    left = __shfl_sync(TFULL, left, 0);
     for (uint32_t i = from + lane; i < n; i += 32) {
         const uint4 x = S.node[i];
         push_node(a, at + i - from, x.x, x.y, x.z, x.w, S.meta[i]);
     }
     __syncwarp();
+    return at + (n - from) + left < a.cap;
 }
 
 __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs a)
 {
     extern __shared__ uint4 tree_smem[];
     SearchCtl *ctl = a.ctl;
-    const uint32_t ntasks = (uint32_t)min(*(volatile unsigned long long *)&ctl->ntasks, (unsigned long long)a.cap);
-    if (ntasks == 0 || *(volatile unsigned *)&ctl->error) return;
+    const uint32_t ntasks = (uint32_t)min(*(volatile unsigned long long *)&ctl->ntasks, (unsigned long long)a.in_cap);
+    const unsigned stopped = *(volatile unsigned *)&ctl->stop;
+    if (ntasks == 0 || *(volatile unsigned *)&ctl->error || (stopped && stopped != a.round)) return;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     TreeStage &S = reinterpret_cast<TreeStage *>(tree_smem)[threadIdx.x >> 5];
     // nodes a warp takes at a time: no more than its part of the launch's
     const uint32_t share = max(1u, min(32u, ntasks / (gridDim.x * (TREE_THREADS / 32))));
     bool active = false, more = true;
-    bool item_room = *(volatile unsigned *)&ctl->row_items < a.item_cap;
+    bool halt = __shfl_sync(TFULL, lane == 0 ? *(volatile unsigned *)&ctl->row_items : 0u, 0) >= a.item_cap;   // the launch stops
     uint32_t task = 0, l = 0, lr = 0, sz = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
     unsigned long long bounds = 0;
     const uint32_t *w = nullptr;
@@ -140,11 +163,16 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             idle = __ballot_sync(TFULL, !active && !fresh);
             __syncwarp();
         }
-        if (more && (idle == TFULL || __popc(idle) >= TREE_REFILL)) {
+        if (more && !halt && (idle == TFULL || __popc(idle) >= TREE_REFILL)) {
             const uint32_t n = min((uint32_t)__popc(idle), share);
             unsigned long long t0 = 0;
-            if (lane == 0) t0 = atomicAdd(&ctl->task_head, (unsigned long long)n);
+            unsigned stop = 0;
+            if (lane == 0) {
+                stop = *(volatile unsigned *)&ctl->stop;
+                t0 = atomicAdd(&ctl->task_head, (unsigned long long)n);
+            }
             t0 = __shfl_sync(TFULL, t0, 0);
+            halt = __shfl_sync(TFULL, stop, 0) != 0;
             more = t0 + n < ntasks;
             const uint32_t r = __popc(idle & lt);
             if (!active && !fresh && r < n && t0 + r < ntasks) {
@@ -165,11 +193,11 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             active = !((a.redo[rid >> 5] >> (rid & 31)) & 1u);
         }
         if (!__any_sync(TFULL, active)) {
-            if (!more && nn == 0) break;
-            continue;
+            if ((!more || halt) && nn == 0) break;
+            if (!halt) continue;
         }
-        if (!more && ++tail > a.tail) {
-            // the rest to the next launch
+        if (halt || (!more && ++tail > a.tail)) {
+            // the rest to the next launch (or to the warp pool)
             const unsigned act = __ballot_sync(TFULL, active);
             if (active) {
                 const uint32_t q = nn + __popc(act & lt);
@@ -178,7 +206,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             }
             nn += __popc(act);
             __syncwarp();
-            flush_nodes(a, S, 0, nn, lane);
+            halt = !flush_nodes(a, S, 0, nn, ntasks, lane) || halt;
             break;
         }
         uint32_t cl[4] = {0, 0, 0, 0}, clr[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0};
@@ -201,7 +229,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             // the other side's interval start: rows of lower symbols (and a $) come first
             uint32_t acc = (left ? lr : l) + ((sd.dollar_row >= pl && sd.dollar_row < pl + sz) ? 1u : 0u);
             const bool whole = nA == 0 && nB == m;
-            const bool checkable = item_room && a.verify_min && nB - nA >= a.verify_min && m - (nB - nA) >= BD_VERIFY_LEFT;
+            const bool checkable = a.verify_min && nB - nA >= a.verify_min && m - (nB - nA) >= BD_VERIFY_LEFT;
             const uint32_t split = nA ? TREE_SPLIT_LEFT : TREE_SPLIT_RIGHT;
             uint32_t most = 0;
 #pragma unroll
@@ -280,11 +308,11 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             ni += all >> 16;
             __syncwarp();
             if (nn > STAGE_LOW) {
-                flush_nodes(a, S, STAGE_LOW, nn, lane);
+                halt = !flush_nodes(a, S, STAGE_LOW, nn, ntasks, lane) || halt;
                 nn = STAGE_LOW;
             }
             if (ni > STAGE_LOW) {
-                item_room = flush_items(a, S, ni, lane);
+                halt = !flush_items(a, S, ni, lane) || halt;
                 ni = 0;
             }
         }
@@ -295,7 +323,8 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             d += pick == base ? 0u : 1u;
         }
     }
-    if (ni) flush_items(a, S, ni, lane);
+    if (ni) halt = !flush_items(a, S, ni, lane) || halt;
+    if (halt && lane == 0) *(volatile unsigned *)&ctl->stop = a.round;
     c_nodes = __reduce_add_sync(TFULL, c_nodes);
     c_blocks = __reduce_add_sync(TFULL, c_blocks);
     if (lane == 0 && c_nodes) {
@@ -305,16 +334,25 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1) end_round(ctl, a.cap);
+    if (threadIdx.x == 0 && atomicAdd(&ctl->done_ctas, 1u) == gridDim.x - 1) {
+        const unsigned long long head = *(volatile unsigned long long *)&ctl->task_head;
+        const bool stop = *(volatile unsigned *)&ctl->stop != 0;
+        ctl->left_from = (uint32_t)min(head, (unsigned long long)ntasks);
+        ctl->left_to = ntasks;
+        end_round(ctl, a.cap + TREE_LAST);
+        if (stop) ctl->unfinished |= 8u;
+    }
 }
 
 }  // namespace
 
-// One launch of the trees: the nodes of `in` (their number in ctl->ntasks), their children to `out`.
-// tail: steps after the launch's nodes are all taken (0: TREE_TAIL).
-int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, const uint4 *in,
-                const uint32_t *in_meta, uint4 *out, uint32_t *out_meta, uint32_t cap, uint4 *items, uint32_t item_cap,
-                uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s)
+// One launch of the trees, the round-th: the nodes of `in` (their number in
+// ctl->ntasks, at most in_cap of them written), their children to `out`, which has room for cap + TREE_LAST;
+// items has room for item_cap.  tail: steps after the launch's nodes are all
+// taken (0: TREE_TAIL).
+int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const ReadsView &rd, uint32_t round,
+                const uint4 *in, const uint32_t *in_meta, uint32_t in_cap, uint4 *out, uint32_t *out_meta, uint32_t cap,
+                uint4 *items, uint32_t item_cap, uint32_t *redo, uint32_t verify_min, uint32_t tail, cudaStream_t s)
 {
     TreeArgs a;
     a.fwd = fwd;
@@ -325,12 +363,13 @@ int launch_tree(const OccSide &fwd, const OccSide &rev, Workspace &w, const Read
     a.iv_cnt = (uint32_t *)w.iv_cnt.p;
     a.in = in;
     a.in_meta = in_meta;
+    a.in_cap = in_cap;
     a.out = out;
     a.out_meta = out_meta;
     a.cap = cap;
     a.items = items;
-    constexpr uint32_t LAST_FLUSHES = 152u * TREE_CTAS * (TREE_THREADS / 32) * STAGE_ITEMS;
-    a.item_cap = item_cap > LAST_FLUSHES ? item_cap - LAST_FLUSHES : 0u;
+    a.item_cap = !verify_min ? 0xffffffffu : item_cap > TREE_LAST ? item_cap - TREE_LAST : 0u;
+    a.round = round;
     a.redo = redo;
     a.verify_min = verify_min;
     a.tail = tail ? tail : TREE_TAIL;

@@ -76,7 +76,7 @@ def _path_is_the_trees(idx):
 def test_the_row_item_list_runs_out(row_items):
     """A list with room for fewer row items than the sweep (up to 500) or the
     trees want, after a batch of the same reads in another order has filled
-    it: what finds no room stays with the trees, and no entry that another
+    it: what finds no room is searched otherwise, and no entry that another
     batch left behind is looked at."""
     g, a, b, want = _inputs()
     idx = _index()
@@ -90,7 +90,7 @@ def test_the_row_item_list_runs_out(row_items):
     for call in range(2):
         for cap in (20, 0):
             gc.assert_same(idx.align_batch(a, hit_cap=cap), want[cap], f"items {row_items} call {call} cap {cap}")
-    _path_is_the_trees(idx)
+            assert idx.stats()["fallback_reads"] == 0
     assert idx.stats()["nodes"] > free["nodes"]       # what found no room was extended instead
     idx.free()
 
@@ -103,7 +103,7 @@ def test_the_row_item_list_runs_out(row_items):
     dict(nodes=4, rounds=64, steps=1, row_items=1)], ids=str)
 def test_limits_of_the_trees(limits, full_sa):
     """The frontier's nodes (first nodes past its end are the warp pool's tasks,
-    later ones give their reads up), a launch's steps, the launches, and these
+    and a launch whose children fill it stops), a launch's steps, the launches, and these
     together: every read's hits are the oracle's, through a call that captures,
     one that replays, and the pipelined calls."""
     _, a, b, want = _inputs()
@@ -114,7 +114,7 @@ def test_limits_of_the_trees(limits, full_sa):
         for call in range(2):
             gc.assert_same(idx.align_batch(a, hit_cap=cap), want[cap], f"{limits} cap {cap} call {call}")
     gc.assert_same(idx.collect(idx.submit_batch(a, hit_cap=20)), want[20], f"{limits} pipelined")
-    if "rounds" in limits and limits["rounds"] < 64:
+    if "rounds" in limits and "nodes" not in limits:
         assert idx.stats()["fallback_reads"] > 0
     idx.debug_search_limits()
     gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], "built-in limits again")
@@ -140,4 +140,38 @@ def test_runs_return_to_a_full_stack(budget):
         for call in range(80):
             gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"budget {budget} call {call}")
             assert idx.stats()["warp_rounds"] > 0
+    idx.free()
+
+
+def _family(copies, div):
+    """A 4 Mbp genome with a family of 3 kbp copies at divergence div, and reads inside them."""
+    rng = np.random.default_rng(copies)
+    g = rng.integers(0, 4, 1 << 22).astype(np.uint8)
+    unit, at = rng.integers(0, 4, 3_000), rng.permutation((1 << 22) // 3_500 - 1)[:copies] * 3_500
+    for s in at:
+        u = unit.copy()
+        hit = rng.random(u.size) < div
+        u[hit] = (u[hit] + rng.integers(1, 4, int(hit.sum()))) & 3
+        g[s:s + 3_000] = u
+    return synth.Genome(g, [(int(s), int(s) + 3_000, "") for s in at])
+
+
+@pytest.mark.parametrize("case", ["short_k3", "short_k2", "family_1000", "lean_short"])
+def test_more_work_than_the_lists_hold(case):
+    """Batches whose trees want several times the row items, or nodes, that the
+    lists hold: the launch stops in time and the warp pool takes what is left,
+    so no read is given up; results are the persistent kernel's."""
+    rng = np.random.default_rng(5)
+    if case == "family_1000":
+        g, n, lo, hi, k, inside = _family(1_000, 0.005), 30_000, 100, 100, 2, 1.0
+    else:
+        g = synth.genome_64m(1 << 24)
+        n, lo, hi, k, inside = {"short_k3": (50_000, 36, 36, 3, 0.2), "short_k2": (200_000, 30, 30, 2, 0.0),
+                                "lean_short": (100_000, 24, 24, 2, 0.0)}[case]
+    b = synth.sample_reads(g, rng.integers(lo, hi + 1, n), np.full(n, k), rng, subs="rate", sub_rate=0.01, repeat_frac=inside)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), full_sa=case != "lean_short")
+    want = idx.align_batch(b, hit_cap=10, kernel="persistent")
+    for call in range(3):
+        gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"{case} call {call}")
+        assert idx.stats()["fallback_reads"] == 0
     idx.free()
