@@ -33,6 +33,7 @@ namespace {
 constexpr unsigned SFULL = 0xffffffffu;
 constexpr int SWEEP_WARPS = 8;
 constexpr int SWEEP_CTAS = 4;     // per SM
+constexpr uint32_t ROWS_SMALL = 16;   // rows of an item that shares a warp's look with others
 constexpr int SWEEP_QUEUE = 64;   // intervals waiting: fewer than 32 left over (each has a row) plus 32 new ones
 
 struct SweepArgs {
@@ -436,61 +437,104 @@ __device__ __forceinline__ void item_windows(const SweepArgs &a, const uint32_t 
     }
 }
 
-// The item list, one item of one read per warp at a time: its rows stream by
-// 32 at a time, those whose left context passes are collected and checked
-// against the text 32 at a time, with the pattern in shared memory.  Intervals
-// of this size come from repeats, a few thousand reads of a batch: here they
-// spread over every warp of the GPU, where the sweep's own warps would each
-// be held by the few they drew.
+// One item of many rows: they stream by 32 at a time, those whose left context
+// passes are collected in st and checked against the text 32 at a time, with
+// the pattern in shared memory (pat).
+__device__ __forceinline__ void rows_of_item(const SweepArgs &a, const uint4 item, uint32_t *pat, uint32_t *st, int lane,
+                                             uint32_t &c_verify, uint32_t &c_vbytes, uint32_t &c_vsect)
+{
+    const uint32_t cnt = item.z & 511u, j = (item.z >> 9) & 3u, ex = (item.z >> 11) & 31u, k = (item.z >> 16) & 3u;
+    const uint32_t at = (item.z >> 18) & 511u, rem = (item.z >> 27) & 3u, rid = item.y >> 1, minus = item.y & 1u;
+    const uint32_t m = a.rd.len[rid];
+    const int wn = (int)((m + 15) >> 4);
+    const uint32_t *w = a.rd.words + a.rd.word_off[rid];
+    if (lane < (int)MAX_WORDS)
+        pat[lane] = minus ? rc_word(raw_word(w, wn - 1 - lane, wn), raw_word(w, wn - 2 - lane, wn), m)
+                          : raw_word(w, lane, wn);
+    __syncwarp();
+    uint32_t have = 0;
+    for (uint32_t r0 = 0; r0 < cnt; r0 += 32) {
+        bool stay = false;
+        uint32_t s = 0;
+        if (r0 + (uint32_t)lane < cnt) {
+            const uint2 x = __ldg(a.sa_ctx + item.x + r0 + (uint32_t)lane);
+            s = x.x - at;
+            uint32_t df = x.y ^ item.w;
+            df = (df | (df >> 1)) & 0x55555555u;
+            if (at < 16u) df &= at ? ~0u << (2u * (16u - at)) : 0u;
+            const bool exact = ex == 0 || (df >> (2u * (16u - ex))) == 0;
+            stay = x.x >= at && (uint64_t)s + m <= a.n && exact && __popc(df) <= rem;
+            c_vbytes += 8u;
+            c_vsect += (lane & 3) == 0;
+        }
+        const unsigned bal = __ballot_sync(SFULL, stay);
+        if (stay) st[have + __popc(bal & ((1u << lane) - 1u))] = s;
+        have += __popc(bal);
+        __syncwarp();
+        if (have >= 32u) {
+            item_windows(a, pat, st, 32u, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
+            have -= 32u;
+            const uint32_t rest = (uint32_t)lane < have ? st[32 + lane] : 0u;
+            __syncwarp();
+            if ((uint32_t)lane < have) st[lane] = rest;
+            __syncwarp();
+        }
+    }
+    if (have) item_windows(a, pat, st, have, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
+    __syncwarp();
+}
+
+// The item list.  Items of many rows come from repeats, a few thousand reads of
+// a batch: they spread over every warp of the GPU, one at a time, where the
+// sweep's own warps would each be held by the few they drew.  A tree's items
+// are mostly of a row or a few, and millions when its seeds are short: a warp
+// takes up to 32 of them and looks at the rows of several together, as the
+// sweep does.  (A warp for each of those too took 2.4 ms for 100k reads of 30
+// bp, k = 2, on a 16 Mbp genome, this way 0.65.)
 __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const SweepArgs a)
 {
     __shared__ uint32_t pat_s[SWEEP_WARPS][MAX_WORDS], start_s[SWEEP_WARPS][64];
+    __shared__ SweepQueue queues[SWEEP_WARPS];
     const uint32_t n_items = min(*(volatile unsigned *)&a.ctl->row_items, a.item_cap);
     if (n_items == 0 || *(volatile unsigned *)&a.ctl->error) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *pat = pat_s[warp], *st = start_s[warp];
+    const unsigned lt = (1u << lane) - 1u;
+    SweepQueue &Q = queues[warp];
     uint32_t c_verify = 0, c_vbytes = 0, c_vsect = 0;
-    for (uint32_t it = blockIdx.x * SWEEP_WARPS + warp; it < n_items; it += gridDim.x * SWEEP_WARPS) {
-        const uint4 item = __ldg(a.items + it);
-        const uint32_t cnt = item.z & 511u, j = (item.z >> 9) & 3u, ex = (item.z >> 11) & 31u, k = (item.z >> 16) & 3u;
-        const uint32_t at = (item.z >> 18) & 511u, rem = (item.z >> 27) & 3u, rid = item.y >> 1, minus = item.y & 1u;
-        const uint32_t m = a.rd.len[rid];
-        const int wn = (int)((m + 15) >> 4);
-        const uint32_t *w = a.rd.words + a.rd.word_off[rid];
-        if (lane < (int)MAX_WORDS)
-            pat[lane] = minus ? rc_word(raw_word(w, wn - 1 - lane, wn), raw_word(w, wn - 2 - lane, wn), m)
-                              : raw_word(w, lane, wn);
-        __syncwarp();
-        uint32_t have = 0;
-        for (uint32_t r0 = 0; r0 < cnt; r0 += 32) {
-            bool stay = false;
-            uint32_t s = 0;
-            if (r0 + (uint32_t)lane < cnt) {
-                const uint2 x = __ldg(a.sa_ctx + item.x + r0 + (uint32_t)lane);
-                s = x.x - at;
-                uint32_t df = x.y ^ item.w;
-                df = (df | (df >> 1)) & 0x55555555u;
-                if (at < 16u) df &= at ? ~0u << (2u * (16u - at)) : 0u;
-                const bool exact = ex == 0 || (df >> (2u * (16u - ex))) == 0;
-                stay = x.x >= at && (uint64_t)s + m <= a.n && exact && __popc(df) <= rem;
-                c_vbytes += 8u;
-                c_vsect += (lane & 3) == 0;
-            }
-            const unsigned bal = __ballot_sync(SFULL, stay);
-            if (stay) st[have + __popc(bal & ((1u << lane) - 1u))] = s;
-            have += __popc(bal);
-            __syncwarp();
-            if (have >= 32u) {
-                item_windows(a, pat, st, 32u, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
-                have -= 32u;
-                const uint32_t rest = (uint32_t)lane < have ? st[32 + lane] : 0u;
-                __syncwarp();
-                if ((uint32_t)lane < have) st[lane] = rest;
-                __syncwarp();
-            }
+    uint32_t top = 0, rows = 0, windows = 0;   // small items queued, their rows, windows queued
+    // (few items: one at a time, so that neighbours on the list, one repeat's, spread over the warps;
+    // with at least 1 / 8 / 32 turns a warp repeats_1m 1.26 / 1.19 / 1.18 ms, uneven_1m 2.11 / 2.07 / 1.99)
+    const uint32_t warps = gridDim.x * SWEEP_WARPS, per = max(1u, min(32u, n_items / (warps * 32u)));
+    for (uint64_t i0 = (uint64_t)(blockIdx.x * SWEEP_WARPS + warp) * per; i0 < n_items; i0 += (uint64_t)warps * per) {
+        uint4 item = make_uint4(0, 0, 0, 0);
+        const bool has = (uint32_t)lane < per && i0 + (uint32_t)lane < n_items;
+        if (has) item = __ldg(a.items + i0 + (uint32_t)lane);
+        const uint32_t cnt = item.z & 511u;
+        const bool small = has && cnt <= ROWS_SMALL;
+        for (unsigned big = __ballot_sync(SFULL, has && !small); big; big &= big - 1) {
+            const int src = __ffs(big) - 1;
+            rows_of_item(a, make_uint4(__shfl_sync(SFULL, item.x, src), __shfl_sync(SFULL, item.y, src),
+                                       __shfl_sync(SFULL, item.z, src), __shfl_sync(SFULL, item.w, src)),
+                         pat_s[warp], start_s[warp], lane, c_verify, c_vbytes, c_vsect);
         }
-        if (have) item_windows(a, pat, st, have, rid, minus, m, k, j, lane, c_verify, c_vbytes, c_vsect);
+        const unsigned bal = __ballot_sync(SFULL, small);
+        if (small) {
+            const uint32_t q = top + __popc(bal & lt);
+            Q.iv[q] = make_uint4(item.x, item.y, cnt | (((item.z >> 9) & 3u) << 16) | (((item.z >> 11) & 31u) << 18) |
+                                 (((item.z >> 27) & 3u) << 23), item.w);
+            Q.at[q] = (uint16_t)((item.z >> 18) & 511u);
+        }
+        top += __popc(bal);
+        rows += __reduce_add_sync(SFULL, small ? cnt : 0u);
         __syncwarp();
+        while (rows >= 32) {
+            sweep_rows(a, Q, top, rows, windows, lane, c_vbytes, c_vsect);
+            if (windows >= 32) sweep_windows(a, Q, windows, lane, c_verify, c_vbytes, c_vsect);
+        }
+    }
+    while (rows | windows) {
+        if (rows) sweep_rows(a, Q, top, rows, windows, lane, c_vbytes, c_vsect);
+        if (windows >= 32 || !rows) sweep_windows(a, Q, windows, lane, c_verify, c_vbytes, c_vsect);
     }
     c_verify = __reduce_add_sync(SFULL, c_verify);
     c_vbytes = __reduce_add_sync(SFULL, c_vbytes);

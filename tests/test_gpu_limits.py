@@ -175,3 +175,39 @@ def test_more_work_than_the_lists_hold(case):
         gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"{case} call {call}")
         assert idx.stats()["fallback_reads"] == 0
     idx.free()
+
+
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 31, 32, 33, 64, 65])
+def test_row_items_of_few_and_many_rows(rows):
+    """Row items at the size up to which several share a warp's look, at the
+    sweep's sizes, and mixed: families of `rows` and of half as many copies,
+    whose copies differ in few bases, some at the genome's very ends."""
+    rng = np.random.default_rng(rows)
+    parts, marks = [], []
+    for copies in (rows, max(1, rows // 2), rows):
+        unit = rng.integers(0, 4, 220)
+        for _ in range(copies):
+            u = unit.copy()
+            hit = rng.random(u.size) < 0.01
+            u[hit] = (u[hit] + rng.integers(1, 4, int(hit.sum()))) & 3
+            marks.append(sum(p.size for p in parts))
+            parts += [u, rng.integers(0, 4, int(rng.integers(0, 30)))]
+    g = np.concatenate(parts).astype(np.uint8)
+    reads, ks = [], []
+    for i in range(400):
+        m = int(rng.integers(24, 180))
+        a = min(int(marks[i % len(marks)] + rng.integers(0, 220 - min(m, 219))), g.size - m)
+        a = {0: 0, 1: g.size - m}.get(i, a)
+        r = g[a:a + m].copy()
+        hit = rng.random(m) < 0.01
+        r[hit] = (r[hit] + rng.integers(1, 4, int(hit.sum()))) & 3
+        reads.append(r if i % 2 else (3 - r)[::-1].copy())
+        ks.append(i % 4)
+    b = gc.batch_from_reads(reads, ks)
+    fm = oracle.FMIndex(g)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g), kmer_q=12, sa_sample=8)
+    for cap in (0, 5):
+        gc.assert_same(idx.align_batch(b, hit_cap=cap), fm.align(b, cap=cap), f"rows {rows} cap {cap}")
+        _path_is_the_trees(idx)
+    assert idx.stats()["verified"] > 0
+    idx.free()
