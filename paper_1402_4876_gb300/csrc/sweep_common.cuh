@@ -13,6 +13,14 @@ namespace mica {
 // uneven 1M reads 1.39 / 1.46 / 1.54 / 1.55 ms.
 constexpr uint32_t TREE_SPLIT_LEFT = 256;
 constexpr uint32_t TREE_SPLIT_RIGHT = 64;
+// ... above this many, in a launch whose lanes are all at work, only once an
+// eighth of the rows that the lane began with have dropped out: copies that do
+// not differ stay one interval to the end, where rows told apart are a leaf
+// each.  A launch of fewer nodes takes as long as its longest chain, which row
+// checks end.  100k reads of 100 bp inside 200 exact copies, cap 10 / cap 1000:
+// 2.52 / 2.59 -> 1.08 / 1.19 ms; uneven 1M reads 2.03 -> 1.79.  With the rule in
+// every launch the best of 100k x 250 bp took 0.97 ms instead of 0.87.
+constexpr uint32_t TREE_SPLIT_FEW = 64;
 
 // An item of rows to check is (row l, task, this word, the read's context): up
 // to 511 rows, scheme j, context bases in the exact piece, budget k, pattern

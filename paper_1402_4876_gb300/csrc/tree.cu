@@ -140,9 +140,11 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
     TreeStage &S = reinterpret_cast<TreeStage *>(tree_smem)[threadIdx.x >> 5];
     // nodes a warp takes at a time: no more than its part of the launch's
     const uint32_t share = max(1u, min(32u, ntasks / (gridDim.x * (TREE_THREADS / 32))));
+    // with at least half as many nodes as the launch has lanes (TREE_SPLIT_FEW's comment)
+    const uint32_t few = 2ull * ntasks >= (unsigned long long)gridDim.x * TREE_THREADS ? TREE_SPLIT_FEW : TREE_SPLIT_LEFT;
     bool active = false, more = true;
     bool halt = __shfl_sync(TFULL, lane == 0 ? *(volatile unsigned *)&ctl->row_items : 0u, 0) >= a.item_cap;   // the launch stops
-    uint32_t task = 0, l = 0, lr = 0, sz = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
+    uint32_t task = 0, l = 0, lr = 0, sz = 0, sz0 = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
     unsigned long long bounds = 0;
     const uint32_t *w = nullptr;
     uint32_t c_nodes = 0, c_blocks = 0, nn = 0, ni = 0, tail = 0;   // staged nodes, staged items
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
         }
         if (fresh) {
             task = it.x; l = it.y; lr = it.z; sz = it.w;
+            sz0 = sz;
             A = bm_a(meta); B = bm_b(meta); d = bm_d(meta); d0 = bm_d0(meta); j = bm_j(meta);
             const uint32_t rid = task >> 1;
             m = a.rd.len[rid];
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
                     clr[c] = left ? acc : start;
                     cs[c] = n_c;
                     if (whole) leafmask |= 1u << c;
-                    else if (checkable && n_c <= split) itemmask |= 1u << c;
+                    else if (checkable && n_c <= split && (n_c <= few || 8u * n_c <= 7u * sz0)) itemmask |= 1u << c;
                     else { nodemask |= 1u << c; most = max(most, n_c); }
                 }
                 acc += n_c;

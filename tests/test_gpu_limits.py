@@ -211,3 +211,23 @@ def test_row_items_of_few_and_many_rows(rows):
         _path_is_the_trees(idx)
     assert idx.stats()["verified"] > 0
     idx.free()
+
+
+@pytest.mark.parametrize("copies", [64, 65, 200, 256, 257])
+@pytest.mark.parametrize("n", [300, 30_000])
+def test_exact_copies_of_few_and_many_reads(copies, n):
+    """Reads inside exact copies: in a batch whose trees fill the GPU's lanes their
+    rows stay one interval (not a leaf each), in a small one they are told
+    apart; results are the persistent kernel's either way, under a cap and
+    without."""
+    g = _family(copies, 0.0)
+    rng = np.random.default_rng(n)
+    b = synth.sample_reads(g, np.full(n, 60), np.full(n, 2), rng, subs="rate", sub_rate=0.01, repeat_frac=1.0)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes))
+    for cap in (10, 0):
+        want = idx.align_batch(b, hit_cap=cap, kernel="persistent")
+        gc.assert_same(idx.align_batch(b, hit_cap=cap), want, f"cap {cap}")
+        _path_is_the_trees(idx)
+        if n == 30_000 and copies > 64:
+            assert idx.stats()["intervals"] < 8 * n
+    idx.free()
