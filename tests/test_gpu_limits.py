@@ -231,3 +231,28 @@ def test_exact_copies_of_few_and_many_reads(copies, n):
         if n == 30_000 and copies > 64:
             assert idx.stats()["intervals"] < 8 * n
     idx.free()
+
+
+@pytest.mark.parametrize("cap", [1, 9, 10, 31, 255, 256])
+def test_reads_over_their_cap_with_one_interval_or_a_few(cap):
+    """Reads over their cap whose lists hold one interval, as many as a warp's
+    lanes, and one more than that."""
+    rng = np.random.default_rng(cap)
+    parts, reads = [rng.integers(0, 4, 800)], []
+    for copies, variants in ((300, 1), (9, 31), (9, 32), (9, 33), (40, 64), (2, 65), (5, 3)):
+        unit = rng.integers(0, 4, 80)
+        reads.append(unit)
+        for v in range(variants):             # each its own interval: a base of its own, or none
+            u = unit.copy()
+            if v:
+                u[v % 80] = (u[v % 80] + 1 + v // 80) & 3
+            parts += [x for _ in range(copies) for x in (u, rng.integers(0, 4, 7))]
+    g = np.concatenate(parts).astype(np.uint8)
+    reads = [r.astype(np.uint8) for r in reads] + [(3 - r.astype(np.uint8))[::-1].copy() for r in reads]
+    fm = oracle.FMIndex(g)
+    for full_sa in (True, False):
+        idx = gc.mica().Index.build(synth.to_acgt_bytes(g), kmer_q=12, sa_sample=8, full_sa=full_sa)
+        for k in (0, 1):
+            b = gc.batch_from_reads(reads, [k] * len(reads))
+            gc.assert_same(idx.align_batch(b, hit_cap=cap), fm.align(b, cap=cap), f"cap {cap} k {k} full {full_sa}")
+        idx.free()
