@@ -29,8 +29,8 @@
 //
 // With the whole suffix array resident the seed sweep (sweep.cu) goes first and
 // the trees it leaves are tree.cu's; the kernel here searches whole tasks
-// where those cannot run (the check off or seeds too short for it), when a small
-// node budget is set, and for schemes that found no room among the nodes.
+// where those do not run (the check off, a small node budget), schemes that
+// found no room among the nodes, and what the trees leave when they stop early.
 //
 // The kernel is a persistent warp pool like k_persistent: each warp holds up
 // to 64 tasks in slots, and two node stacks in shared memory
@@ -1363,17 +1363,23 @@ static bool frontier_trees(const mica_index *idx)
     return idx->tuning.bidir_budget == 0 || idx->tuning.bidir_budget >= 1024;
 }
 
-// The sweep goes first when its task list (8 bytes for each of 2n tasks) fits
-// and its seeds can be checked.  Without the suffix array nothing is checked:
-// it then only turns every seed into a tree's first node (a chain of one row
-// at a time for most, which a lane of tree.cu follows in registers; the warp
-// pool took 0.81 ms for 50k x 100 bp reads on a 16 Mbp genome, 0.31 here).
+// The sweep goes first unless the text check is off (one row at a time for most
+// of a tree then).  Seeds too short to be checked (an index of a small kmer_q,
+// bidir_verify above the seeds' length) become trees, whose intervals are
+// checked once enough bases are matched: over 155 batches (100 to 300k reads,
+// kmer_q 6 to 11 on 0.1-1 Mbp, bidir_verify 16 to 100 on 64 Mbp) 0.80 of the warp
+// pool's time in the geometric mean, up to 1.19 of it on i.i.d. genomes of seeds
+// with a row each, down to 0.3 where they repeat; 300k x 150 bp with bidir_verify
+// 20 1.49 -> 0.73 ms.  Without the suffix array nothing is checked: every seed is then only
+// turned into a tree's first node (a chain of one row at a time for most, which
+// a lane of tree.cu follows in registers; the warp pool took 0.81 ms for 50k x
+// 100 bp reads on a 16 Mbp genome, 0.31 here).
 static bool use_sweep(const mica_index *idx, uint64_t n)
 {
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     if (n > 1ull << 27) return false;
     if (!idx->view.sa_ctx) return frontier_trees(idx);
-    return vmin < 256 && sweep_checks(idx, vmin);
+    return vmin < 256;
 }
 
 // After the sweep the trees grow from the frontier, a thread a node.

@@ -388,10 +388,6 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
                  int grid, cudaStream_t s);
 int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s);
 
-// sweep.cu
-bool sweep_checks(const mica_index *idx, uint32_t verify_min);
-
-
 // post.cu
 int run_post(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, uint32_t hit_cap,
              uint32_t report, cudaStream_t s, uint64_t *n_hits_out);

@@ -1,5 +1,6 @@
-// The seed sweep: the first pass of the bidirectional search (bidir.cu) when
-// the whole suffix array and the text are resident.
+// The seed sweep: the first pass of the bidirectional search (bidir.cu).  With
+// the whole suffix array and the text resident it also checks rows; without them
+// it only makes every seed the first node of a tree.
 //
 // Most schemes of most reads need no search tree: the exact piece's last q
 // bases come up empty in the seed table (a read's other strand, mostly) or
@@ -561,14 +562,6 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
 // kernels, uneven 1M reads 1.38 / 1.39 / 1.50 / 1.55 ms).
 constexpr uint32_t SWEEP_SPLIT = 32;
 constexpr uint32_t SWEEP_SPLIT_MAX = 64;
-
-// Are a seed's bases enough to check its rows against the text, at this verify
-// threshold (matched bases)?
-bool sweep_checks(const mica_index *idx, uint32_t verify_min)
-{
-    const uint32_t q = idx->view.lfwd.table ? idx->view.lfwd.q : idx->view.q;
-    return idx->view.sa_ctx && verify_min && verify_min <= q;
-}
 
 static void base_view(QmerView &q, const uint32_t *table, uint32_t len, uint32_t nshort, const uint32_t *pad,
                       const uint32_t *slen, unsigned long long bloom)

@@ -256,3 +256,29 @@ def test_reads_over_their_cap_with_one_interval_or_a_few(cap):
             b = gc.batch_from_reads(reads, [k] * len(reads))
             gc.assert_same(idx.align_batch(b, hit_cap=cap), fm.align(b, cap=cap), f"cap {cap} k {k} full {full_sa}")
         idx.free()
+
+
+@pytest.mark.parametrize("kmer_q", [1, 4, 8, 11])
+def test_seeds_too_short_to_be_checked(kmer_q):
+    """An index whose seeds are shorter than the text check asks for searches by
+    the sweep and the trees too: every interval is checked once enough bases
+    are matched."""
+    _, a, _, want = _inputs()
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(_inputs()[0]), kmer_q=kmer_q, sa_sample=8)
+    for cap in (20, 0):
+        gc.assert_same(idx.align_batch(a, hit_cap=cap), want[cap], f"q {kmer_q} cap {cap}")
+    assert idx.stats()["verified"] > 0
+    if kmer_q > 4:
+        _path_is_the_trees(idx)
+    idx.free()
+
+
+@pytest.mark.parametrize("verify", [1, 13, 20, 60, 255])
+def test_a_verify_threshold_past_the_seeds(verify):
+    """bidir_verify above the seeds' length leaves the sweep and the trees in place."""
+    _, a, _, want = _inputs()
+    idx = _index()
+    idx.set_tuning(bidir_verify=verify)
+    gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], f"verify {verify}")
+    _path_is_the_trees(idx)
+    idx.free()
