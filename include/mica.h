@@ -389,9 +389,12 @@ void mica_server_params_default(mica_server_params *p);
 /* Start the worker threads on idx's device.  params may be NULL (defaults). */
 int mica_server_start(mica_index *idx, const mica_server_params *params, mica_server **out);
 /* Device bytes a worker's workspace needs to run one tick of n_reads reads
-   held in n_words packed words (the staged batch, the search's buffers incl.
-   the persistent grid's overflow stacks, and the hit assembly's at 4 hits per
-   read): what admission charges against a worker's share. */
+   held in n_words packed words (the staged batch, the search's buffers, and the
+   hit assembly's at 4 hits per read): what admission charges against a
+   worker's share.  For the default kernel: the trees' nodes and row items
+   (some 500 bytes a read, at least 150 MB), the overflow stacks (1 GiB) and
+   what the persistent kernel needs for reads given up; a server with another
+   kernel is charged less, without the nodes and row items. */
 int mica_server_workspace_bytes(const mica_index *idx, uint64_t n_reads, uint64_t n_words, uint64_t *bytes);
 /* Queue a host batch (same layout as mica_align_batch; copied before return).
    MICA_EINVAL for a bad batch, MICA_ENOMEM if a worker's share of the budget

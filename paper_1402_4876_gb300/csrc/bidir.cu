@@ -61,6 +61,7 @@ namespace {
 
 constexpr unsigned BFULL = 0xffffffffu;
 constexpr uint32_t BD_DEEP_MIN = 8192;      // entries of each per-warp overflow stack, at least
+constexpr uint64_t BD_DEEP_BYTES = 1ull << 30;   // all of them, at most (unless the least is more)
 constexpr uint32_t BD_BUDGET = 1u << 12;    // node expansions a task may take before it exports its nodes
 constexpr int VCAP = 64;                    // intervals waiting for that check ...
 constexpr int TCAP = 64;                    // ... and windows of their rows that pass the first look
@@ -1303,7 +1304,7 @@ static uint32_t bidir_deep_cap(Workspace &w, uint64_t warps)
     if (w.bd_deep_cap == 0) {
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); fr = 0; }
-        uint64_t budget = std::min<uint64_t>(fr / 16, 1ull << 30);
+        uint64_t budget = std::min<uint64_t>(fr / 16, BD_DEEP_BYTES);
         uint64_t cap = budget / (warps * 32);
         w.bd_deep_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(cap, BD_DEEP_MIN), 1u << 20);
     }
@@ -1385,6 +1386,24 @@ static bool use_sweep(const mica_index *idx, uint64_t n)
 // After the sweep the trees grow from the frontier, a thread a node.
 static bool use_tree(const mica_index *idx, uint64_t n) { return use_sweep(idx, n) && frontier_trees(idx); }
 
+static uint64_t frontier_bytes(const mica_index *idx, uint64_t n)
+{
+    return (uint64_t)frontier_cap(idx, n) * (2 * 20) + (uint64_t)item_cap(idx, n) * 16 + std::max<uint64_t>(n, 1) * 16;
+}
+
+// Device bytes prepare_bidir reserves for n reads beside what the persistent
+// search's buffers take (search_workspace_bytes; the overflow stacks, `deep`
+// of those bytes, are one buffer for both kernels).
+int bidir_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t deep, uint64_t *bytes)
+{
+    BidirShape &sh = g_bd_shapes[bidir_shape_index(idx)];
+    int grid = 0;
+    if (int rc = bidir_grid(idx->device, sh, grid)) return rc;
+    const uint64_t mine = std::max<uint64_t>((uint64_t)grid * sh.warps * BD_DEEP_MIN * 32, BD_DEEP_BYTES);
+    *bytes = redo_bytes(n) + frontier_bytes(idx, n) + (mine > deep ? mine - deep : 0);
+    return 0;
+}
+
 // Reserve the bidirectional search's buffers for n reads; fills the control
 // block template and the grid.
 int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tmpl, int &grid)
@@ -1401,9 +1420,7 @@ int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tm
     // given-up reads: a bit per read, then a list of them and its length
     if ((rc = dev_reserve(w.redo, redo_bytes(n)))) return rc;
     // nodes: two rounds' buffers of (task, l, lr, sz) and meta; the sweep's row items and task list
-    if ((rc = dev_reserve(w.frontier, (uint64_t)frontier_cap(idx, n) * (2 * 20) + (uint64_t)item_cap(idx, n) * 16 +
-                                      std::max<uint64_t>(n, 1) * 16)))
-        return rc;
+    if ((rc = dev_reserve(w.frontier, frontier_bytes(idx, n)))) return rc;
     tmpl = SearchCtl{};
     tmpl.ntasks = use_sweep(idx, n) ? 0 : 2 * n;   // the sweep counts the tasks (or nodes) it leaves
     tmpl.iv_cap = w.iv_cap;

@@ -373,7 +373,7 @@ int enqueue_persistent(const mica_index *idx, Workspace &w, const ReadsView &rd,
                        const SearchCtl *pinned_tmpl, bool prune, bool prefetch, cudaStream_t s,
                        uint64_t &launches);
 int search_shape_info(int shape, int *scap, int *warps, int *minb);
-int search_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t *bytes);
+int search_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t *bytes, uint64_t *deep);
 
 // bidir.cu
 constexpr int BIDIR_FALLBACK = 2;   // run_search_bidir: an overflow stack filled; run the one-directional search
@@ -381,6 +381,7 @@ bool bidir_available(const mica_index *idx);
 int bidir_shape_index(const mica_index *idx);   // compiled bidirectional shape a call uses
 int bidir_shape_count();
 int prepare_bidir(const mica_index *idx, Workspace &w, uint64_t n, SearchCtl &tmpl, int &grid);
+int bidir_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t deep, uint64_t *bytes);
 constexpr int BIDIR_GROW = 3;       // finish_bidir: the interval buffer overflowed
 int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl &tmpl,
                         bool check, cudaStream_t s, uint64_t &launches);

@@ -1279,8 +1279,8 @@ int search_shape_count() { return N_SHAPES; }
 // only workspace buffers at their first-call sizes): per-read counters, the
 // interval buffer (4 per read + 65,536), lower-bound words, the spill ring
 // (a power of two >= max(n, 2^20) items) and the grid's per-warp overflow
-// stacks, which do not depend on n.
-int search_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t *bytes)
+// stacks, which do not depend on n (*deep: theirs alone).
+int search_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t *bytes, uint64_t *deep)
 {
     int shape = (idx->tuning.shape >= 0 && idx->tuning.shape < N_SHAPES) ? idx->tuning.shape : DEFAULT_SHAPE;
     int bps = 0;
@@ -1288,8 +1288,9 @@ int search_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t *bytes)
     uint64_t warps = (uint64_t)g_num_sms * bps * g_shapes[shape].warps;
     uint64_t iv_cap = std::min<uint64_t>(4 * n + 65536, 1ull << 30);
     uint64_t ring = ring_capacity(n);
+    *deep = warps * DEEP_CAP * 24;
     *bytes = sizeof(SearchCtl) + 64 + 4 * std::max<uint64_t>(n, 1) + iv_cap * sizeof(Interval) +
-             16 * std::max<uint64_t>(n, 1) + ring * (sizeof(WorkItem) + 4) + warps * DEEP_CAP * 24;
+             16 * std::max<uint64_t>(n, 1) + ring * (sizeof(WorkItem) + 4) + *deep;
     return 0;
 }
 

@@ -80,13 +80,19 @@ struct HostBuf {
 }  // namespace
 
 // Device bytes a worker's workspace takes to run one tick of n reads held in
-// nw packed words: the staged batch, the search's buffers and the post
-// pipeline's at the sizes the first call reserves (hits at 4 per read +
-// 65,536; a tick with more grows them).
-int tick_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t nw, uint64_t *bytes)
+// nw packed words: the staged batch, the search's buffers (of the bidirectional
+// search those of the persistent one too, which searches the reads it gives
+// up) and the post pipeline's at the sizes the first call reserves (hits at 4
+// per read + 65,536; a tick with more grows them).
+int tick_workspace_bytes(const mica_index *idx, int kernel, uint64_t n, uint64_t nw, uint64_t *bytes)
 {
-    uint64_t sb = 0;
-    if (int rc = search_workspace_bytes(idx, n, &sb)) return rc;
+    uint64_t sb = 0, deep = 0;
+    if (int rc = search_workspace_bytes(idx, n, &sb, &deep)) return rc;
+    if (kernel == MICA_KERNEL_BIDIRECTIONAL && bidir_available(idx)) {
+        uint64_t bb = 0;
+        if (int rc = bidir_workspace_bytes(idx, n, deep, &bb)) return rc;
+        sb += bb;
+    }
     uint64_t iv_cap = std::min<uint64_t>(4 * n + 65536, 1ull << 30);
     *bytes = std::max<uint64_t>(nw, 1) * 4 + (n + 1) * 8 + 3 * std::max<uint64_t>(n, 1) + sb +
              post_workspace_bytes(n, iv_cap, 4 * n + 65536);
@@ -231,7 +237,7 @@ void form_tick(mica_server *srv, std::vector<Chunk *> &tick, uint64_t &tick_byte
             Chunk &c = r->chunks[r->next_chunk];
             uint64_t nb = 0;
             if (!tick.empty() && reads + c.n > srv->p.max_tick_reads) { ++it; continue; }
-            if (tick_workspace_bytes(srv->idx, reads + c.n, words + c.nw, &nb) || nb > srv->share) {
+            if (tick_workspace_bytes(srv->idx, srv->p.kernel, reads + c.n, words + c.nw, &nb) || nb > srv->share) {
                 ++it;
                 continue;
             }
@@ -328,7 +334,7 @@ int mica_server_workspace_bytes(const mica_index *idx, uint64_t n_reads, uint64_
     if (!idx || !bytes) return MICA_EINVAL;
     DeviceGuard g(idx->device);
     MICA_CUDA_TRY(cudaSetDevice(idx->device));
-    return tick_workspace_bytes(idx, n_reads, n_words, bytes);
+    return tick_workspace_bytes(idx, MICA_KERNEL_BIDIRECTIONAL, n_reads, n_words, bytes);
 }
 
 int mica_server_start(mica_index *idx, const mica_server_params *params, mica_server **out)
@@ -371,7 +377,7 @@ int mica_server_submit(mica_server *srv, const uint32_t *packed_reads, const uin
     MICA_CUDA_TRY(cudaSetDevice(srv->idx->device));
     // a tick of one read must fit a worker's share, or the request could never run
     uint64_t one = 0;
-    if (int rc = tick_workspace_bytes(srv->idx, 1, MICA_MAX_READ_LEN / 16, &one)) return rc;
+    if (int rc = tick_workspace_bytes(srv->idx, srv->p.kernel, 1, MICA_MAX_READ_LEN / 16, &one)) return rc;
     if (one > srv->share) return MICA_ENOMEM;
     Request *r = new Request();
     uint64_t nw = word_offsets[n_reads] - word_offsets[0];
@@ -384,7 +390,7 @@ int mica_server_submit(mica_server *srv, const uint32_t *packed_reads, const uin
     // chunks: at most chunk_reads reads, and no more than a worker's share holds
     uint64_t cmax = std::max<uint64_t>(1, std::min<uint64_t>(srv->p.chunk_reads, srv->p.max_tick_reads));
     for (uint64_t b = 0; b == 0 || cmax > 1;) {
-        if (int rc = tick_workspace_bytes(srv->idx, cmax, cmax * (MICA_MAX_READ_LEN / 16), &b)) { delete r; return rc; }
+        if (int rc = tick_workspace_bytes(srv->idx, srv->p.kernel, cmax, cmax * (MICA_MAX_READ_LEN / 16), &b)) { delete r; return rc; }
         if (b <= srv->share) break;
         cmax /= 2;
     }

@@ -1,0 +1,51 @@
+"""Device memory that a call's workspace takes, against what the library reports,
+and what a workspace keeps between calls."""
+import numpy as np
+import pytest
+
+import synth
+from tests import gpu_common as gc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch", ["plain", "short"])
+def test_reported_workspace_covers_what_a_tick_reserves(batch):
+    """A worker's tick takes no more device memory than
+    mica_server_workspace_bytes reports for it, with the trees alone and with the
+    warp pool (short reads): measured on the device, with a granule per buffer."""
+    import torch
+    m = gc.mica()
+    g = synth.genome_64m(1 << 22)
+    rng = np.random.default_rng(3)
+    n, lens = 600_000, {"plain": 100, "short": 30}[batch]
+    b = synth.sample_reads(g, np.full(n, lens), np.full(n, 2), rng, subs="rate", sub_rate=0.01)
+    few = b.subset(np.arange(1_000))
+    idx = m.Index.build(synth.to_acgt_bytes(g.codes))
+    with m.Server(idx, workers=1, hit_cap=1) as srv:          # everything the process allocates once
+        srv.wait(srv.submit_batch(few))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    with m.Server(idx, workers=1, hit_cap=1, max_tick_reads=n, chunk_reads=n) as srv:
+        srv.wait(srv.submit_batch(b))
+        assert srv.stats()["ticks"] == 1
+        used = before - torch.cuda.mem_get_info()[0]
+        assert srv.stats()["device_bytes_in_use"] == m.Server.workspace_bytes(idx, n, int(b.word_off[-1]))
+    assert used <= m.Server.workspace_bytes(idx, n, int(b.word_off[-1])) + (64 << 20)
+    idx.free()
+
+
+def test_other_kernels_are_charged_for_their_own_buffers():
+    """A budget that holds the persistent kernel's tick but not the default
+    kernel's is enough for a server of the former."""
+    idx = gc.gpu_index("64m")
+    m = gc.mica()
+    b = synth.reads_64m(gc.genome("64m"), n=500)
+    share = m.Server.workspace_bytes(idx, 500, 500 * 16) - (100 << 20)
+    with m.Server(idx, workers=1, max_device_bytes=share) as srv:
+        with pytest.raises(m.MicaError) as e:
+            srv.submit_batch(b)
+        assert e.value.code == m.MICA_ENOMEM
+    with m.Server(idx, workers=1, max_device_bytes=share, kernel="persistent") as srv:
+        res, _ = srv.wait(srv.submit_batch(b))
+        gc.assert_same(res, idx.align_batch(b, hit_cap=1000))
