@@ -143,11 +143,17 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
     // with at least half as many nodes as the launch has lanes (TREE_SPLIT_FEW's comment)
     const uint32_t few = 2ull * ntasks >= (unsigned long long)gridDim.x * TREE_THREADS ? TREE_SPLIT_FEW : TREE_SPLIT_LEFT;
     bool active = false, more = true;
-    bool halt = __shfl_sync(TFULL, lane == 0 ? *(volatile unsigned *)&ctl->row_items : 0u, 0) >= a.item_cap;   // the launch stops
-    uint32_t task = 0, l = 0, lr = 0, sz = 0, sz0 = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
+    uint32_t task = 0, l = 0, lr = 0, sz = 0, lim = 0, A = 0, B = 0, d = 0, d0 = 0, j = 0, m = 0, k = 0;
     unsigned long long bounds = 0;
     const uint32_t *w = nullptr;
     uint32_t c_nodes = 0, c_blocks = 0, nn = 0, ni = 0, tail = 0;   // staged nodes, staged items
+    // the launch stops: no more nodes are taken, and the next step hands on what the warp has
+    const auto halt = [&]() {
+        more = false;
+        tail = 0x7fffffffu;
+        if (lane == 0) *(volatile unsigned *)&ctl->stop = a.round;
+    };
+    if (__shfl_sync(TFULL, lane == 0 ? *(volatile unsigned *)&ctl->row_items : 0u, 0) >= a.item_cap) halt();
     for (;;) {
         // idle lanes take staged nodes, then the launch's
         unsigned idle = __ballot_sync(TFULL, !active);
@@ -165,7 +171,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             idle = __ballot_sync(TFULL, !active && !fresh);
             __syncwarp();
         }
-        if (more && !halt && (idle == TFULL || __popc(idle) >= TREE_REFILL)) {
+        if (more && (idle == TFULL || __popc(idle) >= TREE_REFILL)) {
             const uint32_t n = min((uint32_t)__popc(idle), share);
             unsigned long long t0 = 0;
             unsigned stop = 0;
@@ -174,8 +180,8 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
                 t0 = atomicAdd(&ctl->task_head, (unsigned long long)n);
             }
             t0 = __shfl_sync(TFULL, t0, 0);
-            halt = __shfl_sync(TFULL, stop, 0) != 0;
             more = t0 + n < ntasks;
+            if (__shfl_sync(TFULL, stop, 0)) halt();
             const uint32_t r = __popc(idle & lt);
             if (!active && !fresh && r < n && t0 + r < ntasks) {
                 it = a.in[t0 + r];
@@ -185,7 +191,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
         }
         if (fresh) {
             task = it.x; l = it.y; lr = it.z; sz = it.w;
-            sz0 = sz;
+            lim = max(few, sz - (sz + 7u) / 8u);
             A = bm_a(meta); B = bm_b(meta); d = bm_d(meta); d0 = bm_d0(meta); j = bm_j(meta);
             const uint32_t rid = task >> 1;
             m = a.rd.len[rid];
@@ -196,10 +202,10 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             active = !((a.redo[rid >> 5] >> (rid & 31)) & 1u);
         }
         if (!__any_sync(TFULL, active)) {
-            if ((!more || halt) && nn == 0) break;
-            if (!halt) continue;
+            if (!more && nn == 0) break;
+            continue;
         }
-        if (halt || (!more && ++tail > a.tail)) {
+        if (!more && ++tail > a.tail) {
             // the rest to the next launch (or to the warp pool)
             const unsigned act = __ballot_sync(TFULL, active);
             if (active) {
@@ -209,7 +215,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             }
             nn += __popc(act);
             __syncwarp();
-            halt = !flush_nodes(a, S, 0, nn, ntasks, lane) || halt;
+            if (!flush_nodes(a, S, 0, nn, ntasks, lane)) halt();
             break;
         }
         uint32_t cl[4] = {0, 0, 0, 0}, clr[4] = {0, 0, 0, 0}, cs[4] = {0, 0, 0, 0};
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             uint32_t acc = (left ? lr : l) + ((sd.dollar_row >= pl && sd.dollar_row < pl + sz) ? 1u : 0u);
             const bool whole = nA == 0 && nB == m;
             const bool checkable = a.verify_min && nB - nA >= a.verify_min && m - (nB - nA) >= BD_VERIFY_LEFT;
-            const uint32_t split = nA ? TREE_SPLIT_LEFT : TREE_SPLIT_RIGHT;
+            const uint32_t split = nA ? min(TREE_SPLIT_LEFT, lim) : TREE_SPLIT_RIGHT;
             uint32_t most = 0;
 #pragma unroll
             for (uint32_t c = 0; c < 4; c++) {
@@ -244,7 +250,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
                     clr[c] = left ? acc : start;
                     cs[c] = n_c;
                     if (whole) leafmask |= 1u << c;
-                    else if (checkable && n_c <= split && (n_c <= few || 8u * n_c <= 7u * sz0)) itemmask |= 1u << c;
+                    else if (checkable && n_c <= split) itemmask |= 1u << c;
                     else { nodemask |= 1u << c; most = max(most, n_c); }
                 }
                 acc += n_c;
@@ -311,11 +317,11 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             ni += all >> 16;
             __syncwarp();
             if (nn > STAGE_LOW) {
-                halt = !flush_nodes(a, S, STAGE_LOW, nn, ntasks, lane) || halt;
+                if (!flush_nodes(a, S, STAGE_LOW, nn, ntasks, lane)) halt();
                 nn = STAGE_LOW;
             }
             if (ni > STAGE_LOW) {
-                halt = !flush_items(a, S, ni, lane) || halt;
+                if (!flush_items(a, S, ni, lane)) halt();
                 ni = 0;
             }
         }
@@ -326,8 +332,7 @@ __global__ void __launch_bounds__(TREE_THREADS, TREE_CTAS) k_tree(const TreeArgs
             d += pick == base ? 0u : 1u;
         }
     }
-    if (ni) halt = !flush_items(a, S, ni, lane) || halt;
-    if (halt && lane == 0) *(volatile unsigned *)&ctl->stop = a.round;
+    if (ni && !flush_items(a, S, ni, lane)) halt();
     c_nodes = __reduce_add_sync(TFULL, c_nodes);
     c_blocks = __reduce_add_sync(TFULL, c_blocks);
     if (lane == 0 && c_nodes) {
