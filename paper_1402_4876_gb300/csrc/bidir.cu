@@ -1600,6 +1600,22 @@ int redo_given_up(const mica_index *idx, Workspace &w, mica_stats &st, const Rea
     return run_search_list(idx, w, st, rd, list, nl, out.iv_count, idx->has_rev, s);
 }
 
+// Rounds that a captured batch of this workspace runs: what its last batches
+// needed, to a power of two.  A batch that needs more raises them at once; they
+// fall after ROUNDS_CALLS batches none of which did (a round with nothing to do
+// is two launches, and another number of them another capture).
+constexpr uint32_t ROUNDS_CALLS = 16;
+void settle_rounds(Workspace &w, uint32_t rounds_run)
+{
+    uint32_t need = 2;
+    while (need < rounds_run + 1 && need < BD_MAX_ROUNDS) need *= 2;
+    w.bd_seen = std::max(w.bd_seen, need);
+    if (need > w.bd_rounds || ++w.bd_calls >= ROUNDS_CALLS) {
+        w.bd_rounds = w.bd_seen;
+        w.bd_seen = w.bd_calls = 0;
+    }
+}
+
 // The rest of a search whose control block after `r - 1` rounds is `out`: the
 // rounds that are left, the reads it gave up on, and the call's counters.
 // Returns BIDIR_FALLBACK when the persistent search of those reads overflows a
@@ -1707,8 +1723,7 @@ int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const Read
     st.spills = out.spills;   // nodes exported to later rounds
     st.grid_ctas = (uint64_t)grid;
     w.bd_redo_seen = out.redo_reads > 0;
-    // rounds a captured batch of this workspace runs: what its batches needed so far, to a power of two
-    while (w.bd_rounds < (rows ? rounds_run : out.rounds_run) + 1 && w.bd_rounds < BD_MAX_ROUNDS) w.bd_rounds *= 2;
+    settle_rounds(w, rows ? rounds_run : out.rounds_run);
     if (out.redo_reads) {
         int rc = redo_given_up(idx, w, st, rd, out, s);
         if (rc) return rc;

@@ -398,6 +398,7 @@ static int align_graph_finish(const mica_index *idx, Workspace &w, mica_stats &s
         done = true;
         return 0;
     }
+    if (bidir) settle_rounds(w, out.rounds_run);
     if (nhits > w.hit_capacity) { w.hit_capacity = 2 * nhits; return 0; }
     if (out.n_huge) return 0;   // a read above the shared-memory sort size
     st.tasks = 2 * n;

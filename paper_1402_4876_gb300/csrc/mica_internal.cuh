@@ -219,7 +219,8 @@ struct Workspace {
     DevBuf frontier;                                      // bidirectional search: exported nodes, two rounds
     uint32_t iv_cap = 0, spill_cap = 0;
     uint32_t bd_deep_cap = 0;   // bidirectional search: entries of each warp's overflow stacks
-    uint32_t bd_rounds = 2;     // bidirectional search: frontier rounds of a captured batch
+    uint32_t bd_rounds = 2;     // bidirectional search: frontier rounds of a captured batch,
+    uint32_t bd_seen = 0, bd_calls = 0;   //   the most of the last calls, and how many those are
     bool bd_redo_seen = false;  // bidirectional search: the last call gave reads up (no graph replay then)
     uint64_t hit_cap_total = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};   // call timing
@@ -385,6 +386,7 @@ int bidir_workspace_bytes(const mica_index *idx, uint64_t n, uint64_t deep, uint
 constexpr int BIDIR_GROW = 3;       // finish_bidir: the interval buffer overflowed
 int enqueue_bidir_graph(const mica_index *idx, Workspace &w, const ReadsView &rd, int grid, const SearchCtl &tmpl,
                         bool check, cudaStream_t s, uint64_t &launches);
+void settle_rounds(Workspace &w, uint32_t rounds_run);
 int finish_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, SearchCtl &out, uint32_t r,
                  int grid, cudaStream_t s);
 int run_search_bidir(const mica_index *idx, Workspace &w, mica_stats &st, const ReadsView &rd, cudaStream_t s);

@@ -282,3 +282,25 @@ def test_a_verify_threshold_past_the_seeds(verify):
     gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], f"verify {verify}")
     _path_is_the_trees(idx)
     idx.free()
+
+
+def test_captured_rounds_fall_again_after_a_hard_batch():
+    """A batch that needs many rounds makes the workspace's captured batches hold as
+    many; batches that need few bring them down again."""
+    _, a, b, want = _inputs()
+    idx = _index()
+    easy = a.subset(np.arange(40))
+    fm = oracle.FMIndex(_inputs()[0]).align(easy, cap=20)
+    for _ in range(2):
+        gc.assert_same(idx.align_batch(easy, hit_cap=20), fm, "before")
+    few = idx.stats()["launches"]
+    idx.debug_search_limits(steps=1)
+    for _ in range(2):
+        gc.assert_same(idx.align_batch(a, hit_cap=20), want[20], "hard")
+    idx.debug_search_limits()
+    gc.assert_same(idx.align_batch(easy, hit_cap=20), fm, "after")
+    assert idx.stats()["launches"] > few
+    for _ in range(40):
+        gc.assert_same(idx.align_batch(easy, hit_cap=20), fm, "later")
+    assert idx.stats()["launches"] == few and idx.stats()["graph_replays"] == 1
+    idx.free()
