@@ -49,3 +49,40 @@ def test_other_kernels_are_charged_for_their_own_buffers():
     with m.Server(idx, workers=1, max_device_bytes=share, kernel="persistent") as srv:
         res, _ = srv.wait(srv.submit_batch(b))
         gc.assert_same(res, idx.align_batch(b, hit_cap=1000))
+
+
+@pytest.mark.parametrize("n", [16384 * 512, 16384 * 512 + 1, 16384 * 512 + 513])
+def test_batches_around_the_most_tiles_every_block_adds_up(n):
+    """The prefix sums of a batch of 8.4M reads, at the size from which a kernel
+    scans the tiles' sums: totals, offsets and hits are those of the same reads
+    in batches of a million."""
+    import torch
+    m = gc.mica()
+    g = synth.uniform_genome(1 << 16, 2)
+    idx = m.Index.build(synth.to_acgt_bytes(g.codes), kmer_q=8)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    dev = {"device": "cuda"}
+    at = torch.randint(0, g.n - 16, (n,), generator=gen, **dev)
+    codes = torch.from_numpy(g.codes).cuda().long()
+    words = torch.zeros(n, dtype=torch.int64, **dev)
+    for i in range(16):
+        words |= codes[at + i] << (2 * i)
+    words = torch.where(torch.rand(n, generator=gen, **dev) < 0.1, words ^ 7, words)   # some that do not occur
+    words = torch.where(words >= 1 << 31, words - (1 << 32), words).to(torch.int32)
+    off = torch.arange(n + 1, dtype=torch.int64, **dev)
+    lens, k = torch.full((n,), 16, dtype=torch.int16, **dev), torch.zeros(n, dtype=torch.uint8, **dev)
+    t, o, h = (x.clone() for x in idx.align_device(words, off, lens, k, n, hit_cap=3).tensors())
+    o, h = o.view(torch.int64), h.view(torch.int64)
+    assert int(o[0]) == 0 and int(o[-1]) == h.shape[0]
+    at0 = 0
+    for a in range(0, n, 1_000_000):
+        c = min(1_000_000, n - a)
+        ts, os_, hs = idx.align_device(words[a:a + c].clone(), off[:c + 1], lens[:c], k[:c], c, hit_cap=3).tensors()
+        hs = hs.view(torch.int64)
+        assert torch.equal(t[a:a + c], ts)
+        assert torch.equal(o[a:a + c + 1] - at0, os_.view(torch.int64))
+        assert torch.equal(h[at0:at0 + hs.shape[0]], hs)
+        at0 += int(hs.shape[0])
+    assert at0 == h.shape[0]
+    idx.free()
