@@ -186,7 +186,8 @@ typedef struct {
     uint64_t rev_table_bytes; /* the reversed genome's q-mer table (bidirectional search; 0 without it) */
     uint32_t full_sa;        /* 1 if the whole suffix array, its inverse and the 2-bit text are resident */
     uint64_t full_sa_bytes;  /* their size (0 without them); beside each suffix array entry the index
-                                also keeps 4 bytes of the text before it, not counted here */
+                                also keeps 4 bytes of the text before it, not counted here (see
+                                mica_index_device_bytes) */
     uint32_t long_q;         /* q of the longer seed tables of G$ and G~$ the bidirectional search
                                 seeds from (built from the text with full_sa when log4 N + 1 exceeds
                                 kmer_q; at most 15); 0 without them */
@@ -228,6 +229,10 @@ int mica_index_load(const char *path, int device, mica_index **out);
    collected finish first (their results are dropped).  NULL is a no-op. */
 void mica_index_free(mica_index *idx);
 int mica_index_get_info(const mica_index *idx, mica_index_info *info);
+/* Device memory the index's arrays hold, all of them (the left contexts beside
+   the suffix array too, which mica_index_info does not list), without the
+   workspaces of its calls. */
+int mica_index_device_bytes(const mica_index *idx, uint64_t *bytes);
 
 /*
  * Align a batch given in HOST memory: packed_reads holds 2-bit bases, 16 per

@@ -144,6 +144,7 @@ SIGNATURES = {
     "mica_tuning_shape_info": (_i32, [_i32, P, P, P]),
     "mica_set_tuning": (_i32, [P, P]),
     "mica_get_tuning": (_i32, [P, P]),
+    "mica_index_device_bytes": (_i32, [P, P]),
     "mica_set_wait_limits": (_i32, [P, _u32, _u32]),
     "mica_debug_set_search_limits": (_i32, [P, _u32, _u32, _u32, _u32]),
     "mica_autotune": (_i32, [P, P, P, P, P, _u64, _u32, _u32, P]),
@@ -361,6 +362,12 @@ class Index:
         d = {name: getattr(i, name) for name, _ in IndexInfo._fields_}
         d["C"] = list(i.C)
         return d
+
+    def device_bytes(self) -> int:
+        """Device memory the index's arrays hold (mica_index_device_bytes)."""
+        b = ctypes.c_uint64()
+        _check(_lib.mica_index_device_bytes(self._h, ctypes.byref(b)), "mica_index_device_bytes")
+        return int(b.value)
 
     def set_tuning(self, shape: int = -1, plain_block: int = 0, plain_budget: int = 0, plain_block_len=(0, 0, 0, 0),
                    prefetch: int = -1, bidir_budget: int = 0, bidir_verify: int = 0, bidir_shape: int = -1):

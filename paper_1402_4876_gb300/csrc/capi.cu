@@ -802,6 +802,16 @@ int mica_index_get_info(const mica_index *idx, mica_index_info *info)
     return 0;
 }
 
+int mica_index_device_bytes(const mica_index *idx, uint64_t *bytes)
+{
+    if (!idx || !bytes) return MICA_EINVAL;
+    const DevBuf *all[] = {&idx->occ, &idx->super, &idx->marks, &idx->samples, &idx->table, &idx->variants, &idx->rocc,
+                           &idx->rsuper, &idx->rtable, &idx->sa_ctx, &idx->isa, &idx->text, &idx->ltable, &idx->lrtable};
+    *bytes = 0;
+    for (const DevBuf *b : all) *bytes += b->bytes;
+    return 0;
+}
+
 int mica_get_stats(const mica_index *idx, mica_stats *out)
 {
     if (!idx || !out) return MICA_EINVAL;

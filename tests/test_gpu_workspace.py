@@ -86,3 +86,23 @@ def test_batches_around_the_most_tiles_every_block_adds_up(n):
         at0 += int(hs.shape[0])
     assert at0 == h.shape[0]
     idx.free()
+
+
+@pytest.mark.parametrize("full_sa", [True, False])
+def test_device_bytes_of_an_index(full_sa):
+    """Index.device_bytes() is what the index takes on the device (up to a granule
+    per array), the rows' left contexts included."""
+    import torch
+    m = gc.mica()
+    g = synth.uniform_genome(20_000_000, 6)
+    m.Index.build(synth.to_acgt_bytes(g.codes[:100_000])).free()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    idx = m.Index.build(synth.to_acgt_bytes(g.codes), full_sa=full_sa)
+    used = before - torch.cuda.mem_get_info()[0]
+    info = idx.info()
+    listed = sum(info[x] for x in ("occ_bytes", "mark_bytes", "sample_bytes", "table_bytes", "rev_occ_bytes", "rev_table_bytes",
+                                   "full_sa_bytes", "long_table_bytes"))
+    assert idx.device_bytes() >= listed + (4 * (g.n + 1) if full_sa else 0)
+    assert abs(used - idx.device_bytes()) <= 14 * (2 << 20)
+    idx.free()
