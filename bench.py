@@ -59,7 +59,7 @@ SEARCH_LABEL = {"bidirectional": "k + 1 pieces, one search per leftmost exact pi
                                  "reversed genome's index (same result as exhaustive backtracking)",
                 "persistent": "exhaustive backtracking from the read's end, pruned by mismatch lower bounds "
                               "(same result as unpruned)"}
-ALG_LABEL = {"bidirectional": "32 B x occurrence blocks read + 8 B x seeds (two entries of one table) + the packed "
+ALG_LABEL = {"bidirectional": "32 B x occurrence blocks read + 8 B x seed lookups (two entries of a table) + the packed "
                               "reads once + 16 B x leaf intervals + the bytes of the text checks (8 B of suffix "
                               "array entry and left context per row, the window's text words per row that passes)",
              "persistent": "32 B x occurrence blocks read (search and lower-bound pass) + 8 B x seeds + the "

@@ -138,7 +138,8 @@ typedef struct {
 /* Work counters of the last align call on an index. */
 typedef struct {
     uint64_t tasks;          /* (read, strand) search tasks = 2 * n_reads */
-    uint64_t seeds;          /* q-mer table lookups */
+    uint64_t seeds;          /* q-mer table lookups (two for a seed of the bidirectional search that is
+                                looked up in the reversed genome's table too) */
     uint64_t nodes;          /* backtracking nodes expanded (one interval extension each) */
     uint64_t rank_blocks;    /* 32-byte occurrence blocks read by the search (incl. lower bounds) */
     uint64_t intervals;      /* leaf SA intervals found */

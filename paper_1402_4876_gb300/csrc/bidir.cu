@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_bidir(BidirArgs a)
                         seed_interval_in(ix.rev.table, ix.q, ix.rev.nshort, ix.rev.short_pad, ix.rev.short_len,
                                          ix.rev.short_bloom, rcode, qe, rl, rr);
                     }
-                    c_seeds++;
+                    c_seeds += 2;   // (one lookup in each table)
                     if (fl < fr) {
                         l = fl; lr = rl; sz = fr - fl;
                         const uint32_t a0 = bj - qe;

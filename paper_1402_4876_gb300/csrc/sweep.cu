@@ -311,6 +311,7 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_sweep(const Sw
                         uint32_t lr, rr;
                         seed_interval_in(a.rseed.table, a.rseed.q, a.rseed.nshort, a.rseed.short_pad, a.rseed.short_len,
                                          a.rseed.short_bloom, rev_groups(cj) >> (2u * (16u - qj)), qj, lr, rr);
+                        c_seeds++;
                         const uint32_t bj = bnd(j + 1, m, p);
                         a.nodes[at] = make_uint4((uint32_t)t, lj, lr, sz);
                         a.node_meta[at] = bd_meta(0, bj - qj, bj, 0, 0, j);

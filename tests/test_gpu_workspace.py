@@ -106,3 +106,20 @@ def test_device_bytes_of_an_index(full_sa):
     assert idx.device_bytes() >= listed + (4 * (g.n + 1) if full_sa else 0)
     assert abs(used - idx.device_bytes()) <= 14 * (2 << 20)
     idx.free()
+
+
+def test_every_table_lookup_is_counted():
+    """stats()["seeds"]: a lookup per piece and strand, and another in the reversed
+    genome's table for each seed that becomes a tree (the sweep) or for all (the
+    warp pool)."""
+    g = synth.uniform_genome(50_000, 12)
+    rng = np.random.default_rng(1)
+    n = 1_000
+    b = synth.sample_reads(g, np.full(n, 60), np.full(n, 1), rng, subs="count", max_subs=0)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), kmer_q=10, sa_sample=8, full_sa=False)
+    idx.align_batch(b)
+    assert 4 * n + 2 * n <= idx.stats()["seeds"] <= 8 * n     # both pieces of the read's own strand occur
+    idx.set_tuning(bidir_budget=16)
+    idx.align_batch(b)
+    assert idx.stats()["seeds"] == 8 * n
+    idx.free()
