@@ -331,9 +331,10 @@ int mica_get_tuning(const mica_index *idx, mica_tuning *t);
    call starts afresh.  Small values exist to exercise that path. */
 int mica_set_wait_limits(mica_index *idx, uint32_t idle_rounds, uint32_t ring_spins);
 
-/* Autotuner: time every bidirectional kernel shape with node budgets of 1024
-   and 4096 (when the index has the reversed genome's table), every persistent
-   kernel shape and the plain kernel's block size (over the batch and per
+/* Autotuner: time every shape of the bidirectional search's warp pool with node
+   budgets of 4096 and 1024 (when the index has the reversed genome's table and
+   the pool takes part in the sample's search; else the built-in ones are kept),
+   every persistent kernel shape and the plain kernel's block size (over the batch and per
    read-length class, on that class's reads) on a host sample batch, `repeats`
    timed runs after one warm-up each, and keep the fastest in the index's
    tuning (also copied to *out unless NULL). */

@@ -41,9 +41,10 @@ struct DeviceBatch {
     ~DeviceBatch() { dev_release(words); dev_release(off); dev_release(len); dev_release(k); }
 };
 
-// best (minimum) search-kernel time of `repeats` runs after one warm-up
+// best (minimum) search-kernel time of `repeats` runs after one warm-up; *pool:
+// whether the bidirectional search's warp pool took part
 int time_search(mica_index *idx, Workspace &ws, const ReadsView &rd, int kernel, uint32_t hit_cap,
-                uint32_t repeats, float *best)
+                uint32_t repeats, float *best, bool *pool = nullptr)
 {
     mica_align_params p;
     mica_align_params_default(&p);
@@ -55,6 +56,7 @@ int time_search(mica_index *idx, Workspace &ws, const ReadsView &rd, int kernel,
         uint64_t nh = 0;
         if (int rc = align_on_device(idx, ws, st, rd, p, 0, &nh, false)) return rc;
         if (r > 0) *best = std::min(*best, st.kernel_ms);
+        if (pool) *pool = st.warp_rounds > 0;
     }
     return 0;
 }
@@ -94,17 +96,23 @@ int mica_autotune(mica_index *idx, const uint32_t *packed_reads, const uint64_t 
         DeviceBatch all;
         if ((rc = all.upload(packed_reads, word_offsets, lengths, k, n_reads))) goto done;
         float tbest = 1e30f;
-        // bidirectional shapes (task slots and warps per CTA) and node budgets
+        // the warp pool's shapes (task slots and warps per CTA) and node budgets, the built-in ones
+        // first: where the trees search the whole batch none of them reaches a kernel, and
+        // these stay
         if (bidir_available(idx)) {
-            const uint32_t budgets[] = {1024, 4096};
-            for (int s = 0; s < bidir_shape_count(); s++)
-                for (uint32_t b : budgets) {
+            idx->tuning.bidir_shape = -1;
+            const int s0 = bidir_shape_index(idx);
+            bool pool = true;
+            for (int i = 0; pool && i < bidir_shape_count(); i++)
+                for (uint32_t b : {4096u, 1024u}) {
+                    const int s = (s0 + i) % bidir_shape_count();
                     idx->tuning.bidir_shape = s;
                     idx->tuning.bidir_budget = b;
                     float t;
-                    if ((rc = time_search(idx, ws, all.view, MICA_KERNEL_BIDIRECTIONAL, hit_cap, repeats, &t)))
+                    if ((rc = time_search(idx, ws, all.view, MICA_KERNEL_BIDIRECTIONAL, hit_cap, repeats, &t, &pool)))
                         goto done;
                     if (t < tbest) { tbest = t; best.bidir_shape = s; best.bidir_budget = b; }
+                    if (!pool) break;
                 }
             idx->tuning.bidir_shape = best.bidir_shape;
             idx->tuning.bidir_budget = best.bidir_budget;

@@ -123,3 +123,22 @@ def test_every_table_lookup_is_counted():
     idx.align_batch(b)
     assert idx.stats()["seeds"] == 8 * n
     idx.free()
+
+
+def test_autotune_keeps_the_pools_defaults_where_the_trees_search():
+    """Where no shape or budget of the warp pool reaches a kernel the autotuner does
+    not choose among them, whatever was set before; where the pool searches
+    (an index whose text check is off) it does."""
+    g = synth.uniform_genome(200_000, 3)
+    rng = np.random.default_rng(8)
+    b = synth.sample_reads(g, np.full(2_000, 100), np.full(2_000, 2), rng, subs="rate", sub_rate=0.01)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes))
+    for shape in (0, 1):
+        idx.set_tuning(bidir_shape=shape, bidir_budget=1024)
+        for _ in range(3):
+            t = idx.autotune(b, repeats=1)
+            assert (t["bidir_shape"], t["bidir_budget"]) == (0, 4096)
+    idx.set_tuning(bidir_verify=256)
+    t = idx.autotune(b, repeats=1)
+    assert t["bidir_shape"] in (0, 1) and t["bidir_budget"] in (1024, 4096) and t["bidir_verify"] == 256
+    idx.free()
