@@ -178,13 +178,17 @@ int keep_open(DevBuf &tmp, const uint32_t *in, const uint8_t *flags, uint32_t *o
     return 0;
 }
 
+// The arrays of a suffix sort in a block for each time they live (the rounds'
+// come when the first sort's keys are gone): an allocation and its release
+// take as long as a small genome's kernels.
 struct DoublingBufs {
-    DevBuf k0, k1, v1, rank, open, count, tmp, key_a, key_b, pos_a, pos_b;
+    DevBuf keep, keys, pairs, tmp;
     ~DoublingBufs()
     {
-        for (DevBuf *b : {&k0, &k1, &v1, &rank, &open, &count, &tmp, &key_a, &key_b, &pos_a, &pos_b}) dev_release(*b);
+        for (DevBuf *b : {&keep, &keys, &pairs, &tmp}) dev_release(*b);
     }
 };
+uint64_t padded(uint64_t bytes) { return (bytes + 255) & ~255ull; }
 
 template <typename NumT>
 int doubling(const uint8_t *d_codes, uint64_t n, uint32_t *d_sa, cudaStream_t s)
@@ -192,19 +196,19 @@ int doubling(const uint8_t *d_codes, uint64_t n, uint32_t *d_sa, cudaStream_t s)
     const uint64_t rows = n + 1;
     DoublingBufs B;
     int rc = 0;
-    if ((rc = dev_reserve(B.k0, rows * 4)) || (rc = dev_reserve(B.k1, rows * 4)) || (rc = dev_reserve(B.v1, rows * 4)) ||
-        (rc = dev_reserve(B.rank, rows * 4)) || (rc = dev_reserve(B.open, rows)) || (rc = dev_reserve(B.count, 16)))
-        return rc;
-    uint32_t *rank = (uint32_t *)B.rank.p;
-    uint8_t *open = (uint8_t *)B.open.p;
-    uint64_t *d_count = (uint64_t *)B.count.p;
+    const uint64_t R4 = padded(rows * 4);
+    if ((rc = dev_reserve(B.keys, 2 * R4)) || (rc = dev_reserve(B.keep, 2 * R4 + 256 + rows))) return rc;
+    uint32_t *v1 = (uint32_t *)B.keep.p;
+    uint32_t *rank = (uint32_t *)((char *)B.keep.p + R4);
+    uint64_t *d_count = (uint64_t *)((char *)B.keep.p + 2 * R4);
+    uint8_t *open = (uint8_t *)B.keep.p + 2 * R4 + 256;
     int bits = 1;
     while ((1ull << bits) < rows + 1) bits++;          // rank + 1 <= rows fits in `bits`
     const int g = grid_for(rows);
 
     // by the first 16 bases
-    cub::DoubleBuffer<uint32_t> keys((uint32_t *)B.k0.p, (uint32_t *)B.k1.p);
-    cub::DoubleBuffer<uint32_t> vals(d_sa, (uint32_t *)B.v1.p);
+    cub::DoubleBuffer<uint32_t> keys((uint32_t *)B.keys.p, (uint32_t *)((char *)B.keys.p + R4));
+    cub::DoubleBuffer<uint32_t> vals(d_sa, v1);
     k_init_keys<<<g, 256, 0, s>>>(d_codes, n, std::min<uint64_t>(KEY_SYMS, rows), keys.Current(), vals.Current());
     if ((rc = sort_pairs<uint32_t, NumT>(B.tmp, keys, vals, (NumT)rows, 32, s))) return rc;
     if (vals.Current() != d_sa)
@@ -214,18 +218,17 @@ int doubling(const uint8_t *d_codes, uint64_t n, uint32_t *d_sa, cudaStream_t s)
     if ((rc = scan_in_place(B.tmp, hv, MaxOp(), (NumT)rows, s))) return rc;
     k_scatter_rank<<<g, 256, 0, s>>>(d_sa, hv, rows, rank);
     uint64_t m = 0;
-    if ((rc = keep_open<NumT>(B.tmp, d_sa, open, (uint32_t *)B.v1.p, d_count, (NumT)rows, m, s))) return rc;
+    if ((rc = keep_open<NumT>(B.tmp, d_sa, open, v1, d_count, (NumT)rows, m, s))) return rc;
+    const uint64_t M8 = padded(m * 8), M4 = padded(m * 4);
     if (m) {
-        dev_release(B.k0);
-        dev_release(B.k1);
-        if ((rc = dev_reserve(B.key_a, m * 8)) || (rc = dev_reserve(B.key_b, m * 8)) ||
-            (rc = dev_reserve(B.pos_a, m * 4)) || (rc = dev_reserve(B.pos_b, m * 4)))
-            return rc;
-        MICA_CUDA_TRY(cudaMemcpyAsync(B.pos_a.p, B.v1.p, m * 4, cudaMemcpyDeviceToDevice, s));
+        dev_release(B.keys);
+        if ((rc = dev_reserve(B.pairs, 2 * (M8 + M4)))) return rc;
     }
-    uint32_t *pos = (uint32_t *)B.pos_a.p, *other = (uint32_t *)B.pos_b.p;
+    uint64_t *key_a = (uint64_t *)B.pairs.p, *key_b = (uint64_t *)((char *)B.pairs.p + M8);
+    uint32_t *pos = (uint32_t *)((char *)B.pairs.p + 2 * M8), *other = (uint32_t *)((char *)B.pairs.p + 2 * M8 + M4);
+    if (m) MICA_CUDA_TRY(cudaMemcpyAsync(pos, v1, m * 4, cudaMemcpyDeviceToDevice, s));
     for (uint64_t h = KEY_SYMS; m; h *= 2) {
-        cub::DoubleBuffer<uint64_t> pk((uint64_t *)B.key_a.p, (uint64_t *)B.key_b.p);
+        cub::DoubleBuffer<uint64_t> pk(key_a, key_b);
         cub::DoubleBuffer<uint32_t> pv(pos, other);
         const int gm = grid_for(m);
         k_pair_keys<<<gm, 256, 0, s>>>(pos, rank, m, n, h, bits, pk.Current());
