@@ -303,10 +303,11 @@ typedef struct {
                                their own on every warp (bounds each round's tail; no effect on
                                results); 0 = 4096.  The pool runs instead of the trees' kernel when
                                this is 1 .. 1023, and where the trees cannot */
-    uint32_t bidir_verify;  /* bidirectional kernel with full_sa: an interval of one row whose matched
-                               part is at least this many bases (and which has at least 8 bases
-                               left to match) is checked against the genome's text in one step
-                               instead of being extended base by base; 0 = 12, 256 or more = never */
+    uint32_t bidir_verify;  /* bidirectional search with full_sa: the rows of a small interval (up to
+                               256 of them) whose matched part is at least this many bases (and which
+                               has at least 8 bases left to match) are checked against the genome's
+                               text one by one instead of extending the interval base by base; 0 = 12,
+                               256 or more = never (the warp pool then searches the batch) */
     int32_t bidir_shape;    /* bidirectional kernel shape: 0 = 64 task slots per warp, 6 warps per CTA
                                (fuller rounds when tasks are short); 1 = 32 slots, 8 warps (more warps
                                to hide HBM latency); -1 = automatic (0 when the occurrence blocks fit in
