@@ -22,7 +22,7 @@
 // reversed genome's table too, which only a tree's second interval needs.
 //
 // Measured on one GB300, search kernels of 1M x 150 bp reads, k = 2, on a 64
-// Mbp genome with repeats: 1.57 ms before, 0.87 ms now, 0.45 ms of it the sweep
+// Mbp genome with repeats: 1.57 ms before, 0.93 ms now, 0.49 ms of it the sweep
 // (6M seeds and 3M rows at 30 G random reads/s would take 0.3 ms).
 #include <algorithm>
 
@@ -559,8 +559,8 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_CTAS) k_rows(const Swe
 // Rows of an interval the sweep checks itself, and those it puts on the item
 // list.  Up to 32 are a warp's one look; past 64 a first extension in the trees
 // drops most rows of a repeat family for less than their checks cost (32 / 64 /
-// 128 / 256: 512 Mbp human-like 1M mates 3.57 / 3.57 / 3.58 / 4.00 ms of search
-// kernels, uneven 1M reads 1.38 / 1.39 / 1.50 / 1.55 ms).
+// 128 / 256, when k_rows gave each item a warp: 512 Mbp human-like 1M mates 3.57 /
+// 3.57 / 3.58 / 4.00 ms of search kernels, uneven 1M reads 1.38 / 1.39 / 1.50 / 1.55).
 constexpr uint32_t SWEEP_SPLIT = 32;
 constexpr uint32_t SWEEP_SPLIT_MAX = 64;
 

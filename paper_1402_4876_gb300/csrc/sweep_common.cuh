@@ -8,7 +8,8 @@ namespace mica {
 // Rows of a tree's interval that is checked row by row: while bases are left to
 // match on its left, which the rows' contexts are compared with, and after.
 // Each tree ends sooner the larger they are, each check is more work: search
-// kernels with 64, 16 / 128, 32 / 256, 64 / 400, 128 rows: 512 Mbp human-like 1M
+// kernels with 64, 16 / 128, 32 / 256, 64 / 400, 128 rows (in every launch, an item a
+// warp): 512 Mbp human-like 1M
 // mates 3.57 / 3.22 / 3.27 / 3.14 ms, 250 bp k = 3 0.54 / 0.51 / 0.45 / 0.47 ms,
 // uneven 1M reads 1.39 / 1.46 / 1.54 / 1.55 ms.
 constexpr uint32_t TREE_SPLIT_LEFT = 256;

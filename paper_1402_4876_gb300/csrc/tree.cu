@@ -22,16 +22,17 @@
 // 64 Mbp genome (now 4.8; the pool alone 3.9) and 21.2 ms for 100k reads of 100
 // bp in a family of 1,000 copies at 0.5% (now 9.7).
 //
-// What bounds it: the longest tree of a block.  Of 16.9 cycles between a warp's
-// issues 10.5 are at the barrier before the block's end, 1.4 on global loads (300k x
+// What bounds it: the longest tree of a block.  Of 17.3 cycles between a warp's
+// issues 10.5 are at the barrier before the block's end, 1.7 on global loads (300k x
 // 150 bp reads, 64 Mbp genome with repeats).  A step reads two occurrence blocks
 // (both loaded whole at once; L2 for a genome of up to some 150 Mbp) and does
 // integer work on them.  The warp pool spent 3,000-14,000 cycles a round on its
-// stacks and slots, with 1-5 of 32 lanes at work on these trees.  Measured,
-// search kernels with the pool / with this: 100k reads of 100-250 bp on a 32 Mbp
-// human-like genome 2.36 / 0.39 ms, 1M mates on a 512 Mbp one 5.8 / 3.3 ms, 100k x
-// 250 bp, k = 3 on 16 Mbp 0.53 / 0.45 ms, uneven 1M reads on 64 Mbp 1.56 / 1.54 ms.
-// TREE_TAIL 24 / 48 / 96 / 200: 0.64 / 0.57 / 0.51 / 0.49 ms for the first of these.
+// stacks and slots, with 1-5 of 32 lanes at work on these trees.  Search kernels
+// with the pool in this one's place when it came / now: 100k reads of 100-250 bp
+// on a 32 Mbp human-like genome 2.36 / 0.49 ms, 1M mates on a 512 Mbp one 5.8 /
+// 3.0 ms, 100k x 250 bp, k = 3 on 16 Mbp 0.53 / 0.54 ms, uneven 1M reads on 64 Mbp
+// 1.56 / 1.38 ms.  TREE_TAIL 24 / 48 / 96 / 200 now: 0.82 / 0.70 / 0.61 / 0.49 ms for
+// the first of these, 1.88 / 1.65 / 1.51 / 1.38 for the last.
 #include <algorithm>
 
 #include "sweep_common.cuh"
