@@ -302,7 +302,8 @@ typedef struct {
                                its pending nodes to the next launch round, where they are tasks of
                                their own on every warp (bounds each round's tail; no effect on
                                results); 0 = 4096.  The pool runs instead of the trees' kernel when
-                               this is 1 .. 1023, and where the trees cannot */
+                               this is 1 .. 1023, and where the trees do not; what the trees leave to
+                               it has 65536 at least */
     uint32_t bidir_verify;  /* bidirectional search with full_sa: the rows of a small interval (up to
                                256 of them) whose matched part is at least this many bases (and which
                                has at least 8 bases left to match) are checked against the genome's

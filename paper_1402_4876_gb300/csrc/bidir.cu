@@ -63,6 +63,11 @@ constexpr unsigned BFULL = 0xffffffffu;
 constexpr uint32_t BD_DEEP_MIN = 8192;      // entries of each per-warp overflow stack, at least
 constexpr uint64_t BD_DEEP_BYTES = 1ull << 30;   // all of them, at most (unless the least is more)
 constexpr uint32_t BD_BUDGET = 1u << 12;    // node expansions a task may take before it exports its nodes
+// ... of a batch that the trees began, at least: what they leave is work for every
+// warp for long, and handing nodes on only fills the frontier.  291k reads of 31
+// bp, k = 3, on a 32 Mbp genome with 4,096 / 16,384 / 65,536 / 10^6: 93.7 ms (7,087
+// reads given up) / 54.1 / 54.3 / 54.4; 231k of 24 bp on 29 Mbp 143 / 146 / 116 / 116.
+constexpr uint32_t BD_BUDGET_LEFT = 1u << 16;
 constexpr int VCAP = 64;                    // intervals waiting for that check ...
 constexpr int TCAP = 64;                    // ... and windows of their rows that pass the first look
 constexpr uint32_t BD_SPLIT_LEFT = 32;      // an interval of at most this many rows is checked row by row: while
@@ -1450,6 +1455,7 @@ static void bidir_args(const mica_index *idx, Workspace &w, const ReadsView &rd,
     ba.deep_s = (uint4 *)((char *)w.deep.p + (size_t)grid * sh.warps * w.bd_deep_cap * 16);
     ba.redo = (uint32_t *)w.redo.p;
     ba.budget = idx->tuning.bidir_budget ? idx->tuning.bidir_budget : BD_BUDGET;
+    if (use_tree(idx, rd.n)) ba.budget = std::max(ba.budget, BD_BUDGET_LEFT);
     ba.fr_cap = pool_room(idx, rd.n);
     const uint32_t vmin = idx->tuning.bidir_verify ? idx->tuning.bidir_verify : BD_VERIFY_MIN;
     ba.verify_min = (idx->view.sa_ctx && vmin < 256) ? vmin : 0u;

@@ -304,3 +304,20 @@ def test_captured_rounds_fall_again_after_a_hard_batch():
         gc.assert_same(idx.align_batch(easy, hit_cap=20), fm, "later")
     assert idx.stats()["launches"] == few and idx.stats()["graph_replays"] == 1
     idx.free()
+
+
+@pytest.mark.parametrize("full_sa", [True, False])
+def test_the_pool_gives_no_read_up_for_room(full_sa):
+    """Pieces of six and seven bases, k = 3: the trees stop almost at once, and the
+    warp pool searches nearly everything without handing on more nodes than the
+    frontier holds."""
+    g = synth.uniform_genome(600_000, 4)
+    rng = np.random.default_rng(13)
+    n = 205_000
+    b = synth.sample_reads(g, np.full(n, 25), np.full(n, 3), rng, subs="rate", sub_rate=0.01)
+    idx = gc.mica().Index.build(synth.to_acgt_bytes(g.codes), full_sa=full_sa)
+    want = idx.align_batch(b, hit_cap=10, kernel="persistent")
+    for call in range(2):
+        gc.assert_same(idx.align_batch(b, hit_cap=10), want, f"call {call}")
+        assert idx.stats()["warp_rounds"] > 0 and idx.stats()["fallback_reads"] == 0
+    idx.free()
